@@ -258,6 +258,13 @@ def kernel_model(kernel, lay, nsplit_bytes=0):
     p, d, g, G = lay.dout, lay.din, lay.g, lay.din // lay.g
     if kernel == "target":
         return dict(bound="tensor", work=2.0 * p * g * d, issued=4 * 2.0 * p * g * d)
+    # the sweep's blocks of 256 columns: the average launch of a sweep
+    launches = -(-d // 256)
+    if kernel == "sweep_product":
+        return dict(bound="tensor", work=2.0 * p * d * d / launches,
+                    issued=4 * 2.0 * p * d * d / launches)
+    if kernel == "sweep_babai":
+        return dict(bound="alu", work=1.0 * g * d * p / launches)
     if kernel == "hr_full":
         return dict(bound="tensor", work=2.0 * p * d * d, issued=6 * 2.0 * p * d * d)
     if kernel == "gram":

@@ -6,8 +6,8 @@
 // target-projection shortcut).  Per iteration k = 1..K: the Gram matrices of
 // the current codes and rhs_i = c_i^T P_i, the joint scale solve (gradient
 // rhs - Gram s, objective, early stop), and one Gauss-Seidel sweep over the
-// groups, each group being a target-product phase (T_i) followed by a Babai
-// phase on y = (Pt_i - T_i) / s_i.
+// groups in blocks of a few: the targets' products T_i of a block, then its
+// Babai steps on y = (Pt_i - T_i) / s_i.
 #include <float.h>
 #include <stdlib.h>
 #include <string.h>
@@ -163,8 +163,13 @@ cudaError_t ensure_ws(jarq_hessian *h, int p) {
     if ((e = dalloc(&w.r, (size_t)p * d)) != cudaSuccess) return e;
     if ((e = dalloc(&w.gram, (size_t)p * G * G)) != cudaSuccess) return e;
     if ((e = dalloc(&w.rhs, (size_t)p * G)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.t_hi, (size_t)kMaxSplit * p_pad * g)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.t_lo, (size_t)kMaxSplit * p_pad * g)) != cudaSuccess) return e;
+    // partials of a product: one slot of 256 columns (a block of the sweep) a
+    // row, or more slots while the CTAs of 128 rows x 64 columns fit the SMs
+    // (target_splits), for this row count and every smaller one
+    size_t t_len = (size_t)p_pad * 256;
+    if (t_len < (size_t)num_sms() * 128 * 64) t_len = (size_t)num_sms() * 128 * 64;
+    if ((e = dalloc(&w.t_hi, t_len)) != cudaSuccess) return e;
+    if ((e = dalloc(&w.t_lo, t_len)) != cudaSuccess) return e;
     if ((e = dalloc(&w.Pt_hi, (size_t)p * d)) != cudaSuccess) return e;
     if ((e = dalloc(&w.Pt_lo, (size_t)p * d)) != cudaSuccess) return e;
     if ((e = dalloc(&w.wexp, (size_t)p * G)) != cudaSuccess) return e;
@@ -184,23 +189,6 @@ cudaError_t ensure_ws(jarq_hessian *h, int p) {
     w.cap_rows = p;
     return cudaSuccess;
 }
-
-// Joins the first n extra streams of the sweep to `st` when it goes out of
-// scope: an error return in the middle of a sweep leaves no work of this
-// call running unordered with the caller's stream (best effort: the errors
-// of the join itself are dropped).
-struct ChainJoin {
-    jarq_hessian *h;
-    cudaStream_t st;
-    int n;
-    ~ChainJoin() {
-        if (n == 0) return;
-        for (int c = 0; c < n; ++c)
-            if (cudaEventRecord(h->ev_join[c], h->aux[c]) == cudaSuccess)
-                (void)cudaStreamWaitEvent(st, h->ev_join[c], 0);
-        (void)cudaGetLastError();
-    }
-};
 
 // Device views of the four layer arguments, staging host buffers.
 struct LayerArgs {
@@ -426,6 +414,7 @@ void jarq_hessian_destroy(jarq_hessian *h) {
     cudaFree(h->Hdig10);
     cudaFree(h->expo);
     cudaFree(h->Lf);
+    cudaFree(h->band);
     cudaFree(h->L64);
     cudaFree(h->Rinv);
     cudaFree(h->rdig);
@@ -437,11 +426,6 @@ void jarq_hessian_destroy(jarq_hessian *h) {
     cudaFree(h->qstage);
     cudaFree(h->dstatus);
     cudaFreeHost(h->hstatus);
-    if (h->ev_fork) cudaEventDestroy(h->ev_fork);
-    for (int c = 0; c < kMaxChains - 1; ++c) {
-        if (h->ev_join[c]) cudaEventDestroy(h->ev_join[c]);
-        if (h->aux[c]) cudaStreamDestroy(h->aux[c]);
-    }
     (void)cudaGetLastError();
     delete h;
 }
@@ -477,7 +461,7 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         if ((e = dalloc(&h->expo, (size_t)h->G * h->G)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_bf16(&h->mapD8, h->Hdig8, (uint64_t)6 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_f16(&h->mapD10, h->Hdig10, (uint64_t)4 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->Lf, (size_t)h->G * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        if ((e = dalloc(&h->Lf, (size_t)h->G * factor_floats(group_size))) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->L64, (size_t)h->G * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->Rinv, (size_t)h->G * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->rdig, (size_t)6 * din * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
@@ -487,6 +471,7 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         if ((e = cudaMemsetAsync(h->Htdig, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->expoT, (size_t)h->G * h->G)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_f16(&h->mapHt, h->Htdig, (uint64_t)4 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        if ((e = dalloc(&h->band, (size_t)h->G * (kMaxBlock - 1) * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->dstatus, 1)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = cudaMallocHost((void **)&h->hstatus, sizeof(int))) != cudaSuccess) { rc = cuda_fail(e); break; }
         const float *Hsrc = H;
@@ -508,6 +493,8 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         { ProfScope ps("htilde", st); e = launch_htilde(h->Hs, h->Rinv, Ht_hi, Ht_lo, din, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slice10(Ht_hi, Ht_lo, h->expoT, h->Htdig, din, h->d_pad, group_size, st); ps.done(); count_launches(2); }
+        if (e != cudaSuccess) { rc = cuda_fail(e); break; }
+        { ProfScope ps("slices", st); e = launch_band(h->Htdig, h->band, din, h->d_pad, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slices(h->Hs, h->expo, h->Hdig8, h->Hdig10, din, h->d_pad, group_size, st); ps.done(); count_launches(2); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
@@ -637,14 +624,14 @@ jarq_status jarq_multicode_probe(jarq_hessian *h, const float *W, const float *S
     if (rc != JARQ_OK) return rc;
     Workspace &w = h->ws;
     const int p = dout, d = h->din, g = h->g, G = h->G;
-    const int nsplit = target_splits(w.p_pad, g, G);
+    const int nsplit = target_splits(w.p_pad, g, G, 1);
     RUN("slice_rows", 1, launch_slice_rows(la.W, w.wdig, w.wexp, p, d, h->d_pad, w.p_pad, g, st));
     RUN("proj", 1, launch_tc_proj(w.mapWd, h->mapD8, w.Phi, w.Plo, w.wexp, h->expo, p, w.p_pad, d,
                                   h->d_pad, g, h->dstatus, st));
     // T = sum_h s_h H_ih c_h: the phase product with H's own digits
     RUN("target", 1, launch_tc_target(w.mapC, h->mapD10, w.t_hi, w.t_lo, la.S, h->expo, nullptr, p,
-                                      w.p_pad, h->d_pad, g, G, group, nsplit, 0, p, (1 << bits) - 1,
-                                      h->dstatus, st));
+                                      w.p_pad, h->d_pad, g, G, group, 1, 0, nsplit, (1 << bits) - 1, h->dstatus, st,
+                                      false));
     uint8_t *qo = reinterpret_cast<uint8_t *>(w.Hr);
     RUN("probe", 1, launch_probe(w.Phi, w.Plo, w.t_hi, w.t_lo, h->Hs, h->L64, la.S, la.Q, la.Z, qo,
                                  w.iters, w.accepted, w.ridge, w.L_final, p, w.p_pad, d, g, group,
@@ -692,27 +679,9 @@ jarq_status refine_impl(jarq_hessian *h, const float *W, float *S, uint8_t *Q, c
     const int p = dout, d = h->din, g = h->g, G = h->G, qmax = (1 << bits) - 1;
     RUN("init_rows", 1, launch_init_rows(w.active, w.iters, w.accepted, w.ridge, w.rstat, p, st));
     const ResidualView rv = rview(h);
-    const int nsplit = target_splits(w.p_pad, g, G);
-    // chains of the sweep: the row tiles split into nchain contiguous ranges
-    // only when one phase product needs more than one wave of CTAs (the
-    // chains then fill each other's last wave); otherwise a single chain
-    // with programmatic launches is faster.  Two chains: on the 14336-row
-    // layer three were 2 % faster and four slower.
-    const int tiles = (p + 127) / 128;
-    const int waves = (tiles * (g / 64) * nsplit + num_sms() - 1) / num_sms();
-    int nchain = (tiles >= kSweepSplitTiles && waves > 1) ? 2 : 1;
-    if (nchain > kMaxChains) nchain = kMaxChains;
-    if (nchain > tiles) nchain = tiles;
-    if (nchain < 1) nchain = 1;
-    int chain_row[kMaxChains + 1];
-    for (int c = 0; c <= nchain; ++c) chain_row[c] = c == nchain ? p : (tiles * c / nchain) * 128;
-    for (int c = 0; c < nchain - 1; ++c) {
-        if (!h->aux[c]) {
-            CK(cudaStreamCreateWithFlags(&h->aux[c], cudaStreamNonBlocking));
-            CK(cudaEventCreateWithFlags(&h->ev_join[c], cudaEventDisableTiming));
-        }
-        if (!h->ev_fork) CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-    }
+    // the sweep's blocks of groups, and the split of their products over K
+    const int nblk = G < sweep_block(g) ? G : sweep_block(g);
+    const int nsplit = target_splits(w.p_pad, g, G, nblk);
     // target projection P = W H, w^T H w and the folded Pt, once per call
     RUN("slice_rows", 1, launch_slice_rows(la.W, w.wdig, w.wexp, p, d, h->d_pad, w.p_pad, g, st));
     RUN("proj", 1, launch_tc_proj(w.mapWd, h->mapD8, w.Phi, w.Plo, w.wexp, h->expo, p, w.p_pad, d,
@@ -742,41 +711,16 @@ jarq_status refine_impl(jarq_hessian *h, const float *W, float *S, uint8_t *Q, c
         // The phase product reads the active flags only with the early stop
         // on (to skip tiles whose rows all stopped); a row marked numerical
         // by the scale solve is skipped by Babai, and its partials go unread.
-        // The sweep.  Rows are independent, so the row tiles may form several
-        // ranges, each with its own chain of phase products and Babai steps
-        // on its own stream: one chain's Babai step runs on the SMs that
-        // another chain's phase product leaves free, and each chain's launch
-        // gaps are filled by the others' work.  Programmatic launch only for
-        // a single chain: an early-launched grid waits on its SMs, which the
-        // other chains' kernels need.
-        const bool pdl = nchain == 1;
-        ChainJoin join{h, st, 0};
-        if (nchain > 1) {
-            CK(cudaEventRecord(h->ev_fork, st));
-            for (int c = 0; c < nchain - 1; ++c) {
-                CK(cudaStreamWaitEvent(h->aux[c], h->ev_fork, 0));
-                join.n = c + 1;
-            }
-        }
-        for (int i = 0; i < G; ++i) {
-            for (int c = 0; c < nchain; ++c) {
-                cudaStream_t sc = c == 0 ? st : h->aux[c - 1];
-                const int r0 = chain_row[c], r1 = chain_row[c + 1];
-                RUN_ON("target", 1, sc,
-                       launch_tc_target(w.mapC, h->mapHt, w.t_hi, w.t_lo, la.S, h->expoT,
-                                        o.early_stop ? w.active : nullptr, p, w.p_pad,
-                                        h->d_pad, g, G, i, nsplit, r0, r1 - r0, qmax,
-                                        h->dstatus, sc, pdl));
-                RUN_ON("babai", 1, sc,
-                       launch_babai(w.t_hi, w.t_lo, w.Pt_hi, w.Pt_lo, nsplit, h->Lf, la.S, la.Q,
-                                    la.Z, rv, w.active, w.accepted, h->dstatus, p, g, i, qmax,
-                                    o.eps, r0, r1, sc, pdl));
-            }
-        }
-        join.n = 0;
-        for (int c = 0; c < nchain - 1; ++c) {
-            CK(cudaEventRecord(h->ev_join[c], h->aux[c]));
-            CK(cudaStreamWaitEvent(st, h->ev_join[c], 0));
+        for (int i0 = 0; i0 < G; i0 += nblk) {
+            const int nb = G - i0 < nblk ? G - i0 : nblk;
+            RUN("sweep_product", 1,
+                launch_tc_target(w.mapC, h->mapHt, w.t_hi, w.t_lo, la.S, h->expoT,
+                                 o.early_stop ? w.active : nullptr, p, w.p_pad, h->d_pad, g, G, i0,
+                                 nb, i0 ? nblk : 0, nsplit, qmax, h->dstatus, st, true));
+            RUN("sweep_babai", 1,
+                launch_babai(w.t_hi, w.t_lo, w.Pt_hi, w.Pt_lo, nsplit, h->Lf, h->band, h->expoT,
+                             la.S, la.Q, la.Z, rv, w.active, w.accepted, h->dstatus, p, g, i0, nb,
+                             qmax, o.eps, st));
         }
     }
     // objective of the returned state (and of the input state when K = 0)

@@ -23,11 +23,34 @@ enum : int {
 };
 
 constexpr int kMaxGroups = 128;    // largest supported G for the scale solve
-constexpr int kSweepSplitTiles = 8;   // row tiles from which the sweep may run as several chains
-constexpr int kMaxChains = 4;         // chains of the sweep at most
 constexpr int kMaxSplit = 16;      // largest split-K factor of the phase product
+constexpr int kMaxBlock = 4;       // groups of one block of the sweep at most
+
+// Groups of one block of the sweep for group size g: 256 columns.  The Babai
+// kernel holds the factors of two groups and the blocks Ht_i'i of one group i
+// in shared memory, which for g = 128 leaves room for one such block.  Two
+// groups of 128 in one launch take 58.9 us of product and 27.6 us of Babai
+// steps on 4096 x 4096, a launch per group 2 x 34.7 and 2 x 18.8 us.
+__host__ __device__ constexpr int sweep_block(int g) { return 256 / g; }
 
 __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
+
+// Layout of one group's factor L_i = R_i^T as the Babai kernel reads it
+// (k_babai.cu), float32.  Eight lanes hold a row's g coordinates: lane k of
+// them owns l = 32 a + 4 k + b, a = 0 .. g/32 - 1, b = 0 .. 3 (a quad per a).
+//   rows   h = 0 .. g - 1: h/32 + 1 vectors a of 32 floats, entry (4 k + b)
+//          L[h][32 a + 4 k + b], zero from column 4 (h/4) on (h's own quad
+//          and everything above the diagonal)
+//   tri    per quad 4 q .. 4 q + 3 eight floats: L[3][2], L[3][1], L[3][0],
+//          L[2][1], L[2][0], L[1][0] of the quad's own block, 0, 0
+//   diag   L[l][l];  rdiag  1 / L[l][l]
+__host__ __device__ constexpr int factor_row(int h) {
+    return 512 * (h / 32) * (h / 32 + 1) + (h % 32) * 32 * (h / 32 + 1);
+}
+__host__ __device__ constexpr int factor_tri(int g) { return 512 * (g / 32) * (g / 32 + 1); }
+__host__ __device__ constexpr int factor_diag(int g) { return factor_tri(g) + 2 * g; }
+__host__ __device__ constexpr int factor_rdiag(int g) { return factor_tri(g) + 3 * g; }
+__host__ __device__ constexpr int factor_floats(int g) { return factor_tri(g) + 4 * g; }
 
 // View of the residual r = w - D_s (q - z): float32 [p][d] plus its exact
 // three-plane bf16 split [3][p_pad][d_pad] read by the tensor cores, and the
@@ -72,8 +95,8 @@ struct Workspace {
     float *r = nullptr;          // [p][d]  residual r = w - D_s (q - z)
     float2 *gram = nullptr;      // [p][G][G]  Gram matrices of the current codes (float pairs)
     double *rhs = nullptr;       // [p][G]  rhs_i = c_i^T P_i (also the scratch of grad)
-    float *t_hi = nullptr;       // [nsplit][p_pad][g]  split-K partials of the phase
-    float *t_lo = nullptr;       //   product T_i (double-float)
+    float *t_hi = nullptr;       // [nsplit][p_pad][nb g]  split-K partials of the phase
+    float *t_lo = nullptr;       //   product of nb groups (double-float)
     __nv_bfloat16 *rplanes = nullptr;  // [3][p_pad][d_pad] bf16 split of r
     __half *cplane = nullptr;          // [p_pad][d_pad] codes c = q - z
     CUtensorMap mapR;            // tensor map of rplanes, 128 x 64 boxes
@@ -121,7 +144,11 @@ struct jarq_hessian {
     int *expo = nullptr;          // [G][G] block exponents of the digits
     CUtensorMap mapH128, mapH64;  // tensor maps of Hplanes, 128 x 64 and 64 x 64 boxes
     CUtensorMap mapD8, mapD10;    // tensor maps of Hdig8 / Hdig10, 64 x 64 boxes
-    float *Lf = nullptr;          // [G][g][g] lower factor L_i = R_i^T, row-major
+    float *Lf = nullptr;          // [G][factor_floats(g)] lower factor L_i = R_i^T, packed
+    // digits of the blocks Ht_{i'i}, i' = i + 1 .. i + kMaxBlock - 1, column by
+    // column: [G][kMaxBlock - 1][g columns of i][g rows of i'], each entry the
+    // two 20-bit halves (a_0 2^10 + a_1, a_2 2^10 + a_3) of its digits
+    int2 *band = nullptr;
     double *L64 = nullptr;        // [G][g][g] the same in float64
     double *Rinv = nullptr;       // [G][g][g] R_i^{-1} (upper), row-major, float64
     // R_i^{-1} in six base-2^8 digit planes, transposed per block (row i g + a,
@@ -141,10 +168,6 @@ struct jarq_hessian {
     CUtensorMap mapQ;                  // tensor map of qdig, 64 x 64 boxes
     int *dstatus = nullptr;       // device status word
     int *hstatus = nullptr;       // pinned host mirror
-    // extra streams of the sweep's chains and their fork / join events
-    // (made on first use)
-    cudaStream_t aux[jarq::kMaxChains - 1] = {};
-    cudaEvent_t ev_fork = nullptr, ev_join[jarq::kMaxChains - 1] = {};
     jarq::Workspace ws;
 };
 
@@ -208,28 +231,29 @@ cudaError_t launch_scale_solve(const float2 *gram, const double *rhs, const doub
                                int *iters, int *ridge, int *rstat, int *status, int p, int d,
                                int g, int k, bool eval_only, const jarq_options &o,
                                cudaStream_t s);
-cudaError_t launch_babai(const float *t_hi, const float *t_lo, const float *pt_hi,
-                         const float *pt_lo, int nsplit, const float *Lf, const float *S,
-                         uint8_t *Q, const int32_t *Z, ResidualView rv, const int *active,
-                         int *accepted, int *status, int p, int g, int i, int qmax, float eps, int row0, int row1,
-                         cudaStream_t s, bool pdl = true);
+cudaError_t launch_babai(float *t_hi, float *t_lo, const float *pt_hi,
+                         const float *pt_lo, int nsplit, const float *Lf, const int2 *band,
+                         const int *expoT, const float *S, uint8_t *Q, const int32_t *Z,
+                         ResidualView rv, const int *active, int *accepted, int *status, int p,
+                         int g, int i0, int nb, int qmax, float eps, cudaStream_t s);
+cudaError_t launch_band(const __half *Htdig, int2 *band, int d, int d_pad, int g, cudaStream_t s);
 cudaError_t launch_slice_rinv(const double *Rinv, __nv_bfloat16 *rdig, int *rexp, int d, int g,
                               cudaStream_t s);
 cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, const float *Phi,
                           const float *Plo, __nv_bfloat16 *pdig, int *pexp, const int *rexp,
                           float *out_hi, float *out_lo, int p, int p_pad, int d, int d_pad, int g,
                           int *status, cudaStream_t s);
-int target_splits(int p_pad, int g, int G);
+int target_splits(int p_pad, int g, int G, int nb);
 cudaError_t launch_wait_timeout(int *status, uint32_t polls, cudaStream_t s);
 cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, float *out_hi,
                              float *out_lo, const float *S, const int *expoT, const int *active,
-                             int p, int p_pad, int d_pad, int g, int G, int i, int nsplit,
-                             int row0, int nrows, int qmax, int *status, cudaStream_t s,
-                             bool pdl = true);
+                             int p, int p_pad, int d_pad, int g, int G, int i0, int nb,
+                             int nb_prev, int nsplit, int qmax, int *status, cudaStream_t s,
+                             bool pdl);
 
-// Launch with programmatic stream serialization: the kernel may start while
-// the previous kernel in the stream finishes; it must call griddepcontrol.wait
-// before touching that kernel's inputs or outputs.
+// Launch; with `pdl` under programmatic stream serialization: the kernel may
+// start while the previous kernel in the stream finishes, and must call
+// griddepcontrol.wait before touching that kernel's inputs or outputs.
 template <class... KArgs, class... Args>
 cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                      bool pdl, Args &&...args) {

@@ -7,7 +7,8 @@
 // factor of H_ii (equal to the QR factor up to row signs, to which the
 // Babai recursion is invariant).  The factor and its inverse are computed in
 // float64 in shared memory:
-//   Lf[i]   = L_i = R_i^T          (lower, row-major: Lf[l][m] = R_i[m][l]), float32
+//   Lf[i]   = L_i = R_i^T          (lower, L[l][m] = R_i[m][l]), float32, packed for the
+//             Babai kernel (factor_row in jarq_internal.cuh)
 //   Rinv[i] = R_i^{-1}             (upper, row-major), float64
 // The Babai target of Eq. babai_update needs y = R_i^{-T} (H r)_i / s.  The
 // rows H_i of group i are dominated by the low-rank part of H, which R_i^{-T}
@@ -95,12 +96,24 @@ __global__ void group_factor_kernel(const float *__restrict__ Hs, float *__restr
         if (tid == 0) atomicOr(status, ST_NOT_SPD);
         return;
     }
-    float *Lo = Lf + (size_t)grp * g * g;
+    float *Lo = Lf + (size_t)grp * factor_floats(g);
     double *Ld = L64 + (size_t)grp * g * g;
     for (int idx = tid; idx < g * g; idx += nt) {
-        int a = idx / g, b = idx % g;
-        Lo[idx] = (b <= a) ? (float)A[a * ld + b] : 0.f;
-        Ld[idx] = (b <= a) ? A[a * ld + b] : 0.0;
+        const int h = idx / g, l = idx % g;
+        Ld[idx] = (l <= h) ? A[h * ld + l] : 0.0;
+        if (l < 32 * (h / 32 + 1))
+            Lo[factor_row(h) + l] = (l < 4 * (h / 4)) ? (float)A[h * ld + l] : 0.f;
+    }
+    for (int idx = tid; idx < 2 * g; idx += nt) {
+        const int q = 4 * (idx / 8), e = idx % 8;
+        const int h = e < 3 ? 3 : e < 5 ? 2 : 1;                       // 3 3 3 2 2 1
+        const int l = e < 3 ? 2 - e : e < 5 ? 4 - e : 0;               // 2 1 0 1 0 0
+        Lo[factor_tri(g) + idx] = e < 6 ? (float)A[(q + h) * ld + q + l] : 0.f;
+    }
+    for (int l = tid; l < g; l += nt) {
+        const float v = (float)A[l * ld + l];
+        Lo[factor_diag(g) + l] = v;
+        Lo[factor_rdiag(g) + l] = 1.0f / v;
     }
     __syncthreads();
     // in-place inverse of the lower factor, columns from last to first:
@@ -185,7 +198,36 @@ __global__ void __launch_bounds__(256) htilde_kernel(const float *__restrict__ H
     }
 }
 
+// The band of Ht blocks below the diagonal that the Babai kernel reads column
+// by column (jarq_hessian::band), from Ht's digit planes [4][d_pad][d_pad]:
+// one 32 x 32 tile of one block per CTA, transposed in shared memory.
+__global__ void band_kernel(const __half *__restrict__ dig, int2 *__restrict__ band, int d,
+                            int d_pad, int g) {
+    __shared__ int2 tile[32][33];
+    const int G = d / g, i = blockIdx.y, dd = blockIdx.z, i2 = i + 1 + dd;
+    if (i2 >= G) return;
+    const int nt = g / 32, m0 = (blockIdx.x / nt) * 32, k0 = (blockIdx.x % nt) * 32;
+    const size_t plane = (size_t)d_pad * d_pad;
+    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+    for (int y = ty; y < 32; y += 8) {
+        const size_t off = (size_t)(i2 * g + m0 + y) * d_pad + i * g + k0 + tx;
+        int a[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) a[t] = __half2int_rn(dig[t * plane + off]);
+        tile[y][tx] = make_int2(a[0] * 1024 + a[1], a[2] * 1024 + a[3]);
+    }
+    __syncthreads();
+    int2 *out = band + ((size_t)i * (kMaxBlock - 1) + dd) * g * g;
+    for (int y = ty; y < 32; y += 8) out[(size_t)(k0 + y) * g + m0 + tx] = tile[tx][y];
+}
+
 }  // namespace
+
+cudaError_t launch_band(const __half *Htdig, int2 *band, int d, int d_pad, int g, cudaStream_t s) {
+    band_kernel<<<dim3((g / 32) * (g / 32), d / g, kMaxBlock - 1), dim3(32, 8), 0, s>>>(
+        Htdig, band, d, d_pad, g);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_symmetrize(const float *H, float *Hs, __nv_bfloat16 *Hplanes, int d, int d_pad,
                               float nu2, cudaStream_t s) {

@@ -46,13 +46,14 @@ constexpr int kDrainWarps = 16;
 constexpr int kThreads = 32 * (2 + kDrainWarps);
 
 struct TargetArgs {
-    float *out_hi, *out_lo;   // [nsplit][p_pad][g]
+    float *out_hi, *out_lo;   // [nsplit][p_pad][nb g]
     const float *S;           // [p][G]
     const int *expoT;         // [G][G] block exponents of Ht
     const int *active;        // optional: rows still refined
     int *status;
-    int p, p_pad, d_pad, g, G, i, seg_per_split;
-    int row0;                 // first row of this launch's tiles (a multiple of 128)
+    int p, p_pad, d_pad, g, G, seg_per_split;
+    int i0, nb;               // groups i0 .. i0 + nb - 1 of this launch
+    int prev0;                // groups prev0 .. i0 - 1: the previous grid rewrites their codes
     float round_c;            // 1.5 * 2^(23 - k): rounds to multiples of 2^-k
 };
 
@@ -71,8 +72,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 4);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j0 = a.row0 + blockIdx.x * 128;
-    const int m0 = a.i * a.g + blockIdx.y * 64;          // first row of Ht (output column)
+    const int j0 = blockIdx.x * 128;
+    const int m0 = a.i0 * a.g + blockIdx.y * 64;         // first row of Ht (output column)
     const int h0 = blockIdx.z * a.seg_per_split;
     const int h1 = min(a.G, h0 + a.seg_per_split);
     const int nkc = a.g / 64;
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the previous grid finishes.  With the early stop every thread waits
     // here, before reading the flags; so it does in the first phase, whose
     // previous grid is the scale solve that writes the scales.
-    const bool early = !a.active && a.i > 0;
+    const bool early = !a.active && a.i0 > 0;
     if (!early) tc::pdl_wait();
     // The next grid (Babai of group i) is released at once: before its own
     // wait it reads nothing that this grid or the previous one writes.
@@ -142,8 +143,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
             }
             const int kx = h0 * a.g + c * 64;
-            if (!waited && h0 + c / nkc == a.i - 1) {
-                tc::pdl_wait();   // the codes of group i - 1
+            const int h = h0 + c / nkc;
+            if (!waited && h >= a.prev0 && h < a.i0) {
+                tc::pdl_wait();   // the codes of the previous block
                 waited = true;
             }
             tc::mbar_expect_tx(full(s), kStage);
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         bool ok = true;
         const float *srow = a.S + (size_t)min(row, a.p - 1) * a.G;
-        const int *erow = a.expoT + (size_t)a.i * a.G;
+        const int *erow = a.expoT + (size_t)(m0 / a.g) * a.G;
         float s_next = nseg > 0 ? srow[h0] : 0.f;
         int e_next = nseg > 0 ? erow[h0] : 0;
         for (int u = 0; u < nseg; ++u) {
@@ -260,7 +262,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         // the previous grid reads the partials this drain overwrites
         if (early) tc::pdl_wait();
         if (ok && row < a.p) {
-            const size_t o = (size_t)blockIdx.z * a.p_pad * a.g + (size_t)row * a.g + blockIdx.y * 64 + cq * 16;
+            const size_t ncol = (size_t)a.nb * a.g;
+            const size_t o = ((size_t)blockIdx.z * a.p_pad + row) * ncol + blockIdx.y * 64 + cq * 16;
 #pragma unroll
             for (int e = 0; e < 16; e += 4) {
                 float x[4], y[4];
@@ -283,9 +286,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace
 
-// Split of the K range (groups) over CTAs so that the launch covers the SMs.
-int target_splits(int p_pad, int g, int G) {
-    const int tiles = (p_pad / 128) * (g / 64);
+// Split of the K range (groups) over CTAs so that a launch of nb groups covers
+// the SMs.
+int target_splits(int p_pad, int g, int G, int nb) {
+    const int tiles = (p_pad / 128) * (nb * g / 64);
     int n = num_sms() / tiles;
     if (n < 1) n = 1;
     if (n > kMaxSplit) n = kMaxSplit;
@@ -295,16 +299,14 @@ int target_splits(int p_pad, int g, int G) {
 
 cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, float *out_hi,
                              float *out_lo, const float *S, const int *expoT, const int *active,
-                             int p, int p_pad, int d_pad, int g, int G, int i, int nsplit,
-                             int row0, int nrows, int qmax, int *status, cudaStream_t s,
+                             int p, int p_pad, int d_pad, int g, int G, int i0, int nb,
+                             int nb_prev, int nsplit, int qmax, int *status, cudaStream_t s,
                              bool pdl) {
     static std::atomic<unsigned long long> attr_done{0};
     const cudaError_t e = set_max_dynamic_smem((const void *)tc_target_kernel, kSmem, attr_done);
     if (e != cudaSuccess) return e;
     const int per = (G + nsplit - 1) / nsplit;
-    if (row0 % 128 != 0 || nrows < 0 || row0 + nrows > p_pad) return cudaErrorInvalidValue;
-    const int tiles = (nrows + 127) / 128;
-    if (tiles == 0) return cudaSuccess;
+    const int tiles = (p + 127) / 128;
     // quantum 2^-k of the exact digit split: the largest k with
     // 128 qmax 512 + 2^14 <= 2^(24-k)
     if (qmax < 1 || qmax > 255 || g > 128) return cudaErrorInvalidValue;
@@ -312,9 +314,10 @@ cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, f
     int kq = 0;
     while (kq < 7 && bound <= std::ldexp(1.0, 24 - (kq + 1))) ++kq;
     const float round_c = (float)std::ldexp(1.5, 23 - kq);
-    TargetArgs a{out_hi, out_lo, S, expoT, active, status, p, p_pad, d_pad, g, G, i, per,
-                 row0, round_c};
-    dim3 grid(tiles, g / 64, nsplit);
+    if (nb < 1 || i0 + nb > G || nsplit < 1) return cudaErrorInvalidValue;
+    TargetArgs a{out_hi, out_lo, S, expoT, active, status, p, p_pad, d_pad, g, G, per,
+                 i0, nb, i0 - nb_prev, round_c};
+    dim3 grid(tiles, nb * g / 64, nsplit);
     return launch_k(tc_target_kernel, grid, dim3(kThreads), (size_t)kSmem, s, pdl, mapC, mapT, a);
 }
 

@@ -77,6 +77,26 @@ def test_shapes_parity(jarq, din, dout, g, bits, K):
     assert Q.min() >= 0 and Q.max() <= (1 << bits) - 1
 
 
+@pytest.mark.parametrize("din,dout,g,bits,K", [
+    (384, 1, 128, 3, 2),      # one row; three groups: a block of two and one of one
+    (384, 5, 128, 4, 3),      # a second warp with one row; widest codes summed in 32 bits
+    (320, 7, 64, 4, 3),       # five groups of 64: a block of four and one of one
+    (320, 133, 64, 5, 2),     # a second row tile; digit sums in 64 bits
+    (640, 67, 128, 5, 3),     # the same for groups of 128, three blocks
+])
+def test_sweep_block_edges(jarq, din, dout, g, bits, K):
+    """The sweep's blocks of 256 columns: accepted changes carried to the later
+    groups of a block, short last blocks, partial warps of rows."""
+    lay = small_layer(din, dout, g, bits, K=K, seed=3 * din + dout)
+    prep, res = oracle_run(lay, K, False)
+    S, Q, st = gpu_refine(lay, K)
+    assert st["status"] == 0
+    m = compare_final(lay, prep, res, S, Q, st)
+    assert m["codes_same"] >= CODES_SAME, m
+    assert m["S_rel_max_same_rows"] <= REL_S and m["F_rel_max_same_rows"] <= REL_F, m
+    assert np.array_equal(st["accepted"], res.accepted)
+
+
 def _many_group_layer(din, dout, g, bits, K, seed):
     """A layer with the small-layer recipe whose Hessian is accumulated on
     the GPU (torch generators), returned as NumPy arrays for the oracle."""
