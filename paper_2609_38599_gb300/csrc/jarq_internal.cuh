@@ -29,8 +29,9 @@ constexpr int kMaxBlock = 4;       // groups of one block of the sweep at most
 // Groups of one block of the sweep for group size g: 256 columns.  The Babai
 // kernel holds the factors of two groups and the blocks Ht_i'i of one group i
 // in shared memory, which for g = 128 leaves room for one such block.  Two
-// groups of 128 in one launch take 58.9 us of product and 27.6 us of Babai
-// steps on 4096 x 4096, a launch per group 2 x 34.7 and 2 x 18.8 us.
+// groups of 128 in one launch take 36.7 us of product and 27.6 us of Babai
+// steps on 4096 x 4096; with a launch per group the start of each launch
+// (about 8 us of a product, 4 us of a Babai step) is paid twice.
 __host__ __device__ constexpr int sweep_block(int g) { return 256 / g; }
 
 __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }

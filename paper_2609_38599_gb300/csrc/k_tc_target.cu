@@ -19,14 +19,30 @@
 // Pt_i - T_i, where the low-rank parts of H cancel, loses none of the
 // precision float32 would.
 //
-// One CTA: 128 rows x 64 columns of group i over the groups of one K split.
-//   warp 0       TMA producer: codes tile + its share of the digit tiles
-//   warp 1       TMEM allocation and the single-thread MMA issuer
+// A pair of CTAs (cta_group::2): 256 rows x 64 columns of the block's groups
+// over the groups of one K split.  Per 64-wide K chunk each CTA loads the
+// codes of its own 128 rows and two of the four digit planes, so that an M256
+// x N256 MMA (four planes of 64 columns) reads half of its B from each CTA.
+//   warp 0       TMA producer of its CTA's tiles, onto the even CTA's barriers
+//   warp 1       TMEM allocation; in the even CTA the single-thread MMA issuer
 //   warps 2..17  drain: warp w reads TMEM lanes 32 (w % 4) and 16 columns
 // Four 64-column accumulators per group h, double-buffered (512 columns).
-// The drain does 17 float32 operations per output and group, hence
-// sixteen drain warps; the scale and block exponent of the next group are
-// loaded one group ahead.
+// The drain does 17 float32 operations per output and group (two outputs per
+// instruction), hence sixteen drain warps.
+//
+// What bounds it, per group and CTA (4096 rows, g = 128, clock64 in a copy):
+// about 1560 cycles, of which the MMAs are 1024, the drain's arithmetic 1088
+// at the full float32 rate, and the tile loads and operand reads 128 KB of
+// shared-memory traffic.  Two accumulators keep MMA and drain of consecutive
+// groups overlapped, but a group's MMAs start only when all 32 drain warps
+// have read the accumulator two groups back.  Per launch of two groups (256
+// columns, K = 4096, CUDA events): 36.7 us.  One CTA per tile took 58.9 us
+// (192 KB of shared-memory traffic per group, and an issuing thread that
+// needed 800 cycles per group beside the drain's arithmetic).  Measured and
+// not kept: all digit sums read and the accumulator released before any
+// arithmetic (39.1 us: the four warps of a scheduler drift apart by a whole
+// group), a block barrier among the drain warps per group (39.1 us), one
+// polling lane per warp (37.3 us).
 #include <cmath>
 
 #include "tc_common.cuh"
@@ -36,12 +52,17 @@ namespace {
 
 constexpr int kTileA = 128 * 64 * 2;   // codes: 128 rows x 64 K, fp16
 constexpr int kTileB = 64 * 64 * 2;    // one digit plane: 64 rows of Ht x 64 K
-constexpr int kStage = kTileA + 4 * kTileB;
-constexpr int kStages = 4;
-constexpr int kSmem = 1024 + kStages * kStage + 256;
+constexpr int kStage = kTileA + 2 * kTileB;
+constexpr int kStages = 5;
+constexpr int kSRow = 129;             // pitch (floats) of a group's scales: 128 rows, conflict-free
+// stages, barriers, and per group of the K split the scales and an exponent
+constexpr int smem_bytes(int groups) {
+    return 1024 + kStages * kStage + 256 + groups * (kSRow + 1) * 4;
+}
 // one MMA covers the four digit planes: they are consecutive 64-row tiles
-// in shared memory, and their accumulators consecutive 64-column blocks
-constexpr uint32_t kIdesc = tc::idesc_f16_f32(128, 256);
+// in the two CTAs' shared memory, and their accumulators consecutive
+// 64-column blocks
+constexpr uint32_t kIdesc = tc::idesc_f16_f32(256, 256);
 constexpr int kDrainWarps = 16;
 constexpr int kThreads = 32 * (2 + kDrainWarps);
 
@@ -63,7 +84,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = (a - (s - bb)) + (b - bb);
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_target_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapT,
                      TargetArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -71,8 +92,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint64_t *bars = (uint64_t *)(smem + kStages * kStage);
     uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 4);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+    float *sS = (float *)(smem + kStages * kStage + 256);    // [seg_per_split][kSRow]
+    int *sE = (int *)(sS + a.seg_per_split * kSRow);         // [seg_per_split]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j0 = blockIdx.x * 128;
+    const uint32_t rank = tc::cluster_rank();
+    const int j0 = blockIdx.x * 128, jp = j0 - 128 * (int)rank;   // rows of this CTA, of the pair
     const int m0 = a.i0 * a.g + blockIdx.y * 64;         // first row of Ht (output column)
     const int h0 = blockIdx.z * a.seg_per_split;
     const int h1 = min(a.G, h0 + a.seg_per_split);
@@ -87,19 +111,19 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            tc::mbar_init(full(s), 1);
+            tc::mbar_init(full(s), 1);      // the even CTA's: bytes of both CTAs
             tc::mbar_init(empty(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(afull(b), 1);
-            tc::mbar_init(aempty(b), kDrainWarps);
+            tc::mbar_init(aempty(b), 2 * kDrainWarps);   // the even CTA's: both drains
         }
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
     if (warp == 1) {
-        tc::tmem_alloc(tc::smem_u32(tmem_slot), 512);
-        tc::tmem_relinquish();
+        tc::tmem_alloc_pair(tc::smem_u32(tmem_slot), 512);
+        tc::tmem_relinquish_pair();
     }
     if (warp == 0 && lane == 0) {
         tc::prefetch_tmap(&mapC);
@@ -107,117 +131,158 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     tc::tc_fence_before();
     __syncthreads();
+    tc::cluster_sync();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    // The previous grid (the Babai step of group i - 1) rewrites only the
-    // codes of group i - 1, and reads the phase partials this grid writes.
+    // The previous grid (the Babai steps of the previous block) rewrites only
+    // that block's codes, and reads the phase partials this grid writes.
     // Without the early stop (no active flags to read) each role therefore
     // waits for it only where it must: the producer before the code tile of
-    // a chunk of group i - 1, the drain before writing the partials.  The
+    // a chunk of that block, the drain before writing the partials.  The
     // Ht digit tiles, the other code tiles and the scales do not change
     // during the sweep, so the products of the other groups can run while
     // the previous grid finishes.  With the early stop every thread waits
-    // here, before reading the flags; so it does in the first phase, whose
+    // here, before reading the flags; so it does in the first block, whose
     // previous grid is the scale solve that writes the scales.
     const bool early = !a.active && a.i0 > 0;
     if (!early) tc::pdl_wait();
-    // The next grid (Babai of group i) is released at once: before its own
-    // wait it reads nothing that this grid or the previous one writes.
+    // The next grid (this block's Babai steps) is released at once: before its
+    // own wait it reads nothing that this grid or the previous one writes.
     tc::pdl_launch_dependents();
-    // a tile none of whose rows is still active (early stop, App. E) does
-    // no work: the Babai step reads the partials of active rows only
-    const bool live = early ? j0 < a.p
-                            : __syncthreads_or(threadIdx.x < 128 && j0 + (int)threadIdx.x < a.p &&
-                                               (!a.active || a.active[j0 + threadIdx.x] != 0));
+    // a pair of tiles none of whose rows is still active (early stop, App. E)
+    // does no work: the Babai step reads the partials of active rows only
+    const bool live = early ? jp < a.p
+                            : __syncthreads_or(threadIdx.x < 256 && jp + (int)threadIdx.x < a.p &&
+                                               (!a.active || a.active[jp + threadIdx.x] != 0));
     const int nseg = live ? max(0, h1 - h0) : 0;
     const int nchunks = nseg * nkc;
 
-    if (warp == 0 && lane == 0) {
+    // The three roles run as whole warps with one elected lane for the TMA and
+    // tcgen05 instructions: the control flow stays uniform and the issuing
+    // warps need few issue slots beside the drain's arithmetic.
+    if (warp == 0) {
         // ---------------- producer
-        int issued = 0;
-        bool waited = !early;
+        bool waited = !early, ok = true;
+        const uint32_t full0 = tc::map_rank(full(0), 0);
+        int s = 0, ph = 1;
         for (int c = 0; c < nchunks; ++c) {
-            const int s = c % kStages;
-            if (!tc::mbar_wait(empty(s), ((c / kStages) & 1) ^ 1) || *abort_flag) {
-                *abort_flag = 1;
-                break;
-            }
+            ok = tc::mbar_wait(empty(s), ph);
+            if (!ok) break;
             const int kx = h0 * a.g + c * 64;
-            const int h = h0 + c / nkc;
-            if (!waited && h >= a.prev0 && h < a.i0) {
+            if (!waited && kx >= a.prev0 * a.g && kx < a.i0 * a.g) {
                 tc::pdl_wait();   // the codes of the previous block
                 waited = true;
             }
-            tc::mbar_expect_tx(full(s), kStage);
-            tc::tma_load_2d(tileA(s), &mapC, full(s), kx, j0);
+            if (tc::elect_one()) {
+                if (rank == 0) tc::mbar_expect_tx(full(s), 2 * kStage);
+                const uint32_t bar = full0 + 8 * s;
+                tc::tma_load_2d_pair(tileA(s), &mapC, bar, kx, j0);
 #pragma unroll
-            for (int t = 0; t < 4; ++t)
-                tc::tma_load_2d(tileB(s, t), &mapT, full(s), kx, t * a.d_pad + m0);
-            issued = c + 1;
+                for (int t = 0; t < 2; ++t)
+                    tc::tma_load_2d_pair(tileB(s, t), &mapT, bar, kx, (2 * (int)rank + t) * a.d_pad + m0);
+            }
+            __syncwarp();
+            if (++s == kStages) {
+                s = 0;
+                ph ^= 1;
+            }
         }
         // do not leave before the MMAs have consumed the stages filled here:
         // no copy or commit is in flight afterwards
-        for (int c = issued > kStages ? issued - kStages : 0; c < issued; ++c)
-            if (!tc::mbar_wait(empty(c % kStages), (c / kStages) & 1)) *abort_flag = 1;
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer: one unit per group h
-        for (int u = 0; u < nseg && !*abort_flag; ++u) {
-            const int b = u & 1;
-            if (!tc::mbar_wait(aempty(b), ((u >> 1) & 1) ^ 1)) {
-                *abort_flag = 1;
-                break;
-            }
-            tc::tc_fence_after();
-            for (int kc = 0; kc < nkc; ++kc) {
-                const int c = u * nkc + kc;
-                const int s = c % kStages;
-                if (!tc::mbar_wait(full(s), (c / kStages) & 1) || *abort_flag) {
-                    *abort_flag = 1;
-                    break;
-                }
-                tc::tc_fence_after();
-#pragma unroll
-                for (int sub = 0; sub < 4; ++sub) {
-                    const uint64_t ad = tc::sdesc_sw128(tileA(s)) + 2 * sub;
-                    const uint64_t bd = tc::sdesc_sw128(tileB(s, 0)) + 2 * sub;
-                    tc::mma_bf16(tmem + b * 256, ad, bd, kIdesc, (kc | sub) != 0);
-                }
-                tc::mma_commit(empty(s));
-            }
-            tc::mma_commit(afull(b));
+        for (int c = 0; c < min(nchunks, kStages) && ok; ++c) {
+            // the slots in order from the oldest: s, s + 1, ...
+            const int n = nchunks - min(nchunks, kStages) + c;
+            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
         }
-    } else if (warp >= 2) {
+        if (!ok) *abort_flag = 1;
+    } else if (warp == 1) {
+        // ---------------- MMA issuer of the pair: one unit per group h
+        if (rank == 0) {
+            const uint64_t ad0 = tc::sdesc_sw128(tileA(0)), bd0 = tc::sdesc_sw128(tileB(0, 0));
+            int s = 0, ph = 0;
+            bool ok = true;
+            for (int u = 0; u < nseg && ok; ++u) {
+                const int b = u & 1;
+                // the unit's stages first (they are usually there already),
+                // then its accumulator: nothing but the MMAs' issue lies
+                // between the drain's release and the next products
+                int s1 = s + 1, ph1 = ph;
+                if (s1 == kStages) {
+                    s1 = 0;
+                    ph1 ^= 1;
+                }
+                ok = tc::mbar_wait(full(s), ph);
+                if (nkc == 2) ok = tc::mbar_wait(full(s1), ph1) && ok;
+                ok = tc::mbar_wait(aempty(b), ((u >> 1) & 1) ^ 1) && ok;
+                if (!ok) break;
+                tc::tc_fence_after();
+                if (tc::elect_one()) {
+                    const uint64_t o = (uint64_t)(s * (kStage >> 4));
+#pragma unroll
+                    for (int sub = 0; sub < 4; ++sub)
+                        tc::mma_f16_pair(tmem + b * 256, ad0 + o + 2 * sub, bd0 + o + 2 * sub, kIdesc, sub != 0);
+                    tc::mma_commit_pair(empty(s));
+                    if (nkc == 2) {
+                        const uint64_t o1 = (uint64_t)(s1 * (kStage >> 4));
+#pragma unroll
+                        for (int sub = 0; sub < 4; ++sub)
+                            tc::mma_f16_pair(tmem + b * 256, ad0 + o1 + 2 * sub, bd0 + o1 + 2 * sub, kIdesc, 1);
+                        tc::mma_commit_pair(empty(s1));
+                    }
+                    tc::mma_commit_pair(afull(b));
+                }
+                __syncwarp();
+                s = s1;
+                ph = ph1;
+                if (nkc == 2 && ++s == kStages) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            }
+            if (!ok) *abort_flag = 1;
+        }
+    } else {
         // ---------------- drain: digits -> double-float x s_h 2^(E - 9) -> accumulator
         const int q = warp & 3, cq = (warp - 2) >> 2;    // lane quarter, 16-column quarter
-        const int row = j0 + 32 * q + lane;
-        float hi[16], lo[16];
+        const int rl = 32 * q + lane, row = j0 + rl;
+        // the scales of this tile's rows and the block exponents of this
+        // split's groups, once (neither changes during a sweep)
+        const int t = threadIdx.x - 64;
+        for (int u = lane; u < nseg; u += 32) {
+            constexpr int kR = 128 / kDrainWarps;    // rows of this warp, all loads in flight
+            float sv[kR];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            hi[e] = 0.f;
-            lo[e] = 0.f;
-        }
-        bool ok = true;
-        const float *srow = a.S + (size_t)min(row, a.p - 1) * a.G;
-        const int *erow = a.expoT + (size_t)(m0 / a.g) * a.G;
-        float s_next = nseg > 0 ? srow[h0] : 0.f;
-        int e_next = nseg > 0 ? erow[h0] : 0;
-        for (int u = 0; u < nseg; ++u) {
-            const int b = u & 1, h = h0 + u;
-            const float s_cur = row < a.p ? s_next : 0.f;
-            const int e_cur = e_next;
-            if (u + 1 < nseg) {
-                s_next = srow[h + 1];
-                e_next = erow[h + 1];
+            for (int r = 0; r < kR; ++r) {
+                const int jr = j0 + (t >> 5) + r * kDrainWarps;
+                sv[r] = jr < a.p ? a.S[(size_t)jr * a.G + h0 + u] : 0.f;
             }
-            bool w = tc::mbar_wait(afull(b), (u >> 1) & 1);
-            w = __shfl_sync(0xffffffffu, w && !*abort_flag, 0);
-            tc::tc_fence_after();
-            if (!w) {
+#pragma unroll
+            for (int r = 0; r < kR; ++r) sS[u * kSRow + (t >> 5) + r * kDrainWarps] = sv[r];
+        }
+        for (int u = t; u < nseg; u += 32 * kDrainWarps)
+            sE[u] = a.expoT[(size_t)(m0 / a.g) * a.G + h0 + u] - 9;
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kDrainWarps) : "memory");
+        tc::F2 hi[8], lo[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) hi[e] = lo[e] = tc::f2(0.f);
+        bool ok = true;
+        const tc::F2 c10 = tc::f2(0x1p-10f), c20 = tc::f2(0x1p-20f);
+        const tc::F2 rc = tc::f2(a.round_c);
+        const uint32_t released = tc::map_rank(aempty(0), 0);
+        for (int u = 0; u < nseg; ++u) {
+            const int b = u & 1;
+            const float sv = sS[u * kSRow + rl];
+            const int e2 = sE[u];
+            // s 2^(E - 9): one exact product unless 2^(E - 9) is not normal
+            const float sc = (unsigned)(e2 + 126) <= 252u ? sv * __int_as_float((e2 + 127) << 23)
+                                                          : ldexpf(sv, e2);
+            const tc::F2 scale = tc::f2(sc), nscale = tc::f2(-sc);
+            ok = tc::mbar_wait(afull(b), (u >> 1) & 1);
+            if (!__all_sync(0xffffffffu, ok)) {
                 ok = false;
-                *abort_flag = 1;
                 break;
             }
-            const float scale = ldexpf(s_cur, e_cur - 9);
+            tc::tc_fence_after();
             const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + b * 256 + cq * 16;
 #pragma unroll
             for (int cc = 0; cc < 16; cc += 8) {
@@ -231,10 +296,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // every digit sum of this group is in registers
                     tc::tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(aempty(b));
+                    if (lane == 0) tc::mbar_arrive_cluster(released + 8 * b);
                 }
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
+                for (int e = 0; e < 8; e += 2) {
                     // D_0 + D_1 2^-10 exactly as (vh, vl): the digit sums are
                     // integers with |D_0| <= 128 qmax 512 and |D_1 2^-10| < 2^14;
                     // t = D_1 2^-10 rounded to a multiple of 2^-k (by adding
@@ -242,23 +307,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // so that |D_0 + t| < 2^(24-k): then vh = D_0 + t and
                     // vl = D_1 2^-10 - t (|vl| <= 2^-(k+1)) are exact.  The
                     // D_2, D_3 terms are below 2^-20 of the sum and enter the
-                    // low part.
-                    float s2, e2;
-                    const float d1 = __uint_as_float(v1[e]);
-                    const float tq = __fsub_rn(__fmaf_rn(d1, 0x1p-10f, a.round_c), a.round_c);
-                    const float vh = __fadd_rn(__uint_as_float(v0[e]), tq);
-                    float vl = __fmaf_rn(d1, 0x1p-10f, -tq);
-                    vl = fmaf(__uint_as_float(v2[e]), 0x1p-20f, vl);
-                    vl = fmaf(__uint_as_float(v3[e]), 0x1p-30f, vl);
+                    // low part.  Differences are formed from negated terms,
+                    // so that each is one instruction.
+                    auto pair = [&](const uint32_t (&v)[8]) {
+                        return tc::f2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+                    };
+                    const tc::F2 d1 = pair(v1);
+                    const tc::F2 nt = tc::f2_sub(rc, tc::f2_fma(d1, c10, rc));         // -t
+                    const tc::F2 vh = tc::f2_sub(pair(v0), nt);
+                    const tc::F2 vl = tc::f2_fma(tc::f2_fma(pair(v3), c10, pair(v2)), c20,
+                                                 tc::f2_fma(d1, c10, nt));
                     // (vh + vl) * scale, added to the accumulator
-                    const float ph = vh * scale;
-                    const float pe = fmaf(vh, scale, -ph);
-                    two_sum(hi[cc + e], ph, s2, e2);
-                    hi[cc + e] = s2;
-                    lo[cc + e] += e2 + fmaf(vl, scale, pe);
+                    const tc::F2 np = tc::f2_mul(vh, nscale);                           // -p
+                    const tc::F2 pe = tc::f2_fma(vh, scale, np);
+                    tc::F2 &H = hi[(cc + e) / 2], &L = lo[(cc + e) / 2];
+                    const tc::F2 sm = tc::f2_sub(H, np);
+                    const tc::F2 bb = tc::f2_sub(sm, H);
+                    // (H - (sm - bb)) + (p - bb)
+                    const tc::F2 er = tc::f2_sub(tc::f2_sub(H, tc::f2_sub(sm, bb)), tc::f2_add(np, bb));
+                    H = sm;
+                    L = tc::f2_add(L, tc::f2_add(er, tc::f2_fma(vl, scale, pe)));
                 }
             }
         }
+        if (!ok) *abort_flag = 1;
         // the previous grid reads the partials this drain overwrites
         if (early) tc::pdl_wait();
         if (ok && row < a.p) {
@@ -268,18 +340,27 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int e = 0; e < 16; e += 4) {
                 float x[4], y[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) two_sum(hi[e + k], lo[e + k], x[k], y[k]);
+                for (int k = 0; k < 4; k += 2) {
+                    float h2[2], l2[2];
+                    tc::f2_get(hi[(e + k) / 2], h2[0], h2[1]);
+                    tc::f2_get(lo[(e + k) / 2], l2[0], l2[1]);
+                    two_sum(h2[0], l2[0], x[k], y[k]);
+                    two_sum(h2[1], l2[1], x[k + 1], y[k + 1]);
+                }
                 *reinterpret_cast<float4 *>(a.out_hi + o + e) = make_float4(x[0], x[1], x[2], x[3]);
                 *reinterpret_cast<float4 *>(a.out_lo + o + e) = make_float4(y[0], y[1], y[2], y[3]);
             }
         }
     }
+    // neither CTA leaves while the other may still read its shared memory,
+    // signal its barriers or hold TMEM of the pair
     tc::tc_fence_before();
     __syncwarp();
     __syncthreads();
+    tc::cluster_sync();
     if (warp == 1) {
         tc::tc_fence_after();
-        tc::tmem_dealloc(tmem, 512);
+        tc::tmem_dealloc_pair(tmem, 512);
     }
     if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, ST_TIMEOUT);
 }
@@ -289,8 +370,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Split of the K range (groups) over CTAs so that a launch of nb groups covers
 // the SMs.
 int target_splits(int p_pad, int g, int G, int nb) {
-    const int tiles = (p_pad / 128) * (nb * g / 64);
-    int n = num_sms() / tiles;
+    const int pairs = ((p_pad / 128 + 1) / 2) * (nb * g / 64);
+    int n = num_sms() / 2 / pairs;
     if (n < 1) n = 1;
     if (n > kMaxSplit) n = kMaxSplit;
     if (n > G) n = G;
@@ -303,10 +384,12 @@ cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, f
                              int nb_prev, int nsplit, int qmax, int *status, cudaStream_t s,
                              bool pdl) {
     static std::atomic<unsigned long long> attr_done{0};
-    const cudaError_t e = set_max_dynamic_smem((const void *)tc_target_kernel, kSmem, attr_done);
+    static_assert(smem_bytes(kMaxGroups) <= 227 * 1024, "stages and scales must fit an SM's shared memory");
+    const cudaError_t e =
+        set_max_dynamic_smem((const void *)tc_target_kernel, smem_bytes(kMaxGroups), attr_done);
     if (e != cudaSuccess) return e;
     const int per = (G + nsplit - 1) / nsplit;
-    const int tiles = (p + 127) / 128;
+    const int tiles = (p + 255) / 256 * 2;   // pairs of row tiles
     // quantum 2^-k of the exact digit split: the largest k with
     // 128 qmax 512 + 2^14 <= 2^(24-k)
     if (qmax < 1 || qmax > 255 || g > 128) return cudaErrorInvalidValue;
@@ -318,7 +401,8 @@ cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, f
     TargetArgs a{out_hi, out_lo, S, expoT, active, status, p, p_pad, d_pad, g, G, per,
                  i0, nb, i0 - nb_prev, round_c};
     dim3 grid(tiles, nb * g / 64, nsplit);
-    return launch_k(tc_target_kernel, grid, dim3(kThreads), (size_t)kSmem, s, pdl, mapC, mapT, a);
+    return launch_k(tc_target_kernel, grid, dim3(kThreads), (size_t)smem_bytes(per), s, pdl, mapC,
+                    mapT, a);
 }
 
 }  // namespace jarq
