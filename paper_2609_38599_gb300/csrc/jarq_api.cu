@@ -24,10 +24,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 // 2D tensor map of 2-byte elements (bf16 or fp16) over [rows][cols]
-// (pitch = cols), box_rows x 64 boxes, 128-byte swizzle, out-of-range
-// elements read as zero.
+// (pitch = cols), box_rows x 64 boxes with 128-byte swizzle or box_rows x 32
+// boxes with 64-byte swizzle, out-of-range elements read as zero.
 cudaError_t make_tmap_2b(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
-                         uint32_t box_rows, CUtensorMapDataType dtype) {
+                         uint32_t box_rows, CUtensorMapDataType dtype, uint32_t box_cols) {
     static EncodeTiledFn fn = nullptr;
     if (!fn) {
         void *ptr = nullptr;
@@ -40,22 +40,23 @@ cudaError_t make_tmap_2b(CUtensorMap *m, const void *base, uint64_t rows, uint64
     }
     cuuint64_t dims[2] = {cols, rows};
     cuuint64_t strides[1] = {cols * 2};
-    cuuint32_t box[2] = {64, box_rows};
+    cuuint32_t box[2] = {box_cols, box_rows};
     cuuint32_t es[2] = {1, 1};
     CUresult r = fn(m, dtype, 2, const_cast<void *>(base), dims, strides,
-                    box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                    box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 cudaError_t make_tmap_bf16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
-                           uint32_t box_rows) {
-    return make_tmap_2b(m, base, rows, cols, box_rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
+                           uint32_t box_rows, uint32_t box_cols) {
+    return make_tmap_2b(m, base, rows, cols, box_rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, box_cols);
 }
 
 cudaError_t make_tmap_f16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
                           uint32_t box_rows) {
-    return make_tmap_2b(m, base, rows, cols, box_rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT16);
+    return make_tmap_2b(m, base, rows, cols, box_rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 64);
 }
 
 }  // namespace jarq
@@ -154,7 +155,7 @@ cudaError_t ensure_ws(jarq_hessian *h, int p) {
         return e;
     if ((e = dalloc(&w.wdig, (size_t)6 * p_pad * h->d_pad)) != cudaSuccess) return e;
     if ((e = cudaMemset(w.wdig, 0, (size_t)6 * p_pad * h->d_pad * 2)) != cudaSuccess) return e;
-    if ((e = make_tmap_bf16(&w.mapWd, w.wdig, (uint64_t)4 * p_pad, h->d_pad, 128)) != cudaSuccess)
+    if ((e = make_tmap_bf16(&w.mapWd, w.wdig, (uint64_t)4 * p_pad, h->d_pad, 128, 32)) != cudaSuccess)
         return e;
     if ((e = make_tmap_bf16(&w.mapPd, w.wdig, (uint64_t)6 * p_pad, h->d_pad, 128)) != cudaSuccess)
         return e;
@@ -318,7 +319,7 @@ jarq_status project_by(jarq_hessian *h, const float *M, int p, float *out_hi, fl
         CK(dalloc(&h->qdig, (size_t)6 * h->d_pad * h->d_pad));
         CK(cudaMemset(h->qdig, 0, (size_t)6 * h->d_pad * h->d_pad * 2));
         CK(dalloc(&h->qexp, (size_t)h->G * h->G));
-        CK(make_tmap_bf16(&h->mapQ, h->qdig, (uint64_t)6 * h->d_pad, h->d_pad, 64));
+        CK(make_tmap_bf16(&h->mapQ, h->qdig, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32));
     }
     const float *Md = M;
     if (!is_device_ptr(M)) {
@@ -459,7 +460,7 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         if ((e = dalloc(&h->Hdig10, 4 * pd)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = cudaMemsetAsync(h->Hdig10, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->expo, (size_t)h->G * h->G)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = make_tmap_bf16(&h->mapD8, h->Hdig8, (uint64_t)6 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        if ((e = make_tmap_bf16(&h->mapD8, h->Hdig8, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_f16(&h->mapD10, h->Hdig10, (uint64_t)4 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->Lf, (size_t)h->G * factor_floats(group_size))) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = dalloc(&h->L64, (size_t)h->G * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }

@@ -106,7 +106,7 @@ struct Workspace {
     // hold the six digit planes of P for the folded projection
     __nv_bfloat16 *wdig = nullptr;     // [6][p_pad][d_pad] integer digits of W (4) or P (6)
     int *wexp = nullptr;               // [p][G] exponents of those digits
-    CUtensorMap mapWd;                 // tensor map of wdig's first 4 planes, 128 x 64 boxes
+    CUtensorMap mapWd;                 // tensor map of wdig's first 4 planes, 128 x 32 boxes
     CUtensorMap mapPd;                 // tensor map of all 6 planes, 128 x 64 boxes
     float *Phi = nullptr;        // [p][d]  P = Phi + Plo (double-float)
     float *Plo = nullptr;        // [p][d]
@@ -144,7 +144,7 @@ struct jarq_hessian {
     __half *Hdig10 = nullptr;          // [4][d_pad][d_pad] base 2^10, |digit| <= 512
     int *expo = nullptr;          // [G][G] block exponents of the digits
     CUtensorMap mapH128, mapH64;  // tensor maps of Hplanes, 128 x 64 and 64 x 64 boxes
-    CUtensorMap mapD8, mapD10;    // tensor maps of Hdig8 / Hdig10, 64 x 64 boxes
+    CUtensorMap mapD8, mapD10;    // tensor maps of Hdig8 (64 x 32 boxes) / Hdig10 (64 x 64)
     float *Lf = nullptr;          // [G][factor_floats(g)] lower factor L_i = R_i^T, packed
     // digits of the blocks Ht_{i'i}, i' = i + 1 .. i + kMaxBlock - 1, column by
     // column: [G][kMaxBlock - 1][g columns of i][g rows of i'], each entry the
@@ -166,7 +166,7 @@ struct jarq_hessian {
     __nv_bfloat16 *qdig = nullptr;     // [6][d_pad][d_pad]
     int *qexp = nullptr;               // [G][G]
     float *qstage = nullptr;           // [d][d]
-    CUtensorMap mapQ;                  // tensor map of qdig, 64 x 64 boxes
+    CUtensorMap mapQ;                  // tensor map of qdig, 64 x 32 boxes
     int *dstatus = nullptr;       // device status word
     int *hstatus = nullptr;       // pinned host mirror
     jarq::Workspace ws;
@@ -325,12 +325,13 @@ class DeviceGuard {
 };
 
 // 2D tensor map of 2-byte elements (bf16 or fp16) over [rows][cols]
-// (pitch = cols elements), box_rows x 64 boxes, 128-byte swizzle,
-// out-of-range elements read as zero.
+// (pitch = cols elements), box_rows x box_cols boxes, box_cols = 64 with
+// 128-byte swizzle or 32 with 64-byte swizzle, out-of-range elements read as
+// zero.
 cudaError_t make_tmap_2b(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
-                         uint32_t box_rows, CUtensorMapDataType dtype);
+                         uint32_t box_rows, CUtensorMapDataType dtype, uint32_t box_cols);
 cudaError_t make_tmap_bf16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
-                           uint32_t box_rows);
+                           uint32_t box_rows, uint32_t box_cols = 64);
 cudaError_t make_tmap_f16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
                           uint32_t box_rows);
 

@@ -21,12 +21,26 @@
 // group's contribution to a double-float accumulator.  The dropped products
 // (t + u >= 6) are below 2^-48 of the block scales.
 //
-// Roles: warp 0 TMA producer (4 W planes + 6 H planes per 64-wide K chunk),
-// warp 1 TMEM allocation and MMA issue, warps 2..9 drain (warp w reads TMEM
-// lanes 32 (w % 4) and 32 of the tile's 64 columns).  Tile 128 x 64; the six
-// levels take 384 TMEM columns, single-buffered: the drain warps release
-// them as soon as their loads have landed and combine from registers while
-// the next group's products run.
+// The target projection runs on CTA pairs (cta_group::2): 256 rows x 64
+// columns per pair, each CTA loading its 128 rows of the four W planes and
+// three of the six H planes, 32 of K at a time (five stages of 44 KB).  An MMA
+// takes its B rows half from each CTA, so the planes are split {0, 1, 4 | 2, 3,
+// 5}: W digit t meets planes 0..3 in one N = 256 MMA (levels t .. t + 3) and,
+// for t < 2, planes 4, 5 in one N = 128 MMA (levels t + 4, t + 5).  The
+// products that land on level 6 are not read.
+//   warp 0       TMA producer of its CTA's tiles, onto the even CTA's barriers
+//   warp 1       TMEM allocation; in the even CTA the MMA issuer
+//   warps 2..17  drain: warp w reads TMEM lanes 32 (w % 4) and 16 columns
+// The levels (7 x 64 TMEM columns) are single-buffered and handed back in two
+// steps: levels 4, 5 first, which is all that the N = 128 MMAs of the next
+// group's first tiles need, then levels 0..3.
+//
+// What bounds it: the MMAs.  20 x 64 columns per K step (two of them for level
+// 6) at 4096 x 4096 x 4096 in 1.58 ms are 1.74 PFLOP/s issued, at 4096 x 11008
+// x 11008 in 10.7 ms 1.85 PFLOP/s, of a measured 1.94 PFLOP/s.  One CTA per
+// 128 x 64 tile, with two stages of 112 KB and a drain that combined the
+// levels by two-sums (55 operations an output and group, now 21) before it
+// released them, took 2.43 and 16.2 ms.
 #include "tc_common.cuh"
 
 namespace jarq {
@@ -35,20 +49,23 @@ namespace {
 constexpr int kWDig = 4, kHDig = 6, kLevels = 6;
 constexpr int kTileA = 128 * 64 * 2;   // one W digit plane, 128 rows x 64 K
 constexpr int kTileB = 64 * 64 * 2;    // one H digit plane, 64 rows x 64 K
-// WDIG row-side digit planes (4 for W, 6 for the double-float P of the folded
-// projection); DIAG: only the K block of the tile's own column group (the
-// block-diagonal right-hand side R_i^{-1}), one stage of 144 KB.
-template <int WDIG, bool DIAG>
-struct ProjCfg {
-    static constexpr int kStage = WDIG * kTileA + kHDig * kTileB;
-    static constexpr int kStages = DIAG ? 1 : 2;
-    static constexpr int kSmem = 1024 + kStages * kStage + 256;
-};
-// For a W digit t the H digit planes u are consecutive 64-row tiles and the
-// levels t + u consecutive 64-column blocks, so one MMA covers up to four
-// planes (N = 64 per plane).
+// Folded projection: all digits of the K block of the tile's own column
+// group (the block-diagonal right-hand side R_i^{-1}), one stage of 144 KB.
+constexpr int kFoldStage = kHDig * (kTileA + kTileB);
+constexpr int kFoldSmem = 1024 + kFoldStage + 256;
+// For a row digit t the right-hand digit planes u are consecutive 64-row tiles
+// and the levels t + u consecutive 64-column blocks, so one MMA covers up to
+// four planes (N = 64 per plane).
 __host__ __device__ constexpr uint32_t idesc_n(int n) { return tc::idesc_bf16_f32(128, n); }
-constexpr int kGroupRows = 8;
+// Target projection on CTA pairs
+constexpr int kPairA = 128 * 32 * 2;   // one W digit plane, 128 rows x 32 K
+constexpr int kPairB = 64 * 32 * 2;    // one H digit plane, 64 rows x 32 K
+constexpr int kPairStage = kWDig * kPairA + 3 * kPairB;
+constexpr int kPairStages = 5;
+constexpr int kPairSmem = 1024 + kPairStages * kPairStage + 256;
+constexpr int kPairDrain = 16;
+constexpr int kPairThreads = 32 * (2 + kPairDrain);
+constexpr int kGroupPairs = 4;         // tile pairs per band of the tile order
 
 struct ProjArgs {
     float *Phi, *Plo;    // [p][d] double-float result
@@ -65,11 +82,14 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = (a - (s - bb)) + (b - bb);
 }
 
-template <int WDIG, bool DIAG>
+// Folded projection (launch_ptilde): persistent CTAs over 128 x 64 tiles, one
+// K block each.  Warp 0 TMA producer, warp 1 TMEM allocation and MMA issue,
+// warps 2..9 drain (warp w reads TMEM lanes 32 (w % 4) and 32 of the tile's 64
+// columns).
 __global__ void __launch_bounds__(320, 1)
-    tc_proj_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapH,
+    tc_fold_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapH,
                    ProjArgs a) {
-    constexpr int kStage = ProjCfg<WDIG, DIAG>::kStage, kStages = ProjCfg<WDIG, DIAG>::kStages;
+    constexpr int kStage = kFoldStage, kStages = 1, WDIG = kHDig;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = (uint64_t *)(smem + kStages * kStage);
@@ -77,36 +97,17 @@ __global__ void __launch_bounds__(320, 1)
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkc = a.g / 64;               // K chunks per group
-    // General form: one 128 x 64 tile per CTA in grouped order (bands of
-    // kGroupRows row tiles sweep all column tiles), one segment per group of
-    // K.  Diagonal form: the CTA loops over tiles, item blockIdx.x + v gridDim.x
-    // of (row tiles) x (d / 64 column tiles), one segment each: the K block of
-    // the tile's own column group.
-    int gj0 = 0, gn0 = 0;
-    if (!DIAG) {
-        const int lin = blockIdx.y * gridDim.x + blockIdx.x;
-        const int per_band = kGroupRows * gridDim.y;
-        const int band = lin / per_band, in_band = lin % per_band;
-        const int rows_in_band = min(kGroupRows, (int)gridDim.x - band * kGroupRows);
-        gj0 = (band * kGroupRows + in_band % rows_in_band) * 128;
-        gn0 = (in_band / rows_in_band) * 64;
-    }
+    // item blockIdx.x + v gridDim.x of (row tiles) x (d / 64 column tiles)
     const int nct = a.d / 64;
-    const int nitems = DIAG ? ((a.p + 127) / 128) * nct : 1;
-    const int nseg = DIAG ? ((int)blockIdx.x < nitems ? (nitems - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0)
-                          : a.G;
+    const int nitems = ((a.p + 127) / 128) * nct;
+    const int nseg = (int)blockIdx.x < nitems ? (nitems - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int nchunks = nseg * nkc;
     // tile (first row, first column) of segment v; a 64-wide tile lies in
     // one column group n0 / g
     auto tile_of = [&](int v, int &j0, int &n0) {
-        if (DIAG) {
-            const int it = (int)blockIdx.x + v * (int)gridDim.x;
-            j0 = (it / nct) * 128;
-            n0 = (it % nct) * 64;
-        } else {
-            j0 = gj0;
-            n0 = gn0;
-        }
+        const int it = (int)blockIdx.x + v * (int)gridDim.x;
+        j0 = (it / nct) * 128;
+        n0 = (it % nct) * 64;
     };
 
     auto full = [&](int s) { return tc::smem_u32(bars + s); };
@@ -153,10 +154,8 @@ __global__ void __launch_bounds__(320, 1)
             const int v = c / nkc, kc = c % nkc;
             int j0, n0;
             tile_of(v, j0, n0);
-            // K offsets in the two maps: the right-hand side of the diagonal
-            // form holds only the g columns of each group's block
-            const int kw = DIAG ? (n0 / a.g) * a.g + kc * 64 : c * 64;
-            const int kh = DIAG ? kc * 64 : c * 64;
+            // the right-hand side holds only the g columns of each group's block
+            const int kw = (n0 / a.g) * a.g + kc * 64, kh = kc * 64;
             tc::mbar_expect_tx(full(s), kStage);
 #pragma unroll
             for (int t = 0; t < WDIG; ++t)
@@ -207,180 +206,93 @@ __global__ void __launch_bounds__(320, 1)
         }
     } else if (warp >= 2) {
         // ---------------- drain: levels -> double-float per group -> accumulator
-        if constexpr (DIAG) {
-            // diagonal form: a tile per segment, written when it completes
-            const int q = warp & 3, half = (warp - 2) >> 2;
-            float hi[32], lo[32];
+        // diagonal form: a tile per segment, written when it completes
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        float hi[32], lo[32];
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                hi[e] = 0.f;
-                lo[e] = 0.f;
+        for (int e = 0; e < 32; ++e) {
+            hi[e] = 0.f;
+            lo[e] = 0.f;
+        }
+        const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + half * 32;
+        // exponents of this thread's row and segment v: W's (row, K group)
+        // and the block's; loaded one segment ahead
+        auto seg_exp = [&](int v, int &ew, int &eh) {
+            int j0, n0;
+            tile_of(v, j0, n0);
+            const int row = j0 + 32 * q + lane, hb = n0 / a.g;
+            ew = row < a.p ? a.wexp[(size_t)row * a.G + hb] : 0;
+            eh = a.hexp[hb];
+        };
+        int ew_next = 0, eh_next = 0;
+        if (nseg > 0) seg_exp(0, ew_next, eh_next);
+        for (int sg = 0; sg < nseg; ++sg) {
+            const int ew = ew_next, eh = eh_next;
+            if (sg + 1 < nseg) seg_exp(sg + 1, ew_next, eh_next);
+            bool w = tc::mbar_wait(afull, sg & 1);
+            w = __shfl_sync(0xffffffffu, w && !*abort_flag, 0);
+            tc::tc_fence_after();
+            if (!w) {
+                *abort_flag = 1;
+                break;
             }
-            bool ok = true;
-            const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + half * 32;
-            // exponents of this thread's row and segment v: W's (row, K group)
-            // and H's block (K group, column group); loaded one segment ahead
-            auto seg_exp = [&](int v, int &ew, int &eh) {
-                int j0, n0;
-                tile_of(v, j0, n0);
-                const int row = j0 + 32 * q + lane, hb = n0 / a.g, kg = DIAG ? hb : v;
-                ew = row < a.p ? a.wexp[(size_t)row * a.G + kg] : 0;
-                eh = hb < a.G ? a.hexp[DIAG ? hb : kg * a.G + hb] : 0;
-            };
-            int ew_next = 0, eh_next = 0;
-            if (nseg > 0) seg_exp(0, ew_next, eh_next);
-            for (int sg = 0; sg < nseg; ++sg) {
-                const int ew = ew_next, eh = eh_next;
-                if (sg + 1 < nseg) seg_exp(sg + 1, ew_next, eh_next);
-                bool w = tc::mbar_wait(afull, sg & 1);
-                w = __shfl_sync(0xffffffffu, w && !*abort_flag, 0);
-                tc::tc_fence_after();
-                if (!w) {
-                    ok = false;
-                    *abort_flag = 1;
-                    break;
-                }
-                const float scale = ldexpf(1.0f, ew + eh - 14);
-                // value of the group = sum_l L_l 2^(-8 l), as (vh, vl), 32 columns
-                float vh[32], vl[32];
+            const float scale = ldexpf(1.0f, ew + eh - 14);
+            // value of the group = sum_l L_l 2^(-8 l), as (vh, vl), 32 columns
+            float vh[32], vl[32];
 #pragma unroll
-                for (int l = 0; l < kLevels; ++l) {
-                    uint32_t x[32];
-                    tc::tmem_ld32(base + l * 64, x);
-                    tc::tmem_wait_ld();
-                    if (l == kLevels - 1) {
-                        // every level is in registers: hand the columns back
-                        tc::tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(aempty);
-                    }
-                    const float f = ldexpf(1.0f, -8 * l);
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const float v = __uint_as_float(x[e]) * f;   // exact (power of two)
-                        if (l == 0) {
-                            vh[e] = v;
-                            vl[e] = 0.f;
-                        } else {
-                            float s2, e2;
-                            two_sum(vh[e], v, s2, e2);
-                            vh[e] = s2;
-                            vl[e] += e2;
-                        }
-                    }
+            for (int l = 0; l < kLevels; ++l) {
+                uint32_t x[32];
+                tc::tmem_ld32(base + l * 64, x);
+                tc::tmem_wait_ld();
+                if (l == kLevels - 1) {
+                    // every level is in registers: hand the columns back
+                    tc::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(aempty);
                 }
+                const float f = ldexpf(1.0f, -8 * l);
 #pragma unroll
                 for (int e = 0; e < 32; ++e) {
-                    float s2, e2;
-                    two_sum(hi[e], vh[e] * scale, s2, e2);
-                    hi[e] = s2;
-                    lo[e] += e2 + vl[e] * scale;
-                }
-                // the tile is complete after its last segment (every segment in
-                // the diagonal form)
-                if (DIAG || sg + 1 == nseg) {
-                    int j0, n0;
-                    tile_of(sg, j0, n0);
-                    const int row = j0 + 32 * q + lane, ncol = n0 + half * 32;
-                    if (row < a.p) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) {
-                            const int col = ncol + e;
-                            if (col < a.d) {
-                                float s2, e2;
-                                two_sum(hi[e], lo[e], s2, e2);
-                                a.Phi[(size_t)row * a.d + col] = s2;
-                                a.Plo[(size_t)row * a.d + col] = e2;
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        hi[e] = 0.f;
-                        lo[e] = 0.f;
-                    }
-                }
-            }
-            (void)ok;
-        } else {
-            const int q = warp & 3, half = (warp - 2) >> 2;
-            const int j0 = gj0, n0 = gn0, hblk = n0 / a.g;
-            const int row = j0 + 32 * q + lane;
-            float hi[32], lo[32];
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                hi[e] = 0.f;
-                lo[e] = 0.f;
-            }
-            bool ok = true;
-            const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + half * 32;
-            // exponents of the next group, loaded one group ahead
-            const int *wrow = a.wexp + (size_t)min(row, a.p - 1) * a.G;
-            const int hb = min(hblk, a.G - 1);
-            int ew_next = wrow[0], eh_next = a.hexp[hb];
-            for (int sg = 0; sg < nseg; ++sg) {
-                const int ew = row < a.p ? ew_next : 0;
-                const int eh = hblk < a.G ? eh_next : 0;
-                if (sg + 1 < nseg) {
-                    ew_next = wrow[sg + 1];
-                    eh_next = a.hexp[(sg + 1) * a.G + hb];
-                }
-                bool w = tc::mbar_wait(afull, sg & 1);
-                w = __shfl_sync(0xffffffffu, w && !*abort_flag, 0);
-                tc::tc_fence_after();
-                if (!w) {
-                    ok = false;
-                    *abort_flag = 1;
-                    break;
-                }
-                const float scale = ldexpf(1.0f, ew + eh - 14);
-                // value of the group = sum_l L_l 2^(-8 l), as (vh, vl), 32 columns
-                float vh[32], vl[32];
-#pragma unroll
-                for (int l = 0; l < kLevels; ++l) {
-                    uint32_t x[32];
-                    tc::tmem_ld32(base + l * 64, x);
-                    tc::tmem_wait_ld();
-                    if (l == kLevels - 1) {
-                        // every level is in registers: hand the columns back
-                        tc::tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(aempty);
-                    }
-                    const float f = ldexpf(1.0f, -8 * l);
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const float v = __uint_as_float(x[e]) * f;   // exact (power of two)
-                        if (l == 0) {
-                            vh[e] = v;
-                            vl[e] = 0.f;
-                        } else {
-                            float s2, e2;
-                            two_sum(vh[e], v, s2, e2);
-                            vh[e] = s2;
-                            vl[e] += e2;
-                        }
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    float s2, e2;
-                    two_sum(hi[e], vh[e] * scale, s2, e2);
-                    hi[e] = s2;
-                    lo[e] += e2 + vl[e] * scale;
-                }
-            }
-            if (ok && row < a.p) {
-                const int ncol = n0 + half * 32;
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const int col = ncol + e;
-                    if (col < a.d) {
+                    const float v = __uint_as_float(x[e]) * f;   // exact (power of two)
+                    if (l == 0) {
+                        vh[e] = v;
+                        vl[e] = 0.f;
+                    } else {
                         float s2, e2;
-                        two_sum(hi[e], lo[e], s2, e2);
-                        a.Phi[(size_t)row * a.d + col] = s2;
-                        a.Plo[(size_t)row * a.d + col] = e2;
+                        two_sum(vh[e], v, s2, e2);
+                        vh[e] = s2;
+                        vl[e] += e2;
                     }
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+                float s2, e2;
+                two_sum(hi[e], vh[e] * scale, s2, e2);
+                hi[e] = s2;
+                lo[e] += e2 + vl[e] * scale;
+            }
+            // the tile is complete
+            {
+                int j0, n0;
+                tile_of(sg, j0, n0);
+                const int row = j0 + 32 * q + lane, ncol = n0 + half * 32;
+                if (row < a.p) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        const int col = ncol + e;
+                        if (col < a.d) {
+                            float s2, e2;
+                            two_sum(hi[e], lo[e], s2, e2);
+                            a.Phi[(size_t)row * a.d + col] = s2;
+                            a.Plo[(size_t)row * a.d + col] = e2;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    hi[e] = 0.f;
+                    lo[e] = 0.f;
                 }
             }
         }
@@ -390,6 +302,256 @@ __global__ void __launch_bounds__(320, 1)
     if (warp == 1) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem, 512);
+    }
+    if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, ST_TIMEOUT);
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+    tc_proj_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapH,
+                   ProjArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t *bars = (uint64_t *)(smem + kPairStages * kPairStage);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kPairStages + 3);
+    volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)tc::cluster_rank();
+    // tiles in bands: kGroupPairs pairs of row tiles sweep all column tiles
+    const int npairs = gridDim.x / 2;
+    const int lin = blockIdx.y * npairs + blockIdx.x / 2;
+    const int band = lin / (kGroupPairs * gridDim.y), in_band = lin % (kGroupPairs * gridDim.y);
+    const int in_rows = min(kGroupPairs, npairs - band * kGroupPairs);
+    const int j0 = (band * kGroupPairs + in_band % in_rows) * 256 + 128 * rank;
+    const int n0 = (in_band / in_rows) * 64;
+    const int nsub = a.g / 32;              // 32-wide K chunks per group
+    const int nchunks = a.G * nsub;
+
+    auto full = [&](int s) { return tc::smem_u32(bars + s); };
+    auto empty = [&](int s) { return tc::smem_u32(bars + kPairStages + s); };
+    const uint32_t afull = tc::smem_u32(bars + 2 * kPairStages);
+    const uint32_t afree = tc::smem_u32(bars + 2 * kPairStages + 1);   // [2]: levels 4, 5; 0..3
+    auto tileA = [&](int s, int t) { return tc::smem_u32(smem + s * kPairStage + t * kPairA); };
+    auto tileB = [&](int s, int u) {
+        return tc::smem_u32(smem + s * kPairStage + kWDig * kPairA + u * kPairB);
+    };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kPairStages; ++s) {
+            tc::mbar_init(full(s), 1);      // the even CTA's: bytes of both CTAs
+            tc::mbar_init(empty(s), 1);
+        }
+        tc::mbar_init(afull, 1);
+        tc::mbar_init(afree, 2 * kPairDrain);       // the even CTA's: both drains
+        tc::mbar_init(afree + 8, 2 * kPairDrain);
+        *abort_flag = 0;
+        tc::fence_barrier_init();
+    }
+    if (warp == 1) {
+        tc::tmem_alloc_pair(tc::smem_u32(tmem_slot), 512);
+        tc::tmem_relinquish_pair();
+    }
+    if (warp == 0 && lane == 0) {
+        tc::prefetch_tmap(&mapW);
+        tc::prefetch_tmap(&mapH);
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::cluster_sync();
+    tc::tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        // ---------------- producer
+        bool ok = true;
+        const uint32_t full0 = tc::map_rank(full(0), 0);
+        int s = 0, ph = 1;
+        for (int c = 0; c < nchunks; ++c) {
+            ok = tc::mbar_wait(empty(s), ph);
+            if (!ok) break;
+            if (tc::elect_one()) {
+                if (rank == 0) tc::mbar_expect_tx(full(s), 2 * kPairStage);
+                const uint32_t bar = full0 + 8 * s;
+#pragma unroll
+                for (int t = 0; t < kWDig; ++t)
+                    tc::tma_load_2d_pair(tileA(s, t), &mapW, bar, c * 32, t * a.w_plane + j0);
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                    const int plane = u < 2 ? 2 * rank + u : 4 + rank;
+                    tc::tma_load_2d_pair(tileB(s, u), &mapH, bar, c * 32, plane * a.h_plane + n0);
+                }
+            }
+            __syncwarp();
+            if (++s == kPairStages) {
+                s = 0;
+                ph ^= 1;
+            }
+        }
+        // do not leave before the MMAs have consumed the stages filled here:
+        // no copy or commit is in flight afterwards
+        for (int n = max(0, nchunks - kPairStages); n < nchunks && ok; ++n)
+            ok = tc::mbar_wait(empty(n % kPairStages), (n / kPairStages) & 1);
+        if (!ok) *abort_flag = 1;
+    } else if (warp == 1) {
+        // ---------------- MMA issuer of the pair
+        if (rank == 0) {
+            constexpr uint32_t id256 = tc::idesc_bf16_f32(256, 256), id128 = tc::idesc_bf16_f32(256, 128);
+            const uint64_t ad0 = tc::sdesc_sw64(tileA(0, 0)), bd0 = tc::sdesc_sw64(tileB(0, 0));
+            constexpr uint64_t kPl = kPairA >> 4, kHi = (2 * kPairB) >> 4;   // next W plane; planes 4, 5
+            bool ok = true;
+            int s = 0, ph = 0;
+            for (int sg = 0; sg < a.G && ok; ++sg) {
+                for (int c = 0; c < nsub; ++c) {
+                    ok = tc::mbar_wait(full(s), ph);
+                    if (c == 0) ok = tc::mbar_wait(afree, (sg & 1) ^ 1) && ok;
+                    if (!ok) break;
+                    tc::tc_fence_after();
+                    const uint64_t ad = ad0 + (uint64_t)(s * (kPairStage >> 4));
+                    const uint64_t bd = bd0 + (uint64_t)(s * (kPairStage >> 4));
+                    if (tc::elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < 4; k += 2) {
+                            // planes 4, 5: levels 4, 5 (opened by the first) and 5, 6
+                            tc::mma_f16_pair(tmem + 4 * 64, ad + k, bd + kHi + k, id128, (c | k) != 0);
+                            tc::mma_f16_pair(tmem + 5 * 64, ad + kPl + k, bd + kHi + k, id128, 1);
+                        }
+                    }
+                    __syncwarp();
+                    if (c == 0) {
+                        ok = tc::mbar_wait(afree + 8, (sg & 1) ^ 1);
+                        if (!ok) break;
+                        tc::tc_fence_after();
+                    }
+                    if (tc::elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < 4; k += 2)
+#pragma unroll
+                            for (int t = 0; t < kWDig; ++t)     // planes 0..3: levels t .. t + 3
+                                tc::mma_f16_pair(tmem + t * 64, ad + t * kPl + k, bd + k, id256,
+                                                 t > 0 || (c | k) != 0);
+                        tc::mma_commit_pair(empty(s));
+                        if (c + 1 == nsub) tc::mma_commit_pair(afull);
+                    }
+                    __syncwarp();
+                    if (++s == kPairStages) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+            if (!ok) *abort_flag = 1;
+        }
+    } else {
+        // ---------------- drain: levels -> double-float per group -> accumulator
+        const int q = warp & 3, cq = (warp - 2) >> 2;    // lane quarter, 16-column quarter
+        const int hb = n0 / a.g;
+        const int row = j0 + 32 * q + lane;
+        tc::F2 hi[8], lo[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) hi[e] = lo[e] = tc::f2(0.f);
+        bool ok = true;
+        const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + cq * 16;
+        const uint32_t freed = tc::map_rank(afree, 0);
+        // exponents of the next group, loaded one group ahead
+        const int *wrow = a.wexp + (size_t)min(row, a.p - 1) * a.G;
+        int e_next = wrow[0] + a.hexp[hb];
+        const tc::F2 c8 = tc::f2(0x1p-8f), c16 = tc::f2(0x1p-16f), c24 = tc::f2(0x1p-24f),
+                     c32 = tc::f2(0x1p-32f);
+        for (int sg = 0; sg < a.G; ++sg) {
+            const int ex = e_next - 14;
+            if (sg + 1 < a.G) e_next = wrow[sg + 1] + a.hexp[(sg + 1) * a.G + hb];
+            // 2^ex, from its bits while it is a normal number
+            const tc::F2 scale = tc::f2((unsigned)(ex + 126) <= 252u ? __int_as_float((ex + 127) << 23)
+                                                                     : ldexpf(1.0f, ex));
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(afull, sg & 1));
+            if (!ok) break;
+            tc::tc_fence_after();
+            tc::F2 w[8];     // L_4 + L_5 2^-8
+            {
+                uint32_t x4[16], x5[16];
+                tc::tmem_ld16(base + 4 * 64, x4);
+                tc::tmem_ld16(base + 5 * 64, x5);
+                tc::tmem_wait_ld();
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive_cluster(freed);
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    w[e] = tc::f2_fma(tc::f2(__uint_as_float(x5[2 * e]), __uint_as_float(x5[2 * e + 1])), c8,
+                                      tc::f2(__uint_as_float(x4[2 * e]), __uint_as_float(x4[2 * e + 1])));
+            }
+#pragma unroll
+            for (int cc = 0; cc < 16; cc += 8) {
+                uint32_t x0[8], x1[8], x2[8], x3[8];
+                tc::tmem_ld8(base + 0 * 64 + cc, x0);
+                tc::tmem_ld8(base + 1 * 64 + cc, x1);
+                tc::tmem_ld8(base + 2 * 64 + cc, x2);
+                tc::tmem_ld8(base + 3 * 64 + cc, x3);
+                tc::tmem_wait_ld();
+                if (cc == 8) {
+                    tc::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive_cluster(freed + 8);
+                }
+#pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    // sum_l L_l 2^(-8 l) as (v, r).  L_0 is an integer, and every
+                    // partial sum of the first l levels a multiple of 2^(-8 l)
+                    // (or of a larger power, rounded): an integer multiple of
+                    // the last place of the next term (|L_l| <= 2^23), so that
+                    // three operations give each sum's rounding error exactly
+                    // (Fast2Sum).
+                    auto pair = [&](const uint32_t (&x)[8]) {
+                        return tc::f2(__uint_as_float(x[e]), __uint_as_float(x[e + 1]));
+                    };
+                    auto add_level = [&](tc::F2 &v, const uint32_t (&x)[8], tc::F2 f) {
+                        const tc::F2 v2 = tc::f2_fma(pair(x), f, v);
+                        const tc::F2 r = tc::f2_fma(pair(x), f, tc::f2_sub(v, v2));
+                        v = v2;
+                        return r;
+                    };
+                    tc::F2 v = pair(x0);
+                    tc::F2 r = add_level(v, x1, c8);
+                    r = tc::f2_add(r, add_level(v, x2, c16));
+                    r = tc::f2_add(r, add_level(v, x3, c24));
+                    r = tc::f2_fma(w[(cc + e) / 2], c32, r);
+                    // (v + r) 2^ex (exact products) added to the accumulator
+                    tc::F2 &H = hi[(cc + e) / 2], &L = lo[(cc + e) / 2];
+                    const tc::F2 sm = tc::f2_fma(v, scale, H);
+                    const tc::F2 nb = tc::f2_sub(H, sm);
+                    const tc::F2 er = tc::f2_add(tc::f2_sub(H, tc::f2_add(sm, nb)), tc::f2_fma(v, scale, nb));
+                    H = sm;
+                    L = tc::f2_add(L, tc::f2_fma(r, scale, er));
+                }
+            }
+        }
+        if (!ok) *abort_flag = 1;
+        if (ok && row < a.p) {
+            const size_t o = (size_t)row * a.d + n0 + cq * 16;
+#pragma unroll
+            for (int e = 0; e < 16; e += 4) {
+                float x[4], y[4];
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    float h2[2], l2[2];
+                    tc::f2_get(hi[(e + k) / 2], h2[0], h2[1]);
+                    tc::f2_get(lo[(e + k) / 2], l2[0], l2[1]);
+                    two_sum(h2[0], l2[0], x[k], y[k]);
+                    two_sum(h2[1], l2[1], x[k + 1], y[k + 1]);
+                }
+                *reinterpret_cast<float4 *>(a.Phi + o + e) = make_float4(x[0], x[1], x[2], x[3]);
+                *reinterpret_cast<float4 *>(a.Plo + o + e) = make_float4(y[0], y[1], y[2], y[3]);
+            }
+        }
+    }
+    // neither CTA leaves while the other may still read its shared memory,
+    // signal its barriers or hold TMEM of the pair
+    tc::tc_fence_before();
+    __syncwarp();
+    __syncthreads();
+    tc::cluster_sync();
+    if (warp == 1) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc_pair(tmem, 512);
     }
     if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, ST_TIMEOUT);
 }
@@ -647,16 +809,15 @@ cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, con
         Phi, Plo, pdig, pexp, p, d, d_pad, p_pad, g);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    using C = ProjCfg<kHDig, true>;
     static std::atomic<unsigned long long> attr_done{0};
-    e = set_max_dynamic_smem((const void *)tc_proj_kernel<kHDig, true>, C::kSmem, attr_done);
+    e = set_max_dynamic_smem((const void *)tc_fold_kernel, kFoldSmem, attr_done);
     if (e != cudaSuccess) return e;
     ProjArgs a{out_hi, out_lo, pexp, rexp, status, p, d, g, d / g, p_pad, d};
     // persistent: one CTA per SM over the (p_pad / 128) x (d / 64) tiles
     (void)d_pad;
-    const int items = (p_pad / 128) * (d / 64);
+    const int items = ((p + 127) / 128) * (d / 64);
     const int ctas = items < num_sms() ? items : num_sms();
-    tc_proj_kernel<kHDig, true><<<dim3(ctas, 1, 1), 320, C::kSmem, s>>>(mapPd, mapR, a);
+    tc_fold_kernel<<<dim3(ctas, 1, 1), 320, kFoldSmem, s>>>(mapPd, mapR, a);
     return cudaGetLastError();
 }
 
@@ -671,14 +832,11 @@ cudaError_t launch_slice_rows(const float *W, __nv_bfloat16 *planes, int *wexp, 
 cudaError_t launch_tc_proj(const CUtensorMap &mapW, const CUtensorMap &mapH, float *Phi,
                            float *Plo, const int *wexp, const int *hexp, int p, int p_pad, int d,
                            int d_pad, int g, int *status, cudaStream_t s) {
-    using C = ProjCfg<kWDig, false>;
     static std::atomic<unsigned long long> attr_done{0};
-    const cudaError_t e =
-        set_max_dynamic_smem((const void *)tc_proj_kernel<kWDig, false>, C::kSmem, attr_done);
+    const cudaError_t e = set_max_dynamic_smem((const void *)tc_proj_kernel, kPairSmem, attr_done);
     if (e != cudaSuccess) return e;
     ProjArgs a{Phi, Plo, wexp, hexp, status, p, d, g, d / g, p_pad, d_pad};
-    dim3 grid(p_pad / 128, d_pad / 64, 1);
-    tc_proj_kernel<kWDig, false><<<grid, 320, C::kSmem, s>>>(mapW, mapH, a);
+    tc_proj_kernel<<<dim3((p + 255) / 256 * 2, d / 64), kPairThreads, kPairSmem, s>>>(mapW, mapH, a);
     return cudaGetLastError();
 }
 

@@ -59,6 +59,27 @@ def test_scale_fit_parity(jarq, din, dout, g, bits, method):
         assert np.all(Fa <= Fb * (1 + 1e-9))
 
 
+@pytest.mark.parametrize("din,dout,g", [
+    (64, 1, 64),       # one row, one column tile, one group
+    (192, 129, 64),    # the second CTA of a pair with one row; three column tiles
+    (320, 257, 64),    # a second pair with one row
+    (128, 256, 128),   # one full pair
+    (384, 300, 128),   # three groups of 128
+])
+def test_projection_pair_edges(jarq, din, dout, g):
+    """The target projection on CTA pairs at the edges of its tiles, through
+    the joint fit (same bars as test_scale_fit_parity)."""
+    lay = small_layer(din, dout, g, 3, seed=7 * din + dout)
+    prep = prepare_hessian(lay.H, lay.g)
+    ref32 = joint_scales(prep, lay.W, lay.S0, lay.Q0, lay.Z).astype(np.float32)
+    hess = jarq.prepare(lay.H, lay.g)
+    S = lay.S0.copy()
+    Fb, _ = jarq.fit_scales(hess, lay.W, S, lay.Q0, lay.Z, lay.bits, "joint")
+    hess.close()
+    assert np.all(np.abs(S.astype(np.float64) - ref32) <= 1e-6 * np.abs(ref32))
+    np.testing.assert_allclose(Fb, objective(prep, lay.W, lay.S0, lay.Q0, lay.Z), rtol=1e-6)
+
+
 @pytest.mark.parametrize("din,dout,g,bits", [(256, 80, 64, 3), (384, 64, 128, 3), (256, 48, 64, 4)])
 def test_multicode_probe_parity(jarq, din, dout, g, bits):
     lay = small_layer(din, dout, g, bits, seed=din + dout + 2)
