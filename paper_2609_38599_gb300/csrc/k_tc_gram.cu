@@ -13,16 +13,35 @@
 // integer dots G_t = sum_{m in grp i} c_j[m] D_t[j, m] and
 //     Gram_j[i,h] = 2^(E_ih - 9) (G_0 + G_1 2^-10 + G_2 2^-20 + G_3 2^-30)
 // in float64.  Only h <= i is computed; the block is mirrored.  The pair of
-// groups {i, G-1-i} of a 128-row tile holds G + 1 blocks; a CTA owns one of
-// `nparts` contiguous ranges of them (the host picks nparts so that the
-// CTAs fill the SMs' last wave).
+// groups {i, G-1-i} of a row tile holds G + 1 blocks.  Work items are 256 rows
+// and one of `nparts` contiguous ranges of a group pair's blocks, about four
+// blocks; each pair of CTAs stays on its SMs and takes every npairs-th item, the
+// row tiles of one range first (they share its digit tiles of H in L2).
 //
-// Roles: warp 0 TMA producer; warp 1 TMEM allocation and MMA issuer;
-// warps 2..9 epilogue: warp w reads TMEM lanes 32 (w % 4) .. and 32 of the
-// 64 columns of a unit; the two warps of a lane quarter add their partial
-// dots through shared memory at the end of each block.  One unit of work is
-// (h, column half of group i): 4 accumulators of 64 columns (one per digit
-// plane), double-buffered in 512 TMEM columns.
+// The CTAs of a pair (cta_group::2) share each MMA as in the sweep's product
+// (k_tc_target.cu): each loads the codes of its own 128 rows and two of the four
+// digit planes.  One unit of work is (h, column half of group i): 4 accumulators
+// of 64 columns (one per digit plane), double-buffered in 512 TMEM columns.
+//   warp 0       TMA producer of its CTA's tiles, onto the even CTA's barriers
+//   warp 1       TMEM allocation; in the even CTA the MMA issuer
+//   warps 2..17  epilogue: warp w reads TMEM lanes 32 (w % 4) .. and 16 of the
+//                64 columns of a unit; at the end of a block it leaves its
+//                partial dots in shared memory
+//   warps 18, 19 add the four partial dots of each row and write the entry of
+//                the block: in one of the epilogue warps the conversion and the
+//                stores (about 1000 cycles) would hold back the next unit's
+//                accumulator, which goes back to the issuer when all of them
+//                have read it
+//
+// What bounds it, per unit and CTA (clock64 in a copy): about 2000 cycles, of
+// which the MMAs are 1024 and the epilogue 900 to 1000 issue slots per
+// scheduler (64 digit sums a thread: an add, an integer multiply-add at half
+// rate); the rest is the hand-over between them (a ready barrier costs about
+// 150 cycles, the four TMEM loads 200 to 400).  Without the dots a launch on
+// 4096 x 4096, g = 128 takes 188 us, without the epilogue 162 us, in full 217
+// us; 1424 us on 4096 x 11008.  One CTA per tile with eight epilogue warps took
+// 325 and 2150 us; the block's sum in one of the epilogue warps 231 us, by
+// shared-memory atomics 252 us.
 #include <type_traits>
 
 #include "df.cuh"
@@ -33,25 +52,18 @@ namespace {
 
 constexpr int kTileA = 128 * 64 * 2;   // 128 code rows x 64 K (fp16)
 constexpr int kTileB = 64 * 64 * 2;    // 64 H rows x 64 K, one digit plane (fp16)
-constexpr int kStage = kTileA + 4 * kTileB;
-// Codes of group i are staged per tile as int8 when they fit (|q - z| <= 127,
-// up to 7 bits; then the freed shared memory holds a fourth pipeline stage)
-// and as int16 otherwise.
-template <bool WIDE>
-struct GramCfg {
-    using code_t = typename std::conditional<WIDE, int16_t, int8_t>::type;
-    static constexpr int kStages = WIDE ? 3 : 4;
-    static constexpr int kCodesBytes = 128 * 128 * (int)sizeof(code_t);
-};
-constexpr int kPartBytes = 2 * 4 * 128 * 8;  // int64 partial dots, double-buffered
-template <bool WIDE>
-constexpr int gram_smem() {
-    return 1024 + GramCfg<WIDE>::kStages * kStage + GramCfg<WIDE>::kCodesBytes + kPartBytes + 256;
-}
-constexpr int kThreads = 320;
+constexpr int kStage = kTileA + 2 * kTileB;
+constexpr int kStages = 5;
+constexpr int kDrainWarps = 16, kWriteWarps = 2;
+constexpr int kThreads = 32 * (2 + kDrainWarps + kWriteWarps);
+constexpr int kSlots = 4;              // blocks whose partial dots wait to be written
+constexpr int kPartBytes = kSlots * 4 * 2 * 128 * 8;   // int64 partial dots
+constexpr int kMaxTiles = 4096;        // row tile pairs whose activity is looked up
+constexpr int kSmem = 1024 + kStages * kStage + kPartBytes + 256 + kMaxTiles;
 // one MMA covers the four digit planes: they are consecutive 64-row tiles
-// in shared memory, and their accumulators consecutive 64-column blocks
-constexpr uint32_t kIdesc = tc::idesc_f16_f32(128, 256);
+// in the two CTAs' shared memory, and their accumulators consecutive
+// 64-column blocks
+constexpr uint32_t kIdesc = tc::idesc_f16_f32(256, 256);
 
 struct GramArgs {
     const uint8_t *Q;
@@ -61,83 +73,104 @@ struct GramArgs {
     float2 *gram;        // [p][G][G] as float pairs (hi, lo) of the float64 value
     int *status;
     int p, d, g, G, d_pad;
-    int nparts;          // block ranges per (row tile, group pair): blockIdx.z
+    int nparts;          // block ranges per (row tile pair, group pair)
+    int tiles, nitems;   // row tile pairs; tiles x group pairs x nparts
 };
 
-__device__ __forceinline__ int exact_int(float x) {
-    // x is an integer with |x| < 2^22: add 1.5 * 2^23 and read the low bits
-    return __float_as_int(x + 12582912.0f) - 0x4B400000;
-}
+// Units of a CTA pair: the blocks (i_lo, h <= i_lo), then (i_hi, h <= i_hi), each
+// as its column halves in turn.
+struct GramUnit {
+    int i_lo, i_hi, nhalf;
+    int gi, h, half;
+    __device__ __forceinline__ void start(int blk) {
+        const bool first = blk <= i_lo;
+        gi = first ? i_lo : i_hi;
+        h = first ? blk : blk - i_lo - 1;
+        half = 0;
+    }
+    __device__ __forceinline__ void next() {
+        if (++half < nhalf) return;
+        half = 0;
+        if (++h <= gi) return;
+        h = 0;
+        gi = i_hi;
+    }
+};
 
 // WIDE: codes wider than 4 bits, |D_t| < 2^24 converted by cvt and 64-bit
 // integer dots; otherwise |c| <= 15, |D_t| < 2^20 and every partial dot of
-// 8 terms fits in 32 bits.
+// 32 terms fits in 32 bits.
 template <bool WIDE>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_gram_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapS,
                    GramArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    using code_t = typename GramCfg<WIDE>::code_t;
-    constexpr int kStages = GramCfg<WIDE>::kStages;
-    constexpr int kCodesBytes = GramCfg<WIDE>::kCodesBytes;
-    code_t *codes = (code_t *)(smem + kStages * kStage);   // [128 rows][128]
-    long long *part = (long long *)(smem + kStages * kStage + kCodesBytes);   // [2][4][128]
-    uint64_t *bars = (uint64_t *)(smem + kStages * kStage + kCodesBytes + kPartBytes);
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 4);
+    long long *part = (long long *)(smem + kStages * kStage);   // [kSlots][4 warps][2][128]
+    uint64_t *bars = (uint64_t *)(smem + kStages * kStage + kPartBytes);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 4 + 2 * kSlots);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j0 = blockIdx.x * 128;
+    const int rank = (int)tc::cluster_rank();
+    uint8_t *live = smem + kStages * kStage + kPartBytes + 256;   // [tiles]
     const int G = a.G, g = a.g;
-    const int nhalf = g / 64, nkc = g / 64;   // column halves of group i; K chunks per block
-
-    {
-        int mine = 0;
-        if (threadIdx.x < 128 && j0 + (int)threadIdx.x < a.p)
-            mine = a.active ? a.active[j0 + threadIdx.x] : 1;
-        if (!__syncthreads_or(mine)) return;
-    }
-    // groups handled by this CTA and the unit list: for each group i (h = 0..i,
-    // half = 0..nhalf-1), K chunks kc = 0..nkc-1 per unit
-    const int i_lo = blockIdx.y, i_hi = G - 1 - blockIdx.y;
-    const int ngrp = (i_lo == i_hi) ? 1 : 2;
-    auto group_of = [&](int n) { return n == 0 ? i_lo : i_hi; };
-    const int units0 = (i_lo + 1) * nhalf;
-    const int nunits_pair = units0 + (ngrp == 2 ? (i_hi + 1) * nhalf : 0);
-    // this CTA's blocks: [nblk z / nparts, nblk (z + 1) / nparts) of the pair's
-    const int nblk = nunits_pair / nhalf;
-    const int ub = (nblk * (int)blockIdx.z / a.nparts) * nhalf;
-    const int nunits = (nblk * ((int)blockIdx.z + 1) / a.nparts) * nhalf - ub;
-    auto unit = [&](int u, int &gi, int &h, int &half) {
-        const int n = u < units0 ? 0 : 1;
-        const int r = u < units0 ? u : u - units0;
-        gi = group_of(n);
-        h = r / nhalf;
-        half = r % nhalf;
+    const int nkc = g / 64;                // K chunks per unit (and column halves of a group)
+    const int npairs = gridDim.x / 2, ngp = (G + 1) / 2;
+    // a row tile pair none of whose rows is active is skipped; both CTAs read
+    // the same flags
+    const bool flags = a.active && a.tiles <= kMaxTiles;
+    if (flags)
+        for (int t = warp; t < a.tiles; t += kThreads / 32) {
+            int mine = 0;
+            for (int r = lane; r < 256; r += 32)
+                if (t * 256 + r < a.p) mine |= a.active[t * 256 + r];
+            mine = __any_sync(0xffffffffu, mine);
+            if (lane == 0) live[t] = (uint8_t)mine;
+        }
+    // item -> first row of the tile pair, first unit and number of units
+    // [nblk z / nparts, nblk (z + 1) / nparts) of the group pair's blocks; 0
+    // units for a tile without active rows
+    auto item = [&](int it, int &jp, GramUnit &un) {
+        const int tile = it % a.tiles, gp = (it / a.tiles) % ngp, z = it / (a.tiles * ngp);
+        jp = tile * 256;
+        un.i_lo = gp;
+        un.i_hi = G - 1 - gp;
+        un.nhalf = nkc;
+        if (flags && !live[tile]) return 0;
+        const int nblk = un.i_lo == un.i_hi ? un.i_lo + 1 : G + 1;
+        const int blk0 = nblk * z / a.nparts;
+        un.start(blk0);
+        return (nblk * (z + 1) / a.nparts - blk0) * nkc;
     };
 
     auto full = [&](int s) { return tc::smem_u32(bars + s); };
     auto empty = [&](int s) { return tc::smem_u32(bars + kStages + s); };
     auto afull = [&](int b) { return tc::smem_u32(bars + 2 * kStages + b); };
     auto aempty = [&](int b) { return tc::smem_u32(bars + 2 * kStages + 2 + b); };
+    auto sfull = [&](int s) { return tc::smem_u32(bars + 2 * kStages + 4 + s); };
+    auto sfree = [&](int s) { return tc::smem_u32(bars + 2 * kStages + 4 + kSlots + s); };
     auto tileA = [&](int s) { return tc::smem_u32(smem + s * kStage); };
     auto tileB = [&](int s, int t) { return tc::smem_u32(smem + s * kStage + kTileA + t * kTileB); };
 
     if (threadIdx.x == 0) {
+        for (int s = 0; s < kSlots; ++s) {
+            tc::mbar_init(sfull(s), kDrainWarps);
+            tc::mbar_init(sfree(s), kWriteWarps);
+        }
         for (int s = 0; s < kStages; ++s) {
-            tc::mbar_init(full(s), 1);
+            tc::mbar_init(full(s), 1);      // the even CTA's: bytes of both CTAs
             tc::mbar_init(empty(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(afull(b), 1);
-            tc::mbar_init(aempty(b), 8);
+            tc::mbar_init(aempty(b), 2 * kDrainWarps);   // the even CTA's: both drains
         }
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
     if (warp == 1) {
-        tc::tmem_alloc(tc::smem_u32(tmem_slot), 512);
-        tc::tmem_relinquish();
+        tc::tmem_alloc_pair(tc::smem_u32(tmem_slot), 512);
+        tc::tmem_relinquish_pair();
     }
     if (warp == 0 && lane == 0) {
         tc::prefetch_tmap(&mapC);
@@ -145,207 +178,258 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     tc::tc_fence_before();
     __syncthreads();
+    tc::cluster_sync();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int nchunks = nunits * nkc;
 
-    if (warp == 0 && lane == 0) {
-        // ---------------- producer: per chunk, codes of group h and 4 digit planes
-        int issued = 0;
-        for (int c = 0; c < nchunks; ++c) {
-            const int s = c % kStages;
-            if (!tc::mbar_wait(empty(s), ((c / kStages) & 1) ^ 1) || *abort_flag) {
-                *abort_flag = 1;
-                break;
-            }
-            int gi, h, half;
-            unit(ub + c / nkc, gi, h, half);
-            const int kx = h * g + (c % nkc) * 64;
-            tc::mbar_expect_tx(full(s), kStage);
-            tc::tma_load_2d(tileA(s), &mapC, full(s), kx, j0);
+    if (warp == 0) {
+        // ---------------- producer: per chunk, codes of group h and two digit planes
+        bool ok = true;
+        const uint32_t full0 = tc::map_rank(full(0), 0);
+        GramUnit un;
+        int s = 0, ph = 1, nchunks = 0, jp;
+        for (int it = blockIdx.x / 2; it < a.nitems && ok; it += npairs) {
+            const int nunits = item(it, jp, un);
+            for (int u = 0; u < nunits && ok; ++u, un.next()) {
+                for (int kc = 0; kc < nkc; ++kc) {
+                    ok = tc::mbar_wait(empty(s), ph);
+                    if (!ok) break;
+                    if (tc::elect_one()) {
+                        if (rank == 0) tc::mbar_expect_tx(full(s), 2 * kStage);
+                        const uint32_t bar = full0 + 8 * s;
+                        const int kx = un.h * g + kc * 64;
+                        tc::tma_load_2d_pair(tileA(s), &mapC, bar, kx, jp + 128 * rank);
 #pragma unroll
-            for (int t = 0; t < 4; ++t)
-                tc::tma_load_2d(tileB(s, t), &mapS, full(s), kx, t * a.d_pad + gi * g + half * 64);
-            issued = c + 1;
-        }
-        for (int c = issued > kStages ? issued - kStages : 0; c < issued; ++c)
-            if (!tc::mbar_wait(full(c % kStages), (c / kStages) & 1)) *abort_flag = 1;
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer
-        for (int u = 0; u < nunits && !*abort_flag; ++u) {
-            const int b = u & 1;
-            if (!tc::mbar_wait(aempty(b), ((u >> 1) & 1) ^ 1)) {
-                *abort_flag = 1;
-                break;
-            }
-            tc::tc_fence_after();
-            for (int kc = 0; kc < nkc; ++kc) {
-                const int c = u * nkc + kc;
-                const int s = c % kStages;
-                if (!tc::mbar_wait(full(s), (c / kStages) & 1) || *abort_flag) {
-                    *abort_flag = 1;
-                    break;
-                }
-                tc::tc_fence_after();
-#pragma unroll
-                for (int sub = 0; sub < 4; ++sub) {
-                    const uint64_t ad = tc::sdesc_sw128(tileA(s)) + 2 * sub;
-                    const uint64_t bd = tc::sdesc_sw128(tileB(s, 0)) + 2 * sub;
-                    tc::mma_bf16(tmem + b * 256, ad, bd, kIdesc, (kc | sub) != 0);
-                }
-                tc::mma_commit(empty(s));
-            }
-            tc::mma_commit(afull(b));
-        }
-    } else if (warp >= 2) {
-        // ---------------- epilogue: exact integer dots with the codes of group i
-        const int q = warp & 3, cw = (warp - 2) >> 2;   // lane quarter, 32-column slice
-        const int rl = 32 * q + lane;           // row within the tile
-        const int row = j0 + rl;
-        int cur_g = -1, par = 0;
-        bool dead = false;                      // a wait gave up: skip work, keep the pair barriers
-        long long acc[4] = {0, 0, 0, 0};
-        for (int u = 0; u < nunits; ++u) {
-            int gi, h, half;
-            unit(ub + u, gi, h, half);
-            if (gi != cur_g) {
-                // stage this warp's columns of group gi (row rl written by its own thread)
-                __syncwarp();
-                for (int hf = 0; hf < nhalf; ++hf) {
-                    const int c0 = hf * 64 + cw * 32;
-                    if (row < a.p) {
-                        const int zz = a.Z[(size_t)row * G + gi];
-                        const uint4 *src = reinterpret_cast<const uint4 *>(a.Q + (size_t)row * a.d + gi * g + c0);
-                        for (int m16 = 0; m16 < 2; ++m16) {
-                            const uint4 v = src[m16];
-                            const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                            for (int k = 0; k < 16; ++k)
-                                codes[rl * 128 + c0 + m16 * 16 + k] =
-                                    (code_t)((int)((w4[k >> 2] >> (8 * (k & 3))) & 0xFFu) - zz);
-                        }
-                    } else {
-                        for (int m = 0; m < 32; ++m) codes[rl * 128 + c0 + m] = 0;
+                        for (int t = 0; t < 2; ++t)
+                            tc::tma_load_2d_pair(tileB(s, t), &mapS, bar, kx,
+                                                 (2 * rank + t) * a.d_pad + un.gi * g + un.half * 64);
+                    }
+                    __syncwarp();
+                    ++nchunks;
+                    if (++s == kStages) {
+                        s = 0;
+                        ph ^= 1;
                     }
                 }
-                __syncwarp();
-                cur_g = gi;
             }
-            const int b = u & 1;
-            if (!dead) {
-                bool w = tc::mbar_wait(afull(b), (u >> 1) & 1);
-                w = __shfl_sync(0xffffffffu, w && !*abort_flag, 0);
+        }
+        // do not leave before the MMAs have consumed the stages filled here:
+        // no copy or commit is in flight afterwards
+        for (int n = max(0, nchunks - kStages); n < nchunks && ok; ++n)
+            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
+        if (!ok) *abort_flag = 1;
+    } else if (warp == 1) {
+        // ---------------- MMA issuer of the pair
+        if (rank == 0) {
+            const uint64_t ad0 = tc::sdesc_sw128(tileA(0)), bd0 = tc::sdesc_sw128(tileB(0, 0));
+            int s = 0, ph = 0;
+            bool ok = true;
+            GramUnit un;
+            int jp, total = 0;
+            for (int it = blockIdx.x / 2; it < a.nitems; it += npairs) total += item(it, jp, un);
+            for (int u = 0; u < total && ok; ++u) {
+                const int b = u & 1;
+                int s1 = s + 1, ph1 = ph;
+                if (s1 == kStages) {
+                    s1 = 0;
+                    ph1 ^= 1;
+                }
+                ok = tc::mbar_wait(full(s), ph);
+                if (nkc == 2) ok = tc::mbar_wait(full(s1), ph1) && ok;
+                ok = tc::mbar_wait(aempty(b), ((u >> 1) & 1) ^ 1) && ok;
+                if (!ok) break;
                 tc::tc_fence_after();
-                if (!w) {
-                    *abort_flag = 1;
-                    dead = true;
+                if (tc::elect_one()) {
+                    const uint64_t o = (uint64_t)(s * (kStage >> 4));
+#pragma unroll
+                    for (int sub = 0; sub < 4; ++sub)
+                        tc::mma_f16_pair(tmem + b * 256, ad0 + o + 2 * sub, bd0 + o + 2 * sub, kIdesc, sub != 0);
+                    tc::mma_commit_pair(empty(s));
+                    if (nkc == 2) {
+                        const uint64_t o1 = (uint64_t)(s1 * (kStage >> 4));
+#pragma unroll
+                        for (int sub = 0; sub < 4; ++sub)
+                            tc::mma_f16_pair(tmem + b * 256, ad0 + o1 + 2 * sub, bd0 + o1 + 2 * sub, kIdesc, 1);
+                        tc::mma_commit_pair(empty(s1));
+                    }
+                    tc::mma_commit_pair(afull(b));
+                }
+                __syncwarp();
+                s = s1;
+                ph = ph1;
+                if (nkc == 2 && ++s == kStages) {
+                    s = 0;
+                    ph ^= 1;
                 }
             }
-            if (!dead) {
-                const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + b * 256 + cw * 32;
-                const code_t *crow = codes + rl * 128 + half * 64 + cw * 32;
-                int cr[32];
+            if (!ok) *abort_flag = 1;
+        }
+    } else if (warp < 2 + kDrainWarps) {
+        // ---------------- epilogue: exact integer dots with the codes of group i
+        const int q = warp & 3, cq = (warp - 2) >> 2;   // lane quarter, 16-column quarter
+        const int rl = 32 * q + lane;           // row within the tile
+        const uint32_t released = tc::map_rank(aempty(0), 0);
+        GramUnit un;
+        int z = 0, jp, ug = 0, nb = 0;          // ug, nb: units, blocks of this pair so far
+        uint32_t q4[2][4] = {};                 // this warp's codes of group i, both halves
+        bool ok = true;
+        typedef typename std::conditional<WIDE, long long, int>::type acc_t;
+        acc_t acc[4] = {0, 0, 0, 0};
+        for (int it = blockIdx.x / 2; it < a.nitems && ok; it += npairs) {
+            const int nunits = item(it, jp, un);
+            const int rc = min(jp + 128 * rank + rl, a.p - 1);
+            int cur_g = -1;
+            for (int u = 0; u < nunits; ++u, ++ug, un.next()) {
+                if (un.gi != cur_g) {
+                    cur_g = un.gi;
+                    z = a.Z[(size_t)rc * G + cur_g];
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+                        if (hf < nkc) {
+                            const uint4 v = *reinterpret_cast<const uint4 *>(
+                                a.Q + (size_t)rc * a.d + cur_g * g + hf * 64 + cq * 16);
+                            q4[hf][0] = v.x; q4[hf][1] = v.y; q4[hf][2] = v.z; q4[hf][3] = v.w;
+                        }
+                }
+                int c[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const uint32_t w = un.half ? q4[1][e >> 2] : q4[0][e >> 2];
+                    c[e] = (int)__byte_perm(w, 0, 0x4440 | (e & 3)) - z;
+                }
+                const int b = ug & 1;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(afull(b), (ug >> 1) & 1));
+                if (!ok) break;
+                tc::tc_fence_after();
+                const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + b * 256 + cq * 16;
+                auto release = [&]() {
+                    // every digit sum of this unit is in registers
+                    tc::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive_cluster(released + 8 * b);
+                };
                 if constexpr (WIDE) {
 #pragma unroll
-                    for (int e = 0; e < 32; e += 8) {
-                        const int4 pk = *reinterpret_cast<const int4 *>(crow + e);
-                        const int w4[4] = {pk.x, pk.y, pk.z, pk.w};
+                    for (int t = 0; t < 4; t += 2) {
+                        uint32_t v[2][16];
+                        tc::tmem_ld16(base + t * 64, v[0]);
+                        tc::tmem_ld16(base + (t + 1) * 64, v[1]);
+                        tc::tmem_wait_ld();
+                        if (t == 2) release();
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            cr[e + 2 * k] = (int)(int16_t)(w4[k] & 0xFFFF);
-                            cr[e + 2 * k + 1] = w4[k] >> 16;
-                        }
+                        for (int k = 0; k < 2; ++k)
+#pragma unroll
+                            for (int e = 0; e < 16; ++e)
+                                acc[t + k] += (long long)c[e] * __float2int_rn(__uint_as_float(v[k][e]));
                     }
                 } else {
+                    uint32_t v[4][16];
 #pragma unroll
-                    for (int e = 0; e < 32; e += 16) {
-                        const int4 pk = *reinterpret_cast<const int4 *>(crow + e);
-                        const int w4[4] = {pk.x, pk.y, pk.z, pk.w};
+                    for (int t = 0; t < 4; ++t) tc::tmem_ld16(base + t * 64, v[t]);
+                    tc::tmem_wait_ld();
+                    release();
+                    // D is an integer, |D| < 2^22: the bits of D + 1.5 2^23 are
+                    // 0x4B400000 + D; the offset's share is taken off once
+                    // (modulo 2^32; the dot itself fits)
+                    int cs = 0;
 #pragma unroll
-                        for (int k = 0; k < 16; ++k)
-                            cr[e + k] = (int)(int8_t)((w4[k >> 2] >> (8 * (k & 3))) & 0xFF);
+                    for (int e = 0; e < 16; ++e) cs += c[e];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        uint32_t p0 = 0, p1 = 0;
+#pragma unroll
+                        for (int e = 0; e < 16; e += 2) {
+                            float x0, x1;
+                            tc::f2_get(tc::f2_add(tc::f2(__uint_as_float(v[t][e]), __uint_as_float(v[t][e + 1])),
+                                                  tc::f2(12582912.0f)), x0, x1);
+                            p0 += (uint32_t)c[e] * __float_as_uint(x0);
+                            p1 += (uint32_t)c[e + 1] * __float_as_uint(x1);
+                        }
+                        acc[t] += (int)(p0 + p1 - 0x4B400000u * (uint32_t)cs);
                     }
                 }
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    uint32_t v0[16], v1[16];
-                    tc::tmem_ld16(base + t * 64, v0);
-                    tc::tmem_ld16(base + t * 64 + 16, v1);
-                    tc::tmem_wait_ld();
-                    if (t == 3) {
-                        // every digit of this unit is in registers
-                        tc::tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(aempty(b));
-                    }
-                    if (WIDE) {
-                        long long p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-#pragma unroll
-                        for (int e = 0; e < 16; e += 2) {
-                            p0 += (long long)cr[e] * __float2int_rn(__uint_as_float(v0[e]));
-                            p1 += (long long)cr[e + 1] * __float2int_rn(__uint_as_float(v0[e + 1]));
-                            p2 += (long long)cr[16 + e] * __float2int_rn(__uint_as_float(v1[e]));
-                            p3 += (long long)cr[17 + e] * __float2int_rn(__uint_as_float(v1[e + 1]));
-                        }
-                        acc[t] += (p0 + p1) + (p2 + p3);
+                if (un.half == nkc - 1) {
+                    // two digits to a 64-bit integer (four for narrow codes:
+                    // |acc_t| < 128 * 15 * 2^20 < 2^31 over all columns)
+                    const long long hi = (long long)acc[0] * (1 << 10) + acc[1];
+                    const long long lo = (long long)acc[2] * (1 << 10) + acc[3];
+                    const int slot = nb % kSlots;
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(sfree(slot), ((nb / kSlots) & 1) ^ 1));
+                    if (!ok) break;
+                    long long *pp = part + (size_t)((slot * 4 + cq) * 2) * 128 + rl;
+                    if constexpr (WIDE) {
+                        pp[0] = hi;
+                        pp[128] = lo;
                     } else {
-                        int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-#pragma unroll
-                        for (int e = 0; e < 16; e += 2) {
-                            p0 += cr[e] * exact_int(__uint_as_float(v0[e]));
-                            p1 += cr[e + 1] * exact_int(__uint_as_float(v0[e + 1]));
-                            p2 += cr[16 + e] * exact_int(__uint_as_float(v1[e]));
-                            p3 += cr[17 + e] * exact_int(__uint_as_float(v1[e + 1]));
-                        }
-                        acc[t] += (long long)((p0 + p1) + (p2 + p3));
+                        pp[0] = hi * (1 << 20) + lo;
                     }
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(sfull(slot));
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) acc[t] = 0;
+                    ++nb;
                 }
             }
-            if (half == nhalf - 1) {
-                // the pair of warps of this lane quarter adds its partial dots
-                long long *pp = part + (size_t)par * 4 * 128;
-                if (cw == 1) {
+        }
+        if (!ok) *abort_flag = 1;
+    } else {
+        // ---------------- write the finished blocks, 64 rows a warp
+        const int r0 = 64 * (warp - 2 - kDrainWarps) + lane;
+        GramUnit un;
+        int jp, nb = 0;
+        bool ok = true;
+        for (int it = blockIdx.x / 2; it < a.nitems && ok; it += npairs) {
+            const int nblk = item(it, jp, un) / nkc;
+            for (int k = 0; k < nblk; ++k, ++nb) {
+                const int E = a.expo[un.gi * G + un.h], slot = nb % kSlots;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(sfull(slot), (nb / kSlots) & 1));
+                if (!ok) break;
+                const long long *pp = part + (size_t)slot * 4 * 2 * 128;
+                float2 v2[2];
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) pp[t * 128 + rl] = acc[t];
-                }
-                asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");
-                if (cw == 0 && row < a.p && !dead) {
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) acc[t] += pp[t * 128 + rl];
-                    const int E = a.expo[gi * G + h];
+                for (int r = 0; r < 2; ++r) {
+                    const long long *pr = pp + r0 + 32 * r;
+                    const long long s0 = (pr[0] + pr[256]) + (pr[512] + pr[768]);
                     double v;
-                    if constexpr (!WIDE) {
-                        // |acc_t| < 128 * 15 * 2^20 < 2^31: the digit sum is one
-                        // exact 64-bit integer, converted with a single rounding
-                        // (two float64 operations instead of eleven; float64 is a
-                        // narrow pipe on this GPU)
-                        const long long V = acc[0] * (1LL << 30) + acc[1] * (1LL << 20) +
-                                            acc[2] * (1LL << 10) + acc[3];
-                        v = __ll2double_rn(V) *
-                            __longlong_as_double((long long)(E - 39 + 1023) << 52);
+                    if constexpr (WIDE) {
+                        const long long s1 = (pr[128] + pr[384]) + (pr[640] + pr[896]);
+                        v = ldexp((double)s0, E - 19) + ldexp((double)s1, E - 39);
                     } else {
-                        v = ldexp((double)acc[0] + ldexp((double)acc[1], -10) +
-                                      ldexp((double)acc[2], -20) + ldexp((double)acc[3], -30),
-                                  E - 9);
+                        // one exact 64-bit integer, converted with a single
+                        // rounding (two float64 operations; float64 is a narrow
+                        // pipe on this GPU)
+                        v = __ll2double_rn(s0) * __longlong_as_double((long long)(E - 39 + 1023) << 52);
                     }
                     // stored once as the float pair the scale solve works on
                     const DF vp = split_double(v);
-                    const float2 v2 = make_float2(vp.h, vp.l);
-                    float2 *gr = a.gram + (size_t)row * G * G;
-                    gr[(size_t)gi * G + h] = v2;
-                    gr[(size_t)h * G + gi] = v2;
+                    v2[r] = make_float2(vp.h, vp.l);
                 }
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(sfree(slot));
 #pragma unroll
-                for (int t = 0; t < 4; ++t) acc[t] = 0;
-                par ^= 1;
+                for (int r = 0; r < 2; ++r) {
+                    const int row = jp + 128 * rank + r0 + 32 * r;
+                    if (row < a.p) {
+                        float2 *gr = a.gram + (size_t)row * G * G;
+                        gr[(size_t)un.gi * G + un.h] = v2[r];
+                        gr[(size_t)un.h * G + un.gi] = v2[r];
+                    }
+                }
+                un.half = nkc - 1;      // on to the next block
+                un.next();
             }
         }
+        if (!ok) *abort_flag = 1;
     }
+    // neither CTA leaves while the other may still read its shared memory,
+    // signal its barriers or hold TMEM of the pair
     tc::tc_fence_before();
+    __syncwarp();
     __syncthreads();
+    tc::cluster_sync();
     if (warp == 1) {
         tc::tc_fence_after();
-        tc::tmem_dealloc(tmem, 512);
+        tc::tmem_dealloc_pair(tmem, 512);
     }
     if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, ST_TIMEOUT);
 }
@@ -487,33 +571,33 @@ cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, con
                            int p, int p_pad, int d, int d_pad, int g, int bits, int *status,
                            cudaStream_t s) {
     static std::atomic<unsigned long long> attr_narrow{0}, attr_wide{0};
-    cudaError_t e = set_max_dynamic_smem((const void *)tc_gram_kernel<false>, gram_smem<false>(),
-                                         attr_narrow);
+    cudaError_t e = set_max_dynamic_smem((const void *)tc_gram_kernel<false>, kSmem, attr_narrow);
     if (e == cudaSuccess)
-        e = set_max_dynamic_smem((const void *)tc_gram_kernel<true>, gram_smem<true>(), attr_wide);
+        e = set_max_dynamic_smem((const void *)tc_gram_kernel<true>, kSmem, attr_wide);
     if (e != cudaSuccess) return e;
     const int G = d / g;
-    // parts per (row tile, group pair), 1 to 4: the fewest waves of CTAs,
-    // each wave as long as one part of the pair's blocks plus a fixed cost
-    // of about 5 % of the whole pair
-    const int nsm = num_sms();
-    const long long ctas = (long long)(p_pad / 128) * ((G + 1) / 2);
+    // ranges per (row tile pair, group pair): the fewest blocks for the busiest
+    // CTA pair, each item costing about a sixth of a block beside its blocks
+    // (its rows' codes of the group)
+    const int npairs = num_sms() / 2, tiles = (p + 255) / 256, ngp = (G + 1) / 2;
     int nparts = 1;
     double best = 0.0;
-    for (int n = 1; n <= 4 && n <= G + 1; ++n) {
-        const long long waves = (ctas * n + nsm - 1) / nsm;
-        const double t = (double)waves * (1.0 / n + 0.05);
+    for (int n = 1; n <= G + 1; ++n) {
+        const long long rounds = ((long long)tiles * ngp * n + npairs - 1) / npairs;
+        const double t = (double)rounds * ((double)(G + 1) / n + 0.17);
         if (n == 1 || t < best - 1e-9) {
             best = t;
             nparts = n;
         }
     }
-    GramArgs a{Q, Z, expo, active, gram, status, p, d, g, G, d_pad, nparts};
-    dim3 grid(p_pad / 128, (G + 1) / 2, nparts);
+    const long long items = (long long)tiles * ngp * nparts;
+    if (items > 0x7fffffff) return cudaErrorInvalidValue;
+    GramArgs a{Q, Z, expo, active, gram, status, p, d, g, G, d_pad, nparts, tiles, (int)items};
+    const dim3 grid(2 * (items < npairs ? (int)items : npairs));
     if (bits <= 4)
-        tc_gram_kernel<false><<<grid, kThreads, gram_smem<false>(), s>>>(mapC, mapS, a);
+        tc_gram_kernel<false><<<grid, kThreads, kSmem, s>>>(mapC, mapS, a);
     else
-        tc_gram_kernel<true><<<grid, kThreads, gram_smem<true>(), s>>>(mapC, mapS, a);
+        tc_gram_kernel<true><<<grid, kThreads, kSmem, s>>>(mapC, mapS, a);
     return cudaGetLastError();
 }
 
