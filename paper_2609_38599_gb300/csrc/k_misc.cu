@@ -22,8 +22,9 @@ __global__ void validate_kernel(const uint8_t *__restrict__ Q, const int32_t *__
     if (threadIdx.x == 0 && flag) atomicOr(status, flag);
 }
 
-// The same check, sixteen codes per thread (Q 16-byte aligned, nq a
-// multiple of 16).
+// The same check for Q 16-byte aligned and nq a multiple of 16: qmax is 2^b - 1,
+// so a code is above it iff it has a bit outside qmax; the codes are OR-ed, 64
+// per thread and iteration.
 __global__ void validate16_kernel(const uint4 *__restrict__ Q16, const int32_t *__restrict__ Z,
                                   size_t nq16, size_t nz, int qmax, int *status) {
     __shared__ int flag;
@@ -31,17 +32,23 @@ __global__ void validate16_kernel(const uint4 *__restrict__ Q16, const int32_t *
     __syncthreads();
     int local = 0;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nq16; i += stride) {
-        const uint4 v = Q16[i];
-        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+    const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t seen = 0;
+    size_t i = i0;
+    for (; i + 3 * stride < nq16; i += 4 * stride) {
+        uint4 v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < 4; ++k) v[k] = Q16[i + k * stride];
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-                if ((int)((w4[k] >> (8 * b)) & 0xFFu) > qmax) local |= ST_BAD_CODE;
+        for (int k = 0; k < 4; ++k) seen |= (v[k].x | v[k].y) | (v[k].z | v[k].w);
     }
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nz; i += stride)
-        if (Z[i] < 0 || Z[i] > qmax) local |= ST_BAD_ZERO;
+    for (; i < nq16; i += stride) {
+        const uint4 v = Q16[i];
+        seen |= (v.x | v.y) | (v.z | v.w);
+    }
+    if (seen & ~(0x01010101u * (uint32_t)qmax)) local |= ST_BAD_CODE;
+    for (size_t k = i0; k < nz; k += stride)
+        if (Z[k] < 0 || Z[k] > qmax) local |= ST_BAD_ZERO;
     if (local) atomicOr(&flag, local);
     __syncthreads();
     if (threadIdx.x == 0 && flag) atomicOr(status, flag);
@@ -134,8 +141,9 @@ cudaError_t set_max_dynamic_smem(const void *func, int bytes,
 cudaError_t launch_validate(const uint8_t *Q, const int32_t *Z, int p, int d, int G, int qmax,
                             int *status, cudaStream_t s) {
     size_t nq = (size_t)p * d, nz = (size_t)p * G;
-    int blocks = (int)((nq + 255) / 256);
-    if (blocks > 4 * num_sms()) blocks = 4 * num_sms();
+    size_t work = nq % 16 == 0 ? nq / 16 : nq;
+    if (work < nz) work = nz;
+    int blocks = (int)((work + 255) / 256 < (size_t)(8 * num_sms()) ? (work + 255) / 256 : 8 * num_sms());
     if (blocks < 1) blocks = 1;
     if (nq % 16 == 0 && (uintptr_t)Q % 16 == 0)
         validate16_kernel<<<blocks, 256, 0, s>>>(reinterpret_cast<const uint4 *>(Q), Z, nq / 16, nz,

@@ -55,6 +55,61 @@ def test_dequantize_bit_exact(jarq, dtype):
     assert np.array_equal(out, np.asarray(ref, dtype=np.float64))
 
 
+def _offset_copy(a, off):
+    """A contiguous device copy of `a` whose data starts `off` elements into its storage."""
+    t = torch.as_tensor(a)
+    buf = torch.empty(t.numel() + off, dtype=t.dtype, device="cuda")[off:].view(t.shape)
+    return buf.copy_(t)
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float16", "bfloat16"])
+@pytest.mark.parametrize("g,off", [(64, 0), (64, 1), (48, 0), (24, 0)])
+def test_dequantize_rounds_once_over_the_whole_range(jarq, dtype, g, off):
+    """The 16-code and the single-code kernel (misaligned codes, g not a
+    multiple of 16) on scales from subnormal to overflowing, products at and
+    next to ties: one rounding of the exact product."""
+    rng = np.random.default_rng(g + off)
+    dout, din, bits = 67, 8 * g, 8
+    G = din // g
+    e = rng.integers(-40, 20, size=(dout, G)).astype(np.float64)
+    # the oracle's bfloat16 rounding has no subnormals and no overflow: scales
+    # from 2^-126 there, and 2^128 and above is infinite
+    e[:20] = rng.integers(-126 if dtype == "bfloat16" else -149, 128, size=(20, G))
+    S = (rng.choice([-1.0, 1.0], size=(dout, G)) * rng.uniform(1, 2, size=(dout, G)) * 2.0 ** e).astype(np.float32)
+    S[20:40] = (rng.integers(1, 1 << 12, size=(20, G)) * 2.0 ** -20).astype(np.float32)   # many ties
+    S[40, :3] = [0.0, np.inf, -np.inf]
+    Q = rng.integers(0, 256, size=(dout, din), dtype=np.uint8)
+    Z = rng.integers(0, 256, size=(dout, G)).astype(np.int32)
+    with np.errstate(over="ignore", invalid="ignore"):
+        ref = np.asarray(dequantize_cast(S, Q, Z, g, dtype), dtype=np.float64)
+    if dtype == "bfloat16":
+        ref[np.abs(ref) >= 2.0 ** 128] *= np.inf
+    t = lambda a: torch.as_tensor(a).cuda()
+    out = jarq.dequantize(t(S), _offset_copy(Q, off), t(Z), g, bits, dtype).double().cpu().numpy()
+    np.testing.assert_array_equal(out, ref)
+
+
+@pytest.mark.parametrize("g,off", [(64, 0), (64, 1), (30, 0)])
+def test_canonicalize_paths_agree(jarq, g, off):
+    S, Q, Z = _signed_state(45, 5 * g, g, 4, seed=g)
+    S2, Q2, Z2 = canonicalize(S.astype(np.float64), Q, Z, 4)
+    Sd, Zd, Qd = torch.as_tensor(S).cuda(), torch.as_tensor(Z).cuda(), _offset_copy(Q, off)
+    jarq.canonicalize(Sd, Qd, Zd, g, 4)
+    assert np.array_equal(Sd.cpu().numpy(), S2.astype(np.float32))
+    assert np.array_equal(Qd.cpu().numpy(), Q2) and np.array_equal(Zd.cpu().numpy(), Z2)
+
+
+@pytest.mark.parametrize("bits", [1, 2, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("off", [0, 1])
+def test_pack_codes_whole_words(jarq, bits, off):
+    """Rows of a multiple of 32 codes: 32 codes a thread, or the general kernel
+    for misaligned codes."""
+    rng = np.random.default_rng(bits)
+    Q = rng.integers(0, 1 << bits, size=(37, 96), dtype=np.uint8)
+    got = jarq.pack_codes(_offset_copy(Q, off), bits).cpu().numpy().view(np.uint32)
+    assert np.array_equal(got, pack_codes(Q, bits))
+
+
 @pytest.mark.parametrize("bits", [2, 3, 4, 5, 6, 7, 8])
 def test_pack_codes_bit_exact(jarq, bits):
     rng = np.random.default_rng(bits)
@@ -77,6 +132,11 @@ def test_writeback_rejects_bad_input(jarq):
     with pytest.raises(jarq.JarqError):
         jarq.canonicalize(Sd, Qd, Zd, 64, 3)
     assert torch.equal(Sd, S0)
+    # the cast leaves its output alone as well
+    Wd = torch.full((8, 128), 7.0, dtype=torch.float16, device="cuda")
+    assert lib.jarq_dequantize(Sd.data_ptr(), Qd.data_ptr(), Zd.data_ptr(), 8, 128, 64, 3, 1,
+                               Wd.data_ptr(), None) == jarq.JARQ_ERR_ARG
+    assert bool((Wd == 7.0).all())
 
 
 def test_ridge_acceptance_matches_oracle(jarq):
