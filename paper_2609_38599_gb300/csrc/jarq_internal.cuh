@@ -37,11 +37,9 @@ __host__ __device__ constexpr int sweep_block(int g) { return 256 / g; }
 __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // Layout of one group's factor L_i = R_i^T as the Babai kernel reads it
-// (k_babai.cu), float32.  Eight lanes hold a row's g coordinates: lane k of
-// them owns l = 32 a + 4 k + b, a = 0 .. g/32 - 1, b = 0 .. 3 (a quad per a).
-//   rows   h = 0 .. g - 1: h/32 + 1 vectors a of 32 floats, entry (4 k + b)
-//          L[h][32 a + 4 k + b], zero from column 4 (h/4) on (h's own quad
-//          and everything above the diagonal)
+// (k_babai.cu), float32:
+//   rows   h = 0 .. g - 1: columns 0 .. 32 (h/32 + 1) - 1 of L[h], zero from
+//          column 4 (h/4) on (h's own quad and everything above the diagonal)
 //   tri    per quad 4 q .. 4 q + 3 eight floats: L[3][2], L[3][1], L[3][0],
 //          L[2][1], L[2][0], L[1][0] of the quad's own block, 0, 0
 //   diag   L[l][l];  rdiag  1 / L[l][l]
