@@ -105,88 +105,93 @@ bool is_device_ptr(const void *ptr) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Lays arrays out in one allocation: a first pass without memory adds up the
+// sizes, a second one hands out the pieces.  One cudaMalloc and cudaFree
+// instead of one per array: on a 4096 x 4096 layer, preparing a Hessian went
+// from 3.5 to 3.1 ms, its first layer from 0.74 to 0.2 ms above a later one,
+// and the release from 1.8 to 1.1 ms.
+struct Arena {
+    char *base = nullptr;
+    size_t used = 0;
+    template <class T>
+    void take(T *&ptr, size_t n) {
+        ptr = base ? reinterpret_cast<T *>(base + used) : nullptr;
+        used += (n * sizeof(T) + 255) / 256 * 256;
+    }
+};
+
 void free_ws(Workspace &w) {
-    cudaFree(w.Hr);
-    cudaFree(w.r);
-    cudaFree(w.gram);
-    cudaFree(w.rhs);
-    cudaFree(w.t_hi);
-    cudaFree(w.t_lo);
-    cudaFree(w.Pt_hi);
-    cudaFree(w.Pt_lo);
-    cudaFree(w.wdig);
-    cudaFree(w.wexp);
-    cudaFree(w.Phi);
-    cudaFree(w.Plo);
-    cudaFree(w.wHw);
-    cudaFree(w.aux);
-    cudaFree(w.own);
-    cudaFree(w.L_prev);
-    cudaFree(w.L_host);
-    cudaFree(w.L_final);
-    cudaFree(w.active);
-    cudaFree(w.iters);
-    cudaFree(w.accepted);
-    cudaFree(w.ridge);
-    cudaFree(w.rstat);
+    cudaFree(w.mem);
     cudaFree(w.sW);
     cudaFree(w.sS);
     cudaFree(w.sQ);
     cudaFree(w.sZ);
-    cudaFree(w.rplanes);
-    cudaFree(w.cplane);
     w = Workspace{};
 }
 
-cudaError_t ensure_ws(jarq_hessian *h, int p) {
-    Workspace &w = h->ws;
-    if (p <= w.cap_rows) return cudaSuccess;
-    free_ws(w);
-    const size_t d = h->din, G = h->G, g = h->g;
-    const int p_pad = round_up(p, 128);
-    cudaError_t e;
-    if ((e = dalloc(&w.rplanes, (size_t)3 * p_pad * h->d_pad)) != cudaSuccess) return e;
-    if ((e = cudaMemset(w.rplanes, 0, (size_t)3 * p_pad * h->d_pad * 2)) != cudaSuccess) return e;
-    if ((e = make_tmap_bf16(&w.mapR, w.rplanes, (uint64_t)3 * p_pad, h->d_pad, 128)) != cudaSuccess)
-        return e;
-    if ((e = dalloc(&w.cplane, (size_t)p_pad * h->d_pad)) != cudaSuccess) return e;
-    if ((e = cudaMemset(w.cplane, 0, (size_t)p_pad * h->d_pad * 2)) != cudaSuccess) return e;
-    if ((e = make_tmap_f16(&w.mapC, w.cplane, (uint64_t)p_pad, h->d_pad, 128)) != cudaSuccess)
-        return e;
-    if ((e = dalloc(&w.wdig, (size_t)6 * p_pad * h->d_pad)) != cudaSuccess) return e;
-    if ((e = cudaMemset(w.wdig, 0, (size_t)6 * p_pad * h->d_pad * 2)) != cudaSuccess) return e;
-    if ((e = make_tmap_bf16(&w.mapWd, w.wdig, (uint64_t)4 * p_pad, h->d_pad, 128, 32)) != cudaSuccess)
-        return e;
-    if ((e = make_tmap_bf16(&w.mapPd, w.wdig, (uint64_t)6 * p_pad, h->d_pad, 128)) != cudaSuccess)
-        return e;
-    w.p_pad = p_pad;
-    if ((e = dalloc(&w.Hr, (size_t)p * d)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.r, (size_t)p * d)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.gram, (size_t)p * G * G)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.rhs, (size_t)p * G)) != cudaSuccess) return e;
+void layout_ws(Arena &m, Workspace &w, const jarq_hessian *h, int p, int p_pad) {
+    const size_t d = h->din, G = h->G, pd = (size_t)p_pad * h->d_pad, np = p;
+    m.take(w.rplanes, 3 * pd);
+    m.take(w.cplane, pd);
+    m.take(w.wdig, 6 * pd);
+    m.take(w.Hr, np * d);
+    m.take(w.r, np * d);
+    m.take(w.gram, np * G * G);
+    m.take(w.rhs, np * G);
     // partials of a product: one slot of 256 columns (a block of the sweep) a
     // row, or more slots while the CTAs of 128 rows x 64 columns fit the SMs
     // (target_splits), for this row count and every smaller one
     size_t t_len = (size_t)p_pad * 256;
     if (t_len < (size_t)num_sms() * 128 * 64) t_len = (size_t)num_sms() * 128 * 64;
-    if ((e = dalloc(&w.t_hi, t_len)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.t_lo, t_len)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.Pt_hi, (size_t)p * d)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.Pt_lo, (size_t)p * d)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.wexp, (size_t)p * G)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.Phi, (size_t)p * d)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.Plo, (size_t)p * d)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.wHw, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.aux, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.own, (size_t)p * G)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.L_prev, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.L_host, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.L_final, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.active, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.iters, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.accepted, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.ridge, (size_t)p)) != cudaSuccess) return e;
-    if ((e = dalloc(&w.rstat, (size_t)p)) != cudaSuccess) return e;
+    m.take(w.t_hi, t_len);
+    m.take(w.t_lo, t_len);
+    m.take(w.Pt_hi, np * d);
+    m.take(w.Pt_lo, np * d);
+    m.take(w.wexp, np * G);
+    m.take(w.Phi, np * d);
+    m.take(w.Plo, np * d);
+    m.take(w.wHw, np);
+    m.take(w.aux, np);
+    m.take(w.own, np * G);
+    m.take(w.L_prev, np);
+    m.take(w.L_host, np);
+    m.take(w.L_final, np);
+    m.take(w.active, np);
+    m.take(w.iters, np);
+    m.take(w.accepted, np);
+    m.take(w.ridge, np);
+    m.take(w.rstat, np);
+}
+
+cudaError_t ensure_ws(jarq_hessian *h, int p, cudaStream_t st) {
+    Workspace &w = h->ws;
+    if (p <= w.cap_rows) return cudaSuccess;
+    free_ws(w);
+    const int p_pad = round_up(p, 128);
+    Arena m;
+    layout_ws(m, w, h, p, p_pad);
+    cudaError_t e = dalloc(&m.base, m.used);
+    if (e != cudaSuccess) return e;
+    w.mem = m.base;
+    m.used = 0;
+    layout_ws(m, w, h, p, p_pad);
+    // columns beyond din are read as zeros by the products; rows beyond p only
+    // reach results that nobody reads
+    if (h->d_pad != h->din) {
+        const size_t pd = (size_t)p_pad * h->d_pad;
+        if ((e = cudaMemsetAsync(w.rplanes, 0, 3 * pd * 2, st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(w.cplane, 0, pd * 2, st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(w.wdig, 0, 6 * pd * 2, st)) != cudaSuccess) return e;
+    }
+    if ((e = make_tmap_bf16(&w.mapR, w.rplanes, (uint64_t)3 * p_pad, h->d_pad, 128)) != cudaSuccess)
+        return e;
+    if ((e = make_tmap_f16(&w.mapC, w.cplane, (uint64_t)p_pad, h->d_pad, 128)) != cudaSuccess)
+        return e;
+    if ((e = make_tmap_bf16(&w.mapWd, w.wdig, (uint64_t)4 * p_pad, h->d_pad, 128, 32)) != cudaSuccess)
+        return e;
+    if ((e = make_tmap_bf16(&w.mapPd, w.wdig, (uint64_t)6 * p_pad, h->d_pad, 128)) != cudaSuccess)
+        return e;
+    w.p_pad = p_pad;
     w.cap_rows = p;
     return cudaSuccess;
 }
@@ -252,6 +257,25 @@ cudaError_t stage_layer(jarq_hessian *h, const float *W, const float *S, const u
     return e;
 }
 
+// The arrays of a prepared Hessian (one allocation, h->mem).
+void layout_hessian(Arena &m, jarq_hessian *h) {
+    const size_t d = h->din, G = h->G, g = h->g, pd = (size_t)h->d_pad * h->d_pad;
+    m.take(h->Hs, d * d);
+    m.take(h->Hplanes, 3 * pd);
+    m.take(h->Hdig8, 6 * pd);
+    m.take(h->Hdig10, 4 * pd);
+    m.take(h->expo, G * G);
+    m.take(h->Lf, G * factor_floats((int)g));
+    m.take(h->L64, G * g * g);
+    m.take(h->Rinv, G * g * g);
+    m.take(h->rdig, 6 * d * g);
+    m.take(h->rexp, G);
+    m.take(h->Htdig, 4 * pd);
+    m.take(h->expoT, G * G);
+    m.take(h->band, G * (kMaxBlock - 1) * g * g);
+    m.take(h->dstatus, 1);
+}
+
 jarq_status status_from_bits(int bits) {
     if (bits & ST_NOT_SPD) return JARQ_ERR_NOT_SPD;
     if (bits & (ST_BAD_CODE | ST_BAD_ZERO)) return JARQ_ERR_ARG;
@@ -277,7 +301,7 @@ jarq_status layer_front(jarq_hessian *h, const float *W, const float *S, const u
                         const int32_t *Z, int dout, int bits, LayerArgs &la, cudaStream_t st,
                         bool codes_only = false) {
     CK(cudaSetDevice(h->device));
-    CK(ensure_ws(h, dout));
+    CK(ensure_ws(h, dout, st));
     CK(stage_layer(h, W, S, Q, Z, dout, la, st));
     CK(cudaMemsetAsync(h->dstatus, 0, sizeof(int), st));
     RUN("validate", 1, launch_validate(la.Q, la.Z, dout, h->din, h->G, (1 << bits) - 1, h->dstatus, st));
@@ -409,23 +433,10 @@ void jarq_hessian_destroy(jarq_hessian *h) {
     DeviceGuard dg(h->device);
     cudaDeviceSynchronize();
     free_ws(h->ws);
-    cudaFree(h->Hs);
-    cudaFree(h->Hplanes);
-    cudaFree(h->Hdig8);
-    cudaFree(h->Hdig10);
-    cudaFree(h->expo);
-    cudaFree(h->Lf);
-    cudaFree(h->band);
-    cudaFree(h->L64);
-    cudaFree(h->Rinv);
-    cudaFree(h->rdig);
-    cudaFree(h->rexp);
-    cudaFree(h->Htdig);
-    cudaFree(h->expoT);
+    cudaFree(h->mem);
     cudaFree(h->qdig);
     cudaFree(h->qexp);
     cudaFree(h->qstage);
-    cudaFree(h->dstatus);
     cudaFreeHost(h->hstatus);
     (void)cudaGetLastError();
     delete h;
@@ -444,36 +455,34 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
     h->G = din / group_size;
     h->d_pad = round_up(din, 128);
     jarq_status rc = JARQ_OK;
-    float *Hdev = nullptr, *Ht_hi = nullptr, *Ht_lo = nullptr;
+    float *Hdev = nullptr;
     do {
         if (cudaGetDevice(&h->device) != cudaSuccess) { rc = JARQ_ERR_CUDA; break; }
         const size_t dd = (size_t)din * din;
         cudaError_t e;
-        if ((e = dalloc(&h->Hs, dd)) != cudaSuccess) { rc = cuda_fail(e); break; }
         const size_t pd = (size_t)h->d_pad * h->d_pad;
-        if ((e = dalloc(&h->Hplanes, 3 * pd)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = cudaMemsetAsync(h->Hplanes, 0, 3 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        Arena m;
+        layout_hessian(m, h);
+        if ((e = dalloc(&h->mem, m.used)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        m = Arena{h->mem};
+        layout_hessian(m, h);
+        // the folded rows R_i^{-T} H[grp i, :] as float pairs, only needed to
+        // form their digits: in the memory of H's own base-2^8 digits, which
+        // are formed last
+        float *const Ht_hi = reinterpret_cast<float *>(h->Hdig8), *const Ht_lo = Ht_hi + dd;
+        // columns beyond din are read as zeros by the products
+        const bool padded = h->d_pad != din;
+        if (padded) {
+            if ((e = cudaMemsetAsync(h->Hplanes, 0, 3 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
+            if ((e = cudaMemsetAsync(h->Hdig10, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
+            if ((e = cudaMemsetAsync(h->Htdig, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        }
         if ((e = make_tmap_bf16(&h->mapH128, h->Hplanes, (uint64_t)3 * h->d_pad, h->d_pad, 128)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_bf16(&h->mapH64, h->Hplanes, (uint64_t)3 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->Hdig8, 6 * pd)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = cudaMemsetAsync(h->Hdig8, 0, 6 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->Hdig10, 4 * pd)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = cudaMemsetAsync(h->Hdig10, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->expo, (size_t)h->G * h->G)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_bf16(&h->mapD8, h->Hdig8, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_f16(&h->mapD10, h->Hdig10, (uint64_t)4 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->Lf, (size_t)h->G * factor_floats(group_size))) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->L64, (size_t)h->G * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->Rinv, (size_t)h->G * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->rdig, (size_t)6 * din * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->rexp, (size_t)h->G)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_bf16(&h->mapRi, h->rdig, (uint64_t)6 * din, group_size, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->Htdig, 4 * pd)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = cudaMemsetAsync(h->Htdig, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->expoT, (size_t)h->G * h->G)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_f16(&h->mapHt, h->Htdig, (uint64_t)4 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->band, (size_t)h->G * (kMaxBlock - 1) * group_size * group_size)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&h->dstatus, 1)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = cudaMallocHost((void **)&h->hstatus, sizeof(int))) != cudaSuccess) { rc = cuda_fail(e); break; }
         const float *Hsrc = H;
         if (!is_device_ptr(H)) {
@@ -488,26 +497,22 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slice_rinv(h->Rinv, h->rdig, h->rexp, din, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
-        // folded rows R_i^{-T} H[grp i, :] (double-float, temporary) -> digits
-        if ((e = dalloc(&Ht_hi, dd)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = dalloc(&Ht_lo, dd)) != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("htilde", st); e = launch_htilde(h->Hs, h->Rinv, Ht_hi, Ht_lo, din, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slice10(Ht_hi, Ht_lo, h->expoT, h->Htdig, din, h->d_pad, group_size, st); ps.done(); count_launches(2); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_band(h->Htdig, h->band, din, h->d_pad, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
+        if (padded && (e = cudaMemsetAsync(h->Hdig8, 0, 6 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slices(h->Hs, h->expo, h->Hdig8, h->Hdig10, din, h->d_pad, group_size, st); ps.done(); count_launches(2); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         int sb = 0;
         if ((e = read_status(h, st, &sb)) != cudaSuccess) { rc = cuda_fail(e); break; }
         rc = status_from_bits(sb);
     } while (0);
-    if (Hdev || Ht_hi || Ht_lo) {
+    if (Hdev) {
         cudaStreamSynchronize(st);
         cudaFree(Hdev);
-        cudaFree(Ht_hi);
-        cudaFree(Ht_lo);
     }
     if (rc != JARQ_OK) {
         jarq_hessian_destroy(h);

@@ -89,6 +89,7 @@ __device__ __forceinline__ void store_residual(const ResidualView &v, size_t j, 
 // Library-owned refinement workspace, sized for `cap_rows` output rows.
 struct Workspace {
     int cap_rows = 0;
+    char *mem = nullptr;         // the one allocation that holds the arrays below
     int p_pad = 0;               // rows of the bf16 residual planes (multiple of 128)
     float *Hr = nullptr;         // [p][d]  H r for every row (objective entry point)
     float *r = nullptr;          // [p][d]  residual r = w - D_s (q - z)
@@ -135,6 +136,7 @@ struct jarq_hessian {
     int din = 0, g = 0, G = 0;
     int device = 0;
     int d_pad = 0;
+    char *mem = nullptr;          // the one allocation that holds the arrays below
     float *Hs = nullptr;          // [d][d] symmetrised H (+ nu2 I), fp32
     __nv_bfloat16 *Hplanes = nullptr;  // [3][d_pad][d_pad] exact bf16 split of Hs
     // per-block integer digits of Hs (block exponents in expo):
