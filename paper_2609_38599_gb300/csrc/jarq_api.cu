@@ -345,10 +345,12 @@ jarq_status project_by(jarq_hessian *h, const float *M, int p, float *out_hi, fl
         CK(dalloc(&h->qexp, (size_t)h->G * h->G));
         CK(make_tmap_bf16(&h->mapQ, h->qdig, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32));
     }
+    // the digit kernels read M in 16-byte vectors: a device M that is not
+    // 16-byte aligned is staged like host memory
     const float *Md = M;
-    if (!is_device_ptr(M)) {
+    if (!is_device_ptr(M) || ((uintptr_t)M & 15)) {
         if (!h->qstage) CK(dalloc(&h->qstage, (size_t)d * d));
-        CK(cudaMemcpyAsync(h->qstage, M, (size_t)d * d * sizeof(float), cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(h->qstage, M, (size_t)d * d * sizeof(float), cudaMemcpyDefault, st));
         Md = h->qstage;
     }
     RUN("slices", 2, launch_slices8(Md, h->qexp, h->qdig, d, h->d_pad, g, st));
@@ -467,14 +469,15 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         m = Arena{h->mem};
         layout_hessian(m, h);
         // the folded rows R_i^{-T} H[grp i, :] as float pairs, only needed to
-        // form their digits: in the memory of H's own base-2^8 digits, which
-        // are formed last
+        // form their digits, and the inverse factors as float pairs, only
+        // needed to form those: in the memory of H's own digits, which are
+        // formed last
         float *const Ht_hi = reinterpret_cast<float *>(h->Hdig8), *const Ht_lo = Ht_hi + dd;
+        float2 *const RinvF = reinterpret_cast<float2 *>(Ht_lo + dd);
         // columns beyond din are read as zeros by the products
         const bool padded = h->d_pad != din;
         if (padded) {
             if ((e = cudaMemsetAsync(h->Hplanes, 0, 3 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
-            if ((e = cudaMemsetAsync(h->Hdig10, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
             if ((e = cudaMemsetAsync(h->Htdig, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
         }
         if ((e = make_tmap_bf16(&h->mapH128, h->Hplanes, (uint64_t)3 * h->d_pad, h->d_pad, 128)) != cudaSuccess) { rc = cuda_fail(e); break; }
@@ -493,17 +496,18 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         if ((e = cudaMemsetAsync(h->dstatus, 0, sizeof(int), st)) != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("symmetrize", st); e = launch_symmetrize(Hsrc, h->Hs, h->Hplanes, din, h->d_pad, nu2, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
-        { ProfScope ps("group_factor", st); e = launch_group_factor(h->Hs, h->Lf, h->L64, h->Rinv, din, group_size, h->dstatus, st); ps.done(); count_launches(1); }
+        { ProfScope ps("group_factor", st); e = launch_group_factor(h->Hs, h->Lf, h->L64, h->Rinv, RinvF, din, group_size, h->dstatus, st); ps.done(); count_launches(2); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slice_rinv(h->Rinv, h->rdig, h->rexp, din, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
-        { ProfScope ps("htilde", st); e = launch_htilde(h->Hs, h->Rinv, Ht_hi, Ht_lo, din, group_size, st); ps.done(); count_launches(1); }
+        { ProfScope ps("htilde", st); e = launch_htilde(h->Hs, RinvF, Ht_hi, Ht_lo, din, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slice10(Ht_hi, Ht_lo, h->expoT, h->Htdig, din, h->d_pad, group_size, st); ps.done(); count_launches(2); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_band(h->Htdig, h->band, din, h->d_pad, group_size, st); ps.done(); count_launches(1); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         if (padded && (e = cudaMemsetAsync(h->Hdig8, 0, 6 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        if (padded && (e = cudaMemsetAsync(h->Hdig10, 0, 4 * pd * 2, st)) != cudaSuccess) { rc = cuda_fail(e); break; }
         { ProfScope ps("slices", st); e = launch_slices(h->Hs, h->expo, h->Hdig8, h->Hdig10, din, h->d_pad, group_size, st); ps.done(); count_launches(2); }
         if (e != cudaSuccess) { rc = cuda_fail(e); break; }
         int sb = 0;

@@ -177,8 +177,8 @@ namespace jarq {
 // ---- launchers (each returns the cudaError_t of its launch) ----
 cudaError_t launch_symmetrize(const float *H, float *Hs, __nv_bfloat16 *Hplanes, int d, int d_pad,
                               float nu2, cudaStream_t s);
-cudaError_t launch_group_factor(const float *Hs, float *Lf, double *L64, double *Rinv, int d,
-                                int g, int *status, cudaStream_t s);
+cudaError_t launch_group_factor(const float *Hs, float *Lf, double *L64, double *Rinv,
+                                float2 *RinvF, int d, int g, int *status, cudaStream_t s);
 cudaError_t launch_own_rhs(const float *Hs, const float *W, const uint8_t *Q, const int32_t *Z,
                            double *own, int p, int d, int g, cudaStream_t s);
 cudaError_t launch_scale_fit(const float2 *gram, const double *rhs, const double *own,
@@ -189,7 +189,7 @@ cudaError_t launch_probe(const float *Phi, const float *Plo, const float *t_hi, 
                          const int32_t *Z, uint8_t *q_out, int32_t *moves, int32_t *accepted,
                          int32_t *changed, double *dF, int p, int p_pad, int d, int g, int i,
                          int nsplit, int qmax, float eps, cudaStream_t s);
-cudaError_t launch_htilde(const float *Hs, const double *Rinv, float *out_hi, float *out_lo,
+cudaError_t launch_htilde(const float *Hs, const float2 *RinvF, float *out_hi, float *out_lo,
                           int d, int g, cudaStream_t s);
 cudaError_t launch_slice10(const float *hi, const float *lo, int *expo, __half *dig, int d,
                            int d_pad, int g, cudaStream_t s);

@@ -6,7 +6,8 @@
 // With H = A^T A, R_i^T R_i = H_ii, so R_i is taken as the upper Cholesky
 // factor of H_ii (equal to the QR factor up to row signs, to which the
 // Babai recursion is invariant).  The factor and its inverse are computed in
-// float64 in shared memory:
+// float64 in shared memory (the failing case of a block that is not positive
+// definite leaves its inverse undefined; the call then fails):
 //   Lf[i]   = L_i = R_i^T          (lower, L[l][m] = R_i[m][l]), float32, packed for the
 //             Babai kernel (factor_row in jarq_internal.cuh)
 //   Rinv[i] = R_i^{-1}             (upper, row-major), float64
@@ -51,19 +52,20 @@ __global__ void symmetrize_kernel(const float *__restrict__ H, float *__restrict
     }
 }
 
-// One block per group: float64 Cholesky of H_ii in shared memory, then an
-// in-place inverse of the lower factor.
+// One block per group: float64 Cholesky of H_ii in shared memory.  Bound by
+// float64 (two lanes per clock on an SM, one SM per group): the update of the
+// trailing lower triangle goes row by row over the warps, so that no lane
+// works above the diagonal except in a row's last 32 columns.
 __global__ void group_factor_kernel(const float *__restrict__ Hs, float *__restrict__ Lf,
-                                    double *__restrict__ L64, double *__restrict__ Rinv, int d,
-                                    int g, int *status) {
+                                    double *__restrict__ L64, int d, int g, int *status) {
     extern __shared__ double smem[];
     const int ld = g + 1;
     double *A = smem;               // [g][g+1]
-    double *tmp = smem + g * ld;    // [g]
     __shared__ int failed;
     const int grp = blockIdx.x;
     const int base = grp * g;
     const int tid = threadIdx.x, nt = blockDim.x;
+    const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
     if (tid == 0) failed = 0;
     for (int idx = tid; idx < g * g; idx += nt) {
         int a = idx / g, b = idx % g;
@@ -72,26 +74,22 @@ __global__ void group_factor_kernel(const float *__restrict__ Hs, float *__restr
     __syncthreads();
     // right-looking Cholesky, lower triangle
     for (int k = 0; k < g; ++k) {
-        if (tid == 0) {
-            double piv = A[k * ld + k];
-            if (!(piv > 0.0) || !isfinite(piv)) {
-                failed = 1;
-            } else {
-                A[k * ld + k] = sqrt(piv);
-            }
+        const double piv = A[k * ld + k];
+        if (!(piv > 0.0) || !isfinite(piv)) {       // every thread sees the same pivot
+            if (tid == 0) failed = 1;
+            break;
         }
-        __syncthreads();
-        if (failed) break;
-        const double lkk = A[k * ld + k];
+        const double lkk = sqrt(piv);
         for (int a = k + 1 + tid; a < g; a += nt) A[a * ld + k] /= lkk;
         __syncthreads();
-        const int n = g - k - 1;
-        for (int idx = tid; idx < n * n; idx += nt) {
-            int a = k + 1 + idx / n, b = k + 1 + idx % n;
-            if (b <= a) A[a * ld + b] -= A[a * ld + k] * A[b * ld + k];
+        if (tid == 0) A[k * ld + k] = lkk;
+        for (int a = k + 1 + warp; a < g; a += nw) {
+            const double l = A[a * ld + k];
+            for (int b = k + 1 + lane; b <= a; b += 32) A[a * ld + b] -= l * A[b * ld + k];
         }
         __syncthreads();
     }
+    __syncthreads();
     if (failed) {
         if (tid == 0) atomicOr(status, ST_NOT_SPD);
         return;
@@ -115,27 +113,49 @@ __global__ void group_factor_kernel(const float *__restrict__ Hs, float *__restr
         Lo[factor_diag(g) + l] = v;
         Lo[factor_rdiag(g) + l] = 1.0f / v;
     }
+}
+
+// R_i^{-1} = (L_i^{-1})^T, column j of L^{-1} (= row j of R^{-1}) per warp by
+// forward substitution in float64, kInvCols columns per block: the columns are
+// independent, so the work spreads over g / kInvCols times the SMs that the
+// factorisation uses.  Lane l keeps the entries l + 32 m of its column.  Also
+// written as float pairs (hi, lo) for the folded rows.
+constexpr int kInvCols = 16;
+
+template <int NT>
+__global__ void __launch_bounds__(32 * kInvCols) group_inverse_kernel(const double *__restrict__ L64,
+                                                                      double *__restrict__ Rinv,
+                                                                      float2 *__restrict__ RinvF) {
+    constexpr int g = 32 * NT, ld = g + 1;
+    extern __shared__ double smem[];
+    double *A = smem;               // [g][g+1]
+    double *rd = smem + g * ld;     // [g] 1 / L_bb
+    const size_t off = (size_t)blockIdx.x * g * g;
+    for (int idx = threadIdx.x; idx < g * g; idx += blockDim.x) A[(idx / g) * ld + idx % g] = L64[off + idx];
     __syncthreads();
-    // in-place inverse of the lower factor, columns from last to first:
-    // Linv[j][j] = 1/L[j][j]; Linv[j+1:, j] = -Linv[j][j] * Linv[j+1:, j+1:] L[j+1:, j]
-    for (int j = g - 1; j >= 0; --j) {
-        for (int a = j + 1 + tid; a < g; a += nt) tmp[a] = A[a * ld + j];
-        __syncthreads();
-        const double inv_jj = 1.0 / A[j * ld + j];
-        for (int a = j + 1 + tid; a < g; a += nt) {
-            double acc = 0.0;
-            for (int b = j + 1; b <= a; ++b) acc += A[a * ld + b] * tmp[b];
-            A[a * ld + j] = -acc * inv_jj;
+    for (int b = threadIdx.x; b < g; b += blockDim.x) rd[b] = 1.0 / A[b * ld + b];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, j = blockIdx.y * kInvCols + (threadIdx.x >> 5);
+    double x[NT];
+#pragma unroll
+    for (int m = 0; m < NT; ++m) x[m] = lane + 32 * m == j ? 1.0 : 0.0;
+#pragma unroll
+    for (int mb = 0; mb < NT; ++mb) {
+        for (int bb = max(0, j - 32 * mb); bb < 32; ++bb) {      // warp-uniform
+            const int b = 32 * mb + bb;
+            const double xb = __shfl_sync(0xffffffffu, x[mb], bb) * rd[b];
+            if (lane == bb) x[mb] = xb;
+#pragma unroll
+            for (int m = mb; m < NT; ++m)
+                if (lane + 32 * m > b) x[m] = fma(-A[(lane + 32 * m) * ld + b], xb, x[m]);
         }
-        __syncthreads();
-        if (tid == 0) A[j * ld + j] = inv_jj;
-        __syncthreads();
     }
-    // Rinv = (L^{-1})^T : Rinv[m][l] = Linv[l][m]
-    double *Ri = Rinv + (size_t)grp * g * g;
-    for (int idx = tid; idx < g * g; idx += nt) {
-        int m = idx / g, l = idx % g;
-        Ri[idx] = (l >= m) ? A[l * ld + m] : 0.0;
+#pragma unroll
+    for (int m = 0; m < NT; ++m) {
+        const size_t o = off + (size_t)j * g + lane + 32 * m;
+        const float hi = (float)x[m];
+        Rinv[o] = x[m];
+        RinvF[o] = make_float2(hi, (float)(x[m] - (double)hi));
     }
 }
 
@@ -147,53 +167,81 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
 }
 
 // Ht[i g + a, k] = sum_{b <= a} Rinv_i[b][a] Hs[i g + b, k] for one group i
-// (blockIdx.y) and 64 columns k (blockIdx.x): Rinv_i as float pairs (hi, lo)
-// and the H tile in shared memory, double-float accumulation, written as the
-// float pair (hi, lo) [d][d].
-constexpr int kHtCols = 64;
+// (blockIdx.y) and 128 columns k (blockIdx.x), double-float products and sums
+// (11 float32 operations a term), written as the float pair (hi, lo) [d][d].
+// Rinv_i's pairs and the H tile lie in shared memory; warp w computes the rows
+// 4 w .. 4 w + 3 and their mirror g - 4 - 4 w .., so that every warp has the
+// same number of terms, and lane l the columns 4 l .. 4 l + 3: five 16-byte
+// shared loads for 32 terms (four of them one address for the warp).  One
+// output a thread and step, three shared loads a term, took 1.31 ms on 4096 x
+// 4096.
+constexpr int kHtCols = 128;
 
-__global__ void __launch_bounds__(256) htilde_kernel(const float *__restrict__ Hs,
-                                                     const double *__restrict__ Rinv,
-                                                     float *__restrict__ out_hi,
-                                                     float *__restrict__ out_lo, int d, int g) {
-    extern __shared__ float hsm[];
+template <int NT>
+__global__ void __launch_bounds__(128 * NT, 1) htilde_kernel(const float *__restrict__ Hs,
+                                                             const float2 *__restrict__ RinvF,
+                                                             float *__restrict__ out_hi,
+                                                             float *__restrict__ out_lo, int d) {
+    constexpr int g = 32 * NT;
+    extern __shared__ __align__(16) float hsm[];
     float *rh = hsm;                   // [g][g] hi parts, Rinv[b][a] at b * g + a
     float *rl = rh + g * g;            // [g][g] lo parts
     float *ht = rl + g * g;            // [g][kHtCols] rows of H for this group
     const int i = blockIdx.y, k0 = blockIdx.x * kHtCols;
-    const int tid = threadIdx.x;
-    const double *Ri = Rinv + (size_t)i * g * g;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const float2 *Ri = RinvF + (size_t)i * g * g;
     for (int idx = tid; idx < g * g; idx += blockDim.x) {
-        const double v = Ri[idx];
-        const float hi = (float)v;
-        rh[idx] = hi;
-        rl[idx] = (float)(v - (double)hi);
+        const float2 v = Ri[idx];
+        rh[idx] = v.x;
+        rl[idx] = v.y;
     }
-    for (int idx = tid; idx < g * kHtCols; idx += blockDim.x) {
-        const int b = idx / kHtCols, kk = idx % kHtCols;
-        ht[idx] = (k0 + kk < d) ? Hs[(size_t)(i * g + b) * d + k0 + kk] : 0.f;
+    for (int idx = tid; idx < g * kHtCols / 4; idx += blockDim.x) {
+        const int b = idx / (kHtCols / 4), kk = 4 * (idx % (kHtCols / 4));
+        *reinterpret_cast<float4 *>(ht + b * kHtCols + kk) =
+            k0 + kk < d ? *reinterpret_cast<const float4 *>(Hs + (size_t)(i * g + b) * d + k0 + kk)
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    const int kk = tid % kHtCols, a0 = tid / kHtCols, astep = blockDim.x / kHtCols;
-    for (int a = a0; a < g; a += astep) {
-        float sh = 0.f, sl = 0.f;
-        for (int b = 0; b <= a; ++b) {
-            const float hv = ht[b * kHtCols + kk];
-            const float r_hi = rh[b * g + a], r_lo = rl[b * g + a];
-            const float m = r_hi * hv;
-            float e = fmaf(r_hi, hv, -m);
-            e = fmaf(r_lo, hv, e);
-            float s2, e2;
-            two_sum(sh, m, s2, e2);
-            sh = s2;
-            sl += e2 + e;
-        }
-        if (k0 + kk < d) {
-            float s2, e2;
-            two_sum(sh, sl, s2, e2);
-            const size_t off = (size_t)(i * g + a) * d + k0 + kk;
-            out_hi[off] = s2;
-            out_lo[off] = e2;
+    const int a_lo = 4 * w, a_hi = g - 4 - 4 * w;
+    float sh[8][4] = {}, sl[8][4] = {};     // rows a_lo + r, a_hi + r; columns 4 lane + c
+    auto terms = [&](int r0, const float *prh, const float *prl, const float4 &h4) {
+        const float4 r4 = *reinterpret_cast<const float4 *>(prh), l4 = *reinterpret_cast<const float4 *>(prl);
+        const float hv[4] = {h4.x, h4.y, h4.z, h4.w};
+        const float rv[4] = {r4.x, r4.y, r4.z, r4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float m = rv[r] * hv[c];
+                float e = fmaf(rv[r], hv[c], -m);
+                e = fmaf(lv[r], hv[c], e);
+                float s2, e2;
+                two_sum(sh[r0 + r][c], m, s2, e2);
+                sh[r0 + r][c] = s2;
+                sl[r0 + r][c] += e2 + e;
+            }
+    };
+    // Rinv[b][a] is zero for b > a: the terms up to a row quad's last row
+    int b = 0;
+    for (; b < a_lo + 4; ++b) {
+        const float4 h4 = *reinterpret_cast<const float4 *>(ht + b * kHtCols + 4 * lane);
+        terms(0, rh + b * g + a_lo, rl + b * g + a_lo, h4);
+        terms(4, rh + b * g + a_hi, rl + b * g + a_hi, h4);
+    }
+    for (; b < a_hi + 4; ++b) {
+        const float4 h4 = *reinterpret_cast<const float4 *>(ht + b * kHtCols + 4 * lane);
+        terms(4, rh + b * g + a_hi, rl + b * g + a_hi, h4);
+    }
+    if (k0 + 4 * lane < d) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int a = r < 4 ? a_lo + r : a_hi + r - 4;
+            float x[4], y[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) two_sum(sh[r][c], sl[r][c], x[c], y[c]);
+            const size_t off = (size_t)(i * g + a) * d + k0 + 4 * lane;
+            *reinterpret_cast<float4 *>(out_hi + off) = make_float4(x[0], x[1], x[2], x[3]);
+            *reinterpret_cast<float4 *>(out_lo + off) = make_float4(y[0], y[1], y[2], y[3]);
         }
     }
 }
@@ -236,24 +284,45 @@ cudaError_t launch_symmetrize(const float *H, float *Hs, __nv_bfloat16 *Hplanes,
     return cudaGetLastError();
 }
 
-cudaError_t launch_group_factor(const float *Hs, float *Lf, double *L64, double *Rinv, int d,
-                                int g, int *status, cudaStream_t s) {
-    size_t smem = (size_t)(g * (g + 1) + g) * sizeof(double);
+cudaError_t launch_group_factor(const float *Hs, float *Lf, double *L64, double *Rinv,
+                                float2 *RinvF, int d, int g, int *status, cudaStream_t s) {
+    const int smem = (g * (g + 1) + g) * (int)sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(group_factor_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    group_factor_kernel<<<d / g, 256, smem, s>>>(Hs, Lf, L64, Rinv, d, g, status);
+    group_factor_kernel<<<d / g, 256, smem, s>>>(Hs, Lf, L64, d, g, status);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const dim3 grid(d / g, g / kInvCols);
+    if (g == 128) {
+        e = cudaFuncSetAttribute(group_inverse_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        group_inverse_kernel<4><<<grid, 32 * kInvCols, smem, s>>>(L64, Rinv, RinvF);
+    } else if (g == 64) {
+        e = cudaFuncSetAttribute(group_inverse_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        group_inverse_kernel<2><<<grid, 32 * kInvCols, smem, s>>>(L64, Rinv, RinvF);
+    } else {
+        return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_htilde(const float *Hs, const double *Rinv, float *out_hi, float *out_lo,
-                          int d, int g, cudaStream_t s) {
-    const size_t smem = ((size_t)2 * g * g + (size_t)g * kHtCols) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(htilde_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((d + kHtCols - 1) / kHtCols, d / g);
-    htilde_kernel<<<grid, 256, smem, s>>>(Hs, Rinv, out_hi, out_lo, d, g);
+cudaError_t launch_htilde(const float *Hs, const float2 *RinvF, float *out_hi, float *out_lo, int d,
+                          int g, cudaStream_t s) {
+    const int smem = (2 * g * g + g * kHtCols) * (int)sizeof(float);
+    const dim3 grid((d + kHtCols - 1) / kHtCols, d / g);
+    cudaError_t e;
+    if (g == 128) {
+        e = cudaFuncSetAttribute(htilde_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        htilde_kernel<4><<<grid, 512, smem, s>>>(Hs, RinvF, out_hi, out_lo, d);
+    } else if (g == 64) {
+        e = cudaFuncSetAttribute(htilde_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        htilde_kernel<2><<<grid, 256, smem, s>>>(Hs, RinvF, out_hi, out_lo, d);
+    } else {
+        return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

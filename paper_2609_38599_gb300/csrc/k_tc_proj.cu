@@ -556,33 +556,69 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, ST_TIMEOUT);
 }
 
+// NT consecutive floats / bf16 of one lane.
+template <int NT>
+__device__ __forceinline__ void load_nt(const float *p, float (&v)[NT]) {
+    if constexpr (NT == 4) {
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    } else {
+        const float2 a = *reinterpret_cast<const float2 *>(p);
+        v[0] = a.x; v[1] = a.y;
+    }
+}
+template <int NT>
+__device__ __forceinline__ void store_nt(__nv_bfloat16 *p, const float (&v)[NT]) {
+    __align__(8) __nv_bfloat16 q[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k) q[k] = __float2bfloat16_rn(v[k]);
+    if constexpr (NT == 4)
+        *reinterpret_cast<uint2 *>(p) = *reinterpret_cast<const uint2 *>(q);
+    else
+        *reinterpret_cast<uint32_t *>(p) = *reinterpret_cast<const uint32_t *>(q);
+}
+
 // Digits of W per (row, group): x = W 2^(7 - ew) in [-128, 128] with
 // max |W[j, grp h]| <= 2^ew; a_0 = rint(x), a_t = rint(256 * remainder).
-// One warp per (row, group).
+// One warp per (row, group), lane owns NT = g/32 consecutive entries, loaded as
+// one vector if W is 16-byte aligned (`vec`).
+template <int NT>
 __global__ void slice_rows_kernel(const float *__restrict__ W, __nv_bfloat16 *__restrict__ planes,
-                                  int *__restrict__ wexp, int p, int d, int d_pad, int p_pad, int g) {
+                                  int *__restrict__ wexp, int p, int d, int d_pad, int p_pad, bool vec) {
+    constexpr int g = 32 * NT;
     const int G = d / g;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= (long long)p * G) return;
     const int j = (int)(warp / G), h = (int)(warp % G);
-    const float *src = W + (size_t)j * d + (size_t)h * g;
+    float x[NT];
+    const float *src = W + (size_t)j * d + (size_t)h * g + NT * lane;
+    if (vec) {
+        load_nt<NT>(src, x);
+    } else {
+#pragma unroll
+        for (int k = 0; k < NT; ++k) x[k] = src[k];
+    }
     float mx = 0.f;
-    for (int m = lane; m < g; m += 32) mx = fmaxf(mx, fabsf(src[m]));
+#pragma unroll
+    for (int k = 0; k < NT; ++k) mx = fmaxf(mx, fabsf(x[k]));
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     int e = 0;
     if (mx > 0.f) frexpf(mx, &e);
     if (lane == 0) wexp[(size_t)j * G + h] = e;
     const size_t plane = (size_t)p_pad * d_pad;
-    for (int m = lane; m < g; m += 32) {
-        float x = ldexpf(src[m], 7 - e);
-        const size_t off = (size_t)j * d_pad + (size_t)h * g + m;
+    const size_t off = (size_t)j * d_pad + (size_t)h * g + NT * lane;
 #pragma unroll
-        for (int t = 0; t < kWDig; ++t) {
-            const float dg = rintf(x);
-            planes[t * plane + off] = __float2bfloat16_rn(dg);
-            x = (x - dg) * 256.f;
+    for (int k = 0; k < NT; ++k) x[k] = ldexpf(x[k], 7 - e);
+#pragma unroll
+    for (int t = 0; t < kWDig; ++t) {
+        float dg[NT];
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+            dg[k] = rintf(x[k]);
+            x[k] = (x[k] - dg[k]) * 256.f;
         }
+        store_nt<NT>(planes + t * plane + off, dg);
     }
 }
 
@@ -719,34 +755,46 @@ __global__ void mu_combine_kernel(float *__restrict__ Phi, float *__restrict__ P
 // rint(xh), and the remainder (xh - digit) + xl is renormalised by an exact
 // two-sum before the next digit.  Six digits hold P to 2^-48 of its group
 // maximum (the pair itself carries about 48 bits).
+template <int NT>
 __global__ void slice_df_rows_kernel(const float *__restrict__ Phi, const float *__restrict__ Plo,
                                      __nv_bfloat16 *__restrict__ planes, int *__restrict__ pexp,
-                                     int p, int d, int d_pad, int p_pad, int g) {
+                                     int p, int d, int d_pad, int p_pad) {
+    constexpr int g = 32 * NT;
     const int G = d / g;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= (long long)p * G) return;
     const int j = (int)(warp / G), h = (int)(warp % G);
-    const size_t src = (size_t)j * d + (size_t)h * g;
+    const size_t src = (size_t)j * d + (size_t)h * g + NT * lane;
+    float xh[NT], xl[NT];
+    load_nt<NT>(Phi + src, xh);
+    load_nt<NT>(Plo + src, xl);
     float mx = 0.f;
-    for (int m = lane; m < g; m += 32) mx = fmaxf(mx, fabsf(Phi[src + m]));
+#pragma unroll
+    for (int k = 0; k < NT; ++k) mx = fmaxf(mx, fabsf(xh[k]));
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     int e = 0;
     if (mx > 0.f) frexpf(mx, &e);
     if (lane == 0) pexp[(size_t)j * G + h] = e;
     const size_t plane = (size_t)p_pad * d_pad;
-    for (int m = lane; m < g; m += 32) {
-        float xh = ldexpf(Phi[src + m], 7 - e), xl = ldexpf(Plo[src + m], 7 - e);
-        const size_t off = (size_t)j * d_pad + (size_t)h * g + m;
+    const size_t off = (size_t)j * d_pad + (size_t)h * g + NT * lane;
 #pragma unroll
-        for (int t = 0; t < kHDig; ++t) {
-            const float dg = rintf(xh);
-            planes[t * plane + off] = __float2bfloat16_rn(dg);
+    for (int k = 0; k < NT; ++k) {
+        xh[k] = ldexpf(xh[k], 7 - e);
+        xl[k] = ldexpf(xl[k], 7 - e);
+    }
+#pragma unroll
+    for (int t = 0; t < kHDig; ++t) {
+        float dg[NT];
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+            dg[k] = rintf(xh[k]);
             float s2, e2;
-            two_sum(xh - dg, xl, s2, e2);
-            xh = s2 * 256.f;
-            xl = e2 * 256.f;
+            two_sum(xh[k] - dg[k], xl[k], s2, e2);
+            xh[k] = s2 * 256.f;
+            xl[k] = e2 * 256.f;
         }
+        store_nt<NT>(planes + t * plane + off, dg);
     }
 }
 
@@ -805,8 +853,11 @@ cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, con
                           float *out_hi, float *out_lo, int p, int p_pad, int d, int d_pad, int g,
                           int *status, cudaStream_t s) {
     const long long warps = (long long)p * (d / g);
-    slice_df_rows_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(
-        Phi, Plo, pdig, pexp, p, d, d_pad, p_pad, g);
+    const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
+    if (g == 128)
+        slice_df_rows_kernel<4><<<blocks, 256, 0, s>>>(Phi, Plo, pdig, pexp, p, d, d_pad, p_pad);
+    else
+        slice_df_rows_kernel<2><<<blocks, 256, 0, s>>>(Phi, Plo, pdig, pexp, p, d, d_pad, p_pad);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     static std::atomic<unsigned long long> attr_done{0};
@@ -824,8 +875,12 @@ cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, con
 cudaError_t launch_slice_rows(const float *W, __nv_bfloat16 *planes, int *wexp, int p, int d,
                               int d_pad, int p_pad, int g, cudaStream_t s) {
     const long long warps = (long long)p * (d / g);
-    slice_rows_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(W, planes, wexp, p, d,
-                                                                          d_pad, p_pad, g);
+    const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
+    const bool vec = ((uintptr_t)W & 15) == 0;
+    if (g == 128)
+        slice_rows_kernel<4><<<blocks, 256, 0, s>>>(W, planes, wexp, p, d, d_pad, p_pad, vec);
+    else
+        slice_rows_kernel<2><<<blocks, 256, 0, s>>>(W, planes, wexp, p, d, d_pad, p_pad, vec);
     return cudaGetLastError();
 }
 

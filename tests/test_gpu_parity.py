@@ -204,6 +204,28 @@ def test_host_buffers_match_device_buffers(jarq):
     np.testing.assert_array_equal(std["L_final"], sth.L_final)
 
 
+@pytest.mark.parametrize("g", [64, 128])
+def test_misaligned_device_buffers(jarq, g):
+    """Device tensors that start 4 (float32, int32) or 1 (codes) bytes past a
+    16-byte boundary give the same bits as aligned ones."""
+    lay = small_layer(3 * g, 70, g, 3, seed=24)
+
+    def dev(a, off):
+        t = torch.as_tensor(a)
+        return torch.empty(t.numel() + off, dtype=t.dtype, device="cuda")[off:].view(t.shape).copy_(t)
+
+    out = []
+    for off in (0, 1):
+        hess = jarq.prepare(dev(lay.H, off), g)
+        S, Q = dev(lay.S0, off), dev(lay.Q0, off)
+        st = jarq.refine_mu(hess, dev(lay.W, off), S, Q, dev(lay.Z, off), lay.bits,
+                            dev(lay.H * np.float32(0.9), off), dev(lay.H, off), 0.5, 0.0, max_iters=2)
+        out.append((S.cpu().numpy(), Q.cpu().numpy(), st.L_final.cpu().numpy()))
+        hess.close()
+    for x, y in zip(*out):
+        np.testing.assert_array_equal(x, y)
+
+
 def test_k0_returns_host_state(jarq):
     lay = small_layer(128, 40, 64, 3, seed=23)
     S, Q, st = gpu_refine(lay, 0)
