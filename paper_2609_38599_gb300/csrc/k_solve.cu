@@ -1,6 +1,7 @@
-// Joint scale solve, one warp per output row (Sec. 3.3.1; App. E).
+// Joint scale solve (Sec. 3.3.1; App. E): one warp per output row for up to 32
+// groups, one block of four warps per row for more.
 //
-// For each active row j the warp
+// For each active row j the kernel
 //  1. reads its G x G Gram matrix -- symmetric by construction, since the
 //     Gram kernel computes each block once and writes it to both triangles,
 //     so the symmetrisation of App. E "Solving for scales" is the identity
@@ -32,48 +33,6 @@
 namespace jarq {
 namespace {
 
-// Offset of row a of a lower triangle stored row by row (packed).
-__device__ __forceinline__ int tri(int a) { return (a * (a + 1)) >> 1; }
-
-// In-place lower Cholesky of a G x G matrix stored as a packed lower
-// triangle, by one warp.  Fails when a pivot is not above `thr` or is not
-// finite.  Each lane owns the rows a = lane (mod 32) of the trailing update;
-// A[b][k] is read by all lanes at once (a broadcast).
-__device__ bool warp_cholesky(float *A, int G, float thr) {
-    const int lane = threadIdx.x & 31;
-    for (int k = 0; k < G; ++k) {
-        __syncwarp();
-        const float piv = A[tri(k) + k];
-        if (!(piv > thr) || !isfinite(piv)) return false;
-        const float lkk = sqrtf(piv);
-        __syncwarp();
-        if (lane == 0) A[tri(k) + k] = lkk;
-        for (int a = k + 1 + lane; a < G; a += 32) A[tri(a) + k] /= lkk;
-        __syncwarp();
-        for (int a = k + 1 + lane; a < G; a += 32) {
-            float *Aa = A + tri(a);
-            const float lak = Aa[k];
-            // A[b][k] (rows b > k, column k) and A[a][b] (row a, columns
-            // b > k) never overlap: four of each are loaded before the
-            // four updates are stored
-            int b = k + 1;
-            for (; b + 3 <= a; b += 4) {
-                const int t0 = tri(b) + k;
-                const float c0 = A[t0], c1 = A[t0 + b + 1], c2 = A[t0 + 2 * b + 3],
-                            c3 = A[t0 + 3 * b + 6];
-                const float x0 = Aa[b], x1 = Aa[b + 1], x2 = Aa[b + 2], x3 = Aa[b + 3];
-                Aa[b] = fmaf(-lak, c0, x0);
-                Aa[b + 1] = fmaf(-lak, c1, x1);
-                Aa[b + 2] = fmaf(-lak, c2, x2);
-                Aa[b + 3] = fmaf(-lak, c3, x3);
-            }
-            for (; b <= a; ++b) Aa[b] = fmaf(-lak, A[tri(b) + k], Aa[b]);
-        }
-    }
-    __syncwarp();
-    return true;
-}
-
 __device__ __forceinline__ float warp_max(float v) {
     for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
@@ -91,179 +50,321 @@ struct SolveArgs {
     jarq_options o;
 };
 
-// Per-warp shared memory: the packed lower factor A (G (G + 1) / 2
-// floats), s_old[G], y[G], and the double-float gradient (bh, bl) and
-// increment (ih, il), G each.
-__host__ __device__ inline size_t solve_warp_bytes(int G) {
-    return ((size_t)G * (G + 1) / 2 + 6 * (size_t)G) * sizeof(float);
+// ---------------------------------------------------------------------------
+// Solve for G > 32 (e.g. 64 groups of the 4096-input layers at g = 64, 86 of the
+// 11008-input ones): a block of NT = 64, 96 or 128 threads per row (G rounded
+// up), thread t owning row t of the Gram matrix.  The matrix stays in global
+// memory (L2) and is read column by column, 16 coalesced loads in flight
+// (exactly symmetric, so entry (t, c) is read as (c, t)): once for the gradient
+// and the float32 copy, twice for the refinement residuals, once for the
+// objective.  The float32 factor lives in shared memory and is formed in panels
+// of eight columns: the first warp factors the 8 x 8 diagonal block, every
+// thread solves its row of the panel, and 4 x 4 tiles take the rank-8 update of
+// the trailing triangle.
+// Every dot product with the Gram matrix -- the gradient, the two refinement
+// residuals, the objective -- is summed in double-float on the entries' float
+// pairs.
+//
+// What bounds it: the latency of a row's chain (8 to 11 panels, as many steps of
+// each triangular solve, four passes over the matrix) against the rows that fit
+// an SM (12, 8 or 6 by registers).  4096 rows: 213 us for 64 groups, 427 us for
+// 86.  One warp per row, the trailing triangle updated a column at a time, took
+// 324 and 800 us; both divide by the pivots and add in the same order, so the
+// factor and the ridge decision are those of that kernel bit for bit (with
+// products by the pivots' reciprocals: 181 and 367 us, but other last bits).
+// ---------------------------------------------------------------------------
+
+constexpr int kPanel = 8;
+
+// Row pitch of the float32 factor: a multiple of 4 that is 4 mod 8, so that 16-
+// byte loads of consecutive rows fall into different banks.
+__host__ __device__ inline int solve_ld(int G) { return (G + 7) / 8 * 8 + 4; }
+__host__ __device__ inline size_t solve_bytes(int G) {
+    const int Gp = (G + 7) / 8 * 8;
+    return ((size_t)Gp * solve_ld(G) + 7 * Gp) * sizeof(float);
 }
 
-// Forward and back substitution with the packed float32 factor in A,
-// y <- (L L^T)^{-1} y, for G <= 128: lane l keeps y[l + 32 m] in a
-// register, multiplies by the pivots' reciprocals, and each solved value
-// reaches the other lanes by a shuffle.  y is read and written in shared
-// memory.
-__device__ void warp_chol_solve(const float *A, int G, float *y) {
-    const int lane = threadIdx.x & 31;
-    float v[4], rd[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int t = lane + 32 * m;
-        v[m] = t < G ? y[t] : 0.f;
-        rd[m] = t < G ? 1.0f / A[tri(t) + t] : 0.f;
-    }
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        for (int kk = 0; kk < 32; ++kk) {
-            const int k = 32 * m + kk;
-            if (k >= G) break;   // warp-uniform
-            const float yk = __shfl_sync(0xffffffffu, v[m] * rd[m], kk);
-            if (lane == kk) v[m] = yk;
-#pragma unroll
-            for (int mm = m; mm < 4; ++mm) {
-                const int t = lane + 32 * mm;
-                if (t > k && t < G) v[mm] = fmaf(-A[tri(t) + k], yk, v[mm]);
-            }
-        }
-    }
-#pragma unroll
-    for (int m = 3; m >= 0; --m) {
-        for (int kk = 31; kk >= 0; --kk) {
-            const int k = 32 * m + kk;
-            if (k >= G) continue;   // warp-uniform
-            const float sk = __shfl_sync(0xffffffffu, v[m] * rd[m], kk);
-            if (lane == kk) v[m] = sk;
-#pragma unroll
-            for (int mm = 0; mm <= m; ++mm) {
-                const int t = lane + 32 * mm;
-                if (t < k) v[mm] = fmaf(-A[tri(k) + t], sk, v[mm]);
-            }
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int t = lane + 32 * m;
-        if (t < G) y[t] = v[m];
-    }
-    __syncwarp();
-}
-
-// Row r0 of the (exactly symmetric) Gram matrix times x = xh + xl, in
-// double-float.  Entry (r0, c) is read as (c, r0), so that lanes with
-// consecutive r0 read consecutive addresses, eight loads at a time.
-template <bool kPair>
-__device__ __forceinline__ DF gram_dot(const float2 *gj, int G, int r0, const float *xh,
-                                       const float *xl) {
+// Row t of the Gram matrix times x = xh + xl (xl null: x = xh), in double-float.
+// COPY: also the float32 entries on and below the diagonal into A, entry (c, t)
+// for t <= c, with `finite` false if any entry is not.
+template <bool COPY>
+__device__ __forceinline__ DF big_dot(const float2 *gj, int G, int t, const float *xh, const float *xl,
+                                      float *A, int ld, bool &finite) {
     DF acc{0.f, 0.f};
-    auto term = [&](float2 e, int c) {
-        df_add_prod(acc, e.x, xh[c]);
-        acc.l = fmaf(e.y, xh[c], acc.l);
-        if (kPair) acc.l = fmaf(e.x, xl[c], acc.l);
-    };
-    int c = 0;
-    for (; c + 8 <= G; c += 8) {
-        float2 v[8];
+    constexpr int kU = 16;
+    for (int c0 = 0; c0 < G; c0 += kU) {
+        float2 v[kU];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = __ldg(gj + (size_t)(c + u) * G + r0);
+        for (int u = 0; u < kU; ++u)
+            v[u] = c0 + u < G ? __ldg(gj + (size_t)(c0 + u) * G + t) : make_float2(0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) term(v[u], c + u);
+        for (int u = 0; u < kU; ++u) {
+            const int c = c0 + u;
+            if (c >= G) break;               // uniform
+            df_add_prod(acc, v[u].x, xh[c]);
+            acc.l = fmaf(v[u].y, xh[c], acc.l);
+            if (xl) acc.l = fmaf(v[u].x, xl[c], acc.l);
+            if (COPY) {
+                if (t <= c) A[c * ld + t] = v[u].x;
+                finite &= (bool)isfinite(v[u].x);
+            }
+        }
     }
-    for (; c < G; ++c) term(__ldg(gj + (size_t)c * G + r0), c);
     return acc;
 }
 
-// Solve for G > 32 (e.g. 86 groups of the 11008-input layers): the Gram
-// matrix stays in global memory (L2) and is read row by row; the float32
-// factor lives in shared memory.  Every dot product with the Gram matrix --
-// the gradient, the two refinement residuals, the objective -- is summed in
-// double-float on the entries' float pairs.
-__global__ void scale_solve_kernel(SolveArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int G = a.d / a.g;
-    const int wpb = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j = blockIdx.x * wpb + w;
-    if (j >= a.p || (!a.eval_only && !a.active[j])) return;  // warp-uniform
-    float *A = (float *)(smem_raw + (size_t)w * solve_warp_bytes(G));
-    float *so = A + tri(G);         // s_old
-    float *y = so + G;              // float work vector
-    float *bh = y + G, *bl = bh + G;    // gradient g (double-float)
-    float *ih = bl + G, *il = ih + G;   // increment of the scales (double-float)
+// Sum of one DF per thread, the same in every thread.
+template <int NT>
+__device__ __forceinline__ DF block_sum(DF v, DF *red) {
+    v = df_warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    DF s = red[0];
+    for (int w = 1; w < NT / 32; ++w) s = df_add(s, red[w]);
+    return s;
+}
+
+__device__ __forceinline__ void load_row8(const float *p, float (&l)[kPanel]) {
+    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+    l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w;
+    l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
+}
+
+// In-place lower Cholesky of A (rows and columns beyond G are not touched),
+// rd[a] = 1 / L_aa.  False (in every thread) when a pivot is not above `thr` or
+// not finite.
+template <int NT>
+__device__ bool big_cholesky(float *A, int ld, int G, float thr, float *rd, int *flag) {
+    const int t = threadIdx.x, lane = t & 31;
+    if (t == 0) *flag = 1;
+    for (int k0 = 0; k0 < G; k0 += kPanel) {
+        const int nk = min(kPanel, G - k0);
+        __syncthreads();
+        if (t < 32) {
+            // lane r < 8: row k0 + r of the diagonal block
+            float a[kPanel];
+#pragma unroll
+            for (int c = 0; c < kPanel; ++c)
+                a[c] = (lane < nk && c <= lane) ? A[(k0 + lane) * ld + k0 + c] : 0.f;
+            bool good = true;
+            float inv = 0.f;
+#pragma unroll
+            for (int k = 0; k < kPanel; ++k) {
+                if (k < nk) {                       // uniform
+                    const float piv = __shfl_sync(0xffffffffu, a[k], k);
+                    good = good && piv > thr && isfinite(piv);
+                    const float l = sqrtf(piv);
+                    if (lane == k) {
+                        a[k] = l;
+                        inv = 1.0f / l;
+                    }
+                    if (lane > k) a[k] /= l;
+#pragma unroll
+                    for (int c = k + 1; c < kPanel; ++c) {
+                        const float lc = __shfl_sync(0xffffffffu, a[k], c);
+                        if (lane >= c) a[c] = fmaf(-a[k], lc, a[c]);
+                    }
+                }
+            }
+            if (lane < nk) {
+                rd[k0 + lane] = inv;
+#pragma unroll
+                for (int c = 0; c < kPanel; ++c)
+                    if (c <= lane) A[(k0 + lane) * ld + k0 + c] = a[c];
+            }
+            if (!good && lane == 0) *flag = 0;
+        }
+        __syncthreads();
+        if (!*flag) return false;                   // uniform
+        const int k1 = k0 + kPanel;
+        // rows below: x L_kk^T = a
+        if (t >= k1 && t < G) {
+            float x[kPanel];
+            float4 *row = reinterpret_cast<float4 *>(A + t * ld + k0);
+            const float4 p0 = row[0], p1 = row[1];
+            x[0] = p0.x; x[1] = p0.y; x[2] = p0.z; x[3] = p0.w;
+            x[4] = p1.x; x[5] = p1.y; x[6] = p1.z; x[7] = p1.w;
+#pragma unroll
+            for (int c = 0; c < kPanel; ++c) {
+                float l[kPanel];
+                load_row8(A + (k0 + c) * ld + k0, l);
+#pragma unroll
+                for (int k = 0; k < c; ++k) x[c] = fmaf(-x[k], l[k], x[c]);
+                x[c] /= l[c];
+            }
+            row[0] = make_float4(x[0], x[1], x[2], x[3]);
+            row[1] = make_float4(x[4], x[5], x[6], x[7]);
+        }
+        __syncthreads();
+        // trailing triangle, 4 x 4 tiles (i, j), j <= i
+        const int nt = (G - k1 + 3) / 4;
+        for (int e = t; e < nt * (nt + 1) / 2; e += NT) {
+            int i = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+            if ((i + 1) * (i + 2) / 2 <= e) ++i;
+            if (i * (i + 1) / 2 > e) --i;
+            const int j = e - i * (i + 1) / 2;
+            const float *pa = A + (k1 + 4 * i) * ld + k0, *pb = A + (k1 + 4 * j) * ld + k0;
+            float *pc = A + (k1 + 4 * i) * ld + k1 + 4 * j;
+            float4 b0[4], b1[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                b0[c] = *reinterpret_cast<const float4 *>(pb + c * ld);
+                b1[c] = *reinterpret_cast<const float4 *>(pb + c * ld + 4);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 a0 = *reinterpret_cast<const float4 *>(pa + r * ld);
+                const float4 a1 = *reinterpret_cast<const float4 *>(pa + r * ld + 4);
+                float4 c4 = *reinterpret_cast<const float4 *>(pc + r * ld);
+                float cv[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    cv[c] = fmaf(-a0.x, b0[c].x, cv[c]);
+                    cv[c] = fmaf(-a0.y, b0[c].y, cv[c]);
+                    cv[c] = fmaf(-a0.z, b0[c].z, cv[c]);
+                    cv[c] = fmaf(-a0.w, b0[c].w, cv[c]);
+                    cv[c] = fmaf(-a1.x, b1[c].x, cv[c]);
+                    cv[c] = fmaf(-a1.y, b1[c].y, cv[c]);
+                    cv[c] = fmaf(-a1.z, b1[c].z, cv[c]);
+                    cv[c] = fmaf(-a1.w, b1[c].w, cv[c]);
+                }
+                *reinterpret_cast<float4 *>(pc + r * ld) = make_float4(cv[0], cv[1], cv[2], cv[3]);
+            }
+        }
+    }
+    __syncthreads();
+    return true;
+}
+
+// v <- (L L^T)^{-1} v, thread t holding v_t; x [Gp] is shared scratch.  Per panel
+// every thread solves the 8 x 8 block for itself (rows beyond G are zero, their
+// reciprocal pivots too) and updates its own entry.
+__device__ float big_chol_solve(const float *A, int ld, int G, const float *rd, float *x, float v) {
+    const int t = threadIdx.x;
+    for (int k0 = 0; k0 < G; k0 += kPanel) {
+        if (t >= k0 && t < k0 + kPanel) x[t] = v;
+        __syncthreads();
+        float s[kPanel], r[kPanel];
+        load_row8(x + k0, s);
+        load_row8(rd + k0, r);
+#pragma unroll
+        for (int c = 0; c < kPanel; ++c) {
+            float l[kPanel];
+            load_row8(A + (k0 + c) * ld + k0, l);
+#pragma unroll
+            for (int k = 0; k < c; ++k) s[c] = fmaf(-l[k], s[k], s[c]);
+            s[c] *= r[c];
+            if (t == k0 + c) v = s[c];
+        }
+        if (t >= k0 + kPanel && t < G) {
+            float l[kPanel];
+            load_row8(A + t * ld + k0, l);
+#pragma unroll
+            for (int k = 0; k < kPanel; ++k) v = fmaf(-l[k], s[k], v);
+        }
+    }
+    __syncthreads();        // the last panel's x is written again below
+    for (int k0 = (G - 1) / kPanel * kPanel; k0 >= 0; k0 -= kPanel) {
+        if (t >= k0 && t < k0 + kPanel) x[t] = v;
+        __syncthreads();
+        float s[kPanel], r[kPanel];
+        load_row8(x + k0, s);
+        load_row8(rd + k0, r);
+#pragma unroll
+        for (int c = kPanel - 1; c >= 0; --c) {
+            // x_c is final: take it out of the rows above (columns k < c of row c)
+            s[c] *= r[c];
+            if (t == k0 + c) v = s[c];
+            float l[kPanel];
+            load_row8(A + (k0 + c) * ld + k0, l);
+#pragma unroll
+            for (int k = 0; k < c; ++k) s[k] = fmaf(-l[k], s[c], s[k]);
+        }
+        if (t < k0) {
+#pragma unroll
+            for (int k = kPanel - 1; k >= 0; --k) v = fmaf(-A[(k0 + k) * ld + t], s[k], v);
+        }
+    }
+    return v;
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT, 768 / NT) scale_solve_kernel(SolveArgs a) {
+    extern __shared__ __align__(16) float fsm[];
+    __shared__ DF red[NT / 32];
+    __shared__ int flag;
+    const int G = a.d / a.g, Gp = (G + 7) / 8 * 8, ld = solve_ld(G);
+    const int j = blockIdx.x, t = threadIdx.x, tc = min(t, G - 1);
+    if (!a.eval_only && !a.active[j]) return;   // uniform
+    const bool own = t < G;
+    float *A = fsm;                      // [Gp][ld]
+    float *so = A + Gp * ld;             // s_old, later s_new
+    float *rd = so + Gp, *x = rd + Gp;   // reciprocal pivots; solve scratch
+    float *ih = x + Gp, *il = ih + Gp;   // increment of the scales (double-float)
     const float2 *gj = a.gram + (size_t)j * G * G;
-    const double *rj = a.rhs + (size_t)j * G;
-    // the row's Gram matrix (8 G^2 bytes) is read by five or six passes:
-    // bring it into L2 once, all lines at a time
-    {
-        const char *gb = (const char *)gj;
-        const size_t bytes = (size_t)G * G * sizeof(double);
-        for (size_t off = (size_t)lane * 128; off < bytes; off += 32 * 128)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(gb + off));
-        if (lane == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(gb + bytes - 1));
-    }
-    for (int t = lane; t < G; t += 32) so[t] = a.S[(size_t)j * G + t];
-    __syncwarp();
+    const float s_old = own ? a.S[(size_t)j * G + t] : 0.f;
+    const DF rh = own ? split_double(a.rhs[(size_t)j * G + t]) : DF{0.f, 0.f};
+    if (own) so[t] = s_old;
+    // the rows that pad the last panel; what stands right of the diagonal, the
+    // columns from G on included, is never read into an entry on or below it
+    for (int e = G * ld + t; e < Gp * ld; e += NT) A[e] = 0.f;
+    if (t >= G && t < Gp) rd[t] = 0.f;
+    __syncthreads();
     // gradient g = rhs - Gram s_old and F(s_old) = wHw - s_old^T (rhs + g)
-    bool bfin = true;
+    bool finite = true;
+    const DF gs0 = big_dot<true>(gj, G, tc, so, nullptr, A, ld, finite);
+    const DF gd = df_add(rh, df_neg(gs0));
+    const bool bfin = !own || isfinite(gd.h);
     DF fs{0.f, 0.f};
-    for (int r0 = lane; r0 < G; r0 += 32) {
-        const DF gs = gram_dot<false>(gj, G, r0, so, nullptr);
-        const DF rr = split_double(rj[r0]);
-        const DF gr = df_add(rr, df_neg(gs));
-        bh[r0] = gr.h;
-        bl[r0] = gr.l;
-        const DF rg = df_add(rr, gr);
-        df_add_prod(fs, so[r0], rg.h);
-        fs.l = fmaf(so[r0], rg.l, fs.l);
-        bfin &= (bool)isfinite(gr.h);
+    if (own) {
+        const DF rg = df_add(rh, gd);
+        df_add_prod(fs, s_old, rg.h);
+        fs.l = fmaf(s_old, rg.l, fs.l);
     }
-    const double F_old = a.wHw[j] - df_to_double(df_warp_sum(fs));
-    if (a.L_out && lane == 0) a.L_out[j] = F_old;
+    const double F_old = a.wHw[j] - df_to_double(block_sum<NT>(fs, red));
+    if (a.L_out && t == 0) a.L_out[j] = F_old;
     if (a.eval_only) return;
     if (a.o.fixed_grid) {
         // fixed grid: the scales stay; L^(k) is the objective of the current state
-        bool stop = false;
-        if (a.o.early_stop && a.k >= 2) {
-            const double dec = a.L_prev[j] - F_old;
-            const double den = fmax(fabs(a.L_prev[j]), (double)a.o.eps);
-            stop = (dec / den <= (double)a.o.tau_rel) || (fabs(dec) <= (double)a.o.tau_abs);
-        }
-        if (lane == 0) {
+        if (t == 0) {
+            bool stop = false;
+            if (a.o.early_stop && a.k >= 2) {
+                const double dec = a.L_prev[j] - F_old;
+                const double den = fmax(fabs(a.L_prev[j]), (double)a.o.eps);
+                stop = (dec / den <= (double)a.o.tau_rel) || (fabs(dec) <= (double)a.o.tau_abs);
+            }
             a.L_prev[j] = F_old;
             a.iters[j] = a.k;
             if (stop) a.active[j] = 0;
         }
         return;
     }
-    // float32 copy of the Gram matrix (the high part of a pair is the
-    // correctly rounded float32 of the entry), plus a ridge shift of the
-    // diagonal
-    auto load_sym = [&](float shift) -> bool {
-        bool finite = true;
-#pragma unroll 4
-        for (int r0 = 0; r0 < G; ++r0)
-            for (int c0 = lane; c0 <= r0; c0 += 32) {
-                float v = __ldg(gj + (size_t)r0 * G + c0).x;
-                if (r0 == c0) v += shift;
-                if (!isfinite(v)) finite = false;
-                A[tri(r0) + c0] = v;
-            }
-        __syncwarp();
-        return __all_sync(0xffffffffu, finite);
-    };
-    bool finite = load_sym(0.f);
-    float md = 0.f;
-    for (int t = lane; t < G; t += 32) md = fmaxf(md, A[tri(t) + t]);
-    md = warp_max(md);
-    bool ok = finite && warp_cholesky(A, G, a.o.rcond * fmaxf(md, a.o.eps));
-    int used_ridge = 0;
-    if (!ok) {
-        used_ridge = 1;
-        load_sym(a.o.ridge);
-        ok = warp_cholesky(A, G, 0.f);
+    // float32 factor (the high part of a pair is the correctly rounded float32
+    // of the entry), with the ridge retry
+    finite = __syncthreads_and(finite);
+    __shared__ float wmax[NT / 32];
+    {
+        const float m = warp_max(own ? A[t * ld + t] : 0.f);
+        if ((t & 31) == 0) wmax[t >> 5] = m;
     }
-    ok = ok && __all_sync(0xffffffffu, bfin);
+    __syncthreads();
+    float md = wmax[0];
+    for (int w = 1; w < NT / 32; ++w) md = fmaxf(md, wmax[w]);
+    bool ok = finite && big_cholesky<NT>(A, ld, G, a.o.rcond * fmaxf(md, a.o.eps), rd, &flag);
+    int used_ridge = 0;
+    if (!ok) {                                  // uniform
+        used_ridge = 1;
+        __syncthreads();
+        if (own)
+            for (int c = t; c < G; ++c) A[c * ld + t] = __ldg(gj + (size_t)c * G + t).x + (c == t ? a.o.ridge : 0.f);
+        for (int e = G * ld + t; e < Gp * ld; e += NT) A[e] = 0.f;
+        __syncthreads();
+        ok = big_cholesky<NT>(A, ld, G, 0.f, rd, &flag);
+    }
+    ok = __syncthreads_and(ok && bfin);
     auto fail = [&]() {
-        if (lane == 0) {
+        if (t == 0) {
             a.ridge[j] += used_ridge;
             a.rstat[j] = JARQ_ERR_NUMERICAL;
             a.active[j] = 0;
@@ -277,76 +378,71 @@ __global__ void scale_solve_kernel(SolveArgs a) {
     // (Gram + lambda I) inc = g - lambda s_old, refined twice with
     // double-float residuals
     const float lam = used_ridge ? a.o.ridge : 0.f;
-    for (int t = lane; t < G; t += 32) {
-        ih[t] = 0.f;
-        il[t] = 0.f;
-        DF v{bh[t], bl[t]};
-        df_add_prod(v, -lam, so[t]);
-        y[t] = __fadd_rn(v.h, v.l);
-    }
+    DF rhs0 = gd;
+    df_add_prod(rhs0, -lam, s_old);
+    DF inc{0.f, 0.f};
+    float y = own ? __fadd_rn(rhs0.h, rhs0.l) : 0.f;
     for (int step = 0; step < 3; ++step) {
-        warp_chol_solve(A, G, y);
-        for (int t = lane; t < G; t += 32) {
-            const DF s2 = df_add({ih[t], il[t]}, {y[t], 0.f});
-            ih[t] = s2.h;
-            il[t] = s2.l;
+        y = big_chol_solve(A, ld, G, rd, x, y);
+        if (own) {
+            inc = df_add(inc, DF{y, 0.f});
+            ih[t] = inc.h;
+            il[t] = inc.l;
         }
-        __syncwarp();
         if (step == 2) break;
-        for (int r0 = lane; r0 < G; r0 += 32) {
-            // res = g - lambda (s_old + inc) - Gram inc
-            DF res{bh[r0], bl[r0]};
-            df_add_prod(res, -lam, so[r0]);
-            df_add_prod(res, -lam, ih[r0]);
-            res.l = fmaf(-lam, il[r0], res.l);
-            res = df_add(res, df_neg(gram_dot<true>(gj, G, r0, ih, il)));
-            y[r0] = __fadd_rn(res.h, res.l);
-        }
-        __syncwarp();
+        __syncthreads();
+        // res = g - lambda (s_old + inc) - Gram inc
+        DF res = rhs0;
+        df_add_prod(res, -lam, inc.h);
+        res.l = fmaf(-lam, inc.l, res.l);
+        bool f2 = true;
+        res = df_add(res, df_neg(big_dot<false>(gj, G, tc, ih, il, nullptr, 0, f2)));
+        y = own ? __fadd_rn(res.h, res.l) : 0.f;
+        __syncthreads();
     }
-    bool sfin = true;
-    for (int t = lane; t < G; t += 32) sfin &= (bool)(isfinite(ih[t]) && isfinite(il[t]));
-    if (!__all_sync(0xffffffffu, sfin)) {
+    if (!__syncthreads_and(!own || (isfinite(inc.h) && isfinite(inc.l)))) {
         fail();
         return;
     }
     // s_new = s_old + inc, rounded once to float32
-    for (int t = lane; t < G; t += 32) {
-        const DF s2 = df_add({so[t], 0.f}, {ih[t], il[t]});
-        y[t] = __fadd_rn(s2.h, s2.l);
+    float sn = 0.f;
+    if (own) {
+        const DF s2 = df_add({s_old, 0.f}, inc);
+        sn = __fadd_rn(s2.h, s2.l);
+        so[t] = sn;
     }
-    __syncwarp();
+    __syncthreads();
     // L^{(k)} at the stored float32 scales, from the unridged Gram matrix
+    bool f2 = true;
+    const DF gs = big_dot<false>(gj, G, tc, so, nullptr, nullptr, 0, f2);
     DF t1{0.f, 0.f}, t2{0.f, 0.f};
-    for (int r0 = lane; r0 < G; r0 += 32) {
-        const DF gs = gram_dot<false>(gj, G, r0, y, nullptr);
-        const DF rr = split_double(rj[r0]);
-        df_add_prod(t1, y[r0], rr.h);
-        t1.l = fmaf(y[r0], rr.l, t1.l);
-        df_add_prod(t2, y[r0], gs.h);
-        t2.l = fmaf(y[r0], gs.l, t2.l);
+    if (own) {
+        df_add_prod(t1, sn, rh.h);
+        t1.l = fmaf(sn, rh.l, t1.l);
+        df_add_prod(t2, sn, gs.h);
+        t2.l = fmaf(sn, gs.l, t2.l);
     }
-    double L_new = a.wHw[j] - 2.0 * df_to_double(df_warp_sum(t1)) + df_to_double(df_warp_sum(t2));
+    t1 = block_sum<NT>(t1, red);
+    t2 = block_sum<NT>(t2, red);
+    double L_new = a.wHw[j] - 2.0 * df_to_double(t1) + df_to_double(t2);
     // Remark ridge-acceptance (optional): a ridge-stabilised solve that would
     // raise F_j is dropped and the previous scales stay
     const bool keep_old = used_ridge && a.o.ridge_accept && !(L_new <= F_old);
     if (keep_old) L_new = F_old;
-    bool stop = false;
-    if (a.o.early_stop && a.k >= 2) {
-        const double dec = a.L_prev[j] - L_new;
-        const double den = fmax(fabs(a.L_prev[j]), (double)a.o.eps);
-        stop = (dec / den <= (double)a.o.tau_rel) || (fabs(dec) <= (double)a.o.tau_abs);
-    }
-    if (!keep_old)
-        for (int t = lane; t < G; t += 32) a.S[(size_t)j * G + t] = y[t];
-    if (lane == 0) {
+    if (!keep_old && own) a.S[(size_t)j * G + t] = sn;
+    if (t == 0) {
+        bool stop = false;
+        if (a.o.early_stop && a.k >= 2) {
+            const double dec = a.L_prev[j] - L_new;
+            const double den = fmax(fabs(a.L_prev[j]), (double)a.o.eps);
+            stop = (dec / den <= (double)a.o.tau_rel) || (fabs(dec) <= (double)a.o.tau_abs);
+        }
         a.L_prev[j] = L_new;
         a.iters[j] = a.k;
         a.ridge[j] += used_ridge;
         if (stop) a.active[j] = 0;
     }
 }
-
 
 // ---------------------------------------------------------------------------
 // Register-resident solve for G <= 32 (the g = 128 layers of 4096 inputs).
@@ -358,15 +454,12 @@ __global__ void scale_solve_kernel(SolveArgs a) {
 // Lane l owns row l of the Gram matrix (= column l: it is exactly
 // symmetric) as the double-float pair per entry that the Gram kernel
 // stores.  The float32 Cholesky keeps row l in registers and
-// broadcasts the column of each step with shuffles: the same operations in
-// the same order as warp_cholesky, so the factor (and the ridge decision)
-// is bit-identical.  The triangular solves multiply by the reciprocal of
-// the pivots; the float64-accurate refinement makes the stored scales
-// independent of that rounding.
+// broadcasts the column of each step with shuffles.  The triangular solves
+// multiply by the reciprocal of the pivots; the refinement makes the stored
+// scales independent of that rounding.
 // ---------------------------------------------------------------------------
 
-// In-place lower Cholesky with lane a holding row a in A[]; on and below
-// the diagonal the operations and their order are those of warp_cholesky.
+// In-place lower Cholesky with lane a holding row a in A[].
 __device__ __forceinline__ bool reg_cholesky(float (&A)[32], int G, float thr) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -379,9 +472,8 @@ __device__ __forceinline__ bool reg_cholesky(float (&A)[32], int G, float thr) {
             if (lane > k) lak = A[k] / lkk;
             if (lane == k) A[k] = lkk;
             if (lane > k) A[k] = lak;
-            // entries b <= a take the update of warp_cholesky; the entries
-            // above the diagonal (b > a) are never read again, so they take
-            // it as well instead of a predicate per entry
+            // the entries above the diagonal (b > a) are never read again, so
+            // they take the update as well instead of a predicate per entry
 #pragma unroll
             for (int b = k + 1; b < 32; ++b) {
                 const float lbk = __shfl_sync(0xffffffffu, lak, b);
@@ -594,6 +686,16 @@ __global__ void __launch_bounds__(32 * kSmallWarps, 4) scale_solve_small_kernel(
     }
 }
 
+template <int NT>
+cudaError_t launch_big(const SolveArgs &a, cudaStream_t s) {
+    static std::atomic<unsigned long long> attr_done{0};
+    const cudaError_t e =
+        set_max_dynamic_smem((const void *)scale_solve_kernel<NT>, (int)solve_bytes(NT), attr_done);
+    if (e != cudaSuccess) return e;
+    scale_solve_kernel<NT><<<a.p, NT, solve_bytes(a.d / a.g), s>>>(a);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_scale_solve(const float2 *gram, const double *rhs, const double *wHw, float *S,
@@ -608,18 +710,9 @@ cudaError_t launch_scale_solve(const float2 *gram, const double *rhs, const doub
         scale_solve_small_kernel<<<(p + kSmallWarps - 1) / kSmallWarps, 32 * kSmallWarps, 0, s>>>(a);
         return cudaGetLastError();
     }
-    // at most four warps per block, and blocks small enough that several fit
-    // on an SM: the kernel is bound by the latency of each warp's chain
-    const size_t per_warp = solve_warp_bytes(G);
-    int wpb = (int)((56 * 1024) / per_warp);
-    if (wpb > 4) wpb = 4;
-    if (wpb < 1) wpb = 1;
-    const size_t smem = per_warp * wpb;
-    cudaError_t e = cudaFuncSetAttribute(scale_solve_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    scale_solve_kernel<<<(p + wpb - 1) / wpb, 32 * wpb, smem, s>>>(a);
-    return cudaGetLastError();
+    if (G <= 64) return launch_big<64>(a, s);
+    if (G <= 96) return launch_big<96>(a, s);
+    return launch_big<128>(a, s);
 }
 
 }  // namespace jarq

@@ -13,7 +13,7 @@ torch = pytest.importorskip("torch")
 pytestmark = [pytest.mark.gpu,
               pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
 
-from oracle import Options, group_target, objective, prepare_hessian, refine_layer  # noqa: E402
+from oracle import Options, group_target, joint_scales, objective, prepare_hessian, refine_layer  # noqa: E402
 from synth import Layer, small_layer, tiny_layer  # noqa: E402
 from tests.parity import compare_final, gpu_refine, lockstep  # noqa: E402
 
@@ -123,6 +123,24 @@ def test_many_groups_parity(jarq, din, dout, g, bits, K):
     assert m["S_rel_max_same_rows"] <= REL_S and m["F_rel_max_same_rows"] <= REL_F, m
     assert m["F_rel_all"] <= REL_F, m
     assert m["gpu_no_worse_than_host"], m
+
+
+@pytest.mark.parametrize("G", [33, 40, 63, 64, 65, 95, 96, 97, 127, 128])
+def test_block_solve_group_edges(jarq, G):
+    """The joint fit at the edges of the scale solve for more than 32 groups:
+    the block sizes (64, 96 and 128 groups), whole and partial panels of eight.
+    Both sides round a solution refined in more than float32 to float32, so
+    the scales agree within 1e-6 relative, the objectives within 1e-6."""
+    lay = _many_group_layer(64 * G, 9, 64, 3, 1, seed=G)
+    prep = prepare_hessian(lay.H, lay.g)
+    ref32 = joint_scales(prep, lay.W, lay.S0, lay.Q0, lay.Z).astype(np.float32)
+    hess = jarq.prepare(lay.H, lay.g)
+    S = lay.S0.copy()
+    Fb, Fa = jarq.fit_scales(hess, lay.W, S, lay.Q0, lay.Z, lay.bits, "joint")
+    hess.close()
+    assert np.all(np.abs(S.astype(np.float64) - ref32) <= 1e-6 * np.abs(ref32))
+    np.testing.assert_allclose(Fb, objective(prep, lay.W, lay.S0, lay.Q0, lay.Z), rtol=1e-6)
+    np.testing.assert_allclose(Fa, objective(prep, lay.W, ref32, lay.Q0, lay.Z), rtol=1e-6)
 
 
 @pytest.mark.parametrize("early_stop", [False, True])
