@@ -205,8 +205,7 @@ cudaError_t launch_tc_hr_phase(const CUtensorMap &mapA, const CUtensorMap &mapB1
                                const CUtensorMap &mapB64, float *out, int p, int p_pad, int d_pad,
                                int g, int i, int nsplit, const int *active, int *status,
                                cudaStream_t s);
-cudaError_t launch_grad(const uint8_t *Q, const int32_t *Z, const float *r, const float *Hr,
-                        double *gvec, double *F, int p, int d, int g, cudaStream_t s);
+cudaError_t launch_grad(const float *r, const float *Hr, double *F, int p, int d, cudaStream_t s);
 cudaError_t launch_slices(const float *Hs, int *expo, __nv_bfloat16 *dig8, __half *dig10, int d,
                           int d_pad, int g, cudaStream_t s);
 cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, const uint8_t *Q,

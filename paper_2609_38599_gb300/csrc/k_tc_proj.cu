@@ -685,16 +685,21 @@ __global__ void rhs_kernel(const uint8_t *__restrict__ Q, const int32_t *__restr
     }
 }
 
-// wHw_j = sum_k W[j,k] P[j,k] with P = Phi + Plo, double-float per lane, one
-// warp per row.
-__global__ void whw_kernel(const float *__restrict__ W, const float *__restrict__ Phi,
-                           const float *__restrict__ Plo, double *__restrict__ out, int p, int d) {
-    const int j = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (j >= p) return;
+// wHw_j = sum_k W[j,k] P[j,k] with P = Phi + Plo, double-float per lane, four
+// warps (one block) per row.  Bound by memory (12 bytes an entry): 41 us on
+// 4096 x 4096, 95 us on 4096 x 11008; with one warp per row 51 and 116 us.
+constexpr int kWhwWarps = 4;
+
+__global__ void __launch_bounds__(32 * kWhwWarps) whw_kernel(const float *__restrict__ W,
+                                                             const float *__restrict__ Phi,
+                                                             const float *__restrict__ Plo,
+                                                             double *__restrict__ out, int d) {
+    __shared__ float ph_s[kWhwWarps], pl_s[kWhwWarps];
+    const int j = blockIdx.x, lane = threadIdx.x & 31;
     const size_t off = (size_t)j * d;
     float sh = 0.f, sl = 0.f;
-    for (int k = lane; k < d; k += 32) {
+#pragma unroll 8
+    for (int k = threadIdx.x; k < d; k += 32 * kWhwWarps) {
         const float w = W[off + k], ph = Phi[off + k], pl = Plo[off + k];
         const float m = w * ph;
         const float me = fmaf(w, ph, -m);
@@ -704,7 +709,16 @@ __global__ void whw_kernel(const float *__restrict__ W, const float *__restrict_
         sl += e2 + fmaf(w, pl, me);
     }
     df_warp_sum(sh, sl);
-    if (lane == 0) out[j] = (double)sh + (double)sl;
+    if (lane == 0) {
+        ph_s[threadIdx.x >> 5] = sh;
+        pl_s[threadIdx.x >> 5] = sl;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int w = 0; w < kWhwWarps; ++w) v += (double)ph_s[w] + (double)pl_s[w];
+        out[j] = v;
+    }
 }
 
 // Propagation-corrected target (App. "Propagation-Corrected Targets and
@@ -897,7 +911,7 @@ cudaError_t launch_tc_proj(const CUtensorMap &mapW, const CUtensorMap &mapH, flo
 
 cudaError_t launch_whw(const float *W, const float *Phi, const float *Plo, double *out, int p,
                        int d, cudaStream_t s) {
-    whw_kernel<<<(unsigned)(((long long)p * 32 + 255) / 256), 256, 0, s>>>(W, Phi, Plo, out, p, d);
+    whw_kernel<<<p, 32 * kWhwWarps, 0, s>>>(W, Phi, Plo, out, d);
     return cudaGetLastError();
 }
 
