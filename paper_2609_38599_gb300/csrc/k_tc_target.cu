@@ -27,22 +27,23 @@
 //   warp 1       TMEM allocation; in the even CTA the single-thread MMA issuer
 //   warps 2..17  drain: warp w reads TMEM lanes 32 (w % 4) and 16 columns
 // Four 64-column accumulators per group h, double-buffered (512 columns).
-// The drain does 17 float32 operations per output and group (two outputs per
+// The drain does 14 float32 operations per output and group (two outputs per
 // instruction), hence sixteen drain warps.
 //
-// What bounds it, per group and CTA (4096 rows, g = 128, clock64 in a copy):
-// about 1560 cycles, of which the MMAs are 1024, the drain's arithmetic 1088
-// at the full float32 rate, and the tile loads and operand reads 128 KB of
-// shared-memory traffic.  Two accumulators keep MMA and drain of consecutive
-// groups overlapped, but a group's MMAs start only when all 32 drain warps
-// have read the accumulator two groups back.  Per launch of two groups (256
-// columns, K = 4096, CUDA events): 36.7 us.  One CTA per tile took 58.9 us
-// (192 KB of shared-memory traffic per group, and an issuing thread that
-// needed 800 cycles per group beside the drain's arithmetic).  Measured and
-// not kept: all digit sums read and the accumulator released before any
-// arithmetic (39.1 us: the four warps of a scheduler drift apart by a whole
-// group), a block barrier among the drain warps per group (39.1 us), one
-// polling lane per warp (37.3 us).
+// What bounds it, per group and CTA (4096 rows, g = 128): the MMAs take 1024
+// cycles, the drain's arithmetic 896 at the full float32 rate, the tile loads
+// and operand reads 128 KB of shared-memory traffic.  Two accumulators keep MMA
+// and drain of consecutive groups overlapped, but a group's MMAs start only when
+// all 32 drain warps have read the accumulator two groups back.  Per launch of
+// two groups (256 columns, CUDA events): 33.1 us at K = 4096, 73 us at K = 11008;
+// with 17 operations in the drain (the integer part of D_1 split off by adding a
+// constant, the product's error formed apart) 36.7 and 82 us.  One CTA per tile
+// took 58.9 us at K = 4096 (192 KB of shared-memory traffic per group, and an
+// issuing thread that needed 800 cycles per group beside the drain's
+// arithmetic).  Measured and not kept, at 17 operations: all digit sums read and
+// the accumulator released before any arithmetic (39.1 us: the four warps of a
+// scheduler drift apart by a whole group), a block barrier among the drain warps
+// per group (39.1 us), one polling lane per warp (37.3 us).
 #include <cmath>
 
 #include "tc_common.cuh"
@@ -75,7 +76,6 @@ struct TargetArgs {
     int p, p_pad, d_pad, g, G, seg_per_split;
     int i0, nb;               // groups i0 .. i0 + nb - 1 of this launch
     int prev0;                // groups prev0 .. i0 - 1: the previous grid rewrites their codes
-    float round_c;            // 1.5 * 2^(23 - k): rounds to multiples of 2^-k
 };
 
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
@@ -267,7 +267,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         for (int e = 0; e < 8; ++e) hi[e] = lo[e] = tc::f2(0.f);
         bool ok = true;
         const tc::F2 c10 = tc::f2(0x1p-10f), c20 = tc::f2(0x1p-20f);
-        const tc::F2 rc = tc::f2(a.round_c);
         const uint32_t released = tc::map_rank(aempty(0), 0);
         for (int u = 0; u < nseg; ++u) {
             const int b = u & 1;
@@ -300,33 +299,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 }
 #pragma unroll
                 for (int e = 0; e < 8; e += 2) {
-                    // D_0 + D_1 2^-10 exactly as (vh, vl): the digit sums are
-                    // integers with |D_0| <= 128 qmax 512 and |D_1 2^-10| < 2^14;
-                    // t = D_1 2^-10 rounded to a multiple of 2^-k (by adding
-                    // and subtracting 1.5 2^(23-k)), with k chosen on the host
-                    // so that |D_0 + t| < 2^(24-k): then vh = D_0 + t and
-                    // vl = D_1 2^-10 - t (|vl| <= 2^-(k+1)) are exact.  The
-                    // D_2, D_3 terms are below 2^-20 of the sum and enter the
-                    // low part.  Differences are formed from negated terms,
-                    // so that each is one instruction.
+                    // D_0 + D_1 2^-10 exactly as (vh, vl): vh is the rounded
+                    // sum, D_0 - vh is exact (both are multiples of 2^-10, and
+                    // D_1 2^-10, where it is the larger, is below 2^14), and so
+                    // is what the rounding left out.  The D_2, D_3 terms are
+                    // below 2^-20 of the sum and enter the low part.
                     auto pair = [&](const uint32_t (&v)[8]) {
                         return tc::f2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
                     };
-                    const tc::F2 d1 = pair(v1);
-                    const tc::F2 nt = tc::f2_sub(rc, tc::f2_fma(d1, c10, rc));         // -t
-                    const tc::F2 vh = tc::f2_sub(pair(v0), nt);
+                    const tc::F2 d0 = pair(v0), d1 = pair(v1);
+                    const tc::F2 vh = tc::f2_fma(d1, c10, d0);
                     const tc::F2 vl = tc::f2_fma(tc::f2_fma(pair(v3), c10, pair(v2)), c20,
-                                                 tc::f2_fma(d1, c10, nt));
-                    // (vh + vl) * scale, added to the accumulator
-                    const tc::F2 np = tc::f2_mul(vh, nscale);                           // -p
-                    const tc::F2 pe = tc::f2_fma(vh, scale, np);
+                                                 tc::f2_fma(d1, c10, tc::f2_sub(d0, vh)));
+                    // (vh + vl) * scale, added to the accumulator: a two-sum of
+                    // the rounded product (a sum formed by a multiply-add would
+                    // carry bits below both terms, and the differences would
+                    // not be exact; the product is negated for that reason)
+                    // whose last difference takes the product unrounded and so
+                    // its rounding error as well
                     tc::F2 &H = hi[(cc + e) / 2], &L = lo[(cc + e) / 2];
-                    const tc::F2 sm = tc::f2_sub(H, np);
-                    const tc::F2 bb = tc::f2_sub(sm, H);
-                    // (H - (sm - bb)) + (p - bb)
-                    const tc::F2 er = tc::f2_sub(tc::f2_sub(H, tc::f2_sub(sm, bb)), tc::f2_add(np, bb));
+                    const tc::F2 sm = tc::f2_sub(H, tc::f2_mul(vh, nscale));
+                    const tc::F2 nb = tc::f2_sub(H, sm);        // - (sm - H)
+                    const tc::F2 er = tc::f2_add(tc::f2_sub(H, tc::f2_add(sm, nb)), tc::f2_fma(vh, scale, nb));
                     H = sm;
-                    L = tc::f2_add(L, tc::f2_add(er, tc::f2_fma(vl, scale, pe)));
+                    L = tc::f2_add(L, tc::f2_fma(vl, scale, er));
                 }
             }
         }
@@ -390,16 +386,11 @@ cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, f
     if (e != cudaSuccess) return e;
     const int per = (G + nsplit - 1) / nsplit;
     const int tiles = (p + 255) / 256 * 2;   // pairs of row tiles
-    // quantum 2^-k of the exact digit split: the largest k with
-    // 128 qmax 512 + 2^14 <= 2^(24-k)
+    // the digit sums stay exact: 128 * 255 * 512 < 2^24
     if (qmax < 1 || qmax > 255 || g > 128) return cudaErrorInvalidValue;
-    const double bound = 128.0 * qmax * 512.0 + 16384.0;
-    int kq = 0;
-    while (kq < 7 && bound <= std::ldexp(1.0, 24 - (kq + 1))) ++kq;
-    const float round_c = (float)std::ldexp(1.5, 23 - kq);
     if (nb < 1 || i0 + nb > G || nsplit < 1) return cudaErrorInvalidValue;
     TargetArgs a{out_hi, out_lo, S, expoT, active, status, p, p_pad, d_pad, g, G, per,
-                 i0, nb, i0 - nb_prev, round_c};
+                 i0, nb, i0 - nb_prev};
     dim3 grid(tiles, nb * g / 64, nsplit);
     return launch_k(tc_target_kernel, grid, dim3(kThreads), (size_t)smem_bytes(per), s, pdl, mapC,
                     mapT, a);

@@ -299,6 +299,9 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
+// A product that only feeds an f2_add is fused with it, .rn or not (seen in the
+// results: the sum then carries bits below the rounded product).  Where the
+// product has to be rounded, subtract its negative with f2_sub.
 __device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
     F2 r;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
