@@ -12,22 +12,36 @@
 // features, contiguous; K = tokens, 128 bytes apart; 8-token atoms 1024
 // bytes apart; 64-feature atoms one box, 8 KiB, apart).
 //
-// One CTA computes one 128 x 256 tile (rows r0.., columns c0..) of the upper
-// triangle of X^T X over all n tokens:
-//   warp 0      TMA producer, 4-stage ring of 64-token chunks
-//               (A: 128 features, B: 256 features; a diagonal tile whose A
-//               features lie inside B reads them from B's tile)
-//   warp 1      TMEM allocation and the single-thread MMA issuer: one
-//               M128 x N256 x K16 MMA per 16 tokens
+// A pair of CTAs (cta_group::2) computes 256 x 256 tiles (rows r0.., columns
+// c0..) of the upper triangle of X^T X over all n tokens, every npairs-th tile of
+// an order in which the tiles that run at one time lie in blocks of 12 x 12 tiles
+// (they share their panels of X in L2).  In each CTA:
+//   warp 0      TMA producer, 5-stage ring of 64-token chunks: the features of
+//               its own 128 rows and of its half of the columns (on a diagonal
+//               tile these are the same), onto the even CTA's barriers
+//   warp 1      TMEM allocation; in the even CTA the MMA issuer: one
+//               M256 x N256 x K16 MMA per 16 tokens
 //   warps 2..9  drain: every 512 tokens the TMEM accumulator (restarted at
 //               zero, two of them alternate) is added into float32
-//               registers.  At the end the tile is added to H twice with
-//               coalesced accesses: mirrored, H[col][row], straight from the
-//               registers (a warp's 32 rows are contiguous there), and as
-//               H[row][col] in float4 through shared memory.
+//               registers.  At the end of a tile each warp adds its 32 x 128
+//               part to H, 32 x 32 at a time through its own shared memory, as
+//               H[row][col] and as H[col][row], in float4; the MMAs of the next
+//               tile run meanwhile.
 // Each unordered pair {i, j} belongs to exactly one tile element with
 // col >= row, so every element of H is written exactly once.
+//
+// What bounds it: for many tokens the MMAs (d = 11008, 32768 tokens: 2.56 ms; 2.43
+// ms without the additions to H; the same flops at the 1.75 PFLOP/s that a long
+// run sustains take 2.3 ms), for few the additions to H (d = 4096, 2048 tokens: 61
+// us; 30 us without them).  One CTA per 128 x 256 tile, its ring reused to stage
+// the whole tile, took 2.87 ms and 72 us: 192 bytes of shared memory were written
+// and read per cycle of the MMAs, now 128.  Measured and not kept: tiles in
+// columns over the whole matrix (2.98 ms), a ring of 4 stages (3.05 ms) or 6 (2.69
+// ms), sixteen drain warps (62 us), H prefetched into L2 ahead of the additions
+// (62 us, 2.73 ms).
 #include <math.h>
+
+#include <algorithm>
 
 #include "tc_common.cuh"
 
@@ -35,19 +49,22 @@ namespace jarq {
 namespace {
 
 constexpr int kBox = 64 * 64 * 2;          // one TMA box: 64 tokens x 64 features, fp16
-constexpr int kTileA = 2 * kBox;           // 128 features
-constexpr int kTileB = 4 * kBox;           // 256 features
+constexpr int kTileA = 2 * kBox;           // 128 row features
+constexpr int kTileB = 2 * kBox;           // 128 of the 256 column features
 constexpr int kStage = kTileA + kTileB;
-constexpr int kStages = 4;
-constexpr int kBars = 2 * kStages + 5;     // full, empty, afull[2], aempty[2], done
-constexpr int kSmem = 1024 + kStages * kStage + 8 * kBars + 16;
+constexpr int kStages = 5;
+constexpr int kBars = 2 * kStages + 4;     // full, empty, afull[2], aempty[2]
+constexpr int kDrainWarps = 8;
+constexpr int kTld = 33;                   // row pitch (floats) of a staged 32 x 32 part
+constexpr int kPart = 32 * kTld * 4;
+constexpr int kSmem = 1024 + kStages * kStage + kDrainWarps * kPart + 8 * kBars + 16;
 constexpr int kChunksPerDrain = 8;         // 512 tokens per tensor-core sum
-constexpr int kThreads = 320;
-constexpr int kTld = 257;                  // row pitch (floats) of the staged tile
-static_assert(128 * kTld * 4 <= kStages * kStage, "staged tile must fit the stage ring");
+constexpr int kThreads = 32 * (2 + kDrainWarps);
+constexpr int kBand = 12;                  // tiles per side of a block of the tile order
+static_assert(kSmem <= 227 * 1024, "ring and staged parts must fit an SM's shared memory");
 
-// fp16 x fp16 -> f32, M = 128, N = 256, both operands MN-major.
-constexpr uint32_t kIdesc = tc::idesc_f16_f32(128, 256) | (1u << 15) | (1u << 16);
+// fp16 x fp16 -> f32, M = 256, N = 256, both operands MN-major.
+constexpr uint32_t kIdesc = tc::idesc_f16_f32(256, 256) | (1u << 15) | (1u << 16);
 
 __device__ int g_syrk_status;
 
@@ -69,82 +86,53 @@ struct SyrkArgs {
     float *H;
     float scale;
     int d, n;
-    int ct;          // column tiles of 256
-    int rt;          // row tiles of 128
+    int nt;          // tiles per side
+    int ntiles;      // nt (nt + 1) / 2
 };
 
-// Linear index of an upper tile -> (row tile, column tile); column tile cj
-// holds row tiles 0 .. min(rt, 2 cj + 2) - 1.
-__device__ __forceinline__ void tile_of(int t, int rt, int ct, int &ri, int &cj) {
-    cj = 0;
-    for (; cj < ct; ++cj) {
-        const int m = min(rt, 2 * cj + 2);
-        if (t < m) break;
-        t -= m;
-    }
-    ri = t;
-}
-
-// One pass of the tile update H += scale * T over 256 threads, as float4
-// read-modify-writes of H with 8 loads in flight per thread.  MIRROR false:
-// H[r0+i][c0+j] for c0+j >= r0+i (float4 along j, 128 rows x 64); MIRROR
-// true: H[c0+j][r0+i] for c0+j > r0+i (float4 along i, 256 rows x 32).  A
-// float4 that straddles the diagonal updates its own elements only.
-template <bool MIRROR>
-__device__ __forceinline__ void add_tile_pass(const SyrkArgs &a, const float *T, int t, int r0,
-                                              int c0) {
-    constexpr int kSh = MIRROR ? 5 : 6;           // float4 per H row segment: 32 or 64
-#pragma unroll 1
-    for (int k0 = 0; k0 < 32; k0 += 8) {
-        float4 h[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int idx = t + 256 * (k0 + k);
-            const int u = idx >> kSh, v4 = 4 * (idx & ((1 << kSh) - 1));
-            const int hr = MIRROR ? c0 + u : r0 + u, hc = MIRROR ? r0 + v4 : c0 + v4;
-            // all four elements on the kept side of the diagonal
-            const bool full = hr < a.d && hc < a.d && (MIRROR ? hr > hc + 3 : hc >= hr);
-            h[k] = full ? *reinterpret_cast<const float4 *>(a.H + (size_t)hr * a.d + hc)
-                        : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int idx = t + 256 * (k0 + k);
-            const int u = idx >> kSh, v4 = 4 * (idx & ((1 << kSh) - 1));
-            const int hr = MIRROR ? c0 + u : r0 + u, hc = MIRROR ? r0 + v4 : c0 + v4;
-            if (hr >= a.d || hc >= a.d) continue;
-            // tile element of H[hr][hc + m]
-            auto tv = [&](int m) {
-                return MIRROR ? T[(v4 + m) * kTld + u] : T[u * kTld + v4 + m];
-            };
-            float *hp = a.H + (size_t)hr * a.d + hc;
-            if (MIRROR ? hr > hc + 3 : hc >= hr) {
-                float4 v = h[k];
-                v.x = fmaf(a.scale, tv(0), v.x);
-                v.y = fmaf(a.scale, tv(1), v.y);
-                v.z = fmaf(a.scale, tv(2), v.z);
-                v.w = fmaf(a.scale, tv(3), v.w);
-                *reinterpret_cast<float4 *>(hp) = v;
+// Position t of the tile order, advanced to ever larger t: blocks of kBand x
+// kBand tiles on and above the diagonal, column of blocks by column of blocks.
+struct TileOrder {
+    int nt, bi = 0, bj = 0, base = 0;
+    __device__ explicit TileOrder(int n) : nt(n) {}
+    __device__ void at(int t, int &ri, int &cj) {
+        int nr, nc, cnt;
+        for (;;) {
+            nr = min(kBand, nt - bi * kBand);
+            nc = min(kBand, nt - bj * kBand);
+            cnt = bi == bj ? nc * (nc + 1) / 2 : nr * nc;
+            if (t < base + cnt) break;
+            base += cnt;
+            if (bi == bj) {
+                bi = 0;
+                ++bj;
             } else {
-                for (int m = 0; m < 4; ++m)
-                    if (MIRROR ? hr > hc + m : hc + m >= hr) hp[m] = fmaf(a.scale, tv(m), hp[m]);
+                ++bi;
             }
         }
+        int k = t - base, c = 0;
+        if (bi == bj) {
+            while (k > c) k -= ++c;              // column c holds c + 1 tiles
+        } else {
+            c = k / nr;
+            k %= nr;
+        }
+        ri = bi * kBand + k;
+        cj = bj * kBand + c;
     }
-}
+};
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_syrk_kernel(const __grid_constant__ CUtensorMap mapX, SyrkArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *bars = (uint64_t *)(smem + kStages * kStage);
+    float *parts = (float *)(smem + kStages * kStage);
+    uint64_t *bars = (uint64_t *)(smem + kStages * kStage + kDrainWarps * kPart);
     uint32_t *tmem_slot = (uint32_t *)(bars + kBars);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int ri, cj;
-    tile_of(blockIdx.x, a.rt, a.ct, ri, cj);
-    const int r0 = ri * 128, c0 = cj * 256;
-    const bool a_in_b = r0 >= c0 && r0 < c0 + 256;
+    const int rank = (int)tc::cluster_rank();
+    const int pair = blockIdx.x / 2, npairs = gridDim.x / 2;
     const int nchunks = (a.n + 63) / 64;
     const int nper = (nchunks + kChunksPerDrain - 1) / kChunksPerDrain;
 
@@ -152,157 +140,213 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto empty = [&](int s) { return tc::smem_u32(bars + kStages + s); };
     auto afull = [&](int b) { return tc::smem_u32(bars + 2 * kStages + b); };
     auto aempty = [&](int b) { return tc::smem_u32(bars + 2 * kStages + 2 + b); };
-    const uint32_t done = tc::smem_u32(bars + 2 * kStages + 4);
+    auto tileA = [&](int s) { return tc::smem_u32(smem + s * kStage); };
     auto tileB = [&](int s) { return tc::smem_u32(smem + s * kStage + kTileA); };
-    auto tileA = [&](int s) {
-        return a_in_b ? tileB(s) + (uint32_t)((r0 - c0) / 64) * kBox : tc::smem_u32(smem + s * kStage);
-    };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            tc::mbar_init(full(s), 1);
+            tc::mbar_init(full(s), 1);      // the even CTA's: bytes of both CTAs
             tc::mbar_init(empty(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(afull(b), 1);
-            tc::mbar_init(aempty(b), 8);
+            tc::mbar_init(aempty(b), 2 * kDrainWarps);   // the even CTA's: both drains
         }
-        tc::mbar_init(done, 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
     if (warp == 1) {
-        tc::tmem_alloc(tc::smem_u32(tmem_slot), 512);
-        tc::tmem_relinquish();
+        tc::tmem_alloc_pair(tc::smem_u32(tmem_slot), 512);
+        tc::tmem_relinquish_pair();
     }
     if (warp == 0 && lane == 0) tc::prefetch_tmap(&mapX);
     tc::tc_fence_before();
     __syncthreads();
+    tc::cluster_sync();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- producer
-            int issued = 0;
+        // ---------------- producer
+        bool ok = true;
+        const uint32_t full0 = tc::map_rank(full(0), 0);
+        TileOrder order(a.nt);
+        int s = 0, ph = 1, filled = 0;
+        for (int it = pair; it < a.ntiles && ok; it += npairs) {
+            int ri, cj;
+            order.at(it, ri, cj);
+            const int ra = ri * 256 + 128 * rank, cb = cj * 256 + 128 * rank;
             for (int c = 0; c < nchunks; ++c) {
-                const int s = c % kStages;
-                if (!tc::mbar_wait(empty(s), ((c / kStages) & 1) ^ 1) || *abort_flag) {
-                    *abort_flag = 1;
-                    break;
-                }
-                tc::mbar_expect_tx(full(s), a_in_b ? kTileB : kStage);
-                if (!a_in_b)
-                    for (int m = 0; m < 2; ++m)
-                        tc::tma_load_2d(tc::smem_u32(smem + s * kStage) + m * kBox, &mapX,
-                                        full(s), r0 + 64 * m, c * 64);
-                for (int m = 0; m < 4; ++m)
-                    tc::tma_load_2d(tileB(s) + m * kBox, &mapX, full(s), c0 + 64 * m, c * 64);
-                issued = c + 1;
-            }
-            // leave no copy in flight
-            for (int c = issued > kStages ? issued - kStages : 0; c < issued; ++c)
-                if (!tc::mbar_wait(full(c % kStages), (c / kStages) & 1)) *abort_flag = 1;
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer: accumulator b = per & 1 for each 512 tokens
-            for (int per = 0; per < nper && !*abort_flag; ++per) {
-                const int b = per & 1;
-                if (!tc::mbar_wait(aempty(b), ((per >> 1) & 1) ^ 1)) {
-                    *abort_flag = 1;
-                    break;
-                }
-                tc::tc_fence_after();
-                const int cbeg = per * kChunksPerDrain;
-                const int cend = min(nchunks, cbeg + kChunksPerDrain);
-                bool ok = true;
-                for (int c = cbeg; c < cend; ++c) {
-                    const int s = c % kStages;
-                    if (!tc::mbar_wait(full(s), (c / kStages) & 1) || *abort_flag) {
-                        ok = false;
-                        break;
-                    }
-                    tc::tc_fence_after();
+                ok = tc::mbar_wait(empty(s), ph);
+                if (!ok) break;
+                if (tc::elect_one()) {
+                    if (rank == 0) tc::mbar_expect_tx(full(s), 2 * (ri == cj ? kTileB : kStage));
+                    const uint32_t bar = full0 + 8 * s;
 #pragma unroll
-                    for (int sub = 0; sub < 4; ++sub) {
-                        // 16 tokens = two 8-token atoms = 2048 bytes along K
-                        const uint64_t ad = sdesc_mn_sw128(tileA(s)) + (uint64_t)(128 * sub);
-                        const uint64_t bd = sdesc_mn_sw128(tileB(s)) + (uint64_t)(128 * sub);
-                        tc::mma_bf16(tmem + b * 256, ad, bd, kIdesc, (c > cbeg || sub > 0) ? 1u : 0u);
+                    for (int m = 0; m < 2; ++m) {
+                        if (ri != cj) tc::tma_load_2d_pair(tileA(s) + m * kBox, &mapX, bar, ra + 64 * m, c * 64);
+                        tc::tma_load_2d_pair(tileB(s) + m * kBox, &mapX, bar, cb + 64 * m, c * 64);
                     }
-                    tc::mma_commit(empty(s));
                 }
-                if (!ok) {
-                    *abort_flag = 1;
-                    break;
+                __syncwarp();
+                ++filled;
+                if (++s == kStages) {
+                    s = 0;
+                    ph ^= 1;
                 }
-                tc::mma_commit(afull(b));
             }
-            // every MMA issued has finished before TMEM is released
-            tc::mma_commit(done);
-            if (!tc::mbar_wait(done, 0)) *abort_flag = 1;
+        }
+        // do not leave before the MMAs have consumed the stages filled here:
+        // no copy or commit is in flight afterwards
+        for (int n = max(0, filled - kStages); n < filled && ok; ++n)
+            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
+        if (!ok) *abort_flag = 1;
+    } else if (warp == 1) {
+        // ---------------- MMA issuer of the pair: an accumulator per 512 tokens
+        if (rank == 0) {
+            bool ok = true;
+            TileOrder order(a.nt);
+            const uint64_t a0 = sdesc_mn_sw128(tileA(0)), b0 = sdesc_mn_sw128(tileB(0));
+            int s = 0, ph = 0, pc = 0;
+            for (int it = pair; it < a.ntiles && ok; it += npairs) {
+                int ri, cj;
+                order.at(it, ri, cj);
+                const uint64_t ad0 = ri == cj ? b0 : a0;
+                for (int c0 = 0; c0 < nchunks && ok; c0 += kChunksPerDrain, ++pc) {
+                    const int b = pc & 1, c1 = min(nchunks, c0 + kChunksPerDrain);
+                    ok = tc::mbar_wait(aempty(b), ((pc >> 1) & 1) ^ 1);
+                    for (int c = c0; c < c1 && ok; ++c) {
+                        ok = tc::mbar_wait(full(s), ph);
+                        if (!ok) break;
+                        tc::tc_fence_after();
+                        if (tc::elect_one()) {
+                            const uint64_t o = (uint64_t)(s * (kStage >> 4));
+                            // 16 tokens = two 8-token atoms = 2048 bytes along K
+#pragma unroll
+                            for (int sub = 0; sub < 4; ++sub)
+                                tc::mma_f16_pair(tmem + b * 256, ad0 + o + 128 * sub, b0 + o + 128 * sub, kIdesc,
+                                                 c > c0 || sub > 0);
+                            tc::mma_commit_pair(empty(s));
+                            if (c + 1 == c1) tc::mma_commit_pair(afull(b));
+                        }
+                        __syncwarp();
+                        if (++s == kStages) {
+                            s = 0;
+                            ph ^= 1;
+                        }
+                    }
+                }
+            }
+            if (!ok) *abort_flag = 1;
         }
     } else {
-        // ---------------- drain: TMEM -> float32 registers
-        const int q = warp & 3, half = (warp - 2) >> 2;
-        float acc[128];
+        // ---------------- drain: TMEM -> float32 registers -> H
+        const int q = warp & 3, half = (warp - 2) >> 2;   // lane quarter, 128-column half
+        const uint32_t released = tc::map_rank(aempty(0), 0);
+        float *T = parts + (warp - 2) * (kPart / 4);
+        bool ok = true;
+        TileOrder order(a.nt);
+        int pc = 0;
+        for (int it = pair; it < a.ntiles && ok; it += npairs) {
+            float acc[128];
 #pragma unroll
-        for (int e = 0; e < 128; ++e) acc[e] = 0.f;
-        for (int per = 0; per < nper; ++per) {
-            const int b = per & 1;
-            bool w = tc::mbar_wait(afull(b), (per >> 1) & 1);
-            w = __shfl_sync(0xffffffffu, w, 0) && !*abort_flag;
-            if (!__all_sync(0xffffffffu, w)) {
-                if (lane == 0) *abort_flag = 1;
-                break;
+            for (int e = 0; e < 128; ++e) acc[e] = 0.f;
+            int ri, cj;
+            order.at(it, ri, cj);
+            const int row0 = ri * 256 + 128 * rank + 32 * q, colh = cj * 256 + half * 128;
+            for (int per = 0; per < nper; ++per, ++pc) {
+                const int b = pc & 1;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(afull(b), (pc >> 1) & 1));
+                if (!ok) break;
+                tc::tc_fence_after();
+                const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + b * 256 + half * 128;
+#pragma unroll
+                for (int cc = 0; cc < 128; cc += 16) {
+                    uint32_t v[16];
+                    tc::tmem_ld16(base + cc, v);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) acc[cc + e] += __uint_as_float(v[e]);
+                }
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive_cluster(released + 8 * b);
             }
-            tc::tc_fence_after();
-            const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + b * 256 + half * 128;
+            if (!ok) break;
+            const int u = lane >> 3, v4 = 4 * (lane & 7);
 #pragma unroll
             for (int cc = 0; cc < 128; cc += 32) {
-                uint32_t v[32];
-                tc::tmem_ld32(base + cc, v);
-                tc::tmem_wait_ld();
+                __syncwarp();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) acc[cc + e] += __uint_as_float(v[e]);
+                for (int e = 0; e < 32; ++e) T[lane * kTld + e] = acc[cc + e];
+                __syncwarp();
+                const int col0 = colh + cc;
+                // the 32 x 32 part lies above, on or below the diagonal as a whole
+                if (row0 >= a.d || col0 >= a.d || col0 < row0) continue;
+                const bool diag = col0 == row0;
+                if (diag) {
+                    // H[j][i] takes the element of H[i][j], i < j, as well
+#pragma unroll 1
+                    for (int j = lane + 1; j < 32; ++j) T[j * kTld + lane] = T[lane * kTld + j];
+                    __syncwarp();
+                }
+                // H[row0 + 4 k + u][col0 + v4 ..] and H[col0 + 4 k + u][row0 + v4 ..]
+                float *hp = a.H + (size_t)(row0 + u) * a.d + col0 + v4;
+                float *hm = a.H + (size_t)(col0 + u) * a.d + row0 + v4;
+                const size_t step = (size_t)4 * a.d;
+                // rows 4 k + u of the two parts that exist: 4 k below these
+                const int np = col0 + v4 < a.d ? a.d - row0 - u : 0;
+                const int nm = row0 + v4 < a.d && !diag ? a.d - col0 - u : 0;
+                const float *tp = T + u * kTld + v4, *tm = T + v4 * kTld + u;
+#pragma unroll 1
+                for (int k0 = 0; k0 < 32; k0 += 16) {        // 16 rows of each part
+                    float4 h[4], m[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k0 + 4 * k < np) h[k] = *reinterpret_cast<const float4 *>(hp + k * step);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k0 + 4 * k < nm) m[k] = *reinterpret_cast<const float4 *>(hm + k * step);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k0 + 4 * k < np) {
+                            const float *t = tp + 4 * k * kTld;
+                            h[k].x = fmaf(a.scale, t[0], h[k].x);
+                            h[k].y = fmaf(a.scale, t[1], h[k].y);
+                            h[k].z = fmaf(a.scale, t[2], h[k].z);
+                            h[k].w = fmaf(a.scale, t[3], h[k].w);
+                            *reinterpret_cast<float4 *>(hp + k * step) = h[k];
+                        }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k0 + 4 * k < nm) {
+                            const float *t = tm + 4 * k;
+                            m[k].x = fmaf(a.scale, t[0], m[k].x);
+                            m[k].y = fmaf(a.scale, t[kTld], m[k].y);
+                            m[k].z = fmaf(a.scale, t[2 * kTld], m[k].z);
+                            m[k].w = fmaf(a.scale, t[3 * kTld], m[k].w);
+                            *reinterpret_cast<float4 *>(hm + k * step) = m[k];
+                        }
+                    hp += 4 * step;
+                    hm += 4 * step;
+                    tp += 16 * kTld;
+                    tm += 16;
+                }
             }
-            tc::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(aempty(b));
         }
-        // the stage ring is idle once the last accumulator has been read:
-        // stage the tile as T[row][col]
-        float *T = (float *)smem;
-        if (!*abort_flag) {
-            const int i = 32 * q + lane;
-#pragma unroll
-            for (int e = 0; e < 128; ++e) T[i * kTld + half * 128 + e] = acc[e];
-        }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (!*abort_flag) {
-            const int t = threadIdx.x - 64;
-            // H[row][col] for col >= row: a tile row is 64 float4 of H's row
-            add_tile_pass<false>(a, T, t, r0, c0);
-            // H[col][row] for col > row: a tile column is 32 float4 of H's row `col`
-            add_tile_pass<true>(a, T, t, r0, c0);
-        }
+        if (!ok) *abort_flag = 1;
     }
+    // neither CTA leaves while the other may still read its shared memory,
+    // signal its barriers or hold TMEM of the pair
     tc::tc_fence_before();
+    __syncwarp();
     __syncthreads();
+    tc::cluster_sync();
     if (warp == 1) {
         tc::tc_fence_after();
-        tc::tmem_dealloc(tmem, 512);
+        tc::tmem_dealloc_pair(tmem, 512);
     }
     if (threadIdx.x == 0 && *abort_flag) atomicOr(&g_syrk_status, ST_TIMEOUT);
-}
-
-// Number of 128 x 256 tiles that meet the upper triangle of a d x d matrix.
-int syrk_tiles(int d) {
-    const int rt = (d + 127) / 128, ct = (d + 255) / 256;
-    int n = 0;
-    for (int cj = 0; cj < ct; ++cj) n += min(rt, 2 * cj + 2);
-    return n;
 }
 
 }  // namespace
@@ -329,9 +373,10 @@ extern "C" jarq_status jarq_accumulate_hessian(const void *X, int n, int d, floa
         e = cudaFuncSetAttribute(tc_syrk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
     if (e == cudaSuccess) {
-        SyrkArgs args{H, scale, d, n, (d + 255) / 256, (d + 127) / 128};
+        const int nt = (d + 255) / 256, ntiles = nt * (nt + 1) / 2;
+        SyrkArgs args{H, scale, d, n, nt, ntiles};
         ProfScope ps("syrk", st);
-        tc_syrk_kernel<<<syrk_tiles(d), kThreads, kSmem, st>>>(map, args);
+        tc_syrk_kernel<<<2 * std::min(ntiles, num_sms() / 2), kThreads, kSmem, st>>>(map, args);
         e = cudaGetLastError();
         ps.done();
         count_launches(1);

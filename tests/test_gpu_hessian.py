@@ -51,6 +51,23 @@ def test_integer_activations_bit_exact(jarq, n, d):
     np.testing.assert_array_equal(H.cpu().numpy(), ref.astype(np.float32))
 
 
+@pytest.mark.parametrize("n,d", [
+    (64, 256),       # one whole tile
+    (513, 264),      # a tile side of 8 features; one token in the second sum
+    (65, 3592),      # 120 tiles, more than the pairs of CTAs; two blocks of the tile order
+    (600, 6408),     # 351 tiles, a ragged last block
+])
+def test_tile_order_edges_bit_exact(jarq, n, d):
+    """Integer activations, every product and sum exact: each pair of features
+    is added once, in both places, by the tiles of CTA pairs."""
+    X = integer_activations_np(n, d, amax=8, seed=n + d)
+    H0 = torch.randint(-1000, 1000, (d, d), device="cuda").float()    # not symmetric
+    Xd = torch.as_tensor(X, device="cuda")
+    ref = H0.double() + Xd.double().T @ Xd.double()
+    H = jarq.accumulate_hessian(Xd, H0.clone())
+    assert torch.equal(H.double(), ref)
+
+
 def test_streamed_batches_and_scale_bit_exact(jarq):
     d = 392
     X = integer_activations_np(5000, d, amax=6, seed=11)
