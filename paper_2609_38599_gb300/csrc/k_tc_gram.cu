@@ -33,15 +33,16 @@
 //                accumulator, which goes back to the issuer when all of them
 //                have read it
 //
-// What bounds it, per unit and CTA (clock64 in a copy): about 2000 cycles, of
-// which the MMAs are 1024 and the epilogue 900 to 1000 issue slots per
+// What bounds it, per unit and CTA (clock64 in a copy, 4-bit codes): about 2000
+// cycles, of which the MMAs are 1024 and the epilogue 900 to 1000 issue slots per
 // scheduler (64 digit sums a thread: an add, an integer multiply-add at half
 // rate); the rest is the hand-over between them (a ready barrier costs about
 // 150 cycles, the four TMEM loads 200 to 400).  Without the dots a launch on
 // 4096 x 4096, g = 128 takes 188 us, without the epilogue 162 us, in full 217
-// us; 1424 us on 4096 x 11008.  One CTA per tile with eight epilogue warps took
-// 325 and 2150 us; the block's sum in one of the epilogue warps 231 us, by
-// shared-memory atomics 252 us.
+// us; 1424 us on 4096 x 11008.  Codes of up to three bits: 200 us, and 409 us with
+// groups of 64 (218 and 450 us with the integer dots).  One CTA per tile with
+// eight epilogue warps took 325 and 2150 us; the block's sum in one of the
+// epilogue warps 231 us, by shared-memory atomics 252 us.
 #include <type_traits>
 
 #include "df.cuh"
@@ -97,10 +98,18 @@ struct GramUnit {
     }
 };
 
-// WIDE: codes wider than 4 bits, |D_t| < 2^24 converted by cvt and 64-bit
-// integer dots; otherwise |c| <= 15, |D_t| < 2^20 and every partial dot of
-// 32 terms fits in 32 bits.
-template <bool WIDE>
+// How an epilogue warp forms its dots, by the width of the codes:
+//   up to 3 bits  |c| <= 7, |D_t| <= 128 * 7 * 512, so float32 sums of four
+//                 products are exact integers (< 2^24); a conversion and an
+//                 integer addition per four products instead of a multiply-add
+//                 at half rate for each
+//   4 bits        |c| <= 15, |D_t| < 2^20: integer products, every partial dot of
+//                 32 terms fits in 32 bits.  Float32 would hold one product, and
+//                 a conversion for each takes 328 us where this takes 217 us.
+//   wider         |D_t| < 2^24 converted by cvt, 64-bit integer dots
+enum { kWideDots = -1, kIntDots = 0 };    // or the number of terms of a float32 sum
+
+template <int kMode>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_gram_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapS,
                    GramArgs a) {
@@ -273,7 +282,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         int z = 0, jp, ug = 0, nb = 0;          // ug, nb: units, blocks of this pair so far
         uint32_t q4[2][4] = {};                 // this warp's codes of group i, both halves
         bool ok = true;
-        typedef typename std::conditional<WIDE, long long, int>::type acc_t;
+        typedef typename std::conditional<kMode == kWideDots, long long, int>::type acc_t;
         acc_t acc[4] = {0, 0, 0, 0};
         for (int it = blockIdx.x / 2; it < a.nitems && ok; it += npairs) {
             const int nunits = item(it, jp, un);
@@ -291,11 +300,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                             q4[hf][0] = v.x; q4[hf][1] = v.y; q4[hf][2] = v.z; q4[hf][3] = v.w;
                         }
                 }
+                // c = q - z, as integers or as float pairs (the bits of 2^23 + q
+                // are 0x4B000000 + q; both differences are exact)
                 int c[16];
+                tc::F2 cf[8];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
                     const uint32_t w = un.half ? q4[1][e >> 2] : q4[0][e >> 2];
-                    c[e] = (int)__byte_perm(w, 0, 0x4440 | (e & 3)) - z;
+                    c[e] = kMode > 0 ? (int)__byte_perm(w, 0x4B000000u, 0x7440 | (e & 3))
+                                               : (int)__byte_perm(w, 0, 0x4440 | (e & 3)) - z;
+                }
+                if (kMode > 0) {
+                    const tc::F2 off = tc::f2(-8388608.0f - (float)z);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        cf[e] = tc::f2_add(tc::f2(__int_as_float(c[2 * e]), __int_as_float(c[2 * e + 1])), off);
                 }
                 const int b = ug & 1;
                 ok = __all_sync(0xffffffffu, tc::mbar_wait(afull(b), (ug >> 1) & 1));
@@ -308,7 +327,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive_cluster(released + 8 * b);
                 };
-                if constexpr (WIDE) {
+                if constexpr (kMode == kWideDots) {
 #pragma unroll
                     for (int t = 0; t < 4; t += 2) {
                         uint32_t v[2][16];
@@ -321,6 +340,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
                             for (int e = 0; e < 16; ++e)
                                 acc[t + k] += (long long)c[e] * __float2int_rn(__uint_as_float(v[k][e]));
+                    }
+                } else if constexpr (kMode > 0) {
+                    uint32_t v[4][16];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) tc::tmem_ld16(base + t * 64, v[t]);
+                    tc::tmem_wait_ld();
+                    release();
+                    // |c D| <= 7 * 7 * 128 * 512: sums of four are below 2^24
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        auto dg = [&](int e) {
+                            return tc::f2(__uint_as_float(v[t][2 * e]), __uint_as_float(v[t][2 * e + 1]));
+                        };
+#pragma unroll
+                        for (int h = 0; h < 8; h += kMode) {
+                            tc::F2 sum = tc::f2_fma(cf[h], dg(h), tc::f2(0.f));
+#pragma unroll
+                            for (int e = h + 1; e < h + kMode; ++e) sum = tc::f2_fma(cf[e], dg(e), sum);
+                            float x0, x1;
+                            tc::f2_get(sum, x0, x1);
+                            acc[t] += __float2int_rn(x0) + __float2int_rn(x1);
+                        }
                     }
                 } else {
                     uint32_t v[4][16];
@@ -357,7 +398,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     ok = __all_sync(0xffffffffu, tc::mbar_wait(sfree(slot), ((nb / kSlots) & 1) ^ 1));
                     if (!ok) break;
                     long long *pp = part + (size_t)((slot * 4 + cq) * 2) * 128 + rl;
-                    if constexpr (WIDE) {
+                    if constexpr (kMode == kWideDots) {
                         pp[0] = hi;
                         pp[128] = lo;
                     } else {
@@ -391,7 +432,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     const long long *pr = pp + r0 + 32 * r;
                     const long long s0 = (pr[0] + pr[256]) + (pr[512] + pr[768]);
                     double v;
-                    if constexpr (WIDE) {
+                    if constexpr (kMode == kWideDots) {
                         const long long s1 = (pr[128] + pr[384]) + (pr[640] + pr[896]);
                         v = ldexp((double)s0, E - 19) + ldexp((double)s1, E - 39);
                     } else {
@@ -610,11 +651,6 @@ cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, con
                            const int32_t *Z, const int *expo, const int *active, float2 *gram,
                            int p, int p_pad, int d, int d_pad, int g, int bits, int *status,
                            cudaStream_t s) {
-    static std::atomic<unsigned long long> attr_narrow{0}, attr_wide{0};
-    cudaError_t e = set_max_dynamic_smem((const void *)tc_gram_kernel<false>, kSmem, attr_narrow);
-    if (e == cudaSuccess)
-        e = set_max_dynamic_smem((const void *)tc_gram_kernel<true>, kSmem, attr_wide);
-    if (e != cudaSuccess) return e;
     const int G = d / g;
     // ranges per (row tile pair, group pair): the fewest blocks for the busiest
     // CTA pair, each item costing about a sixth of a block beside its blocks
@@ -634,11 +670,16 @@ cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, con
     if (items > 0x7fffffff) return cudaErrorInvalidValue;
     GramArgs a{Q, Z, expo, active, gram, status, p, d, g, G, d_pad, nparts, tiles, (int)items};
     const dim3 grid(2 * (items < npairs ? (int)items : npairs));
-    if (bits <= 4)
-        tc_gram_kernel<false><<<grid, kThreads, kSmem, s>>>(mapC, mapS, a);
-    else
-        tc_gram_kernel<true><<<grid, kThreads, kSmem, s>>>(mapC, mapS, a);
-    return cudaGetLastError();
+    auto run = [&](auto *kernel, std::atomic<unsigned long long> &done) {
+        const cudaError_t e = set_max_dynamic_smem((const void *)kernel, kSmem, done);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, kThreads, kSmem, s>>>(mapC, mapS, a);
+        return cudaGetLastError();
+    };
+    static std::atomic<unsigned long long> done[3];
+    if (bits <= 3) return run(tc_gram_kernel<4>, done[0]);
+    if (bits <= 4) return run(tc_gram_kernel<kIntDots>, done[1]);
+    return run(tc_gram_kernel<kWideDots>, done[2]);
 }
 
 }  // namespace jarq

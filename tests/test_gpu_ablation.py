@@ -124,6 +124,28 @@ def test_fixed_grid_parity(jarq):
     np.testing.assert_allclose(F_gpu_state, hist[-1], rtol=1e-4)
 
 
+@pytest.mark.parametrize("g", [64, 128])
+@pytest.mark.parametrize("bits", [2, 3, 4, 5, 8])
+def test_gram_at_the_largest_digit_sums(jarq, g, bits):
+    """Codes at both ends of their range against a matrix whose off-diagonal
+    blocks are near their block maximum: the largest digit sums that each way
+    of forming the dots has to hold.  Every term of F has one sign (W <= 0 <= c),
+    so F is off by no more than its terms: H and W by 2^-38 of an entry, the
+    products by less; 2^-35 is allowed."""
+    rng = np.random.default_rng(bits + g)
+    din, dout, qmax = 6 * g, 300, (1 << bits) - 1
+    H = 1.0 - rng.uniform(0, 2.0 ** -6, (din, din))
+    H = ((H + H.T) / 2 + np.diag(rng.uniform(0.5, 1, din))).astype(np.float32)
+    W = -rng.uniform(0.5, 1, (dout, din)).astype(np.float32)
+    Q = np.where(rng.random((dout, din)) < 0.9, qmax, qmax - 1).astype(np.uint8)
+    Z = np.zeros((dout, 6), np.int32)
+    S = rng.uniform(0.5, 1, (dout, 6)).astype(np.float32)
+    prep, hess = prepare_hessian(H, g), jarq.prepare(H, g)
+    F, _ = jarq.fit_scales(hess, W, S.copy(), Q, Z, bits, "joint")
+    hess.close()
+    np.testing.assert_allclose(F, objective(prep, W, S, Q, Z), rtol=2.0 ** -35)
+
+
 def test_full_size_scale_fits_and_probe_sampled_rows(jarq):
     """The q_proj layer (4096 x 4096, g = 128, 3-bit) from its RTN state: the
     three scale fits and the multi-code probe of two groups on the whole layer;
