@@ -645,43 +645,70 @@ __device__ __forceinline__ void df_warp_sum(float &sh, float &sl) {
 }
 
 // rhs_j[i] = sum_{l in grp i} (q_l - z_i) P_j[l], one warp per row, lane owns
-// NT = g/32 consecutive entries of every group.
-template <int NT>
-__global__ void rhs_kernel(const uint8_t *__restrict__ Q, const int32_t *__restrict__ Z,
-                           const float *__restrict__ Phi, const float *__restrict__ Plo,
-                           const int *__restrict__ active, double *__restrict__ rhs, int p, int d) {
+// NT = g/32 consecutive entries of every group; NB groups are loaded and reduced
+// together.  What bounds it: memory (9 bytes an entry), at the loads that a row's
+// warp keeps in flight.  4096 x 4096: 37 us for g = 128 (NB = 8; 39 with 4), 47 us
+// for g = 64 (NB = 2; 52 and 57 with 4 and 8); 14336 x 4096 83 us, 4096 x 11008 96
+// us.  One group at a time: 42, 68, 102 and 98 us.
+constexpr int kRhsThreads = 64;
+
+template <int NT, int NB>
+__global__ void __launch_bounds__(kRhsThreads) rhs_kernel(const uint8_t *__restrict__ Q,
+                                                          const int32_t *__restrict__ Z,
+                                                          const float *__restrict__ Phi,
+                                                          const float *__restrict__ Plo,
+                                                          const int *__restrict__ active,
+                                                          double *__restrict__ rhs, int p, int d) {
     constexpr int g = 32 * NT;
     const int G = d / g;
     const int j = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (j >= p || (active && !active[j])) return;   // warp-uniform
     const size_t off = (size_t)j * d + NT * lane;
-    for (int i = 0; i < G; ++i) {
-        const float z = (float)Z[(size_t)j * G + i];
-        const size_t o = off + (size_t)i * g;
-        float ph[NT], pl[NT], qc[NT];
-        if constexpr (NT == 4) {
-            const float4 a4 = *reinterpret_cast<const float4 *>(Phi + o);
-            const float4 b4 = *reinterpret_cast<const float4 *>(Plo + o);
-            const uint32_t q4 = *reinterpret_cast<const uint32_t *>(Q + o);
-            ph[0] = a4.x; ph[1] = a4.y; ph[2] = a4.z; ph[3] = a4.w;
-            pl[0] = b4.x; pl[1] = b4.y; pl[2] = b4.z; pl[3] = b4.w;
+    const int32_t *zj = Z + (size_t)j * G;
+#pragma unroll 1
+    for (int i = 0; i < G; i += NB) {
+        float ph[NB][NT], pl[NB][NT];
+        uint32_t q[NB];
+        int z[NB];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) qc[t] = (float)((q4 >> (8 * t)) & 0xFFu);
-        } else {
-            const float2 a2 = *reinterpret_cast<const float2 *>(Phi + o);
-            const float2 b2 = *reinterpret_cast<const float2 *>(Plo + o);
-            const uint32_t q2 = *reinterpret_cast<const uint16_t *>(Q + o);
-            ph[0] = a2.x; ph[1] = a2.y;
-            pl[0] = b2.x; pl[1] = b2.y;
-            qc[0] = (float)(q2 & 0xFFu);
-            qc[1] = (float)(q2 >> 8);
+        for (int u = 0; u < NB; ++u) {
+            const int iu = min(i + u, G - 1);       // past the end: the last group again, not stored
+            const size_t o = off + (size_t)iu * g;
+            if constexpr (NT == 4) {
+                const float4 a4 = __ldg(reinterpret_cast<const float4 *>(Phi + o));
+                const float4 b4 = __ldg(reinterpret_cast<const float4 *>(Plo + o));
+                q[u] = __ldg(reinterpret_cast<const uint32_t *>(Q + o));
+                ph[u][0] = a4.x; ph[u][1] = a4.y; ph[u][2] = a4.z; ph[u][3] = a4.w;
+                pl[u][0] = b4.x; pl[u][1] = b4.y; pl[u][2] = b4.z; pl[u][3] = b4.w;
+            } else {
+                const float2 a2 = __ldg(reinterpret_cast<const float2 *>(Phi + o));
+                const float2 b2 = __ldg(reinterpret_cast<const float2 *>(Plo + o));
+                q[u] = __ldg(reinterpret_cast<const uint16_t *>(Q + o));
+                ph[u][0] = a2.x; ph[u][1] = a2.y;
+                pl[u][0] = b2.x; pl[u][1] = b2.y;
+            }
+            z[u] = __ldg(zj + iu);
         }
-        float sh = 0.f, sl = 0.f;
+        float sh[NB], sl[NB];
 #pragma unroll
-        for (int t = 0; t < NT; ++t) df_axpy(qc[t] - z, ph[t], pl[t], sh, sl);
-        df_warp_sum(sh, sl);
-        if (lane == 0) rhs[(size_t)j * G + i] = (double)sh + (double)sl;
+        for (int u = 0; u < NB; ++u) {
+            sh[u] = sl[u] = 0.f;
+            const float zf = (float)z[u];
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+                df_axpy((float)((q[u] >> (8 * t)) & 0xFFu) - zf, ph[u][t], pl[u][t], sh[u], sl[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < NB; ++u) df_warp_sum(sh[u], sl[u]);
+        // every lane holds the sums: lane u stores group i + u
+        float h = sh[0], l = sl[0];
+#pragma unroll
+        for (int u = 1; u < NB; ++u) {
+            h = lane == u ? sh[u] : h;
+            l = lane == u ? sl[u] : l;
+        }
+        if (lane < NB && i + lane < G) rhs[(size_t)j * G + i + lane] = (double)h + (double)l;
     }
 }
 
@@ -925,11 +952,11 @@ cudaError_t launch_mu_combine(float *Phi, float *Plo, const float *Khi, const fl
 
 cudaError_t launch_rhs(const uint8_t *Q, const int32_t *Z, const float *Phi, const float *Plo,
                        const int *active, double *rhs, int p, int d, int g, cudaStream_t s) {
-    const unsigned blocks = (unsigned)(((long long)p * 32 + 255) / 256);
+    const unsigned blocks = (unsigned)(((long long)p * 32 + kRhsThreads - 1) / kRhsThreads);
     if (g == 128)
-        rhs_kernel<4><<<blocks, 256, 0, s>>>(Q, Z, Phi, Plo, active, rhs, p, d);
+        rhs_kernel<4, 8><<<blocks, kRhsThreads, 0, s>>>(Q, Z, Phi, Plo, active, rhs, p, d);
     else if (g == 64)
-        rhs_kernel<2><<<blocks, 256, 0, s>>>(Q, Z, Phi, Plo, active, rhs, p, d);
+        rhs_kernel<2, 2><<<blocks, kRhsThreads, 0, s>>>(Q, Z, Phi, Plo, active, rhs, p, d);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
