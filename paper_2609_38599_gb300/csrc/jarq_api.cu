@@ -189,7 +189,7 @@ cudaError_t ensure_ws(jarq_hessian *h, int p, cudaStream_t st) {
         return e;
     if ((e = make_tmap_bf16(&w.mapWd, w.wdig, (uint64_t)4 * p_pad, h->d_pad, 128, 32)) != cudaSuccess)
         return e;
-    if ((e = make_tmap_bf16(&w.mapPd, w.wdig, (uint64_t)6 * p_pad, h->d_pad, 128)) != cudaSuccess)
+    if ((e = make_tmap_bf16(&w.mapPd, w.wdig, (uint64_t)6 * p_pad, h->d_pad, 128, 32)) != cudaSuccess)
         return e;
     w.p_pad = p_pad;
     w.cap_rows = p;
@@ -484,7 +484,7 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         if ((e = make_tmap_bf16(&h->mapH64, h->Hplanes, (uint64_t)3 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_bf16(&h->mapD8, h->Hdig8, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_f16(&h->mapD10, h->Hdig10, (uint64_t)4 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
-        if ((e = make_tmap_bf16(&h->mapRi, h->rdig, (uint64_t)6 * din, group_size, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
+        if ((e = make_tmap_bf16(&h->mapRi, h->rdig, (uint64_t)6 * din, group_size, 64, 32)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = make_tmap_f16(&h->mapHt, h->Htdig, (uint64_t)4 * h->d_pad, h->d_pad, 64)) != cudaSuccess) { rc = cuda_fail(e); break; }
         if ((e = cudaMallocHost((void **)&h->hstatus, sizeof(int))) != cudaSuccess) { rc = cuda_fail(e); break; }
         const float *Hsrc = H;

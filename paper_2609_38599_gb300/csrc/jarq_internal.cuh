@@ -106,7 +106,7 @@ struct Workspace {
     __nv_bfloat16 *wdig = nullptr;     // [6][p_pad][d_pad] integer digits of W (4) or P (6)
     int *wexp = nullptr;               // [p][G] exponents of those digits
     CUtensorMap mapWd;                 // tensor map of wdig's first 4 planes, 128 x 32 boxes
-    CUtensorMap mapPd;                 // tensor map of all 6 planes, 128 x 64 boxes
+    CUtensorMap mapPd;                 // tensor map of all 6 planes, 128 x 32 boxes
     float *Phi = nullptr;        // [p][d]  P = Phi + Plo (double-float)
     float *Plo = nullptr;        // [p][d]
     float *Pt_hi = nullptr;      // [p][d]  folded projection Pt_i = R_i^{-T} P_i
@@ -156,7 +156,7 @@ struct jarq_hessian {
     // column b: digit of R_i^{-1}[b][a]), one exponent per group
     __nv_bfloat16 *rdig = nullptr;     // [6][d][g]
     int *rexp = nullptr;               // [G]
-    CUtensorMap mapRi;                 // tensor map of rdig, 64 x 64 boxes
+    CUtensorMap mapRi;                 // tensor map of rdig, 64 x 32 boxes
     // folded rows Ht[grp i, :] = R_i^{-T} H[grp i, :] in the base-2^10 digit scheme
     __half *Htdig = nullptr;      // [4][d_pad][d_pad] fp16 digits, |digit| <= 512
     int *expoT = nullptr;         // [G][G] block exponents of Ht

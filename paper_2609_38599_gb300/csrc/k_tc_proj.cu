@@ -47,12 +47,6 @@ namespace jarq {
 namespace {
 
 constexpr int kWDig = 4, kHDig = 6, kLevels = 6;
-constexpr int kTileA = 128 * 64 * 2;   // one W digit plane, 128 rows x 64 K
-constexpr int kTileB = 64 * 64 * 2;    // one H digit plane, 64 rows x 64 K
-// Folded projection: all digits of the K block of the tile's own column
-// group (the block-diagonal right-hand side R_i^{-1}), one stage of 144 KB.
-constexpr int kFoldStage = kHDig * (kTileA + kTileB);
-constexpr int kFoldSmem = 1024 + kFoldStage + 256;
 // For a row digit t the right-hand digit planes u are consecutive 64-row tiles
 // and the levels t + u consecutive 64-column blocks, so one MMA covers up to
 // four planes (N = 64 per plane).
@@ -60,6 +54,10 @@ __host__ __device__ constexpr uint32_t idesc_n(int n) { return tc::idesc_bf16_f3
 // Target projection on CTA pairs
 constexpr int kPairA = 128 * 32 * 2;   // one W digit plane, 128 rows x 32 K
 constexpr int kPairB = 64 * 32 * 2;    // one H digit plane, 64 rows x 32 K
+// Folded projection: all digits of 128 rows and 64 columns, 32 of K at a time
+constexpr int kFoldStage = kHDig * (kPairA + kPairB);
+constexpr int kFoldStages = 3;
+constexpr int kFoldSmem = 1024 + kFoldStages * kFoldStage + 256;
 constexpr int kPairStage = kWDig * kPairA + 3 * kPairB;
 constexpr int kPairStages = 5;
 constexpr int kPairSmem = 1024 + kPairStages * kPairStage + 256;
@@ -82,41 +80,61 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = (a - (s - bb)) + (b - bb);
 }
 
-// Folded projection (launch_ptilde): persistent CTAs over 128 x 64 tiles, one
-// K block each.  Warp 0 TMA producer, warp 1 TMEM allocation and MMA issue,
-// warps 2..9 drain (warp w reads TMEM lanes 32 (w % 4) and 32 of the tile's 64
-// columns).
-__global__ void __launch_bounds__(320, 1)
+// Levels 0..3 and w = L_4 + L_5 2^-8 of two columns: sum_l L_l 2^(-8 l) as (v, r).
+// L_0 is an integer, and every partial sum of the first l levels a multiple of
+// 2^(-8 l) (or of a larger power, rounded): an integer multiple of the last place
+// of the next term (|L_l| <= 2^23), so that three operations give each sum's
+// rounding error exactly (Fast2Sum).
+__device__ __forceinline__ void sum_levels(tc::F2 l0, tc::F2 l1, tc::F2 l2, tc::F2 l3, tc::F2 w, tc::F2 &v,
+                                           tc::F2 &r) {
+    v = l0;
+    auto add_level = [&](tc::F2 x, float f) {
+        const tc::F2 v2 = tc::f2_fma(x, tc::f2(f), v);
+        const tc::F2 e = tc::f2_fma(x, tc::f2(f), tc::f2_sub(v, v2));
+        v = v2;
+        return e;
+    };
+    r = add_level(l1, 0x1p-8f);
+    r = tc::f2_add(r, add_level(l2, 0x1p-16f));
+    r = tc::f2_add(r, add_level(l3, 0x1p-24f));
+    r = tc::f2_fma(w, tc::f2(0x1p-32f), r);
+}
+
+// Folded projection (launch_ptilde): persistent CTAs over 128 x 64 tiles, the K
+// block of the tile's own column group only, and of that the rows of R_i^{-1}
+// (upper triangular) that reach the tile's columns.
+//   warp 0       TMA producer (three stages of 32 of K, 72 KB each)
+//   warp 1       TMEM allocation and MMA issue
+//   warps 2..17  drain: warp w reads TMEM lanes 32 (w % 4) and 16 of the tile's
+//                64 columns
+// What bounds it: memory (the digit planes and the result, 20 bytes an entry)
+// and, tile by tile, the MMAs and the drain one after the other: six levels of 64
+// columns leave no room for a second accumulator.  4096 x 4096, g = 128: 108 us,
+// 175 with the digits of P before it; 465 us on 4096 x 11008, 582 on 14336 x 4096.
+// A single stage of 64 of K, all rows of R_i^{-1} and a drain of eight warps that
+// combined the levels by two-sums took 325, 920 and 1100 us.
+__global__ void __launch_bounds__(kPairThreads, 1)
     tc_fold_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapH,
                    ProjArgs a) {
-    constexpr int kStage = kFoldStage, kStages = 1, WDIG = kHDig;
+    constexpr int kStages = kFoldStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *bars = (uint64_t *)(smem + kStages * kStage);
+    uint64_t *bars = (uint64_t *)(smem + kStages * kFoldStage);
     uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 2);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nkc = a.g / 64;               // K chunks per group
-    // item blockIdx.x + v gridDim.x of (row tiles) x (d / 64 column tiles)
-    const int nct = a.d / 64;
-    const int nitems = ((a.p + 127) / 128) * nct;
-    const int nseg = (int)blockIdx.x < nitems ? (nitems - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const int nchunks = nseg * nkc;
-    // tile (first row, first column) of segment v; a 64-wide tile lies in
-    // one column group n0 / g
-    auto tile_of = [&](int v, int &j0, int &n0) {
-        const int it = (int)blockIdx.x + v * (int)gridDim.x;
-        j0 = (it / nct) * 128;
-        n0 = (it % nct) * 64;
-    };
+    // tile it: row tile it / nct, column tile it % nct (in one group: g is a
+    // multiple of 64); K chunks of 32 up to the tile's last column
+    const int nct = a.d / 64, nitems = ((a.p + 127) / 128) * nct;
+    auto chunks_of = [&](int it) { return ((it % nct) * 64 % a.g + 64) / 32; };
 
     auto full = [&](int s) { return tc::smem_u32(bars + s); };
     auto empty = [&](int s) { return tc::smem_u32(bars + kStages + s); };
     const uint32_t afull = tc::smem_u32(bars + 2 * kStages);
     const uint32_t aempty = tc::smem_u32(bars + 2 * kStages + 1);
-    auto tileA = [&](int s, int t) { return tc::smem_u32(smem + s * kStage + t * kTileA); };
+    auto tileA = [&](int s, int t) { return tc::smem_u32(smem + s * kFoldStage + t * kPairA); };
     auto tileB = [&](int s, int u) {
-        return tc::smem_u32(smem + s * kStage + WDIG * kTileA + u * kTileB);
+        return tc::smem_u32(smem + s * kFoldStage + kHDig * kPairA + u * kPairB);
     };
 
     if (threadIdx.x == 0) {
@@ -125,7 +143,7 @@ __global__ void __launch_bounds__(320, 1)
             tc::mbar_init(empty(s), 1);
         }
         tc::mbar_init(afull, 1);
-        tc::mbar_init(aempty, 8);
+        tc::mbar_init(aempty, kPairDrain);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -142,162 +160,139 @@ __global__ void __launch_bounds__(320, 1)
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // ---------------- producer
-        int issued = 0;
-        for (int c = 0; c < nchunks; ++c) {
-            const int s = c % kStages;
-            if (!tc::mbar_wait(empty(s), ((c / kStages) & 1) ^ 1) || *abort_flag) {
-                *abort_flag = 1;
-                break;
-            }
-            const int v = c / nkc, kc = c % nkc;
-            int j0, n0;
-            tile_of(v, j0, n0);
-            // the right-hand side holds only the g columns of each group's block
-            const int kw = (n0 / a.g) * a.g + kc * 64, kh = kc * 64;
-            tc::mbar_expect_tx(full(s), kStage);
+        bool ok = true;
+        int s = 0, ph = 1, filled = 0;
+        for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
+            const int j0 = it / nct * 128, n0 = it % nct * 64, k0 = n0 / a.g * a.g, nc = chunks_of(it);
+            for (int c = 0; c < nc; ++c) {
+                ok = tc::mbar_wait(empty(s), ph);
+                if (!ok) break;
+                if (tc::elect_one()) {
+                    tc::mbar_expect_tx(full(s), kFoldStage);
+                    // the right-hand side holds only the g columns of each group's block
 #pragma unroll
-            for (int t = 0; t < WDIG; ++t)
-                tc::tma_load_2d(tileA(s, t), &mapW, full(s), kw, t * a.w_plane + j0);
-#pragma unroll
-            for (int u = 0; u < kHDig; ++u)
-                tc::tma_load_2d(tileB(s, u), &mapH, full(s), kh, u * a.h_plane + n0);
-            issued = c + 1;
-        }
-        // do not leave with copies in flight
-        for (int c = issued > kStages ? issued - kStages : 0; c < issued; ++c)
-            if (!tc::mbar_wait(full(c % kStages), (c / kStages) & 1)) *abort_flag = 1;
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer
-        for (int sg = 0; sg < nseg && !*abort_flag; ++sg) {
-            if (!tc::mbar_wait(aempty, (sg & 1) ^ 1)) {
-                *abort_flag = 1;
-                break;
-            }
-            tc::tc_fence_after();
-            for (int kc = 0; kc < nkc; ++kc) {
-                const int c = sg * nkc + kc;
-                const int s = c % kStages;
-                if (!tc::mbar_wait(full(s), (c / kStages) & 1) || *abort_flag) {
-                    *abort_flag = 1;
-                    break;
-                }
-                tc::tc_fence_after();
-#pragma unroll
-                for (int sub = 0; sub < 4; ++sub) {
-#pragma unroll
-                    for (int t = 0; t < WDIG; ++t) {
-                        const uint64_t ad = tc::sdesc_sw128(tileA(s, t)) + 2 * sub;
-                        // the products of W digit t with H digits u < kLevels - t,
-                        // in runs of at most four planes; t = 0 opens every level
-                        const uint32_t acc = (kc | sub | t) != 0;
-#pragma unroll
-                        for (int u0 = 0; u0 < kLevels - t; u0 += 4) {
-                            const int nu = min(4, kLevels - t - u0);
-                            const uint64_t bd = tc::sdesc_sw128(tileB(s, u0)) + 2 * sub;
-                            tc::mma_bf16(tmem + (t + u0) * 64, ad, bd, idesc_n(64 * nu), acc);
-                        }
+                    for (int t = 0; t < kHDig; ++t) {
+                        tc::tma_load_2d(tileA(s, t), &mapW, full(s), k0 + c * 32, t * a.w_plane + j0);
+                        tc::tma_load_2d(tileB(s, t), &mapH, full(s), c * 32, t * a.h_plane + n0);
                     }
                 }
-                tc::mma_commit(empty(s));
+                __syncwarp();
+                ++filled;
+                if (++s == kStages) {
+                    s = 0;
+                    ph ^= 1;
+                }
             }
-            tc::mma_commit(afull);
         }
-    } else if (warp >= 2) {
-        // ---------------- drain: levels -> double-float per group -> accumulator
-        // diagonal form: a tile per segment, written when it completes
-        const int q = warp & 3, half = (warp - 2) >> 2;
-        float hi[32], lo[32];
+        // do not leave before the MMAs have consumed the stages filled here
+        for (int n = max(0, filled - kStages); n < filled && ok; ++n)
+            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
+        if (!ok) *abort_flag = 1;
+    } else if (warp == 1) {
+        // ---------------- MMA issuer
+        const uint64_t ad0 = tc::sdesc_sw64(tileA(0, 0)), bd0 = tc::sdesc_sw64(tileB(0, 0));
+        bool ok = true;
+        int s = 0, ph = 0, n = 0;
+        for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x, ++n) {
+            const int nc = chunks_of(it);
+            for (int c = 0; c < nc; ++c) {
+                ok = tc::mbar_wait(full(s), ph);
+                if (c == 0) ok = tc::mbar_wait(aempty, (n & 1) ^ 1) && ok;
+                if (!ok) break;
+                tc::tc_fence_after();
+                if (tc::elect_one()) {
+                    const uint64_t o = (uint64_t)(s * (kFoldStage >> 4));
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-            hi[e] = 0.f;
-            lo[e] = 0.f;
+                    for (int k = 0; k < 4; k += 2)
+#pragma unroll
+                        for (int t = 0; t < kHDig; ++t)
+                            // the products of row digit t with digits u < kLevels - t,
+                            // in runs of at most four planes; t = 0 opens every level
+#pragma unroll
+                            for (int u0 = 0; u0 < kLevels - t; u0 += 4)
+                                tc::mma_bf16(tmem + (t + u0) * 64, ad0 + o + t * (kPairA >> 4) + k,
+                                             bd0 + o + u0 * (kPairB >> 4) + k,
+                                             idesc_n(64 * min(4, kLevels - t - u0)), (c | k | t) != 0);
+                    tc::mma_commit(empty(s));
+                    if (c + 1 == nc) tc::mma_commit(afull);
+                }
+                __syncwarp();
+                if (++s == kStages) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            }
         }
-        const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + half * 32;
-        // exponents of this thread's row and segment v: W's (row, K group)
-        // and the block's; loaded one segment ahead
-        auto seg_exp = [&](int v, int &ew, int &eh) {
-            int j0, n0;
-            tile_of(v, j0, n0);
-            const int row = j0 + 32 * q + lane, hb = n0 / a.g;
-            ew = row < a.p ? a.wexp[(size_t)row * a.G + hb] : 0;
-            eh = a.hexp[hb];
-        };
-        int ew_next = 0, eh_next = 0;
-        if (nseg > 0) seg_exp(0, ew_next, eh_next);
-        for (int sg = 0; sg < nseg; ++sg) {
-            const int ew = ew_next, eh = eh_next;
-            if (sg + 1 < nseg) seg_exp(sg + 1, ew_next, eh_next);
-            bool w = tc::mbar_wait(afull, sg & 1);
-            w = __shfl_sync(0xffffffffu, w && !*abort_flag, 0);
+        if (!ok) *abort_flag = 1;
+    } else {
+        // ---------------- drain: levels -> double-float
+        const int q = warp & 3, cq = (warp - 2) >> 2;    // lane quarter, 16-column quarter
+        const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + cq * 16;
+        bool ok = true;
+        int n = 0;
+        for (int it = blockIdx.x; it < nitems; it += gridDim.x, ++n) {
+            const int row = it / nct * 128 + 32 * q + lane, n0 = it % nct * 64, hb = n0 / a.g;
+            const int ex = a.wexp[(size_t)min(row, a.p - 1) * a.G + hb] + a.hexp[hb] - 14;
+            const tc::F2 scale = tc::f2(ldexpf(1.0f, ex));
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(afull, n & 1));
+            if (!ok) break;
             tc::tc_fence_after();
-            if (!w) {
-                *abort_flag = 1;
-                break;
-            }
-            const float scale = ldexpf(1.0f, ew + eh - 14);
-            // value of the group = sum_l L_l 2^(-8 l), as (vh, vl), 32 columns
-            float vh[32], vl[32];
-#pragma unroll
-            for (int l = 0; l < kLevels; ++l) {
-                uint32_t x[32];
-                tc::tmem_ld32(base + l * 64, x);
+            tc::F2 w[8];     // L_4 + L_5 2^-8
+            {
+                uint32_t x4[16], x5[16];
+                tc::tmem_ld16(base + 4 * 64, x4);
+                tc::tmem_ld16(base + 5 * 64, x5);
                 tc::tmem_wait_ld();
-                if (l == kLevels - 1) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    w[e] = tc::f2_fma(tc::f2(__uint_as_float(x5[2 * e]), __uint_as_float(x5[2 * e + 1])),
+                                      tc::f2(0x1p-8f),
+                                      tc::f2(__uint_as_float(x4[2 * e]), __uint_as_float(x4[2 * e + 1])));
+            }
+            const size_t o = (size_t)row * a.d + n0 + cq * 16;
+#pragma unroll
+            for (int cc = 0; cc < 16; cc += 8) {
+                uint32_t x[4][8];
+#pragma unroll
+                for (int l = 0; l < 4; ++l) tc::tmem_ld8(base + l * 64 + cc, x[l]);
+                tc::tmem_wait_ld();
+                if (cc == 8) {
                     // every level is in registers: hand the columns back
                     tc::tc_fence_before();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(aempty);
                 }
-                const float f = ldexpf(1.0f, -8 * l);
+                float xh[8], xl[8];
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const float v = __uint_as_float(x[e]) * f;   // exact (power of two)
-                    if (l == 0) {
-                        vh[e] = v;
-                        vl[e] = 0.f;
-                    } else {
-                        float s2, e2;
-                        two_sum(vh[e], v, s2, e2);
-                        vh[e] = s2;
-                        vl[e] += e2;
+                for (int e = 0; e < 8; e += 2) {
+                    auto lv = [&](int l) {
+                        return tc::f2(__uint_as_float(x[l][e]), __uint_as_float(x[l][e + 1]));
+                    };
+                    tc::F2 v, r;
+                    sum_levels(lv(0), lv(1), lv(2), lv(3), w[(cc + e) / 2], v, r);
+                    // (v + r) 2^ex, normalised
+                    float v0, v1, r0, r1;
+                    tc::f2_get(tc::f2_mul(v, scale), v0, v1);
+                    tc::f2_get(tc::f2_mul(r, scale), r0, r1);
+                    two_sum(v0, r0, xh[e], xl[e]);
+                    two_sum(v1, r1, xh[e + 1], xl[e + 1]);
+                }
+                if (row < a.p)
+#pragma unroll
+                    for (int e = 0; e < 8; e += 4) {
+                        *reinterpret_cast<float4 *>(a.Phi + o + cc + e) =
+                            make_float4(xh[e], xh[e + 1], xh[e + 2], xh[e + 3]);
+                        *reinterpret_cast<float4 *>(a.Plo + o + cc + e) =
+                            make_float4(xl[e], xl[e + 1], xl[e + 2], xl[e + 3]);
                     }
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                float s2, e2;
-                two_sum(hi[e], vh[e] * scale, s2, e2);
-                hi[e] = s2;
-                lo[e] += e2 + vl[e] * scale;
-            }
-            // the tile is complete
-            {
-                int j0, n0;
-                tile_of(sg, j0, n0);
-                const int row = j0 + 32 * q + lane, ncol = n0 + half * 32;
-                if (row < a.p) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const int col = ncol + e;
-                        if (col < a.d) {
-                            float s2, e2;
-                            two_sum(hi[e], lo[e], s2, e2);
-                            a.Phi[(size_t)row * a.d + col] = s2;
-                            a.Plo[(size_t)row * a.d + col] = e2;
-                        }
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    hi[e] = 0.f;
-                    lo[e] = 0.f;
-                }
             }
         }
+        if (!ok) *abort_flag = 1;
     }
     tc::tc_fence_before();
+    __syncwarp();
     __syncthreads();
     if (warp == 1) {
         tc::tc_fence_after();
@@ -454,8 +449,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         // exponents of the next group, loaded one group ahead
         const int *wrow = a.wexp + (size_t)min(row, a.p - 1) * a.G;
         int e_next = wrow[0] + a.hexp[hb];
-        const tc::F2 c8 = tc::f2(0x1p-8f), c16 = tc::f2(0x1p-16f), c24 = tc::f2(0x1p-24f),
-                     c32 = tc::f2(0x1p-32f);
+        const tc::F2 c8 = tc::f2(0x1p-8f);
         for (int sg = 0; sg < a.G; ++sg) {
             const int ex = e_next - 14;
             if (sg + 1 < a.G) e_next = wrow[sg + 1] + a.hexp[(sg + 1) * a.G + hb];
@@ -494,26 +488,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 }
 #pragma unroll
                 for (int e = 0; e < 8; e += 2) {
-                    // sum_l L_l 2^(-8 l) as (v, r).  L_0 is an integer, and every
-                    // partial sum of the first l levels a multiple of 2^(-8 l)
-                    // (or of a larger power, rounded): an integer multiple of
-                    // the last place of the next term (|L_l| <= 2^23), so that
-                    // three operations give each sum's rounding error exactly
-                    // (Fast2Sum).
                     auto pair = [&](const uint32_t (&x)[8]) {
                         return tc::f2(__uint_as_float(x[e]), __uint_as_float(x[e + 1]));
                     };
-                    auto add_level = [&](tc::F2 &v, const uint32_t (&x)[8], tc::F2 f) {
-                        const tc::F2 v2 = tc::f2_fma(pair(x), f, v);
-                        const tc::F2 r = tc::f2_fma(pair(x), f, tc::f2_sub(v, v2));
-                        v = v2;
-                        return r;
-                    };
-                    tc::F2 v = pair(x0);
-                    tc::F2 r = add_level(v, x1, c8);
-                    r = tc::f2_add(r, add_level(v, x2, c16));
-                    r = tc::f2_add(r, add_level(v, x3, c24));
-                    r = tc::f2_fma(w[(cc + e) / 2], c32, r);
+                    tc::F2 v, r;
+                    sum_levels(pair(x0), pair(x1), pair(x2), pair(x3), w[(cc + e) / 2], v, r);
                     // (v + r) 2^ex (exact products) added to the accumulator
                     tc::F2 &H = hi[(cc + e) / 2], &L = lo[(cc + e) / 2];
                     const tc::F2 sm = tc::f2_fma(v, scale, H);
@@ -909,7 +888,7 @@ cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, con
     (void)d_pad;
     const int items = ((p + 127) / 128) * (d / 64);
     const int ctas = items < num_sms() ? items : num_sms();
-    tc_fold_kernel<<<dim3(ctas, 1, 1), 320, kFoldSmem, s>>>(mapPd, mapR, a);
+    tc_fold_kernel<<<dim3(ctas, 1, 1), kPairThreads, kFoldSmem, s>>>(mapPd, mapR, a);
     return cudaGetLastError();
 }
 
