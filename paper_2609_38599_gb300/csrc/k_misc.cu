@@ -71,10 +71,15 @@ __global__ void residual_kernel(const float *__restrict__ W, const float *__rest
     }
 }
 
-// Only the code plane c = q - z, eight codes per thread (one group: g is a
-// multiple of 8; Q 8-byte aligned; 16-byte stores into the plane).
-__global__ void codes_kernel(const uint8_t *__restrict__ Q, const int32_t *__restrict__ Z,
-                             ResidualView rv, int p, int g) {
+// The same, eight entries per thread (one group: g is a multiple of 8; Q 8-byte,
+// W 16-byte aligned; 16-byte accesses); FULL with the residual.  Bound by memory:
+// 17 us for the code plane of 4096 x 4096 (3 bytes an entry), 48 us with the
+// residual (17 bytes); one entry a thread took 83 us with the residual.
+template <bool FULL>
+__global__ void __launch_bounds__(256) residual8_kernel(const float *__restrict__ W, const float *__restrict__ S,
+                                                        const uint8_t *__restrict__ Q,
+                                                        const int32_t *__restrict__ Z, ResidualView rv, int p,
+                                                        int g) {
     const int d = rv.d, G = d / g;
     const size_t n8 = (size_t)p * d / 8;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -85,10 +90,33 @@ __global__ void codes_kernel(const uint8_t *__restrict__ Q, const int32_t *__res
         const int z = Z[j * G + col / g];
         const uint2 q8 = *reinterpret_cast<const uint2 *>(Q + idx);
         const uint32_t w2[2] = {q8.x, q8.y};
+        int c[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) c[k] = (int)((w2[k >> 2] >> (8 * (k & 3))) & 0xFFu) - z;
+        const size_t o = j * rv.d_pad + col;
+        if constexpr (FULL) {
+            const float4 wa = *reinterpret_cast<const float4 *>(W + idx);
+            const float4 wb = *reinterpret_cast<const float4 *>(W + idx + 4);
+            const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+            const float ns = -S[j * G + col / g];
+            float r[8];
+            __align__(16) __nv_bfloat16 x[3][8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                r[k] = fmaf(ns, (float)c[k], w[k]);
+                split3(r[k], x[0][k], x[1][k], x[2][k]);
+            }
+            *reinterpret_cast<float4 *>(rv.r + idx) = make_float4(r[0], r[1], r[2], r[3]);
+            *reinterpret_cast<float4 *>(rv.r + idx + 4) = make_float4(r[4], r[5], r[6], r[7]);
+            const size_t plane = (size_t)rv.p_pad * rv.d_pad;
+#pragma unroll
+            for (int t = 0; t < 3; ++t)
+                *reinterpret_cast<uint4 *>(rv.planes + t * plane + o) = *reinterpret_cast<const uint4 *>(x[t]);
+        }
         __align__(16) __half h[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) h[k] = __int2half_rn((int)((w2[k >> 2] >> (8 * (k & 3))) & 0xFFu) - z);
-        *reinterpret_cast<uint4 *>(rv.cplane + j * rv.d_pad + col) = *reinterpret_cast<const uint4 *>(h);
+        for (int k = 0; k < 8; ++k) h[k] = __int2half_rn(c[k]);
+        *reinterpret_cast<uint4 *>(rv.cplane + o) = *reinterpret_cast<const uint4 *>(h);
     }
 }
 
@@ -159,8 +187,11 @@ cudaError_t launch_residual(const float *W, const float *S, const uint8_t *Q, co
     int blocks = (int)((n + 255) / 256);
     if (blocks > 8 * num_sms()) blocks = 8 * num_sms();
     if (blocks < 1) blocks = 1;
-    if (!rv.r && g % 8 == 0 && (uintptr_t)Q % 8 == 0 && rv.d_pad % 8 == 0)
-        codes_kernel<<<blocks, 256, 0, s>>>(Q, Z, rv, p, g);
+    const bool eight = g % 8 == 0 && (uintptr_t)Q % 8 == 0 && rv.d_pad % 8 == 0;
+    if (eight && !rv.r)
+        residual8_kernel<false><<<blocks, 256, 0, s>>>(W, S, Q, Z, rv, p, g);
+    else if (eight && (uintptr_t)W % 16 == 0 && (uintptr_t)rv.r % 16 == 0)
+        residual8_kernel<true><<<blocks, 256, 0, s>>>(W, S, Q, Z, rv, p, g);
     else
         residual_kernel<<<blocks, 256, 0, s>>>(W, S, Q, Z, rv, p, g);
     return cudaGetLastError();

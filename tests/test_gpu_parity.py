@@ -244,6 +244,24 @@ def test_misaligned_device_buffers(jarq, g):
         np.testing.assert_array_equal(x, y)
 
 
+@pytest.mark.parametrize("g", [64, 128])
+def test_objective_misaligned_buffers(jarq, g):
+    """The objective forms its residual eight entries at a time from aligned
+    codes and weights, one at a time otherwise: the same bits."""
+    lay = small_layer(3 * g, 71, g, 3, seed=25)
+
+    def dev(a, off):
+        t = torch.as_tensor(a)
+        return torch.empty(t.numel() + off, dtype=t.dtype, device="cuda")[off:].view(t.shape).copy_(t)
+
+    hess = jarq.prepare(lay.H, g)
+    out = [jarq.objective(hess, dev(lay.W, w), dev(lay.S0, 0), dev(lay.Q0, q), dev(lay.Z, 0), lay.bits).cpu().numpy()
+           for w, q in ((0, 0), (1, 0), (0, 1), (4, 8))]
+    hess.close()
+    for x in out[1:]:
+        np.testing.assert_array_equal(out[0], x)
+
+
 def test_k0_returns_host_state(jarq):
     lay = small_layer(128, 40, 64, 3, seed=23)
     S, Q, st = gpu_refine(lay, 0)
