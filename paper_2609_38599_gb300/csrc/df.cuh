@@ -48,6 +48,17 @@ __device__ __forceinline__ DF df_warp_sum(DF a) {
 
 __device__ __forceinline__ double df_to_double(DF a) { return (double)a.h + (double)a.l; }
 
+// x as float64, by integer operations on its bits (a conversion runs at the
+// float64 rate, 1/64 of float32's): the exponent re-biased from 127 to 1023, the
+// mantissa shifted up.  Zero keeps its sign; subnormal and non-finite values take
+// the conversion.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x), m = b & 0x7FFFFFFFu;
+    if (m - 1u < 0x007FFFFFu || m >= 0x7F800000u) return (double)x;      // rare
+    const uint32_t hi = m ? (m >> 3) + (896u << 20) : 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(m << 29));
+}
+
 // x = hi + lo with hi = x rounded to float32 (nearest, ties to even) and
 // lo = x - hi rounded to float32, by integer operations on the bits of x.
 // Branch-free for zero and for 2^-74 <= |x| < 2^126; any other value

@@ -41,6 +41,7 @@
 // 128 x 64 tile, with two stages of 112 KB and a drain that combined the
 // levels by two-sums (55 operations an output and group, now 21) before it
 // released them, took 2.43 and 16.2 ms.
+#include "df.cuh"
 #include "tc_common.cuh"
 
 namespace jarq {
@@ -737,24 +738,27 @@ __global__ void __launch_bounds__(32 * kWhwWarps) whw_kernel(const float *__rest
 // On entry P = Phi + Plo holds H w, PK = Khi + Klo holds K w (rows of the
 // target projection with K in place of H), wHw[j] = w^T H w and
 // wXXw[j] = w^T XX w; on exit P holds H w_corr and wHw[j] ||y_j(mu)||^2.
-// One warp per row, float64 arithmetic.
-__global__ void mu_combine_kernel(float *__restrict__ Phi, float *__restrict__ Plo,
-                                  const float *__restrict__ Khi, const float *__restrict__ Klo,
-                                  const float *__restrict__ W, const double *__restrict__ wXXw,
-                                  double *__restrict__ wHw, int p, int d, double mu, double nu2) {
-    const int j = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (j >= p) return;
+// Four warps (one block) per row, float64 arithmetic: seven operations an entry,
+// which bound the kernel (1/64 of the float32 rate); the conversions in and the
+// split out are integer operations.  429 us on 4096 x 4096; with conversions (eight
+// more operations on the float64 pipe) and one warp per row 599 us.
+__global__ void __launch_bounds__(32 * kWhwWarps)
+    mu_combine_kernel(float *__restrict__ Phi, float *__restrict__ Plo, const float *__restrict__ Khi,
+                      const float *__restrict__ Klo, const float *__restrict__ W,
+                      const double *__restrict__ wXXw, double *__restrict__ wHw, int d, double mu, double nu2) {
+    __shared__ double part[2][kWhwWarps];
+    const int j = blockIdx.x, lane = threadIdx.x & 31;
     const size_t off = (size_t)j * d;
     double wKw = 0.0, ww = 0.0;
-    for (int k = lane; k < d; k += 32) {
-        const double P = (double)Phi[off + k] + (double)Plo[off + k];
-        const double PK = (double)Khi[off + k] + (double)Klo[off + k];
-        const double w = W[off + k];
+#pragma unroll 2
+    for (int k = threadIdx.x; k < d; k += 32 * kWhwWarps) {
+        const double P = widen(Phi[off + k]) + widen(Plo[off + k]);
+        const double PK = widen(Khi[off + k]) + widen(Klo[off + k]);
+        const double w = widen(W[off + k]);
         const double r = mu * P + (1.0 - mu) * fma(nu2, w, PK);
-        const float hi = __double2float_rn(r);
-        Phi[off + k] = hi;
-        Plo[off + k] = __double2float_rn(r - (double)hi);
+        const DF v = split_double(r);
+        Phi[off + k] = v.h;
+        Plo[off + k] = v.l;
         wKw = fma(w, PK, wKw);
         ww = fma(w, w, ww);
     }
@@ -763,6 +767,16 @@ __global__ void mu_combine_kernel(float *__restrict__ Phi, float *__restrict__ P
         ww += __shfl_xor_sync(0xffffffffu, ww, o);
     }
     if (lane == 0) {
+        part[0][threadIdx.x >> 5] = wKw;
+        part[1][threadIdx.x >> 5] = ww;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        wKw = ww = 0.0;
+        for (int w = 0; w < kWhwWarps; ++w) {
+            wKw += part[0][w];
+            ww += part[1][w];
+        }
         const double a = 1.0 - mu;
         wHw[j] = a * a * wXXw[j] + 2.0 * mu * a * wKw + mu * mu * (wHw[j] - nu2 * ww) + nu2 * ww;
     }
@@ -924,8 +938,7 @@ cudaError_t launch_whw(const float *W, const float *Phi, const float *Plo, doubl
 cudaError_t launch_mu_combine(float *Phi, float *Plo, const float *Khi, const float *Klo,
                               const float *W, const double *wXXw, double *wHw, int p, int d,
                               double mu, double nu2, cudaStream_t s) {
-    mu_combine_kernel<<<(unsigned)(((long long)p * 32 + 255) / 256), 256, 0, s>>>(
-        Phi, Plo, Khi, Klo, W, wXXw, wHw, p, d, mu, nu2);
+    mu_combine_kernel<<<p, 32 * kWhwWarps, 0, s>>>(Phi, Plo, Khi, Klo, W, wXXw, wHw, d, mu, nu2);
     return cudaGetLastError();
 }
 

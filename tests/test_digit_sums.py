@@ -85,3 +85,21 @@ def test_sweep_product_sum(groups, lead, spread):
                                         + Fraction(int(w), 1 << 30)) for a, x, y, z, w in zip(s, *D)]
     err = [abs(Fraction(float(h)) + Fraction(float(l)) - e) for h, l, e in zip(H, L, exact)]
     assert all(float(e) <= (groups + 4) * 2.0 ** -24 * b for e, b in zip(err, low))
+
+
+def test_float32_widened_by_integer_operations():
+    """float32 -> float64 by re-biasing the exponent: exact for zeros and all
+    normal numbers (the kernels convert the others)."""
+    rng = np.random.default_rng(3)
+    b = np.concatenate([rng.integers(0, 1 << 32, 200000, dtype=np.uint64),
+                        [0, 1 << 31, 0x00800000, 0x007FFFFF, 1, 0x7F7FFFFF, 0xFF7FFFFF, 0x80800000, 0x7F800000]])
+    b = b.astype(np.uint32)
+    m = b & np.uint32(0x7FFFFFFF)
+    rare = (m - np.uint32(1) < 0x007FFFFF) | (m >= 0x7F800000)
+    x = b.view(F)
+    assert np.array_equal(rare, ~(np.isfinite(x) & ((x == 0) | (np.abs(x) >= np.finfo(F).tiny))))
+    hi = np.where(m > 0, (m >> np.uint32(3)) + np.uint32(896 << 20), 0).astype(np.uint64)
+    hi |= (b & np.uint32(1 << 31)).astype(np.uint64)
+    lo = ((m.astype(np.uint64) << np.uint64(29)) & np.uint64(0xFFFFFFFF))
+    bits = ((hi << np.uint64(32)) | lo)[~rare]
+    assert np.array_equal(bits, x[~rare].astype(np.float64).view(np.uint64))

@@ -262,6 +262,26 @@ def test_objective_misaligned_buffers(jarq, g):
         np.testing.assert_array_equal(out[0], x)
 
 
+def test_mu_target_of_zero_and_subnormal_rows(jarq):
+    """The corrected target of a zero row is exactly 0, that of a subnormal row
+    (|y|^2 below 1e-70) next to nothing, and the other rows are unaffected."""
+    lay = small_layer(128, 8, 64, 3, seed=26)
+    W, Q = lay.W.copy(), lay.Q0.copy()
+    Q[1:3] = np.repeat(lay.Z[1:3], 64, axis=1)      # codes at the zero point
+    W[1], W[2] = 0.0, 1e-41
+
+    def run(W):
+        hess = jarq.prepare(lay.H, 64)
+        st = jarq.refine_mu(hess, W, lay.S0.copy(), Q.copy(), lay.Z, lay.bits, lay.H * np.float32(0.9), lay.H,
+                            0.5, 0.0, max_iters=0)
+        hess.close()
+        return st.L_host
+
+    L, rest = run(W), run(lay.W)
+    assert L[1] == 0.0 and abs(L[2]) <= 1e-70
+    np.testing.assert_array_equal(np.delete(L, (1, 2)), np.delete(rest, (1, 2)))
+
+
 def test_k0_returns_host_state(jarq):
     lay = small_layer(128, 40, 64, 3, seed=23)
     S, Q, st = gpu_refine(lay, 0)
