@@ -4,8 +4,8 @@ One step = one ``jarq_refine_layer`` call refining the Llama-2-7B q_proj
 layer (4096 x 4096, g = 128, 3-bit, RTN host, K = 10 iterations, early stop
 off) from its host state: the whole hot path (once the target projection
 P = W H and its folded form; per iteration the Gram matrices, right-hand
-sides and joint scale solve, then the 32-group sweep of phase products and
-Babai proposals).  Inputs are seeded synthetic tensors resident in HBM; the
+sides and joint scale solve, then the sweep, a product and a Babai step per
+block of two groups).  Inputs are seeded synthetic tensors resident in HBM; the
 working set per step (W, P and the folded P 64 MB each, the digit planes of
 H 336 MB) exceeds the 129 MB L2.
 
@@ -266,7 +266,7 @@ def kernel_model(kernel, lay, nsplit_bytes=0):
     if kernel == "sweep_babai":
         return dict(bound="alu", work=1.0 * g * d * p / launches)
     if kernel == "hr_full":
-        return dict(bound="tensor", work=2.0 * p * d * d, issued=6 * 2.0 * p * d * d)
+        return dict(bound="tensor", work=2.0 * p * d * d, issued=8 * 2.0 * p * d * d)
     if kernel == "gram":
         blocks = G * (G + 1) / 2
         return dict(bound="tensor", work=2.0 * p * g * g * blocks, issued=4 * 2.0 * p * g * g * blocks)

@@ -143,7 +143,7 @@ struct jarq_hessian {
     __nv_bfloat16 *Hdig8 = nullptr;    // [6][d_pad][d_pad] base 2^8, |digit| <= 128
     __half *Hdig10 = nullptr;          // [4][d_pad][d_pad] base 2^10, |digit| <= 512
     int *expo = nullptr;          // [G][G] block exponents of the digits
-    CUtensorMap mapH128, mapH64;  // tensor maps of Hplanes, 128 x 64 and 64 x 64 boxes
+    CUtensorMap mapH128;          // tensor map of Hplanes, 128 x 64 boxes
     CUtensorMap mapD8, mapD10;    // tensor maps of Hdig8 (64 x 32 boxes) / Hdig10 (64 x 64)
     float *Lf = nullptr;          // [G][factor_floats(g)] lower factor L_i = R_i^T, packed
     // digits of the blocks Ht_{i'i}, i' = i + 1 .. i + kMaxBlock - 1, column by
@@ -201,10 +201,6 @@ cudaError_t launch_residual(const float *W, const float *S, const uint8_t *Q, co
 cudaError_t launch_tc_hr_full(const CUtensorMap &mapA, const CUtensorMap &mapB, float *out,
                               int ldo, int p, int p_pad, int d, int d_pad, int *status,
                               cudaStream_t s);
-cudaError_t launch_tc_hr_phase(const CUtensorMap &mapA, const CUtensorMap &mapB128,
-                               const CUtensorMap &mapB64, float *out, int p, int p_pad, int d_pad,
-                               int g, int i, int nsplit, const int *active, int *status,
-                               cudaStream_t s);
 cudaError_t launch_grad(const float *r, const float *Hr, double *F, int p, int d, cudaStream_t s);
 cudaError_t launch_slices(const float *Hs, int *expo, __nv_bfloat16 *dig8, __half *dig10, int d,
                           int d_pad, int g, cudaStream_t s);

@@ -3,19 +3,15 @@
 // The residual r = w - D_s (q - z) (Eq. quantized_group) and the symmetric
 // Hessian H are both split exactly into three bf16 planes,
 // x = x1 + x2 + x3 (truncation splits of the float32 value), and
-//     H r ~= sum over the six products r_a H_b with a + b <= 4
-// (a, b = 1..3; the three dropped products are below float32 resolution),
+//     H r ~= sum over the eight products r_a H_b but r_3 H_3
+// (a, b = 1..3; the dropped product is below float32 resolution),
 // accumulated in float32.  Tensor-core accumulation truncates, so its error
 // grows with the number of products summed into one accumulator; the kernel
-// therefore (a) keeps the leading product r_1 H_1 and the five small products
+// therefore (a) keeps the leading product r_1 H_1 and the seven small products
 // in separate TMEM accumulators, and (b) drains both into float32 registers
-// (round to nearest) every 128 columns of K, restarting the TMEM sums at zero.
-// Two accumulator pairs alternate so the MMAs of one 128-wide K period overlap
-// the drain of the previous one.  Used for
-//   * the full product H r at the start of an iteration (objective of
-//     Eq. bbmils_columns and the scale gradient c_i^T (H r)_i), and
-//   * the per-group phase product (H r)_i of the Gauss-Seidel sweep
-//     (Eq. conditional_residual), split over K across CTAs.
+// (round to nearest) every 64 columns of K, restarting the TMEM sums at zero.
+// Two accumulator pairs alternate so the MMAs of one 64-wide K period overlap
+// the drain of the previous one.  Used for the objective (Eq. bbmils_columns).
 //
 // One CTA computes a 128-row x BN-column output tile:
 //   warp 0      TMA producer: 3 A planes + 3 B planes per 64-wide K chunk
@@ -265,12 +261,11 @@ __global__ void __launch_bounds__(320, 1)
 
 template <int BN>
 cudaError_t launch_tc_hr_bn(const CUtensorMap &mapA, const CUtensorMap &mapB, const HrArgs &a,
-                            dim3 grid, cudaStream_t s, bool programmatic = false) {
+                            dim3 grid, cudaStream_t s) {
     using C = HrCfg<BN>;
     static std::atomic<unsigned long long> attr_done{0};
     const cudaError_t e = set_max_dynamic_smem((const void *)tc_hr_kernel<BN>, C::kSmem, attr_done);
     if (e != cudaSuccess) return e;
-    if (programmatic) return launch_pdl(tc_hr_kernel<BN>, grid, dim3(320), C::kSmem, s, mapA, mapB, a);
     tc_hr_kernel<BN><<<grid, 320, C::kSmem, s>>>(mapA, mapB, a);
     return cudaGetLastError();
 }
@@ -285,21 +280,5 @@ cudaError_t launch_tc_hr_full(const CUtensorMap &mapA, const CUtensorMap &mapB, 
     dim3 grid(p_pad / 128, d_pad / 128, 1);
     return launch_tc_hr_bn<128>(mapA, mapB, a, grid, s);
 }
-
-// Phase product (H r)_i for group i, split over K: out[split][p][g].
-cudaError_t launch_tc_hr_phase(const CUtensorMap &mapA, const CUtensorMap &mapB128,
-                               const CUtensorMap &mapB64, float *out, int p, int p_pad, int d_pad,
-                               int g, int i, int nsplit, const int *active, int *status,
-                               cudaStream_t s) {
-    const int kc_total = d_pad / 64;
-    const int kc_per = (kc_total + nsplit - 1) / nsplit;
-    HrArgs a{out, (size_t)p_pad * g, g, p, p_pad, d_pad, i * g, g, kc_total, kc_per, active, status};
-    dim3 grid(p_pad / 128, 1, nsplit);
-    if (g == 128) return launch_tc_hr_bn<128>(mapA, mapB128, a, grid, s, true);
-    if (g == 64) return launch_tc_hr_bn<64>(mapA, mapB64, a, grid, s, true);
-    return cudaErrorInvalidValue;
-}
-
-int tc_hr_smem_bytes(int bn) { return bn == 128 ? HrCfg<128>::kSmem : HrCfg<64>::kSmem; }
 
 }  // namespace jarq
