@@ -705,18 +705,26 @@ jarq_status refine_impl(jarq_hessian *h, const float *W, float *S, uint8_t *Q, c
     }
     RUN("ptilde", 2, launch_ptilde(w.mapPd, h->mapRi, w.Phi, w.Plo, w.wdig, w.wexp, h->rexp, w.Pt_hi,
                                    w.Pt_lo, p, w.p_pad, d, h->d_pad, g, h->dstatus, st));
+    // Gram, right-hand side and solve of a small layer are launched
+    // programmatically too, so that launch latency and prologues run under the
+    // kernel before: 256 x 256 455 -> 427 us, 1024 x 512 530 -> 500 us, 64 x 4096
+    // 3.26 -> 3.21 ms.  Above 2^19 weights the early grids take room from the
+    // running one: 1000 x 1344 1.05 -> 1.10 ms, 256 x 4096 2.82 -> 2.88 ms, 4096 x
+    // 4096 13.02 -> 13.15 ms.
+    constexpr long long kChainedWeights = 1ll << 19;
+    const bool chained = (long long)p * d <= kChainedWeights;
     for (int k = 1; k <= o.max_iters; ++k) {
         // with the early stop off every row is refined (a row marked numerical
         // is skipped by the solve and Babai), so the Gram and the right-hand
         // side need not read the active flags
         const int *act_es = o.early_stop ? w.active : nullptr;
         RUN("gram", 1, launch_tc_gram(w.mapC, h->mapD10, la.Q, la.Z, h->expo, act_es, w.gram, p,
-                                      w.p_pad, d, h->d_pad, g, bits, h->dstatus, st));
-        RUN("rhs", 1, launch_rhs(la.Q, la.Z, w.Phi, w.Plo, act_es, w.rhs, p, d, g, st));
+                                      w.p_pad, d, h->d_pad, g, bits, h->dstatus, st, chained));
+        RUN("rhs", 1, launch_rhs(la.Q, la.Z, w.Phi, w.Plo, act_es, w.rhs, p, d, g, st, chained));
         double *L_out = (k == 1 && stats && stats->L_host) ? w.L_host : nullptr;
         RUN("scale_solve", 1, launch_scale_solve(w.gram, w.rhs, w.wHw, la.S, w.L_prev, L_out,
                                                  w.active, w.iters, w.ridge, w.rstat, h->dstatus,
-                                                 p, d, g, k, false, o, st));
+                                                 p, d, g, k, false, o, st, chained));
         // The phase product reads the active flags only with the early stop
         // on (to skip tiles whose rows all stopped); a row marked numerical
         // by the scale solve is skipped by Babai, and its partials go unread.
@@ -737,11 +745,11 @@ jarq_status refine_impl(jarq_hessian *h, const float *W, float *S, uint8_t *Q, c
     const bool want_host0 = stats && stats->L_host && o.max_iters == 0;
     if (want_final || want_host0) {
         RUN("gram", 1, launch_tc_gram(w.mapC, h->mapD10, la.Q, la.Z, h->expo, nullptr, w.gram, p,
-                                      w.p_pad, d, h->d_pad, g, bits, h->dstatus, st));
-        RUN("rhs", 1, launch_rhs(la.Q, la.Z, w.Phi, w.Plo, nullptr, w.rhs, p, d, g, st));
+                                      w.p_pad, d, h->d_pad, g, bits, h->dstatus, st, chained));
+        RUN("rhs", 1, launch_rhs(la.Q, la.Z, w.Phi, w.Plo, nullptr, w.rhs, p, d, g, st, chained));
         RUN("scale_solve", 1, launch_scale_solve(w.gram, w.rhs, w.wHw, la.S, w.L_prev, w.L_final,
                                                  w.active, w.iters, w.ridge, w.rstat, h->dstatus,
-                                                 p, d, g, 0, true, o, st));
+                                                 p, d, g, 0, true, o, st, chained));
         if (want_host0)
             CK(cudaMemcpyAsync(w.L_host, w.L_final, p * sizeof(double), cudaMemcpyDeviceToDevice, st));
     }

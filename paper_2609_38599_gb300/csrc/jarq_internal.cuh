@@ -207,7 +207,7 @@ cudaError_t launch_slices(const float *Hs, int *expo, __nv_bfloat16 *dig8, __hal
 cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, const uint8_t *Q,
                            const int32_t *Z, const int *expo, const int *active, float2 *gram,
                            int p, int p_pad, int d, int d_pad, int g, int bits, int *status,
-                           cudaStream_t s);
+                           cudaStream_t s, bool pdl = false);
 cudaError_t launch_slices8(const float *M, int *expo, __nv_bfloat16 *dig8, int d, int d_pad,
                            int g, cudaStream_t s);
 cudaError_t launch_mu_combine(float *Phi, float *Plo, const float *Khi, const float *Klo,
@@ -221,12 +221,13 @@ cudaError_t launch_tc_proj(const CUtensorMap &mapW, const CUtensorMap &mapH, flo
 cudaError_t launch_whw(const float *W, const float *Phi, const float *Plo, double *out, int p,
                        int d, cudaStream_t s);
 cudaError_t launch_rhs(const uint8_t *Q, const int32_t *Z, const float *Phi, const float *Plo,
-                       const int *active, double *rhs, int p, int d, int g, cudaStream_t s);
+                       const int *active, double *rhs, int p, int d, int g, cudaStream_t s,
+                       bool pdl = false);
 cudaError_t launch_scale_solve(const float2 *gram, const double *rhs, const double *wHw, float *S,
                                double *L_prev, double *L_out, int *active,
                                int *iters, int *ridge, int *rstat, int *status, int p, int d,
                                int g, int k, bool eval_only, const jarq_options &o,
-                               cudaStream_t s);
+                               cudaStream_t s, bool pdl = false);
 cudaError_t launch_babai(float *t_hi, float *t_lo, const float *pt_hi,
                          const float *pt_lo, int nsplit, const float *Lf, const int2 *band,
                          const int *expoT, const float *S, uint8_t *Q, const int32_t *Z,

@@ -28,7 +28,7 @@
 #include <float.h>
 
 #include "df.cuh"
-#include "jarq_internal.cuh"
+#include "tc_common.cuh"
 
 namespace jarq {
 namespace {
@@ -296,6 +296,8 @@ __global__ void __launch_bounds__(NT, 768 / NT) scale_solve_kernel(SolveArgs a) 
     __shared__ int flag;
     const int G = a.d / a.g, Gp = (G + 7) / 8 * 8, ld = solve_ld(G);
     const int j = blockIdx.x, t = threadIdx.x, tc = min(t, G - 1);
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
     if (!a.eval_only && !a.active[j]) return;   // uniform
     const bool own = t < G;
     float *A = fsm;                      // [Gp][ld]
@@ -507,6 +509,8 @@ constexpr int kSmallWarps = 4;   // rows (warps) per block of the G <= 32 kernel
 
 __global__ void __launch_bounds__(32 * kSmallWarps, 4) scale_solve_small_kernel(SolveArgs a) {
     __shared__ float Lsh[kSmallWarps][32 * 33];
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
     const int G = a.d / a.g;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j = blockIdx.x * kSmallWarps + w;
@@ -687,13 +691,12 @@ __global__ void __launch_bounds__(32 * kSmallWarps, 4) scale_solve_small_kernel(
 }
 
 template <int NT>
-cudaError_t launch_big(const SolveArgs &a, cudaStream_t s) {
+cudaError_t launch_big(const SolveArgs &a, bool pdl, cudaStream_t s) {
     static std::atomic<unsigned long long> attr_done{0};
     const cudaError_t e =
         set_max_dynamic_smem((const void *)scale_solve_kernel<NT>, (int)solve_bytes(NT), attr_done);
     if (e != cudaSuccess) return e;
-    scale_solve_kernel<NT><<<a.p, NT, solve_bytes(a.d / a.g), s>>>(a);
-    return cudaGetLastError();
+    return launch_k(scale_solve_kernel<NT>, dim3(a.p), dim3(NT), solve_bytes(a.d / a.g), s, pdl, a);
 }
 
 }  // namespace
@@ -702,17 +705,16 @@ cudaError_t launch_scale_solve(const float2 *gram, const double *rhs, const doub
                                double *L_prev, double *L_out, int *active,
                                int *iters, int *ridge, int *rstat, int *status, int p, int d,
                                int g, int k, bool eval_only, const jarq_options &o,
-                               cudaStream_t s) {
+                               cudaStream_t s, bool pdl) {
     const int G = d / g;
     SolveArgs a{gram, rhs, wHw, S, L_prev, L_out, active, iters, ridge, rstat,
                 status, p, d, g, k, eval_only, o};
-    if (G <= 32) {
-        scale_solve_small_kernel<<<(p + kSmallWarps - 1) / kSmallWarps, 32 * kSmallWarps, 0, s>>>(a);
-        return cudaGetLastError();
-    }
-    if (G <= 64) return launch_big<64>(a, s);
-    if (G <= 96) return launch_big<96>(a, s);
-    return launch_big<128>(a, s);
+    if (G <= 32)
+        return launch_k(scale_solve_small_kernel, dim3((p + kSmallWarps - 1) / kSmallWarps),
+                        dim3(32 * kSmallWarps), 0, s, pdl, a);
+    if (G <= 64) return launch_big<64>(a, pdl, s);
+    if (G <= 96) return launch_big<96>(a, pdl, s);
+    return launch_big<128>(a, pdl, s);
 }
 
 }  // namespace jarq

@@ -128,14 +128,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // a row tile pair none of whose rows is active is skipped; both CTAs read
     // the same flags
     const bool flags = a.active && a.tiles <= kMaxTiles;
-    if (flags)
-        for (int t = warp; t < a.tiles; t += kThreads / 32) {
-            int mine = 0;
-            for (int r = lane; r < 256; r += 32)
-                if (t * 256 + r < a.p) mine |= a.active[t * 256 + r];
-            mine = __any_sync(0xffffffffu, mine);
-            if (lane == 0) live[t] = (uint8_t)mine;
-        }
     // item -> first row of the tile pair, first unit and number of units
     // [nblk z / nparts, nblk (z + 1) / nparts) of the group pair's blocks; 0
     // units for a tile without active rows
@@ -185,6 +177,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tc::prefetch_tmap(&mapC);
         tc::prefetch_tmap(&mapS);
     }
+    // launched programmatically the previous grid may still run: all that it
+    // writes (codes, flags) is read, and the next grid released, after it
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
+    if (flags)
+        for (int t = warp; t < a.tiles; t += kThreads / 32) {
+            int mine = 0;
+            for (int r = lane; r < 256; r += 32)
+                if (t * 256 + r < a.p) mine |= a.active[t * 256 + r];
+            mine = __any_sync(0xffffffffu, mine);
+            if (lane == 0) live[t] = (uint8_t)mine;
+        }
     tc::tc_fence_before();
     __syncthreads();
     tc::cluster_sync();
@@ -650,7 +654,7 @@ cudaError_t launch_slices8(const float *M, int *expo, __nv_bfloat16 *dig8, int d
 cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, const uint8_t *Q,
                            const int32_t *Z, const int *expo, const int *active, float2 *gram,
                            int p, int p_pad, int d, int d_pad, int g, int bits, int *status,
-                           cudaStream_t s) {
+                           cudaStream_t s, bool pdl) {
     const int G = d / g;
     // ranges per (row tile pair, group pair): the fewest blocks for the busiest
     // CTA pair, each item costing about a sixth of a block beside its blocks
@@ -673,8 +677,7 @@ cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, con
     auto run = [&](auto *kernel, std::atomic<unsigned long long> &done) {
         const cudaError_t e = set_max_dynamic_smem((const void *)kernel, kSmem, done);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, kThreads, kSmem, s>>>(mapC, mapS, a);
-        return cudaGetLastError();
+        return launch_k(kernel, grid, dim3(kThreads), (size_t)kSmem, s, pdl, mapC, mapS, a);
     };
     static std::atomic<unsigned long long> done[3];
     if (bits <= 3) return run(tc_gram_kernel<4>, done[0]);

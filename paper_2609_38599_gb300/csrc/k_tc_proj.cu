@@ -640,6 +640,8 @@ __global__ void __launch_bounds__(kRhsThreads) rhs_kernel(const uint8_t *__restr
                                                           const int *__restrict__ active,
                                                           double *__restrict__ rhs, int p, int d) {
     constexpr int g = 32 * NT;
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
     const int G = d / g;
     const int j = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -943,15 +945,16 @@ cudaError_t launch_mu_combine(float *Phi, float *Plo, const float *Khi, const fl
 }
 
 cudaError_t launch_rhs(const uint8_t *Q, const int32_t *Z, const float *Phi, const float *Plo,
-                       const int *active, double *rhs, int p, int d, int g, cudaStream_t s) {
+                       const int *active, double *rhs, int p, int d, int g, cudaStream_t s,
+                       bool pdl) {
     const unsigned blocks = (unsigned)(((long long)p * 32 + kRhsThreads - 1) / kRhsThreads);
     if (g == 128)
-        rhs_kernel<4, 8><<<blocks, kRhsThreads, 0, s>>>(Q, Z, Phi, Plo, active, rhs, p, d);
-    else if (g == 64)
-        rhs_kernel<2, 2><<<blocks, kRhsThreads, 0, s>>>(Q, Z, Phi, Plo, active, rhs, p, d);
-    else
-        return cudaErrorInvalidValue;
-    return cudaGetLastError();
+        return launch_k(rhs_kernel<4, 8>, dim3(blocks), dim3(kRhsThreads), 0, s, pdl, Q, Z, Phi, Plo, active, rhs,
+                        p, d);
+    if (g == 64)
+        return launch_k(rhs_kernel<2, 2>, dim3(blocks), dim3(kRhsThreads), 0, s, pdl, Q, Z, Phi, Plo, active, rhs,
+                        p, d);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace jarq

@@ -97,6 +97,19 @@ def test_sweep_block_edges(jarq, din, dout, g, bits, K):
     assert np.array_equal(st["accepted"], res.accepted)
 
 
+@pytest.mark.parametrize("dout", [1024, 1025])
+def test_small_layer_launch_rule(jarq, dout):
+    """Both sides of 2^19 weights: every kernel of an iteration launched
+    programmatically, and only the sweep's; early stop on."""
+    lay = small_layer(512, dout, 128, 3, K=4, seed=dout)
+    prep, res = oracle_run(lay, 4, True)
+    S, Q, st = gpu_refine(lay, 4, early_stop=True)
+    assert st["status"] == 0 and np.mean(st["iters"] == res.iters) >= 0.99
+    m = compare_final(lay, prep, res, S, Q, st)
+    assert m["codes_same"] >= CODES_SAME, m
+    assert m["S_rel_max_same_rows"] <= REL_S and m["F_rel_max_same_rows"] <= REL_F, m
+
+
 def _many_group_layer(din, dout, g, bits, K, seed):
     """A layer with the small-layer recipe whose Hessian is accumulated on
     the GPU (torch generators), returned as NumPy arrays for the oracle."""
