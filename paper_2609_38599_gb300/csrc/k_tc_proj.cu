@@ -838,7 +838,12 @@ __global__ void slice_df_rows_kernel(const float *__restrict__ Phi, const float 
 // Hessian): plane u, row i g + a, column b holds digit u of R_i^{-1}[b][a]
 // (zero below the diagonal), so that the 64 x 64 tiles of the projection
 // kernel read the transposed block; exponent E_i with max |R_i^{-1}| < 2^E_i,
-// six balanced base-256 digits of R_i^{-1} 2^(7-E_i) in float64.
+// six balanced base-256 digits of R_i^{-1} 2^(7-E_i) in float64.  Bound by float64
+// (some thirty operations an entry): four blocks a group, each of which finds
+// the maximum for itself, and no arithmetic for the zeros.  32 groups of 128:
+// 51 us; one block a group took 152 us.
+constexpr int kRinvParts = 4;
+
 __global__ void slice_rinv_kernel(const double *__restrict__ Rinv, __nv_bfloat16 *__restrict__ rdig,
                                   int *__restrict__ rexp, int d, int g) {
     __shared__ double red[32];
@@ -858,12 +863,17 @@ __global__ void slice_rinv_kernel(const double *__restrict__ Rinv, __nv_bfloat16
     mx = red[0];
     int E = 0;
     if (mx > 0.0) frexp(mx, &E);
-    if (threadIdx.x == 0) rexp[i] = E;
+    if (threadIdx.x == 0 && blockIdx.y == 0) rexp[i] = E;
     const size_t plane = (size_t)d * g;
-    for (int idx = threadIdx.x; idx < g * g; idx += blockDim.x) {
+    for (int idx = blockIdx.y * blockDim.x + threadIdx.x; idx < g * g; idx += gridDim.y * blockDim.x) {
         const int a = idx / g, b = idx % g;
-        double x = b <= a ? ldexp(Ri[(size_t)b * g + a], 7 - E) : 0.0;
         const size_t off = ((size_t)i * g + a) * g + b;
+        if (b > a) {
+#pragma unroll
+            for (int u = 0; u < kHDig; ++u) rdig[u * plane + off] = __float2bfloat16_rn(0.f);
+            continue;
+        }
+        double x = ldexp(Ri[(size_t)b * g + a], 7 - E);
 #pragma unroll
         for (int u = 0; u < kHDig; ++u) {
             const double dg = rint(x);
@@ -877,7 +887,7 @@ __global__ void slice_rinv_kernel(const double *__restrict__ Rinv, __nv_bfloat16
 
 cudaError_t launch_slice_rinv(const double *Rinv, __nv_bfloat16 *rdig, int *rexp, int d, int g,
                               cudaStream_t s) {
-    slice_rinv_kernel<<<d / g, 256, 0, s>>>(Rinv, rdig, rexp, d, g);
+    slice_rinv_kernel<<<dim3(d / g, kRinvParts), 256, 0, s>>>(Rinv, rdig, rexp, d, g);
     return cudaGetLastError();
 }
 
