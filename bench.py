@@ -41,23 +41,23 @@ DTYPE = "f32 (integer-digit fp16/bf16 tensor-core products with exact partial su
 
 # DRAM bytes (read + write) per launch from one ncu capture of the main
 # workload (q_proj; other workloads report null; the sweep kernels' figures
-# are those of the first phase; the Hessian
-# kernel's is a capture at 32768 tokens scaled to the full token count); the
-# summaries kept with the profiles give each capture's command.  A figure is
+# are those of the first block, with ncu's cache flush before each launch; the
+# Hessian kernel has none at the bench's token count); the summary kept with
+# the profiles gives the capture's command.  A figure is
 # valid while the kernel's source file is unchanged (first 12 hex digits of
 # its SHA-1); otherwise the bench reports null.
 TRAFFIC = {
-    "target": ("k_tc_target.cu", "d243a12fe467", 38.299e6 + 0.000512e6),
-    "babai": ("k_babai.cu", "22add12322a6", 14.275e6 + 0.002048e6),
-    "gram": ("k_tc_gram.cu", "0a673536a73b", 146.070e6 + 24.520e6),
-    "proj": ("k_tc_proj.cu", "6cf1b3d8cc4f", 1371.689e6 + 153.910e6),
-    "ptilde": ("k_tc_proj.cu", "6cf1b3d8cc4f", 134.248e6 + 150.687e6 + 222.887e6 + 103.208e6),
-    "rhs": ("k_tc_proj.cu", "6cf1b3d8cc4f", 151.550e6 + 0.264e6),
-    "whw": ("k_tc_proj.cu", "6cf1b3d8cc4f", 201.371e6 + 0.190e6),
-    "slice_rows": ("k_tc_proj.cu", "6cf1b3d8cc4f", 67.122e6 + 81.168e6),
-    "scale_solve": ("k_solve.cu", "6176a6787f3e", 35.289e6 + 0.0),
-    # captured at 32768 tokens, scaled to 262144
-    "syrk": ("k_syrk.cu", "3896afedc783", 8 * 537.171e6 + 40.712e6),
+    "target": ("k_tc_target.cu", "0e24dd5faf51", 42.625e6 + 0.140e6),
+    "sweep_product": ("k_tc_target.cu", "0e24dd5faf51", 42.625e6 + 0.140e6),
+    "babai": ("k_babai.cu", "672bc1eb4b99", 19.160e6 + 0.0),
+    "sweep_babai": ("k_babai.cu", "672bc1eb4b99", 19.160e6 + 0.0),
+    "gram": ("k_tc_gram.cu", "caa812655db4", 141.735e6 + 22.765e6),
+    "proj": ("k_tc_proj.cu", "18c811b3e91e", 1350.252e6 + 139.033e6),
+    "ptilde": ("k_tc_proj.cu", "18c811b3e91e", 134.258e6 + 143.617e6 + 288.578e6 + 97.168e6),
+    "rhs": ("k_tc_proj.cu", "18c811b3e91e", 151.551e6 + 0.272e6),
+    "whw": ("k_tc_proj.cu", "18c811b3e91e", 201.350e6 + 0.297e6),
+    "slice_rows": ("k_tc_proj.cu", "18c811b3e91e", 67.122e6 + 73.267e6),
+    "scale_solve": ("k_solve.cu", "c4ababeb8bae", 35.289e6 + 0.0),
 }
 HESSIAN_WORKLOAD = "llama2_7b_attn_in_4096_n262144"
 
