@@ -320,6 +320,28 @@ class DeviceGuard {
     bool ok_ = false, switched_ = false;
 };
 
+// A status word of the current device for the length of one call that has no
+// handle: calls on other streams and host threads have other words, so a
+// kernel may decide by its call's word whether to write.  The words are one
+// static array; a call waits for a free one (each call ends by itself).
+class StatusWord {
+  public:
+    explicit StatusWord(cudaStream_t s);
+    // gives the word back, after the stream's work if read() has not waited
+    ~StatusWord();
+    int *ptr() const { return ptr_; }    // null: the device has no such array
+    cudaError_t clear();                 // enqueued on the call's stream
+    cudaError_t read(int *bits);         // the word after all of the stream's work
+    StatusWord(const StatusWord &) = delete;
+    StatusWord &operator=(const StatusWord &) = delete;
+
+  private:
+    cudaStream_t s_;
+    int index_;
+    int *ptr_ = nullptr;
+    bool idle_ = true;
+};
+
 // 2D tensor map of 2-byte elements (bf16 or fp16) over [rows][cols]
 // (pitch = cols elements), box_rows x box_cols boxes, box_cols = 64 with
 // 128-byte swizzle or 32 with 64-byte swizzle, out-of-range elements read as

@@ -1,8 +1,27 @@
 // Elementwise and bookkeeping kernels of the refinement path.
+#include <condition_variable>
+#include <mutex>
+
 #include "tc_common.cuh"
 
 namespace jarq {
 namespace {
+
+constexpr int kStatusWords = 64;       // calls that hold one at a time
+__device__ int g_status_words[kStatusWords];
+
+// Which words are taken.  An index is taken on all devices at once.  Never
+// destroyed: a call may still run while the process ends.
+struct StatusPool {
+    std::mutex mu;
+    std::condition_variable freed;
+    unsigned long long taken = 0;
+};
+StatusPool &status_pool() {
+    static StatusPool *p = new StatusPool;
+    return *p;
+}
+static_assert(kStatusWords == 64, "one bit of `taken` per word");
 
 // Codes and zero points must lie in [0, qmax] (Sec. 3.1: q in B^{d_i};
 // integer zero points kept from the host).
@@ -133,6 +152,45 @@ __global__ void init_rows_kernel(int *active, int *iters, int *accepted, int *ri
 }
 
 }  // namespace
+
+StatusWord::StatusWord(cudaStream_t s) : s_(s) {
+    StatusPool &pool = status_pool();
+    {
+        std::unique_lock<std::mutex> lock(pool.mu);
+        pool.freed.wait(lock, [&] { return pool.taken != ~0ull; });
+        index_ = 0;
+        while (pool.taken >> index_ & 1) ++index_;
+        pool.taken |= 1ull << index_;
+    }
+    void *base = nullptr;
+    if (cudaGetSymbolAddress(&base, g_status_words) != cudaSuccess || !base)
+        (void)cudaGetLastError();
+    else
+        ptr_ = static_cast<int *>(base) + index_;
+}
+
+StatusWord::~StatusWord() {
+    // an error between clear() and read() leaves work that may use the word
+    if (!idle_ && cudaStreamSynchronize(s_) != cudaSuccess) (void)cudaGetLastError();
+    StatusPool &pool = status_pool();
+    {
+        std::lock_guard<std::mutex> lock(pool.mu);
+        pool.taken &= ~(1ull << index_);
+    }
+    pool.freed.notify_one();
+}
+
+cudaError_t StatusWord::clear() {
+    idle_ = false;
+    return cudaMemsetAsync(ptr_, 0, sizeof(int), s_);
+}
+
+cudaError_t StatusWord::read(int *bits) {
+    cudaError_t e = cudaMemcpyAsync(bits, ptr_, sizeof(int), cudaMemcpyDeviceToHost, s_);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s_);
+    idle_ = e == cudaSuccess;
+    return e;
+}
 
 int num_sms() {
     constexpr int kDevs = 64;

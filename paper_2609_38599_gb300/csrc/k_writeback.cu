@@ -8,11 +8,8 @@
 namespace jarq {
 namespace {
 
-// status word of the write-back calls (device address taken per call)
-__device__ int g_writeback_status;
-
-// Every kernel below does nothing when the validation before it (same stream)
-// has set the status word.
+// Every kernel below does nothing when the validation before it (same call)
+// has set the call's status word.
 
 // if s < 0, s' = -s, z' = qmax - z, q' = qmax - q.  A warp looks at 32 (row,
 // group) scales at once and takes the negative ones in turn, so that a layer
@@ -182,21 +179,18 @@ int grid_for(size_t n) {
 // Validate codes (and zero points when Z is given); then `launch(stream,
 // status)` a kernel that does nothing when the status word is set.  One
 // synchronisation for both: waiting for the verdict before the launch cost
-// about 15 us a call.
+// about 15 us a call.  The word is this call's alone: another call's verdict
+// must not stop this kernel halfway, nor its start let this one run on bad codes.
 template <class F>
 jarq_status checked_run(const uint8_t *Q, const int32_t *Z, int p, int d, int G, int qmax,
                         cudaStream_t st, F launch) {
-    int *status = nullptr;
-    if (cudaGetSymbolAddress((void **)&status, g_writeback_status) != cudaSuccess || !status) {
-        (void)cudaGetLastError();
-        return JARQ_ERR_CUDA;
-    }
+    StatusWord status(st);
+    if (!status.ptr()) return JARQ_ERR_CUDA;
     int host = 0;
-    cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = launch_validate(Q, Z, p, d, Z ? G : 0, qmax, status, st);
-    if (e == cudaSuccess) e = launch(st, status);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&host, status, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaError_t e = status.clear();
+    if (e == cudaSuccess) e = launch_validate(Q, Z, p, d, Z ? G : 0, qmax, status.ptr(), st);
+    if (e == cudaSuccess) e = launch(st, status.ptr());
+    if (e == cudaSuccess) e = status.read(&host);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return JARQ_ERR_CUDA;

@@ -139,6 +139,60 @@ def test_writeback_rejects_bad_input(jarq):
     assert bool((Wd == 7.0).all())
 
 
+def test_valid_and_invalid_layers_on_two_streams(jarq):
+    """Two host threads, each on a stream of its own, one writing back a valid
+    layer and one passing codes out of range, over and over: every valid result
+    is whole, every invalid call is refused and changes nothing."""
+    import threading
+    dout, din, g, bits = 1031, 2048, 64, 3
+    S, Q, Z = _signed_state(dout, din, g, bits, seed=77)
+    S2, Q2, Z2 = canonicalize(S.astype(np.float64), Q, Z, bits)
+    want = {"S": S2.astype(np.float32), "Q": Q2, "Z": Z2, "P": pack_codes(Q2, bits).view(np.int32),
+            "W": np.asarray(dequantize_cast(S2.astype(np.float32), Q2, Z2, g, "float16"), dtype=np.float16)}
+    want = {k: torch.as_tensor(v).cuda() for k, v in want.items()}
+    t = lambda a: torch.as_tensor(a).cuda()
+    Sd, Qd, Zd = t(S), t(Q), t(Z)
+    Qbad = Qd.clone()
+    Qbad[-1, -1] = 1 << bits            # seen by the last blocks of the check
+    torch.cuda.synchronize()
+    wrong, done = [], threading.Event()
+
+    def valid():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(150):
+                    s, q, z = Sd.clone(), Qd.clone(), Zd.clone()
+                    jarq.canonicalize(s, q, z, g, bits)
+                    got = {"S": s, "Q": q, "Z": z, "W": jarq.dequantize(s, q, z, g, bits, "float16"),
+                           "P": jarq.pack_codes(q, bits)}
+                    wrong.extend(k for k, v in got.items() if not torch.equal(v, want[k]))
+        except Exception as e:      # a valid call refused
+            wrong.append(e)
+        done.set()
+
+    def invalid():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            s, q, z = Sd.clone(), Qbad.clone(), Zd.clone()
+            while not done.is_set():
+                for call in (lambda: jarq.canonicalize(s, q, z, g, bits), lambda: jarq.pack_codes(q, bits),
+                             lambda: jarq.dequantize(s, q, z, g, bits, "float16")):
+                    try:
+                        call()
+                        wrong.append("an invalid layer was accepted")
+                    except jarq.JarqError as e:
+                        if e.status != jarq.JARQ_ERR_ARG:
+                            wrong.append(e)
+            if not (torch.equal(s, Sd) and torch.equal(q, Qbad) and torch.equal(z, Zd)):
+                wrong.append("an invalid layer was changed")
+
+    threads = [threading.Thread(target=f) for f in (valid, invalid)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join(120)
+    assert done.is_set() and not wrong, wrong[:5]
+
+
 def test_ridge_acceptance_matches_oracle(jarq):
     """A row whose starting scales are its exact least-squares scales and
     whose Gram matrix is singular (one group at its zero point, H scaled so

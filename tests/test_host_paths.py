@@ -1,0 +1,125 @@
+"""The library's host code on the CPU: its own objects linked with a CUDA
+runtime that has no device (``fake_cudart.cpp``), so that the order, streams,
+buffers and failures of a call's device operations can be looked at.  Kernels
+do not run; nothing here says anything about results."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HOOK = ctypes.CFUNCTYPE(None, ctypes.c_char_p, ctypes.c_void_p, ctypes.c_size_t)
+STREAM = 0x5150
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_2609_38599_gb300 import build as b
+    srcs = [os.path.join(b.CSRC, f) for f in os.listdir(b.CSRC)] + [os.path.join(ROOT, "include", "jarq.h")]
+    objs = [os.path.join(b.BUILD, f[:-3] + ".o") for f in os.listdir(b.CSRC) if f.endswith(".cu")]
+    newest = max(os.path.getmtime(f) for f in srcs)
+    if not all(os.path.exists(o) and os.path.getmtime(o) >= newest for o in objs):
+        b.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libjarq_host.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(b.nvcc())), "include")
+    subprocess.run(["g++", "-O1", "-fPIC", "-shared", "-std=c++17", "-Wl,-Bsymbolic", "-I" + cuda,
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp"), *objs, "-o", out, "-pthread"], check=True)
+    lib = ctypes.CDLL(out)
+    lib.fake_log.restype = ctypes.c_char_p
+    lib.fake_live.restype = ctypes.c_size_t
+    lib.fake_hook.argtypes = [HOOK]
+    return lib
+
+
+class Device:
+    """Buffers, handles and the log of one test."""
+
+    def __init__(self, lib):
+        self.lib, self.hooks, self.bufs, self.handles = lib, [], [], []
+        lib.fake_reset()
+
+    def buf(self, nbytes):
+        p = ctypes.c_void_p()
+        assert self.lib.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(nbytes)) == 0
+        self.bufs.append(p)
+        return p
+
+    def prepare(self, din, g, stream=STREAM):
+        h = ctypes.c_void_p()
+        rc = self.lib.jarq_prepare_hessian(self.buf(4 * din * din), din, g, ctypes.c_float(0), ctypes.byref(h),
+                                           ctypes.c_void_p(stream))
+        if rc == 0:
+            self.handles.append(h)
+        return rc, h
+
+    def layer(self, din, dout, g):
+        G = din // g
+        return self.buf(4 * din * dout), self.buf(4 * dout * G), self.buf(din * dout), self.buf(4 * dout * G)
+
+    def refine(self, h, lay, dout, bits=3, stream=STREAM):
+        return self.lib.jarq_refine_layer(h, *lay, dout, bits, None, None, ctypes.c_void_p(stream))
+
+    def refine_mu(self, h, lay, dout, K, XX, bits=3, stream=STREAM):
+        return self.lib.jarq_refine_layer_mu(h, *lay, dout, bits, K, XX, ctypes.c_float(0.5), ctypes.c_float(0),
+                                             None, None, ctypes.c_void_p(stream))
+
+    def hook(self, fn):
+        """`fn(what, pointer, bytes)` inside every operation from now on."""
+        h = HOOK(lambda what, p, n: fn(what.decode(), p, n))
+        self.hooks.append(h)
+        self.lib.fake_hook(h)
+
+    def log(self):
+        """Operations so far: (what, stream, rest)."""
+        return [tuple(x.split(" ", 2)) for x in self.lib.fake_log().decode().splitlines()]
+
+    def close(self):
+        self.lib.fake_reset()
+        for h in self.handles:
+            self.lib.jarq_hessian_destroy(h)
+        for p in self.bufs:
+            self.lib.cudaFree(p)
+
+
+@pytest.fixture
+def dev(lib):
+    d = Device(lib)
+    yield d
+    d.close()
+
+
+def _overlapped(dev, call):
+    """Runs `call(stream)` and, while it waits for its stream, a second one;
+    the addresses of the status words that the two clear."""
+    cleared = {}
+    state = {"inside": False}
+
+    def note(what, p, n):
+        who = "second" if state["inside"] else "first"
+        if what == "memset" and n == 4:
+            cleared[who] = p
+        if what == "sync" and not state["inside"] and "second" not in cleared:
+            state["inside"] = True
+            assert call(STREAM + 1) == 0
+            state["inside"] = False
+
+    dev.hook(note)
+    assert call(STREAM) == 0
+    assert set(cleared) == {"first", "second"}
+    return cleared
+
+
+def test_overlapping_writeback_calls_have_a_status_word_each(dev):
+    """The write-back kernels write only while their call's status word is
+    clear: a call on another stream must not set or clear that word."""
+    lib = dev.lib
+    S, Q, Z, out = dev.buf(4 * 8 * 2), dev.buf(8 * 128), dev.buf(4 * 8 * 2), dev.buf(4 * 8 * 128)
+    calls = {
+        "canonicalize": lambda s: lib.jarq_canonicalize(S, Q, Z, 8, 128, 64, 3, ctypes.c_void_p(s)),
+        "dequantize": lambda s: lib.jarq_dequantize(S, Q, Z, 8, 128, 64, 3, 1, out, ctypes.c_void_p(s)),
+        "pack": lambda s: lib.jarq_pack_codes(Q, 8, 128, 3, out, ctypes.c_void_p(s)),
+    }
+    for name, call in calls.items():
+        words = _overlapped(dev, call)
+        assert words["first"] != words["second"], name
