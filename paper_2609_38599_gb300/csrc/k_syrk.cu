@@ -66,8 +66,6 @@ static_assert(kSmem <= 227 * 1024, "ring and staged parts must fit an SM's share
 // fp16 x fp16 -> f32, M = 256, N = 256, both operands MN-major.
 constexpr uint32_t kIdesc = tc::idesc_f16_f32(256, 256) | (1u << 15) | (1u << 16);
 
-__device__ int g_syrk_status;
-
 // Descriptor of an MN-major operand written by TMA with 128-byte swizzle:
 // 64 contiguous MN elements per 128-byte row, K rows 128 bytes apart,
 // 8-row atoms SBO = 1024 bytes apart along K, 64-element MN atoms
@@ -84,6 +82,7 @@ __device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr) {
 
 struct SyrkArgs {
     float *H;
+    int *status;     // the call's own word
     float scale;
     int d, n;
     int nt;          // tiles per side
@@ -346,7 +345,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tc::tc_fence_after();
         tc::tmem_dealloc_pair(tmem, 512);
     }
-    if (threadIdx.x == 0 && *abort_flag) atomicOr(&g_syrk_status, ST_TIMEOUT);
+    if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, ST_TIMEOUT);
 }
 
 }  // namespace
@@ -366,23 +365,21 @@ extern "C" jarq_status jarq_accumulate_hessian(const void *X, int n, int d, floa
         (void)cudaGetLastError();
         return JARQ_ERR_ARG;
     }
-    int *status = nullptr;
+    StatusWord status(st);
+    if (!status.ptr()) return JARQ_ERR_CUDA;
     int host = 0;
-    cudaError_t e = cudaGetSymbolAddress((void **)&status, g_syrk_status);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_syrk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
+    cudaError_t e = cudaFuncSetAttribute(tc_syrk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e == cudaSuccess) e = status.clear();
     if (e == cudaSuccess) {
         const int nt = (d + 255) / 256, ntiles = nt * (nt + 1) / 2;
-        SyrkArgs args{H, scale, d, n, nt, ntiles};
+        SyrkArgs args{H, status.ptr(), scale, d, n, nt, ntiles};
         ProfScope ps("syrk", st);
         tc_syrk_kernel<<<2 * std::min(ntiles, num_sms() / 2), kThreads, kSmem, st>>>(map, args);
         e = cudaGetLastError();
         ps.done();
         count_launches(1);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&host, status, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = status.read(&host);
     prof_collect();
     if (e != cudaSuccess) {
         (void)cudaGetLastError();

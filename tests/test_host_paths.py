@@ -123,3 +123,12 @@ def test_overlapping_writeback_calls_have_a_status_word_each(dev):
     for name, call in calls.items():
         words = _overlapped(dev, call)
         assert words["first"] != words["second"], name
+
+
+def test_overlapping_hessian_calls_have_a_status_word_each(dev):
+    """A call that starts while another one runs must not clear the word in
+    which that one's kernel reports a wait that gave up."""
+    X, H = dev.buf(2 * 64 * 64), dev.buf(4 * 64 * 64)
+    words = _overlapped(dev, lambda s: dev.lib.jarq_accumulate_hessian(X, 64, 64, ctypes.c_float(1), H,
+                                                                       ctypes.c_void_p(s)))
+    assert words["first"] != words["second"]
