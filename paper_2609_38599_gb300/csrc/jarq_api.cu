@@ -341,7 +341,9 @@ jarq_status project_by(jarq_hessian *h, const float *M, int p, float *out_hi, fl
     const int d = h->din, g = h->g;
     if (!h->qdig) {
         CK(dalloc(&h->qdig, (size_t)6 * h->d_pad * h->d_pad));
-        CK(cudaMemset(h->qdig, 0, (size_t)6 * h->d_pad * h->d_pad * 2));
+        // on the call's stream: one that does not block is not ordered with
+        // the default stream, whose fill could land on digits already written
+        if (h->d_pad != d) CK(cudaMemsetAsync(h->qdig, 0, (size_t)6 * h->d_pad * h->d_pad * 2, st));
         CK(dalloc(&h->qexp, (size_t)h->G * h->G));
         CK(make_tmap_bf16(&h->mapQ, h->qdig, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32));
     }

@@ -132,3 +132,26 @@ def test_overlapping_hessian_calls_have_a_status_word_each(dev):
     words = _overlapped(dev, lambda s: dev.lib.jarq_accumulate_hessian(X, 64, 64, ctypes.c_float(1), H,
                                                                        ctypes.c_void_p(s)))
     assert words["first"] != words["second"]
+
+
+def _mu_handle(dev, din=192, dout=40, g=64):
+    """A handle whose padding (din no multiple of 128) has to be zeroed, a
+    layer, K and XX."""
+    rc, h = dev.prepare(din, g)
+    assert rc == 0
+    return h, dev.layer(din, dout, g), dout, dev.buf(4 * din * din), dev.buf(4 * din * din)
+
+
+def test_a_call_works_on_its_own_stream_only(dev):
+    """Every call of a handle, from its first on: each copy, fill and launch on
+    the caller's stream.  One on the default stream is not ordered with a
+    non-blocking stream's."""
+    h, lay, dout, K, XX = _mu_handle(dev)
+    st, F = ctypes.c_void_p(STREAM), dev.buf(8 * dout)
+    assert dev.refine(h, lay, dout) == 0 and dev.refine_mu(h, lay, dout, K, XX) == 0
+    assert dev.lib.jarq_objective(h, *lay, dout, 3, F, st) == 0
+    assert dev.lib.jarq_multicode_probe(h, *lay, dout, 3, 1, None, None, None, None, None, st) == 0
+    for method in range(3):
+        assert dev.lib.jarq_fit_scales(h, *lay, dout, 3, method, 2, F, F, st) == 0
+    others = [op for op in dev.log() if op[0] != "attribute" and op[1] != str(STREAM)]
+    assert not others
