@@ -340,12 +340,28 @@ jarq_status project_by(jarq_hessian *h, const float *M, int p, float *out_hi, fl
     Workspace &w = h->ws;
     const int d = h->din, g = h->g;
     if (!h->qdig) {
-        CK(dalloc(&h->qdig, (size_t)6 * h->d_pad * h->d_pad));
+        // the handle takes the planes only when all that goes with them is
+        // there: a call after a failed one starts again from here
+        Arena m;
+        __nv_bfloat16 *dig;
+        int *expo;
+        const size_t pd = (size_t)h->d_pad * h->d_pad;
+        auto layout = [&] {
+            m.take(dig, 6 * pd);
+            m.take(expo, (size_t)h->G * h->G);
+        };
+        layout();
+        CK(dalloc(&m.base, m.used));
+        m.used = 0;
+        layout();
         // on the call's stream: one that does not block is not ordered with
         // the default stream, whose fill could land on digits already written
-        if (h->d_pad != d) CK(cudaMemsetAsync(h->qdig, 0, (size_t)6 * h->d_pad * h->d_pad * 2, st));
-        CK(dalloc(&h->qexp, (size_t)h->G * h->G));
-        CK(make_tmap_bf16(&h->mapQ, h->qdig, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32));
+        cudaError_t e = h->d_pad != d ? cudaMemsetAsync(dig, 0, 6 * pd * 2, st) : cudaSuccess;
+        if (e == cudaSuccess) e = make_tmap_bf16(&h->mapQ, dig, (uint64_t)6 * h->d_pad, h->d_pad, 64, 32);
+        if (e != cudaSuccess) cudaFree(m.base);
+        CK(e);
+        h->qdig = dig;
+        h->qexp = expo;
     }
     // the digit kernels read M in 16-byte vectors: a device M that is not
     // 16-byte aligned is staged like host memory
@@ -439,7 +455,6 @@ void jarq_hessian_destroy(jarq_hessian *h) {
     free_ws(h->ws);
     cudaFree(h->mem);
     cudaFree(h->qdig);
-    cudaFree(h->qexp);
     cudaFree(h->qstage);
     cudaFreeHost(h->hstatus);
     (void)cudaGetLastError();

@@ -163,8 +163,8 @@ struct jarq_hessian {
     CUtensorMap mapHt;            // tensor map of Htdig, 64 x 64 boxes
     // mu-target (allocated on first use): digits of K or XX, base 2^8, six
     // planes, with a symmetric block-exponent map; staging for host K / XX
-    __nv_bfloat16 *qdig = nullptr;     // [6][d_pad][d_pad]
-    int *qexp = nullptr;               // [G][G]
+    __nv_bfloat16 *qdig = nullptr;     // [6][d_pad][d_pad], the allocation's start
+    int *qexp = nullptr;               // [G][G], in qdig's allocation
     float *qstage = nullptr;           // [d][d]
     CUtensorMap mapQ;                  // tensor map of qdig, 64 x 32 boxes
     int *dstatus = nullptr;       // device status word

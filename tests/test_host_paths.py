@@ -155,3 +155,26 @@ def test_a_call_works_on_its_own_stream_only(dev):
         assert dev.lib.jarq_fit_scales(h, *lay, dout, 3, method, 2, F, F, st) == 0
     others = [op for op in dev.log() if op[0] != "attribute" and op[1] != str(STREAM)]
     assert not others
+
+
+def test_a_corrected_target_call_after_a_failed_allocation(dev):
+    """Each allocation of a handle's first corrected-target call fails once;
+    the call says so, and the next one has all buffers and tensor maps."""
+    lib, n = dev.lib, 1
+    while True:
+        h, lay, dout, K, XX = _mu_handle(dev)
+        K1 = ctypes.c_void_p(dev.buf(4 * 192 * 192 + 16).value + 4)     # misaligned: staged
+        lib.fake_fail_malloc(n)
+        rc = dev.refine_mu(h, lay, dout, K1, XX)
+        lib.fake_fail_malloc(0)
+        if rc == 0:
+            break
+        assert rc == 6, n                           # out of memory
+        lib.fake_watch(b"12slice_kernel", 1)        # the block exponents
+        lib.fake_watch(b"tc_proj_kernel", 1)        # the base of the digits' tensor map
+        start = len(dev.log())
+        assert dev.refine_mu(h, lay, dout, K1, XX) == 0
+        seen = [op[2].split()[1] for op in dev.log()[start:] if len(op) > 2 and op[0] == "launch" and " " in op[2]]
+        assert len(seen) == 5 and "0" not in seen, (n, seen)       # two slicings, three projections
+        n += 1
+    assert n > 3
