@@ -23,6 +23,7 @@ enum : int {
 };
 
 constexpr int kMaxGroups = 128;    // largest supported G for the scale solve
+constexpr int kMaxGroupSize = 128; // the larger of the two group sizes
 constexpr int kMaxSplit = 16;      // largest split-K factor of the phase product
 constexpr int kMaxBlock = 4;       // groups of one block of the sweep at most
 
@@ -277,7 +278,9 @@ cudaError_t launch_init_rows(int *active, int *iters, int *accepted, int *ridge,
 // Multiprocessor count of the current device (cached per device ordinal).
 int num_sms();
 
-// Enable `bytes` of dynamic shared memory for `func` on the current device.
+// Enable `bytes` of dynamic shared memory for `func` on the current device:
+// the most that any call of it needs, since the limit is the process's and a
+// smaller one, set by another thread, would refuse a launch on its way.
 // The attribute is per device and a process may drive several devices, so
 // `done` is a bit mask over device ordinals; ordinals of 64 and above set
 // the attribute on every call.

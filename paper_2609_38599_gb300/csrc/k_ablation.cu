@@ -331,9 +331,10 @@ __global__ void __launch_bounds__(32 * kProbeWarps) probe_kernel(ProbeArgs a) {
 
 cudaError_t launch_own_rhs(const float *Hs, const float *W, const uint8_t *Q, const int32_t *Z,
                            double *own, int p, int d, int g, cudaStream_t s) {
-    const size_t smem = (size_t)g * (g + 1) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(own_rhs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    auto bytes = [](int n) { return n * (n + 1) * (int)sizeof(float); };
+    const size_t smem = (size_t)bytes(g);
+    static std::atomic<unsigned long long> attr_done{0};
+    const cudaError_t e = set_max_dynamic_smem((const void *)own_rhs_kernel, bytes(kMaxGroupSize), attr_done);
     if (e != cudaSuccess) return e;
     own_rhs_kernel<<<dim3((p + 31) / 32, d / g), 256, smem, s>>>(Hs, W, Q, Z, own, p, d, g);
     return cudaGetLastError();
@@ -354,12 +355,14 @@ cudaError_t launch_probe(const float *Phi, const float *Plo, const float *t_hi, 
                          const int32_t *Z, uint8_t *q_out, int32_t *moves, int32_t *accepted,
                          int32_t *changed, double *dF, int p, int p_pad, int d, int g, int i,
                          int nsplit, int qmax, float eps, cudaStream_t s) {
-    const size_t ld = (size_t)g + 1;
-    const size_t fl = ((size_t)g * ld + 1) & ~(size_t)1;
-    const size_t smem = (size_t)g * ld * sizeof(double) + fl * sizeof(float) +
-                        (size_t)kProbeWarps * 2 * g * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    auto bytes = [](int n) {
+        const size_t ld = (size_t)n + 1, fl = (n * ld + 1) & ~(size_t)1;
+        return n * ld * sizeof(double) + fl * sizeof(float) + (size_t)kProbeWarps * 2 * n * sizeof(double);
+    };
+    const size_t smem = bytes(g);
+    static std::atomic<unsigned long long> attr_done{0};
+    const cudaError_t e =
+        set_max_dynamic_smem((const void *)probe_kernel, (int)bytes(kMaxGroupSize), attr_done);
     if (e != cudaSuccess) return e;
     ProbeArgs a{Phi, Plo, t_hi, t_lo, Hs, L64, S, Q, Z, q_out, moves, accepted, changed, dF,
                 p, p_pad, d, g, i, nsplit, qmax, eps};

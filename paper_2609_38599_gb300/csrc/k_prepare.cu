@@ -286,9 +286,10 @@ cudaError_t launch_symmetrize(const float *H, float *Hs, __nv_bfloat16 *Hplanes,
 
 cudaError_t launch_group_factor(const float *Hs, float *Lf, double *L64, double *Rinv,
                                 float2 *RinvF, int d, int g, int *status, cudaStream_t s) {
-    const int smem = (g * (g + 1) + g) * (int)sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(group_factor_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    auto bytes = [](int n) { return (n * (n + 1) + n) * (int)sizeof(double); };
+    const int smem = bytes(g);
+    static std::atomic<unsigned long long> attr_done{0};
+    cudaError_t e = set_max_dynamic_smem((const void *)group_factor_kernel, bytes(kMaxGroupSize), attr_done);
     if (e != cudaSuccess) return e;
     group_factor_kernel<<<d / g, 256, smem, s>>>(Hs, Lf, L64, d, g, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

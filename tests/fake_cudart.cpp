@@ -44,6 +44,7 @@ State &st() {
     return *s;
 }
 thread_local Launch g_pushed;
+thread_local cudaError_t g_last = cudaSuccess;
 
 void note(const char *what, cudaStream_t s, const void *p, size_t n) {
     Hook hook;
@@ -60,7 +61,7 @@ cudaError_t launch(const void *fn, size_t smem, cudaStream_t s, void **args) {
     const std::string &name = st().kernels[fn];
     const auto lim = st().smem_limit.find(fn);
     if (smem > 48 * 1024 && (lim == st().smem_limit.end() || smem > (size_t)lim->second))
-        return cudaErrorInvalidValue;
+        return g_last = cudaErrorInvalidValue;
     st().log << "launch " << (size_t)s << ' ' << name;
     for (const auto &w : st().watched)
         if (name.find(w.first) != std::string::npos) st().log << ' ' << *(size_t *)args[w.second];
@@ -215,7 +216,11 @@ cudaError_t cudaStreamSynchronize(cudaStream_t s) {
     note("sync", s, nullptr, 0);
     return cudaSuccess;
 }
-cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+cudaError_t cudaGetLastError(void) {
+    const cudaError_t e = g_last;
+    g_last = cudaSuccess;
+    return e;
+}
 cudaError_t cudaEventCreate(cudaEvent_t *e) {
     *e = (cudaEvent_t)malloc(1);
     return cudaSuccess;

@@ -178,3 +178,31 @@ def test_a_corrected_target_call_after_a_failed_allocation(dev):
         assert len(seen) == 5 and "0" not in seen, (n, seen)       # two slicings, three projections
         n += 1
     assert n > 3
+
+
+@pytest.mark.parametrize("call", ["prepare", "independent fit", "probe"])
+def test_the_other_group_size_at_the_same_time(dev, call):
+    """A kernel's limit of dynamic shared memory belongs to the process: a call
+    with groups of 64 that runs while one with 128 is on its way must not lower
+    it under a launch that needs more."""
+    lib, dout, state = dev.lib, 40, {"busy": False}
+    handle = {g: dev.prepare(256, g)[1] for g in (64, 128)}
+    layer = {g: dev.layer(256, dout, g) for g in (64, 128)}
+
+    def run(g, stream):
+        st = ctypes.c_void_p(stream)
+        if call == "prepare":
+            return dev.prepare(256, g, stream)[0]
+        if call == "probe":
+            return lib.jarq_multicode_probe(handle[g], *layer[g], dout, 3, 1, None, None, None, None, None, st)
+        return lib.jarq_fit_scales(handle[g], *layer[g], dout, 3, 1, 1, None, None, st)
+
+    def note(what, p, n):
+        if what == "attribute" and not state["busy"]:
+            state["busy"] = True
+            assert run(64, STREAM + 1) == 0
+            state["busy"] = False
+
+    assert run(128, STREAM) == 0        # limits that are set once are set
+    dev.hook(note)
+    assert run(128, STREAM) == 0
