@@ -556,7 +556,7 @@ jarq_status jarq_objective(jarq_hessian *h, const float *W, const float *S, cons
     if (rc != JARQ_OK) return rc;
     Workspace &w = h->ws;
     CK(cudaMemsetAsync(h->dstatus, 0, sizeof(int), st));
-    RUN("hr_full", 1, launch_tc_hr_full(w.mapR, h->mapH128, w.Hr, h->din, dout, w.p_pad, h->din, h->d_pad, h->dstatus, st));
+    RUN("hr_full", 1, launch_tc_hr_full(w.mapR, h->mapH128, w.Hr, dout, w.p_pad, h->din, h->d_pad, h->dstatus, st));
     RUN("grad", 1, launch_grad(w.r, w.Hr, w.L_final, dout, h->din, st));
     CK(cudaMemcpyAsync(F_per_row, w.L_final, (size_t)dout * sizeof(double), cudaMemcpyDefault, st));
     int sb = 0;
@@ -577,7 +577,7 @@ jarq_status jarq_residual_product(jarq_hessian *h, const float *W, const float *
     if (rc != JARQ_OK) return rc;
     Workspace &w = h->ws;
     CK(cudaMemsetAsync(h->dstatus, 0, sizeof(int), st));
-    RUN("hr_full", 1, launch_tc_hr_full(w.mapR, h->mapH128, w.Hr, h->din, dout, w.p_pad, h->din, h->d_pad, h->dstatus, st));
+    RUN("hr_full", 1, launch_tc_hr_full(w.mapR, h->mapH128, w.Hr, dout, w.p_pad, h->din, h->d_pad, h->dstatus, st));
     CK(cudaMemcpyAsync(HR, w.Hr, (size_t)dout * h->din * sizeof(float), cudaMemcpyDefault, st));
     int sb = 0;
     CK(read_status(h, st, &sb));

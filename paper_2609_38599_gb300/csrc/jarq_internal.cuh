@@ -199,9 +199,8 @@ cudaError_t launch_validate(const uint8_t *Q, const int32_t *Z, int p, int d, in
                             int *status, cudaStream_t s);
 cudaError_t launch_residual(const float *W, const float *S, const uint8_t *Q, const int32_t *Z,
                             ResidualView rv, int p, int g, cudaStream_t s);
-cudaError_t launch_tc_hr_full(const CUtensorMap &mapA, const CUtensorMap &mapB, float *out,
-                              int ldo, int p, int p_pad, int d, int d_pad, int *status,
-                              cudaStream_t s);
+cudaError_t launch_tc_hr_full(const CUtensorMap &mapA, const CUtensorMap &mapB, float *out, int p,
+                              int p_pad, int d, int d_pad, int *status, cudaStream_t s);
 cudaError_t launch_grad(const float *r, const float *Hr, double *F, int p, int d, cudaStream_t s);
 cudaError_t launch_slices(const float *Hs, int *expo, __nv_bfloat16 *dig8, __half *dig10, int d,
                           int d_pad, int g, cudaStream_t s);

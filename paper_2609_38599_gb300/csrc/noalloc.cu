@@ -120,7 +120,7 @@ extern "C" jarq_status jarq_objective_noalloc(jarq_hessian *h, const float *W, c
     if (e == cudaSuccess) e = cudaMemsetAsync(cplane, 0, (size_t)p_pad * d_pad * 2, st);
     if (e == cudaSuccess) e = launch_residual(W, S, Q, Z, rv, dout, g, st);
     if (e == cudaSuccess)
-        e = launch_tc_hr_full(mapR, h->mapH128, Hr, d, dout, p_pad, d, d_pad, h->dstatus, st);
+        e = launch_tc_hr_full(mapR, h->mapH128, Hr, dout, p_pad, d, d_pad, h->dstatus, st);
     if (e == cudaSuccess) e = launch_grad(r, Hr, F_per_row, dout, d, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->hstatus, h->dstatus, sizeof(int), cudaMemcpyDeviceToHost, st);
