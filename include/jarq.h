@@ -342,13 +342,22 @@ long long jarq_launch_count(void);
 
 /* Test hook for the bounded device waits (no counterpart in the paper).
  * Every wait of the library's kernels on a barrier gives up after a fixed
- * number of polls; the kernel then records the timeout, finishes its copies
- * in flight and returns, and the call reports JARQ_ERR_TIMEOUT.  This call
+ * number of polls; the kernel then waits, again with a limit, for its copies
+ * and tensor-core products in flight, records the timeout and returns, and the
+ * call reports JARQ_ERR_TIMEOUT.  This call
  * launches one thread that waits on a barrier nothing completes, with a
  * short poll limit, and returns the status the same path produces:
  * JARQ_ERR_TIMEOUT when it works.  The CUDA context stays usable.  `stream`
  * as for every entry point; returns after the stream work has finished. */
 jarq_status jarq_selftest_wait_timeout(void *stream);
+
+/* The same for the tensor-core kernels: one of them ("target", "gram",
+ * "proj", "ptilde", "hr_full" or "syrk") on a small layer of its own, with a
+ * short poll limit and its issuing warp told to stop after the first unit of
+ * work, so that the waits of the other warps run out while copies lie
+ * unused in shared memory.  Returns what that launch reports:
+ * JARQ_ERR_TIMEOUT when it works; JARQ_ERR_ARG for another name. */
+jarq_status jarq_selftest_stalled_kernel(const char *kernel, void *stream);
 
 #ifdef __cplusplus
 }

@@ -12,6 +12,9 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <memory>
+#include <vector>
+
 #include <new>
 
 #include "jarq_internal.cuh"
@@ -670,6 +673,69 @@ jarq_status jarq_multicode_probe(jarq_hessian *h, const float *W, const float *S
     int sb = 0;
     CK(read_status(h, st, &sb));
     return status_from_bits(sb);
+}
+
+jarq_status jarq_selftest_stalled_kernel(const char *kernel, void *stream) try {
+    if (!kernel) return JARQ_ERR_ARG;
+    auto is = [&](const char *name) { return !strcmp(kernel, name); };
+    // a small layer refined and scored first, so that every buffer holds what
+    // its kernel reads
+    constexpr int d = 512, g = 128, G = d / g, p = 300, bits = 3, n = 1200;
+    cudaStream_t st = (cudaStream_t)stream;
+    std::vector<float> H((size_t)d * d), W((size_t)p * d), S((size_t)p * G, 0.1f);
+    std::vector<uint8_t> Q((size_t)p * d);
+    std::vector<int32_t> Z((size_t)p * G, 3);
+    std::vector<double> F(p);
+    for (int i = 0; i < d; ++i) H[(size_t)i * d + i] = 1.f;
+    for (size_t i = 0; i < W.size(); ++i) {
+        Q[i] = (uint8_t)(i * 5 % 8);
+        W[i] = 0.1f * (float)((int)Q[i] - 3) + 0.01f * (float)(i % 7);
+    }
+    jarq_hessian *h = nullptr;
+    jarq_status rc = jarq_prepare_hessian(H.data(), d, g, 0.f, &h, stream);
+    if (rc != JARQ_OK) return rc;
+    std::unique_ptr<jarq_hessian, void (*)(jarq_hessian *)> owner(h, jarq_hessian_destroy);
+    rc = jarq_refine_layer(h, W.data(), S.data(), Q.data(), Z.data(), p, bits, nullptr, nullptr, stream);
+    if (rc == JARQ_OK)
+        rc = jarq_objective(h, W.data(), S.data(), Q.data(), Z.data(), p, bits, F.data(), stream);
+    if (rc != JARQ_OK) return rc;
+    Workspace &w = h->ws;
+    CK(cudaMemsetAsync(h->dstatus, 0, sizeof(int), st));
+    char *scratch = nullptr;
+    if (is("target")) {
+        CK(launch_tc_target(w.mapC, h->mapHt, w.t_hi, w.t_lo, w.sS, h->expoT, nullptr, p, w.p_pad, h->d_pad, g, G,
+                            0, sweep_block(g), 0, 1, (1 << bits) - 1, h->dstatus, st, false, true));
+    } else if (is("gram")) {
+        CK(launch_tc_gram(w.mapC, h->mapD10, w.sQ, w.sZ, h->expo, nullptr, w.gram, p, w.p_pad, d, h->d_pad, g,
+                          bits, h->dstatus, st, false, true));
+    } else if (is("proj")) {
+        CK(launch_tc_proj(w.mapWd, h->mapD8, w.Phi, w.Plo, w.wexp, h->expo, p, w.p_pad, d, h->d_pad, g, h->dstatus,
+                          st, true));
+    } else if (is("ptilde")) {
+        CK(launch_ptilde(w.mapPd, h->mapRi, w.Phi, w.Plo, w.wdig, w.wexp, h->rexp, w.Pt_hi, w.Pt_lo, p, w.p_pad, d,
+                         h->d_pad, g, h->dstatus, st, true));
+    } else if (is("hr_full")) {
+        CK(launch_tc_hr_full(w.mapR, h->mapH128, w.Hr, p, w.p_pad, d, h->d_pad, h->dstatus, st, true));
+    } else if (is("syrk")) {
+        const size_t hb = (size_t)d * d * sizeof(float), xb = (size_t)n * d * 2;
+        CUtensorMap map;
+        CK(dalloc(&scratch, hb + xb));
+        cudaError_t e = cudaMemsetAsync(scratch, 0, hb + xb, st);
+        if (e == cudaSuccess) e = make_tmap_f16(&map, scratch + hb, n, d, 64);
+        if (e == cudaSuccess)
+            e = launch_tc_syrk(map, reinterpret_cast<float *>(scratch), h->dstatus, 1.f, d, n, st, true);
+        if (e != cudaSuccess) cudaFree(scratch);
+        CK(e);
+    } else {
+        return JARQ_ERR_ARG;
+    }
+    int sb = 0;
+    const cudaError_t e = read_status(h, st, &sb);
+    cudaFree(scratch);
+    CK(e);
+    return status_from_bits(sb);
+} catch (const std::bad_alloc &) {
+    return JARQ_ERR_NOMEM;
 }
 
 jarq_status jarq_refine_layer_mu(jarq_hessian *h, const float *W, float *S, uint8_t *Q,

@@ -176,6 +176,8 @@ struct jarq_hessian {
 namespace jarq {
 
 // ---- launchers (each returns the cudaError_t of its launch) ----
+// `stalled`: the self-test's form of the kernel, whose MMA issuer stops early
+// and whose waits give up after milliseconds
 cudaError_t launch_symmetrize(const float *H, float *Hs, __nv_bfloat16 *Hplanes, int d, int d_pad,
                               float nu2, cudaStream_t s);
 cudaError_t launch_group_factor(const float *Hs, float *Lf, double *L64, double *Rinv,
@@ -200,14 +202,17 @@ cudaError_t launch_validate(const uint8_t *Q, const int32_t *Z, int p, int d, in
 cudaError_t launch_residual(const float *W, const float *S, const uint8_t *Q, const int32_t *Z,
                             ResidualView rv, int p, int g, cudaStream_t s);
 cudaError_t launch_tc_hr_full(const CUtensorMap &mapA, const CUtensorMap &mapB, float *out, int p,
-                              int p_pad, int d, int d_pad, int *status, cudaStream_t s);
+                              int p_pad, int d, int d_pad, int *status, cudaStream_t s,
+                              bool stalled = false);
+cudaError_t launch_tc_syrk(const CUtensorMap &mapX, float *H, int *status, float scale, int d, int n,
+                           cudaStream_t s, bool stalled = false);
 cudaError_t launch_grad(const float *r, const float *Hr, double *F, int p, int d, cudaStream_t s);
 cudaError_t launch_slices(const float *Hs, int *expo, __nv_bfloat16 *dig8, __half *dig10, int d,
                           int d_pad, int g, cudaStream_t s);
 cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, const uint8_t *Q,
                            const int32_t *Z, const int *expo, const int *active, float2 *gram,
                            int p, int p_pad, int d, int d_pad, int g, int bits, int *status,
-                           cudaStream_t s, bool pdl = false);
+                           cudaStream_t s, bool pdl = false, bool stalled = false);
 cudaError_t launch_slices8(const float *M, int *expo, __nv_bfloat16 *dig8, int d, int d_pad,
                            int g, cudaStream_t s);
 cudaError_t launch_mu_combine(float *Phi, float *Plo, const float *Khi, const float *Klo,
@@ -217,7 +222,7 @@ cudaError_t launch_slice_rows(const float *W, __nv_bfloat16 *planes, int *wexp, 
                               int d_pad, int p_pad, int g, cudaStream_t s);
 cudaError_t launch_tc_proj(const CUtensorMap &mapW, const CUtensorMap &mapH, float *Phi,
                            float *Plo, const int *wexp, const int *hexp, int p, int p_pad, int d,
-                           int d_pad, int g, int *status, cudaStream_t s);
+                           int d_pad, int g, int *status, cudaStream_t s, bool stalled = false);
 cudaError_t launch_whw(const float *W, const float *Phi, const float *Plo, double *out, int p,
                        int d, cudaStream_t s);
 cudaError_t launch_rhs(const uint8_t *Q, const int32_t *Z, const float *Phi, const float *Plo,
@@ -239,14 +244,14 @@ cudaError_t launch_slice_rinv(const double *Rinv, __nv_bfloat16 *rdig, int *rexp
 cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, const float *Phi,
                           const float *Plo, __nv_bfloat16 *pdig, int *pexp, const int *rexp,
                           float *out_hi, float *out_lo, int p, int p_pad, int d, int d_pad, int g,
-                          int *status, cudaStream_t s);
+                          int *status, cudaStream_t s, bool stalled = false);
 int target_splits(int p_pad, int g, int G, int nb);
 cudaError_t launch_wait_timeout(int *status, uint32_t polls, cudaStream_t s);
 cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, float *out_hi,
                              float *out_lo, const float *S, const int *expoT, const int *active,
                              int p, int p_pad, int d_pad, int g, int G, int i0, int nb,
                              int nb_prev, int nsplit, int qmax, int *status, cudaStream_t s,
-                             bool pdl);
+                             bool pdl, bool stalled = false);
 
 // Launch; with `pdl` under programmatic stream serialization: the kernel may
 // start while the previous kernel in the stream finishes, and must call

@@ -436,8 +436,8 @@ __global__ void __launch_bounds__(32 * (kMaxWarps + 1), 1) babai_kernel(BabaiArg
     __syncthreads();
     if (*abort_f && threadIdx.x == 0) {
         for (int n = 0; n < a.nb; ++n) {
-            (void)tc::mbar_wait(full(n % kFactorSlots), (n / kFactorSlots) & 1);
-            for (int t = 0; t < a.nb - 1 - n; ++t) (void)tc::mbar_wait(pfull(t), n & 1);
+            (void)tc::mbar_wait<tc::kCloseIters>(full(n % kFactorSlots), (n / kFactorSlots) & 1);
+            for (int t = 0; t < a.nb - 1 - n; ++t) (void)tc::mbar_wait<tc::kCloseIters>(pfull(t), n & 1);
         }
         atomicOr(a.status, ST_TIMEOUT);
     }

@@ -53,7 +53,7 @@ constexpr int kTileA = 2 * kBox;           // 128 row features
 constexpr int kTileB = 2 * kBox;           // 128 of the 256 column features
 constexpr int kStage = kTileA + kTileB;
 constexpr int kStages = 5;
-constexpr int kBars = 2 * kStages + 4;     // full, empty, afull[2], aempty[2]
+constexpr int kBars = 2 * kStages + 5;     // full, empty, afull[2], aempty[2], closing
 constexpr int kDrainWarps = 8;
 constexpr int kTld = 33;                   // row pitch (floats) of a staged 32 x 32 part
 constexpr int kPart = 32 * kTld * 4;
@@ -121,8 +121,11 @@ struct TileOrder {
     }
 };
 
+// kStalled: for the self-test, the issuer stops after one accumulator.
+template <bool kStalled>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_syrk_kernel(const __grid_constant__ CUtensorMap mapX, SyrkArgs a) {
+    constexpr uint32_t kPolls = tc::wait_polls(kStalled);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     float *parts = (float *)(smem + kStages * kStage);
@@ -139,6 +142,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     auto empty = [&](int s) { return tc::smem_u32(bars + kStages + s); };
     auto afull = [&](int b) { return tc::smem_u32(bars + 2 * kStages + b); };
     auto aempty = [&](int b) { return tc::smem_u32(bars + 2 * kStages + 2 + b); };
+    const uint32_t closing = tc::smem_u32(bars + 2 * kStages + 4);
     auto tileA = [&](int s) { return tc::smem_u32(smem + s * kStage); };
     auto tileB = [&](int s) { return tc::smem_u32(smem + s * kStage + kTileA); };
 
@@ -151,6 +155,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tc::mbar_init(afull(b), 1);
             tc::mbar_init(aempty(b), 2 * kDrainWarps);   // the even CTA's: both drains
         }
+        tc::mbar_init(closing, 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -176,7 +181,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             order.at(it, ri, cj);
             const int ra = ri * 256 + 128 * rank, cb = cj * 256 + 128 * rank;
             for (int c = 0; c < nchunks; ++c) {
-                ok = tc::mbar_wait(empty(s), ph);
+                ok = tc::mbar_wait<kPolls>(empty(s), ph);
                 if (!ok) break;
                 if (tc::elect_one()) {
                     if (rank == 0) tc::mbar_expect_tx(full(s), 2 * (ri == cj ? kTileB : kStage));
@@ -198,8 +203,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         // do not leave before the MMAs have consumed the stages filled here:
         // no copy or commit is in flight afterwards
         for (int n = max(0, filled - kStages); n < filled && ok; ++n)
-            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
-        if (!ok) *abort_flag = 1;
+            ok = tc::mbar_wait<kPolls>(empty(n % kStages), (n / kStages) & 1);
+        if (!ok) {
+            *abort_flag = 1;
+            tc::abandon_ring(full(0), kStages, filled, rank == 0);
+        }
     } else if (warp == 1) {
         // ---------------- MMA issuer of the pair: an accumulator per 512 tokens
         if (rank == 0) {
@@ -208,14 +216,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const uint64_t a0 = sdesc_mn_sw128(tileA(0)), b0 = sdesc_mn_sw128(tileB(0));
             int s = 0, ph = 0, pc = 0;
             for (int it = pair; it < a.ntiles && ok; it += npairs) {
+                if (kStalled && pc > 0) break;
                 int ri, cj;
                 order.at(it, ri, cj);
                 const uint64_t ad0 = ri == cj ? b0 : a0;
-                for (int c0 = 0; c0 < nchunks && ok; c0 += kChunksPerDrain, ++pc) {
+                for (int c0 = 0; c0 < nchunks && ok && !(kStalled && pc > 0); c0 += kChunksPerDrain, ++pc) {
                     const int b = pc & 1, c1 = min(nchunks, c0 + kChunksPerDrain);
-                    ok = tc::mbar_wait(aempty(b), ((pc >> 1) & 1) ^ 1);
+                    ok = tc::mbar_wait<kPolls>(aempty(b), ((pc >> 1) & 1) ^ 1);
                     for (int c = c0; c < c1 && ok; ++c) {
-                        ok = tc::mbar_wait(full(s), ph);
+                        ok = tc::mbar_wait<kPolls>(full(s), ph);
                         if (!ok) break;
                         tc::tc_fence_after();
                         if (tc::elect_one()) {
@@ -236,7 +245,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     }
                 }
             }
-            if (!ok) *abort_flag = 1;
+            if (!tc::mma_done_pair<kPolls>(closing, tc::elect_one()) || !ok) *abort_flag = 1;
         }
     } else {
         // ---------------- drain: TMEM -> float32 registers -> H
@@ -255,7 +264,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const int row0 = ri * 256 + 128 * rank + 32 * q, colh = cj * 256 + half * 128;
             for (int per = 0; per < nper; ++per, ++pc) {
                 const int b = pc & 1;
-                ok = __all_sync(0xffffffffu, tc::mbar_wait(afull(b), (pc >> 1) & 1));
+                ok = __all_sync(0xffffffffu, tc::mbar_wait<kPolls>(afull(b), (pc >> 1) & 1));
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + b * 256 + half * 128;
@@ -349,6 +358,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 }
 
 }  // namespace
+
+cudaError_t launch_tc_syrk(const CUtensorMap &mapX, float *H, int *status, float scale, int d, int n,
+                           cudaStream_t s, bool stalled) {
+    const int nt = (d + 255) / 256, ntiles = nt * (nt + 1) / 2;
+    const SyrkArgs args{H, status, scale, d, n, nt, ntiles};
+    auto run = [&](auto *kernel, std::atomic<unsigned long long> &done) {
+        const cudaError_t e = set_max_dynamic_smem((const void *)kernel, kSmem, done);
+        if (e != cudaSuccess) return e;
+        return launch_k(kernel, dim3(2 * std::min(ntiles, num_sms() / 2)), dim3(kThreads), (size_t)kSmem, s, false,
+                        mapX, args);
+    };
+    static std::atomic<unsigned long long> done[2];
+    return stalled ? run(tc_syrk_kernel<true>, done[1]) : run(tc_syrk_kernel<false>, done[0]);
+}
+
 }  // namespace jarq
 
 using namespace jarq;
@@ -368,14 +392,10 @@ extern "C" jarq_status jarq_accumulate_hessian(const void *X, int n, int d, floa
     StatusWord status(st);
     if (!status.ptr()) return JARQ_ERR_CUDA;
     int host = 0;
-    cudaError_t e = cudaFuncSetAttribute(tc_syrk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (e == cudaSuccess) e = status.clear();
+    cudaError_t e = status.clear();
     if (e == cudaSuccess) {
-        const int nt = (d + 255) / 256, ntiles = nt * (nt + 1) / 2;
-        SyrkArgs args{H, status.ptr(), scale, d, n, nt, ntiles};
         ProfScope ps("syrk", st);
-        tc_syrk_kernel<<<2 * std::min(ntiles, num_sms() / 2), kThreads, kSmem, st>>>(map, args);
-        e = cudaGetLastError();
+        e = launch_tc_syrk(map, H, status.ptr(), scale, d, n, st);
         ps.done();
         count_launches(1);
     }

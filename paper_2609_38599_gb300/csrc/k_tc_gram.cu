@@ -109,15 +109,17 @@ struct GramUnit {
 //   wider         |D_t| < 2^24 converted by cvt, 64-bit integer dots
 enum { kWideDots = -1, kIntDots = 0 };    // or the number of terms of a float32 sum
 
-template <int kMode>
+// kStalled: for the self-test, the issuer stops after one unit.
+template <int kMode, bool kStalled>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_gram_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapS,
                    GramArgs a) {
+    constexpr uint32_t kPolls = tc::wait_polls(kStalled);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     long long *part = (long long *)(smem + kStages * kStage);   // [kSlots][4 warps][2][128]
     uint64_t *bars = (uint64_t *)(smem + kStages * kStage + kPartBytes);
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 4 + 2 * kSlots);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 5 + 2 * kSlots);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)tc::cluster_rank();
@@ -150,6 +152,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     auto aempty = [&](int b) { return tc::smem_u32(bars + 2 * kStages + 2 + b); };
     auto sfull = [&](int s) { return tc::smem_u32(bars + 2 * kStages + 4 + s); };
     auto sfree = [&](int s) { return tc::smem_u32(bars + 2 * kStages + 4 + kSlots + s); };
+    const uint32_t closing = tc::smem_u32(bars + 2 * kStages + 4 + 2 * kSlots);
     auto tileA = [&](int s) { return tc::smem_u32(smem + s * kStage); };
     auto tileB = [&](int s, int t) { return tc::smem_u32(smem + s * kStage + kTileA + t * kTileB); };
 
@@ -166,6 +169,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tc::mbar_init(afull(b), 1);
             tc::mbar_init(aempty(b), 2 * kDrainWarps);   // the even CTA's: both drains
         }
+        tc::mbar_init(closing, 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -205,7 +209,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const int nunits = item(it, jp, un);
             for (int u = 0; u < nunits && ok; ++u, un.next()) {
                 for (int kc = 0; kc < nkc; ++kc) {
-                    ok = tc::mbar_wait(empty(s), ph);
+                    ok = tc::mbar_wait<kPolls>(empty(s), ph);
                     if (!ok) break;
                     if (tc::elect_one()) {
                         if (rank == 0) tc::mbar_expect_tx(full(s), 2 * kStage);
@@ -229,8 +233,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         // do not leave before the MMAs have consumed the stages filled here:
         // no copy or commit is in flight afterwards
         for (int n = max(0, nchunks - kStages); n < nchunks && ok; ++n)
-            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
-        if (!ok) *abort_flag = 1;
+            ok = tc::mbar_wait<kPolls>(empty(n % kStages), (n / kStages) & 1);
+        if (!ok) {
+            *abort_flag = 1;
+            tc::abandon_ring(full(0), kStages, nchunks, rank == 0);
+        }
     } else if (warp == 1) {
         // ---------------- MMA issuer of the pair
         if (rank == 0) {
@@ -240,6 +247,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             GramUnit un;
             int jp, total = 0;
             for (int it = blockIdx.x / 2; it < a.nitems; it += npairs) total += item(it, jp, un);
+            if (kStalled) total = min(total, 1);
             for (int u = 0; u < total && ok; ++u) {
                 const int b = u & 1;
                 int s1 = s + 1, ph1 = ph;
@@ -247,9 +255,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     s1 = 0;
                     ph1 ^= 1;
                 }
-                ok = tc::mbar_wait(full(s), ph);
-                if (nkc == 2) ok = tc::mbar_wait(full(s1), ph1) && ok;
-                ok = tc::mbar_wait(aempty(b), ((u >> 1) & 1) ^ 1) && ok;
+                ok = tc::mbar_wait<kPolls>(full(s), ph);
+                if (nkc == 2) ok = tc::mbar_wait<kPolls>(full(s1), ph1) && ok;
+                ok = tc::mbar_wait<kPolls>(aempty(b), ((u >> 1) & 1) ^ 1) && ok;
                 if (!ok) break;
                 tc::tc_fence_after();
                 if (tc::elect_one()) {
@@ -275,7 +283,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     ph ^= 1;
                 }
             }
-            if (!ok) *abort_flag = 1;
+            if (!tc::mma_done_pair<kPolls>(closing, tc::elect_one()) || !ok) *abort_flag = 1;
         }
     } else if (warp < 2 + kDrainWarps) {
         // ---------------- epilogue: exact integer dots with the codes of group i
@@ -321,7 +329,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         cf[e] = tc::f2_add(tc::f2(__int_as_float(c[2 * e]), __int_as_float(c[2 * e + 1])), off);
                 }
                 const int b = ug & 1;
-                ok = __all_sync(0xffffffffu, tc::mbar_wait(afull(b), (ug >> 1) & 1));
+                ok = __all_sync(0xffffffffu, tc::mbar_wait<kPolls>(afull(b), (ug >> 1) & 1));
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + b * 256 + cq * 16;
@@ -399,7 +407,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     const long long hi = (long long)acc[0] * (1 << 10) + acc[1];
                     const long long lo = (long long)acc[2] * (1 << 10) + acc[3];
                     const int slot = nb % kSlots;
-                    ok = __all_sync(0xffffffffu, tc::mbar_wait(sfree(slot), ((nb / kSlots) & 1) ^ 1));
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait<kPolls>(sfree(slot), ((nb / kSlots) & 1) ^ 1));
                     if (!ok) break;
                     long long *pp = part + (size_t)((slot * 4 + cq) * 2) * 128 + rl;
                     if constexpr (kMode == kWideDots) {
@@ -427,7 +435,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const int nblk = item(it, jp, un) / nkc;
             for (int k = 0; k < nblk; ++k, ++nb) {
                 const int E = a.expo[un.gi * G + un.h], slot = nb % kSlots;
-                ok = __all_sync(0xffffffffu, tc::mbar_wait(sfull(slot), (nb / kSlots) & 1));
+                ok = __all_sync(0xffffffffu, tc::mbar_wait<kPolls>(sfull(slot), (nb / kSlots) & 1));
                 if (!ok) break;
                 const long long *pp = part + (size_t)slot * 4 * 2 * 128;
                 float2 v2[2];
@@ -654,7 +662,7 @@ cudaError_t launch_slices8(const float *M, int *expo, __nv_bfloat16 *dig8, int d
 cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, const uint8_t *Q,
                            const int32_t *Z, const int *expo, const int *active, float2 *gram,
                            int p, int p_pad, int d, int d_pad, int g, int bits, int *status,
-                           cudaStream_t s, bool pdl) {
+                           cudaStream_t s, bool pdl, bool stalled) {
     const int G = d / g;
     // ranges per (row tile pair, group pair): the fewest blocks for the busiest
     // CTA pair, each item costing about a sixth of a block beside its blocks
@@ -679,10 +687,11 @@ cudaError_t launch_tc_gram(const CUtensorMap &mapC, const CUtensorMap &mapS, con
         if (e != cudaSuccess) return e;
         return launch_k(kernel, grid, dim3(kThreads), (size_t)kSmem, s, pdl, mapC, mapS, a);
     };
-    static std::atomic<unsigned long long> done[3];
-    if (bits <= 3) return run(tc_gram_kernel<4>, done[0]);
-    if (bits <= 4) return run(tc_gram_kernel<kIntDots>, done[1]);
-    return run(tc_gram_kernel<kWideDots>, done[2]);
+    static std::atomic<unsigned long long> done[4];
+    if (stalled) return run(tc_gram_kernel<kIntDots, true>, done[3]);
+    if (bits <= 3) return run(tc_gram_kernel<4, false>, done[0]);
+    if (bits <= 4) return run(tc_gram_kernel<kIntDots, false>, done[1]);
+    return run(tc_gram_kernel<kWideDots, false>, done[2]);
 }
 
 }  // namespace jarq

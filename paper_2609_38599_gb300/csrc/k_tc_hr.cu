@@ -52,13 +52,16 @@ struct HrArgs {
     int *status;
 };
 
+// kStalled: for the self-test, the issuer stops after one chunk.
+template <bool kStalled>
 __global__ void __launch_bounds__(320, 1)
     tc_hr_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                  HrArgs a) {
+    constexpr uint32_t kPolls = tc::wait_polls(kStalled);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = (uint64_t *)(smem + kStages * kStage);
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 4);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 5);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tile order: grouped so that consecutive CTAs share column tiles within
@@ -75,6 +78,7 @@ __global__ void __launch_bounds__(320, 1)
     auto empty = [&](int s) { return tc::smem_u32(bars + kStages + s); };
     auto afull = [&](int b) { return tc::smem_u32(bars + 2 * kStages + b); };
     auto aempty = [&](int b) { return tc::smem_u32(bars + 2 * kStages + 2 + b); };
+    const uint32_t closing = tc::smem_u32(bars + 2 * kStages + 4);
     auto tileA = [&](int s, int t) { return tc::smem_u32(smem + s * kStage + t * kTile); };
     auto tileB = [&](int s, int t) { return tc::smem_u32(smem + s * kStage + (3 + t) * kTile); };
 
@@ -87,6 +91,7 @@ __global__ void __launch_bounds__(320, 1)
             tc::mbar_init(afull(b), 1);
             tc::mbar_init(aempty(b), 8);   // one arrival per drain warp
         }
+        tc::mbar_init(closing, 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -109,7 +114,7 @@ __global__ void __launch_bounds__(320, 1)
         for (int c = 0; c < nk; ++c) {
             const int s = c % kStages;
             const uint32_t ph = (c / kStages) & 1;
-            if (!tc::mbar_wait(empty(s), ph ^ 1) || *abort_flag) {
+            if (!tc::mbar_wait<kPolls>(empty(s), ph ^ 1) || *abort_flag) {
                 *abort_flag = 1;
                 break;
             }
@@ -120,19 +125,20 @@ __global__ void __launch_bounds__(320, 1)
             for (int t = 0; t < 3; ++t) tc::tma_load_2d(tileB(s, t), &mapB, full(s), c * 64, n0 + t * a.d_pad);
             issued = c + 1;
         }
-        // copies still in flight complete on their barriers before we leave
-        for (int c = issued > kStages ? issued - kStages : 0; c < issued; ++c)
-            if (!tc::mbar_wait(full(c % kStages), (c / kStages) & 1)) *abort_flag = 1;
+        // do not leave before the copies have landed
+        for (int c = issued > kStages ? issued - kStages : 0; c < issued && !*abort_flag; ++c)
+            if (!tc::mbar_wait<kPolls>(full(c % kStages), (c / kStages) & 1)) *abort_flag = 1;
+        if (*abort_flag) tc::abandon_ring(full(0), kStages, issued, true);
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
-        for (int c = 0; c < nk && !*abort_flag; ++c) {
+        for (int c = 0; c < (kStalled ? 1 : nk) && !*abort_flag; ++c) {
             const int b = c & 1, s = c % kStages;
-            if (!tc::mbar_wait(aempty(b), ((c >> 1) & 1) ^ 1)) {
+            if (!tc::mbar_wait<kPolls>(aempty(b), ((c >> 1) & 1) ^ 1)) {
                 *abort_flag = 1;
                 break;
             }
             const uint32_t acc_big = tmem + b * 256, acc_small = acc_big + 128;
-            if (!tc::mbar_wait(full(s), (c / kStages) & 1) || *abort_flag) {
+            if (!tc::mbar_wait<kPolls>(full(s), (c / kStages) & 1) || *abort_flag) {
                 *abort_flag = 1;
                 break;
             }
@@ -152,6 +158,7 @@ __global__ void __launch_bounds__(320, 1)
             tc::mma_commit(empty(s));
             tc::mma_commit(afull(b));
         }
+        if (!tc::mma_done<kPolls>(closing, true)) *abort_flag = 1;
     } else if (warp >= 2) {
         // ---------------- drain + store (decisions warp-uniform: tcgen05.ld is .aligned)
         constexpr int HB = 64;                     // columns per drain warp
@@ -163,7 +170,7 @@ __global__ void __launch_bounds__(320, 1)
         bool ok = true;
         for (int c = 0; c < nk; ++c) {
             const int b = c & 1;
-            bool w = tc::mbar_wait(afull(b), (c >> 1) & 1);
+            bool w = tc::mbar_wait<kPolls>(afull(b), (c >> 1) & 1);
             w = __shfl_sync(0xffffffffu, w && !*abort_flag, 0);
             tc::tc_fence_after();
             if (!w) {
@@ -214,13 +221,16 @@ __global__ void __launch_bounds__(320, 1)
 
 // Full product H r for all rows: out[p][d].
 cudaError_t launch_tc_hr_full(const CUtensorMap &mapA, const CUtensorMap &mapB, float *out, int p,
-                              int p_pad, int d, int d_pad, int *status, cudaStream_t s) {
-    static std::atomic<unsigned long long> attr_done{0};
-    const cudaError_t e = set_max_dynamic_smem((const void *)tc_hr_kernel, kSmem, attr_done);
-    if (e != cudaSuccess) return e;
+                              int p_pad, int d, int d_pad, int *status, cudaStream_t s,
+                              bool stalled) {
     HrArgs a{out, p, d, p_pad, d_pad, status};
-    tc_hr_kernel<<<dim3(p_pad / 128, d_pad / 128), 320, kSmem, s>>>(mapA, mapB, a);
-    return cudaGetLastError();
+    auto run = [&](auto *kernel, std::atomic<unsigned long long> &done) {
+        const cudaError_t e = set_max_dynamic_smem((const void *)kernel, kSmem, done);
+        if (e != cudaSuccess) return e;
+        return launch_k(kernel, dim3(p_pad / 128, d_pad / 128), dim3(320), (size_t)kSmem, s, false, mapA, mapB, a);
+    };
+    static std::atomic<unsigned long long> done[2];
+    return stalled ? run(tc_hr_kernel<true>, done[1]) : run(tc_hr_kernel<false>, done[0]);
 }
 
 }  // namespace jarq

@@ -114,14 +114,17 @@ __device__ __forceinline__ void sum_levels(tc::F2 l0, tc::F2 l1, tc::F2 l2, tc::
 // 175 with the digits of P before it; 465 us on 4096 x 11008, 582 on 14336 x 4096.
 // A single stage of 64 of K, all rows of R_i^{-1} and a drain of eight warps that
 // combined the levels by two-sums took 325, 920 and 1100 us.
+// kStalled: for the self-test, the issuer does nothing.
+template <bool kStalled>
 __global__ void __launch_bounds__(kPairThreads, 1)
     tc_fold_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapH,
                    ProjArgs a) {
+    constexpr uint32_t kPolls = tc::wait_polls(kStalled);
     constexpr int kStages = kFoldStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = (uint64_t *)(smem + kStages * kFoldStage);
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 2);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 3);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tile it: row tile it / nct, column tile it % nct (in one group: g is a
@@ -133,6 +136,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     auto empty = [&](int s) { return tc::smem_u32(bars + kStages + s); };
     const uint32_t afull = tc::smem_u32(bars + 2 * kStages);
     const uint32_t aempty = tc::smem_u32(bars + 2 * kStages + 1);
+    const uint32_t closing = tc::smem_u32(bars + 2 * kStages + 2);
     auto tileA = [&](int s, int t) { return tc::smem_u32(smem + s * kFoldStage + t * kPairA); };
     auto tileB = [&](int s, int u) {
         return tc::smem_u32(smem + s * kFoldStage + kHDig * kPairA + u * kPairB);
@@ -145,6 +149,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
         tc::mbar_init(afull, 1);
         tc::mbar_init(aempty, kPairDrain);
+        tc::mbar_init(closing, 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -168,7 +173,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
             const int j0 = it / nct * 128, n0 = it % nct * 64, k0 = n0 / a.g * a.g, nc = chunks_of(it);
             for (int c = 0; c < nc; ++c) {
-                ok = tc::mbar_wait(empty(s), ph);
+                ok = tc::mbar_wait<kPolls>(empty(s), ph);
                 if (!ok) break;
                 if (tc::elect_one()) {
                     tc::mbar_expect_tx(full(s), kFoldStage);
@@ -189,18 +194,21 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
         // do not leave before the MMAs have consumed the stages filled here
         for (int n = max(0, filled - kStages); n < filled && ok; ++n)
-            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
-        if (!ok) *abort_flag = 1;
+            ok = tc::mbar_wait<kPolls>(empty(n % kStages), (n / kStages) & 1);
+        if (!ok) {
+            *abort_flag = 1;
+            tc::abandon_ring(full(0), kStages, filled, true);
+        }
     } else if (warp == 1) {
         // ---------------- MMA issuer
         const uint64_t ad0 = tc::sdesc_sw64(tileA(0, 0)), bd0 = tc::sdesc_sw64(tileB(0, 0));
         bool ok = true;
         int s = 0, ph = 0, n = 0;
-        for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x, ++n) {
+        for (int it = blockIdx.x; it < (kStalled ? 0 : nitems) && ok; it += gridDim.x, ++n) {
             const int nc = chunks_of(it);
             for (int c = 0; c < nc; ++c) {
-                ok = tc::mbar_wait(full(s), ph);
-                if (c == 0) ok = tc::mbar_wait(aempty, (n & 1) ^ 1) && ok;
+                ok = tc::mbar_wait<kPolls>(full(s), ph);
+                if (c == 0) ok = tc::mbar_wait<kPolls>(aempty, (n & 1) ^ 1) && ok;
                 if (!ok) break;
                 tc::tc_fence_after();
                 if (tc::elect_one()) {
@@ -226,7 +234,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                 }
             }
         }
-        if (!ok) *abort_flag = 1;
+        if (!tc::mma_done<kPolls>(closing, tc::elect_one()) || !ok) *abort_flag = 1;
     } else {
         // ---------------- drain: levels -> double-float
         const int q = warp & 3, cq = (warp - 2) >> 2;    // lane quarter, 16-column quarter
@@ -237,7 +245,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             const int row = it / nct * 128 + 32 * q + lane, n0 = it % nct * 64, hb = n0 / a.g;
             const int ex = a.wexp[(size_t)min(row, a.p - 1) * a.G + hb] + a.hexp[hb] - 14;
             const tc::F2 scale = tc::f2(ldexpf(1.0f, ex));
-            ok = __all_sync(0xffffffffu, tc::mbar_wait(afull, n & 1));
+            ok = __all_sync(0xffffffffu, tc::mbar_wait<kPolls>(afull, n & 1));
             if (!ok) break;
             tc::tc_fence_after();
             tc::F2 w[8];     // L_4 + L_5 2^-8
@@ -302,13 +310,16 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, ST_TIMEOUT);
 }
 
+// kStalled: for the self-test, the issuer stops after one group.
+template <bool kStalled>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     tc_proj_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapH,
                    ProjArgs a) {
+    constexpr uint32_t kPolls = tc::wait_polls(kStalled);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = (uint64_t *)(smem + kPairStages * kPairStage);
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kPairStages + 3);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kPairStages + 4);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)tc::cluster_rank();
@@ -326,6 +337,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     auto empty = [&](int s) { return tc::smem_u32(bars + kPairStages + s); };
     const uint32_t afull = tc::smem_u32(bars + 2 * kPairStages);
     const uint32_t afree = tc::smem_u32(bars + 2 * kPairStages + 1);   // [2]: levels 4, 5; 0..3
+    const uint32_t closing = tc::smem_u32(bars + 2 * kPairStages + 3);
     auto tileA = [&](int s, int t) { return tc::smem_u32(smem + s * kPairStage + t * kPairA); };
     auto tileB = [&](int s, int u) {
         return tc::smem_u32(smem + s * kPairStage + kWDig * kPairA + u * kPairB);
@@ -339,6 +351,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         tc::mbar_init(afull, 1);
         tc::mbar_init(afree, 2 * kPairDrain);       // the even CTA's: both drains
         tc::mbar_init(afree + 8, 2 * kPairDrain);
+        tc::mbar_init(closing, 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -360,9 +373,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         // ---------------- producer
         bool ok = true;
         const uint32_t full0 = tc::map_rank(full(0), 0);
-        int s = 0, ph = 1;
-        for (int c = 0; c < nchunks; ++c) {
-            ok = tc::mbar_wait(empty(s), ph);
+        int s = 0, ph = 1, c = 0;
+        for (; c < nchunks; ++c) {
+            ok = tc::mbar_wait<kPolls>(empty(s), ph);
             if (!ok) break;
             if (tc::elect_one()) {
                 if (rank == 0) tc::mbar_expect_tx(full(s), 2 * kPairStage);
@@ -385,8 +398,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         // do not leave before the MMAs have consumed the stages filled here:
         // no copy or commit is in flight afterwards
         for (int n = max(0, nchunks - kPairStages); n < nchunks && ok; ++n)
-            ok = tc::mbar_wait(empty(n % kPairStages), (n / kPairStages) & 1);
-        if (!ok) *abort_flag = 1;
+            ok = tc::mbar_wait<kPolls>(empty(n % kPairStages), (n / kPairStages) & 1);
+        if (!ok) {
+            *abort_flag = 1;
+            tc::abandon_ring(full(0), kPairStages, c, rank == 0);
+        }
     } else if (warp == 1) {
         // ---------------- MMA issuer of the pair
         if (rank == 0) {
@@ -395,10 +411,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             constexpr uint64_t kPl = kPairA >> 4, kHi = (2 * kPairB) >> 4;   // next W plane; planes 4, 5
             bool ok = true;
             int s = 0, ph = 0;
-            for (int sg = 0; sg < a.G && ok; ++sg) {
+            const int ngroups = kStalled ? 1 : a.G;
+            for (int sg = 0; sg < ngroups && ok; ++sg) {
                 for (int c = 0; c < nsub; ++c) {
-                    ok = tc::mbar_wait(full(s), ph);
-                    if (c == 0) ok = tc::mbar_wait(afree, (sg & 1) ^ 1) && ok;
+                    ok = tc::mbar_wait<kPolls>(full(s), ph);
+                    if (c == 0) ok = tc::mbar_wait<kPolls>(afree, (sg & 1) ^ 1) && ok;
                     if (!ok) break;
                     tc::tc_fence_after();
                     const uint64_t ad = ad0 + (uint64_t)(s * (kPairStage >> 4));
@@ -413,7 +430,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                     }
                     __syncwarp();
                     if (c == 0) {
-                        ok = tc::mbar_wait(afree + 8, (sg & 1) ^ 1);
+                        ok = tc::mbar_wait<kPolls>(afree + 8, (sg & 1) ^ 1);
                         if (!ok) break;
                         tc::tc_fence_after();
                     }
@@ -434,7 +451,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                     }
                 }
             }
-            if (!ok) *abort_flag = 1;
+            if (!tc::mma_done_pair<kPolls>(closing, tc::elect_one()) || !ok) *abort_flag = 1;
         }
     } else {
         // ---------------- drain: levels -> double-float per group -> accumulator
@@ -457,7 +474,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             // 2^ex, from its bits while it is a normal number
             const tc::F2 scale = tc::f2((unsigned)(ex + 126) <= 252u ? __int_as_float((ex + 127) << 23)
                                                                      : ldexpf(1.0f, ex));
-            ok = __all_sync(0xffffffffu, tc::mbar_wait(afull, sg & 1));
+            ok = __all_sync(0xffffffffu, tc::mbar_wait<kPolls>(afull, sg & 1));
             if (!ok) break;
             tc::tc_fence_after();
             tc::F2 w[8];     // L_4 + L_5 2^-8
@@ -897,7 +914,7 @@ cudaError_t launch_slice_rinv(const double *Rinv, __nv_bfloat16 *rdig, int *rexp
 cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, const float *Phi,
                           const float *Plo, __nv_bfloat16 *pdig, int *pexp, const int *rexp,
                           float *out_hi, float *out_lo, int p, int p_pad, int d, int d_pad, int g,
-                          int *status, cudaStream_t s) {
+                          int *status, cudaStream_t s, bool stalled) {
     const long long warps = (long long)p * (d / g);
     const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
     if (g == 128)
@@ -906,16 +923,18 @@ cudaError_t launch_ptilde(const CUtensorMap &mapPd, const CUtensorMap &mapR, con
         slice_df_rows_kernel<2><<<blocks, 256, 0, s>>>(Phi, Plo, pdig, pexp, p, d, d_pad, p_pad);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    static std::atomic<unsigned long long> attr_done{0};
-    e = set_max_dynamic_smem((const void *)tc_fold_kernel, kFoldSmem, attr_done);
-    if (e != cudaSuccess) return e;
     ProjArgs a{out_hi, out_lo, pexp, rexp, status, p, d, g, d / g, p_pad, d};
     // persistent: one CTA per SM over the (p_pad / 128) x (d / 64) tiles
     (void)d_pad;
     const int items = ((p + 127) / 128) * (d / 64);
     const int ctas = items < num_sms() ? items : num_sms();
-    tc_fold_kernel<<<dim3(ctas, 1, 1), kPairThreads, kFoldSmem, s>>>(mapPd, mapR, a);
-    return cudaGetLastError();
+    auto run = [&](auto *kernel, std::atomic<unsigned long long> &done) {
+        const cudaError_t r = set_max_dynamic_smem((const void *)kernel, kFoldSmem, done);
+        if (r != cudaSuccess) return r;
+        return launch_k(kernel, dim3(ctas), dim3(kPairThreads), (size_t)kFoldSmem, s, false, mapPd, mapR, a);
+    };
+    static std::atomic<unsigned long long> done[2];
+    return stalled ? run(tc_fold_kernel<true>, done[1]) : run(tc_fold_kernel<false>, done[0]);
 }
 
 cudaError_t launch_slice_rows(const float *W, __nv_bfloat16 *planes, int *wexp, int p, int d,
@@ -932,13 +951,16 @@ cudaError_t launch_slice_rows(const float *W, __nv_bfloat16 *planes, int *wexp, 
 
 cudaError_t launch_tc_proj(const CUtensorMap &mapW, const CUtensorMap &mapH, float *Phi,
                            float *Plo, const int *wexp, const int *hexp, int p, int p_pad, int d,
-                           int d_pad, int g, int *status, cudaStream_t s) {
-    static std::atomic<unsigned long long> attr_done{0};
-    const cudaError_t e = set_max_dynamic_smem((const void *)tc_proj_kernel, kPairSmem, attr_done);
-    if (e != cudaSuccess) return e;
+                           int d_pad, int g, int *status, cudaStream_t s, bool stalled) {
     ProjArgs a{Phi, Plo, wexp, hexp, status, p, d, g, d / g, p_pad, d_pad};
-    tc_proj_kernel<<<dim3((p + 255) / 256 * 2, d / 64), kPairThreads, kPairSmem, s>>>(mapW, mapH, a);
-    return cudaGetLastError();
+    auto run = [&](auto *kernel, std::atomic<unsigned long long> &done) {
+        const cudaError_t e = set_max_dynamic_smem((const void *)kernel, kPairSmem, done);
+        if (e != cudaSuccess) return e;
+        return launch_k(kernel, dim3((p + 255) / 256 * 2, d / 64), dim3(kPairThreads), (size_t)kPairSmem, s, false,
+                        mapW, mapH, a);
+    };
+    static std::atomic<unsigned long long> done[2];
+    return stalled ? run(tc_proj_kernel<true>, done[1]) : run(tc_proj_kernel<false>, done[0]);
 }
 
 cudaError_t launch_whw(const float *W, const float *Phi, const float *Plo, double *out, int p,

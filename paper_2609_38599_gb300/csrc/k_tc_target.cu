@@ -84,13 +84,16 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = (a - (s - bb)) + (b - bb);
 }
 
+// kStalled: for the self-test, the issuer stops after one group.
+template <bool kStalled>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_target_kernel(const __grid_constant__ CUtensorMap mapC, const __grid_constant__ CUtensorMap mapT,
                      TargetArgs a) {
+    constexpr uint32_t kPolls = tc::wait_polls(kStalled);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = (uint64_t *)(smem + kStages * kStage);
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 4);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * kStages + 5);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     float *sS = (float *)(smem + kStages * kStage + 256);    // [seg_per_split][kSRow]
     int *sE = (int *)(sS + a.seg_per_split * kSRow);         // [seg_per_split]
@@ -106,6 +109,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     auto empty = [&](int s) { return tc::smem_u32(bars + kStages + s); };
     auto afull = [&](int b) { return tc::smem_u32(bars + 2 * kStages + b); };
     auto aempty = [&](int b) { return tc::smem_u32(bars + 2 * kStages + 2 + b); };
+    const uint32_t closing = tc::smem_u32(bars + 2 * kStages + 4);
     auto tileA = [&](int s) { return tc::smem_u32(smem + s * kStage); };
     auto tileB = [&](int s, int t) { return tc::smem_u32(smem + s * kStage + kTileA + t * kTileB); };
 
@@ -118,6 +122,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tc::mbar_init(afull(b), 1);
             tc::mbar_init(aempty(b), 2 * kDrainWarps);   // the even CTA's: both drains
         }
+        tc::mbar_init(closing, 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -164,9 +169,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         // ---------------- producer
         bool waited = !early, ok = true;
         const uint32_t full0 = tc::map_rank(full(0), 0);
-        int s = 0, ph = 1;
-        for (int c = 0; c < nchunks; ++c) {
-            ok = tc::mbar_wait(empty(s), ph);
+        int s = 0, ph = 1, c = 0;
+        for (; c < nchunks; ++c) {
+            ok = tc::mbar_wait<kPolls>(empty(s), ph);
             if (!ok) break;
             const int kx = h0 * a.g + c * 64;
             if (!waited && kx >= a.prev0 * a.g && kx < a.i0 * a.g) {
@@ -189,19 +194,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         // do not leave before the MMAs have consumed the stages filled here:
         // no copy or commit is in flight afterwards
-        for (int c = 0; c < min(nchunks, kStages) && ok; ++c) {
+        for (int e = 0; e < min(nchunks, kStages) && ok; ++e) {
             // the slots in order from the oldest: s, s + 1, ...
-            const int n = nchunks - min(nchunks, kStages) + c;
-            ok = tc::mbar_wait(empty(n % kStages), (n / kStages) & 1);
+            const int n = nchunks - min(nchunks, kStages) + e;
+            ok = tc::mbar_wait<kPolls>(empty(n % kStages), (n / kStages) & 1);
         }
-        if (!ok) *abort_flag = 1;
+        if (!ok) {
+            *abort_flag = 1;
+            tc::abandon_ring(full(0), kStages, c, rank == 0);
+        }
     } else if (warp == 1) {
         // ---------------- MMA issuer of the pair: one unit per group h
         if (rank == 0) {
             const uint64_t ad0 = tc::sdesc_sw128(tileA(0)), bd0 = tc::sdesc_sw128(tileB(0, 0));
             int s = 0, ph = 0;
             bool ok = true;
-            for (int u = 0; u < nseg && ok; ++u) {
+            const int nunits = kStalled ? min(nseg, 1) : nseg;
+            for (int u = 0; u < nunits && ok; ++u) {
                 const int b = u & 1;
                 // the unit's stages first (they are usually there already),
                 // then its accumulator: nothing but the MMAs' issue lies
@@ -211,9 +220,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     s1 = 0;
                     ph1 ^= 1;
                 }
-                ok = tc::mbar_wait(full(s), ph);
-                if (nkc == 2) ok = tc::mbar_wait(full(s1), ph1) && ok;
-                ok = tc::mbar_wait(aempty(b), ((u >> 1) & 1) ^ 1) && ok;
+                ok = tc::mbar_wait<kPolls>(full(s), ph);
+                if (nkc == 2) ok = tc::mbar_wait<kPolls>(full(s1), ph1) && ok;
+                ok = tc::mbar_wait<kPolls>(aempty(b), ((u >> 1) & 1) ^ 1) && ok;
                 if (!ok) break;
                 tc::tc_fence_after();
                 if (tc::elect_one()) {
@@ -239,7 +248,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     ph ^= 1;
                 }
             }
-            if (!ok) *abort_flag = 1;
+            if (!tc::mma_done_pair<kPolls>(closing, tc::elect_one()) || !ok) *abort_flag = 1;
         }
     } else {
         // ---------------- drain: digits -> double-float x s_h 2^(E - 9) -> accumulator
@@ -276,7 +285,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const float sc = (unsigned)(e2 + 126) <= 252u ? sv * __int_as_float((e2 + 127) << 23)
                                                           : ldexpf(sv, e2);
             const tc::F2 scale = tc::f2(sc), nscale = tc::f2(-sc);
-            ok = tc::mbar_wait(afull(b), (u >> 1) & 1);
+            ok = tc::mbar_wait<kPolls>(afull(b), (u >> 1) & 1);
             if (!__all_sync(0xffffffffu, ok)) {
                 ok = false;
                 break;
@@ -378,12 +387,8 @@ cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, f
                              float *out_lo, const float *S, const int *expoT, const int *active,
                              int p, int p_pad, int d_pad, int g, int G, int i0, int nb,
                              int nb_prev, int nsplit, int qmax, int *status, cudaStream_t s,
-                             bool pdl) {
-    static std::atomic<unsigned long long> attr_done{0};
+                             bool pdl, bool stalled) {
     static_assert(smem_bytes(kMaxGroups) <= 227 * 1024, "stages and scales must fit an SM's shared memory");
-    const cudaError_t e =
-        set_max_dynamic_smem((const void *)tc_target_kernel, smem_bytes(kMaxGroups), attr_done);
-    if (e != cudaSuccess) return e;
     const int per = (G + nsplit - 1) / nsplit;
     const int tiles = (p + 255) / 256 * 2;   // pairs of row tiles
     // the digit sums stay exact: 128 * 255 * 512 < 2^24
@@ -392,8 +397,13 @@ cudaError_t launch_tc_target(const CUtensorMap &mapC, const CUtensorMap &mapT, f
     TargetArgs a{out_hi, out_lo, S, expoT, active, status, p, p_pad, d_pad, g, G, per,
                  i0, nb, i0 - nb_prev};
     dim3 grid(tiles, nb * g / 64, nsplit);
-    return launch_k(tc_target_kernel, grid, dim3(kThreads), (size_t)smem_bytes(per), s, pdl, mapC,
-                    mapT, a);
+    auto run = [&](auto *kernel, std::atomic<unsigned long long> &done) {
+        const cudaError_t e = set_max_dynamic_smem((const void *)kernel, smem_bytes(kMaxGroups), done);
+        if (e != cudaSuccess) return e;
+        return launch_k(kernel, grid, dim3(kThreads), (size_t)smem_bytes(per), s, pdl, mapC, mapT, a);
+    };
+    static std::atomic<unsigned long long> done[2];
+    return stalled ? run(tc_target_kernel<true>, done[1]) : run(tc_target_kernel<false>, done[0]);
 }
 
 }  // namespace jarq

@@ -1,7 +1,11 @@
 // Blackwell (sm_103a) building blocks: mbarriers, TMA tile loads, TMEM and
 // tcgen05.mma, written as inline PTX.  Every wait is bounded: after
-// kWaitIters polls a wait gives up and reports failure so the kernel can set
-// the timeout status, drain its own copies and MMAs and return.
+// kWaitIters polls a role gives up and sets its CTA's abort flag, and each role
+// that is left waiting runs out in its turn.  A producer
+// that gives up then waits, again with a limit, for its copies in flight
+// (abandon_ring), as the issuing warp does for its MMAs in any case
+// (mma_done), TMEM is freed, the CTAs of a pair leave together, and the timeout
+// status is set.
 #pragma once
 
 #include <cuda.h>
@@ -12,7 +16,16 @@
 namespace jarq {
 namespace tc {
 
+// A poll of a barrier that is not ready takes about 1.5 us (the hardware
+// suspends the thread): a wait gives up after some 50 s, and one for what is
+// then still in flight after some 6 ms.  In the self-test of this path
+// (jarq_selftest_stalled_kernel) a wait gives up after 1.5 ms.  The limits are
+// constants: passed as an argument, or with a look at the abort flag every 64
+// polls, the same kernels took 3 to 7 % longer (Gram 198 -> 207 and 211 us,
+// target projection 1.58 -> 1.63 and 1.62 ms on 4096 x 4096).
 constexpr uint32_t kWaitIters = 1u << 25;
+constexpr uint32_t kCloseIters = 1u << 12;
+__host__ __device__ constexpr uint32_t wait_polls(bool stalled) { return stalled ? 1u << 10 : kWaitIters; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -42,12 +55,25 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Wait for the phase with the given parity; false after kWaitIters polls.
+// Wait for the phase with the given parity; false after kPolls polls.
+template <uint32_t kPolls = kWaitIters>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 #pragma unroll 1
-    for (uint32_t i = 0; i < kWaitIters; ++i)
+    for (uint32_t i = 0; i < kPolls; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
+}
+
+// A producer gives up, `filled` stages of its ring of `stages` filled so far:
+// until its copies have landed, with a short limit.  They complete on the
+// barriers full0 + 8 s of this CTA; in the odd CTA of a pair (`owner` false)
+// on the even one's, which waits for them there, and this CTA stays as long
+// (nothing arrives on its own).  Out of line: only a give-up gets here.
+static __device__ __noinline__ void abandon_ring(uint32_t full0, int stages, int filled, bool owner) {
+    // a wait that runs out has given the copies issued with it their time too
+    bool landed = true;
+    for (int n = filled > stages ? filled - stages : 0; n < filled && landed; ++n)
+        landed = mbar_wait<kCloseIters>(full0 + 8 * (owner ? n % stages : 0), owner ? (n / stages) & 1 : 0);
 }
 
 // True in one lane of a converged warp, the same lane each time.
@@ -190,6 +216,14 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
         : "memory");
 }
 
+// End of the issuing warp, given up or not: true once the MMAs that its lane
+// `mine` issued are done (`bar`: count 1, used for nothing else).
+template <uint32_t kPolls>
+__device__ __forceinline__ bool mma_done(uint32_t bar, bool mine) {
+    if (mine) mma_commit(bar);
+    return mbar_wait<kPolls>(bar, 0);
+}
+
 // ---------------------------------------------------------------- CTA pairs (cta_group::2)
 // Two CTAs of a cluster of two share one MMA: 256 rows of A (128 in each
 // CTA's shared memory), N columns of B (N/2 rows of B in each), and each CTA
@@ -250,14 +284,20 @@ __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t adesc, ui
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// Arrive on the barrier at this offset in both CTAs of the pair once every
-// tcgen05 operation this thread issued so far is done.
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
+// Arrive on the barrier at this offset in the CTAs of `mask` (both of the
+// pair) once every tcgen05 operation this thread issued so far is done.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t mask = 3) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
         " [%0], %1;" ::"r"(bar),
-        "h"((uint16_t)3)
+        "h"(mask)
         : "memory");
+}
+// mma_done of a pair, by the even CTA.
+template <uint32_t kPolls>
+__device__ __forceinline__ bool mma_done_pair(uint32_t bar, bool mine) {
+    if (mine) mma_commit_pair(bar, 1);
+    return mbar_wait<kPolls>(bar, 0);
 }
 
 // ---------------------------------------------------------------- packed float32 pairs

@@ -33,7 +33,7 @@ EXPORTS = ("jarq_default_options", "jarq_prepare_hessian", "jarq_refine_layer",
            "jarq_objective_noalloc", "jarq_residual_product", "jarq_canonicalize",
            "jarq_dequantize", "jarq_pack_codes", "jarq_accumulate_hessian",
            "jarq_refine_layer_mu", "jarq_fit_scales", "jarq_multicode_probe",
-           "jarq_selftest_wait_timeout")
+           "jarq_selftest_wait_timeout", "jarq_selftest_stalled_kernel")
 
 
 class JarqError(RuntimeError):
@@ -109,6 +109,8 @@ def _load():
     lib.jarq_launch_count.argtypes = []
     lib.jarq_selftest_wait_timeout.restype = ci
     lib.jarq_selftest_wait_timeout.argtypes = [vp]
+    lib.jarq_selftest_stalled_kernel.restype = ci
+    lib.jarq_selftest_stalled_kernel.argtypes = [ctypes.c_char_p, vp]
     return lib
 
 
@@ -154,6 +156,14 @@ def selftest_wait_timeout() -> int:
     the bounded-wait path works), on the current torch stream."""
     import torch
     return int(_lib.jarq_selftest_wait_timeout(ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)))
+
+
+def selftest_stalled_kernel(kernel: str) -> int:
+    """Status of one tensor-core kernel whose waits run out (JARQ_ERR_TIMEOUT),
+    on the current torch stream."""
+    import torch
+    return int(_lib.jarq_selftest_stalled_kernel(
+        kernel.encode(), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)))
 
 
 def status_string(status: int) -> str:

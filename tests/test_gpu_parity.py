@@ -416,6 +416,10 @@ def test_bounded_wait_reports_timeout_and_context_survives(jarq):
     every kernel's bounded waits use; the context stays usable afterwards:
     the tiny layer still refines as the oracle does."""
     assert jarq.selftest_wait_timeout() == jarq.JARQ_ERR_TIMEOUT
+    _refines_as_the_oracle()
+
+
+def _refines_as_the_oracle():
     lay = tiny_layer()
     prep, res = oracle_run(lay, 2, False)
     S, Q, st = gpu_refine(lay, 2, early_stop=False)
@@ -423,3 +427,16 @@ def test_bounded_wait_reports_timeout_and_context_survives(jarq):
     m = compare_final(lay, prep, res, S, Q, st)
     assert m["codes_same"] >= CODES_SAME, m
     assert m["F_rel_all"] <= REL_F, m
+
+
+@pytest.mark.parametrize("kernel", ["hr_full", "ptilde", "target", "gram", "proj", "syrk"])
+def test_stalled_kernel_reports_timeout_and_context_survives(jarq, kernel):
+    """A tensor-core kernel whose issuing warp stops after its first unit of
+    work: every other warp of the CTA (both CTAs of a pair) gives up, waits for
+    what is in flight and leaves; the call reports the timeout within seconds
+    and the next refinement is the oracle's."""
+    import time
+    t0 = time.perf_counter()
+    assert jarq.selftest_stalled_kernel(kernel) == jarq.JARQ_ERR_TIMEOUT
+    assert time.perf_counter() - t0 < 10
+    _refines_as_the_oracle()

@@ -206,3 +206,14 @@ def test_the_other_group_size_at_the_same_time(dev, call):
     assert run(128, STREAM) == 0        # limits that are set once are set
     dev.hook(note)
     assert run(128, STREAM) == 0
+
+
+@pytest.mark.parametrize("kernel,part", [
+    (b"target", "tc_target_kernel"), (b"gram", "tc_gram_kernel"), (b"proj", "tc_proj_kernel"),
+    (b"ptilde", "tc_fold_kernel"), (b"hr_full", "tc_hr_kernel"), (b"syrk", "tc_syrk_kernel")])
+def test_stalled_kernel_selftest_launches_the_kernel_named(dev, kernel, part):
+    live = dev.lib.fake_live()
+    assert dev.lib.jarq_selftest_stalled_kernel(kernel, ctypes.c_void_p(STREAM)) == 0
+    launches = [op[2] for op in dev.log() if op[0] == "launch"]
+    assert part in launches[-1] and dev.lib.fake_live() == live
+    assert dev.lib.jarq_selftest_stalled_kernel(b"no such kernel", ctypes.c_void_p(STREAM)) == 1
