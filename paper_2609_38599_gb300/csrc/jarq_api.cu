@@ -275,7 +275,7 @@ void layout_hessian(Arena &m, jarq_hessian *h) {
     m.take(h->rexp, G);
     m.take(h->Htdig, 4 * pd);
     m.take(h->expoT, G * G);
-    m.take(h->band, G * (kMaxBlock - 1) * g * g);
+    m.take(h->band, G * (sweep_block(h->g) - 1) * g * g);
     m.take(h->dstatus, 1);
 }
 

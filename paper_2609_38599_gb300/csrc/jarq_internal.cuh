@@ -25,7 +25,6 @@ enum : int {
 constexpr int kMaxGroups = 128;    // largest supported G for the scale solve
 constexpr int kMaxGroupSize = 128; // the larger of the two group sizes
 constexpr int kMaxSplit = 16;      // largest split-K factor of the phase product
-constexpr int kMaxBlock = 4;       // groups of one block of the sweep at most
 
 // Groups of one block of the sweep for group size g: 256 columns.  The Babai
 // kernel holds the factors of two groups and the blocks Ht_i'i of one group i
@@ -147,8 +146,8 @@ struct jarq_hessian {
     CUtensorMap mapH128;          // tensor map of Hplanes, 128 x 64 boxes
     CUtensorMap mapD8, mapD10;    // tensor maps of Hdig8 (64 x 32 boxes) / Hdig10 (64 x 64)
     float *Lf = nullptr;          // [G][factor_floats(g)] lower factor L_i = R_i^T, packed
-    // digits of the blocks Ht_{i'i}, i' = i + 1 .. i + kMaxBlock - 1, column by
-    // column: [G][kMaxBlock - 1][g columns of i][g rows of i'], each entry the
+    // digits of the blocks Ht_{i'i}, i' = i + 1 .. i + sweep_block(g) - 1, column by
+    // column: [G][sweep_block(g) - 1][g columns of i][g rows of i'], each entry the
     // two 20-bit halves (a_0 2^10 + a_1, a_2 2^10 + a_3) of its digits
     int2 *band = nullptr;
     double *L64 = nullptr;        // [G][g][g] the same in float64

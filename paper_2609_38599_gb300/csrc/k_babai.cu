@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(32 * (kMaxWarps + 1), 1) babai_kernel(BabaiArg
                     }
                     tc::mbar_expect_tx(pfull(t), g * g * sizeof(int2));
                     tc::bulk_load(tc::smem_u32(pairs + (size_t)t * g * g),
-                                  a.band + ((size_t)(a.i0 + n) * (kMaxBlock - 1) + t) * g * g,
+                                  a.band + ((size_t)(a.i0 + n) * kPairs + t) * g * g,
                                   g * g * sizeof(int2), pfull(t));
                 }
             }

@@ -265,14 +265,14 @@ __global__ void band_kernel(const __half *__restrict__ dig, int2 *__restrict__ b
         tile[y][tx] = make_int2(a[0] * 1024 + a[1], a[2] * 1024 + a[3]);
     }
     __syncthreads();
-    int2 *out = band + ((size_t)i * (kMaxBlock - 1) + dd) * g * g;
+    int2 *out = band + ((size_t)i * gridDim.z + dd) * g * g;
     for (int y = ty; y < 32; y += 8) out[(size_t)(k0 + y) * g + m0 + tx] = tile[tx][y];
 }
 
 }  // namespace
 
 cudaError_t launch_band(const __half *Htdig, int2 *band, int d, int d_pad, int g, cudaStream_t s) {
-    band_kernel<<<dim3((g / 32) * (g / 32), d / g, kMaxBlock - 1), dim3(32, 8), 0, s>>>(
+    band_kernel<<<dim3((g / 32) * (g / 32), d / g, sweep_block(g) - 1), dim3(32, 8), 0, s>>>(
         Htdig, band, d, d_pad, g);
     return cudaGetLastError();
 }

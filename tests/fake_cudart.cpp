@@ -56,15 +56,15 @@ void note(const char *what, cudaStream_t s, const void *p, size_t n) {
     if (hook) hook(what, const_cast<void *>(p), n);
 }
 
-cudaError_t launch(const void *fn, size_t smem, cudaStream_t s, void **args) {
+cudaError_t launch(const void *fn, dim3 grid, size_t smem, cudaStream_t s, void **args) {
     std::lock_guard<std::recursive_mutex> l(st().mu);
     const std::string &name = st().kernels[fn];
     const auto lim = st().smem_limit.find(fn);
     if (smem > 48 * 1024 && (lim == st().smem_limit.end() || smem > (size_t)lim->second))
         return g_last = cudaErrorInvalidValue;
-    st().log << "launch " << (size_t)s << ' ' << name;
+    st().log << "launch " << (size_t)s << ' ' << name << " grid=" << grid.x << ',' << grid.y << ',' << grid.z;
     for (const auto &w : st().watched)
-        if (name.find(w.first) != std::string::npos) st().log << ' ' << *(size_t *)args[w.second];
+        if (name.find(w.first) != std::string::npos) st().log << " arg=" << *(size_t *)args[w.second];
     st().log << '\n';
     return cudaSuccess;
 }
@@ -134,11 +134,11 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *fn) {
     *k = (cudaKernel_t)fn;
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t smem, cudaStream_t s) {
-    return launch((const void *)k, smem, s, args);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **args, size_t smem, cudaStream_t s) {
+    return launch((const void *)k, grid, smem, s, args);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **args) {
-    return launch(fn, c->dynamicSmemBytes, c->stream, args);
+    return launch(fn, c->gridDim, c->dynamicSmemBytes, c->stream, args);
 }
 cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute a, int v) {
     if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {

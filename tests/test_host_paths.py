@@ -174,7 +174,7 @@ def test_a_corrected_target_call_after_a_failed_allocation(dev):
         lib.fake_watch(b"tc_proj_kernel", 1)        # the base of the digits' tensor map
         start = len(dev.log())
         assert dev.refine_mu(h, lay, dout, K1, XX) == 0
-        seen = [op[2].split()[1] for op in dev.log()[start:] if len(op) > 2 and op[0] == "launch" and " " in op[2]]
+        seen = [op[2].split("arg=")[1] for op in dev.log()[start:] if op[0] == "launch" and "arg=" in op[2]]
         assert len(seen) == 5 and "0" not in seen, (n, seen)       # two slicings, three projections
         n += 1
     assert n > 3
@@ -217,3 +217,13 @@ def test_stalled_kernel_selftest_launches_the_kernel_named(dev, kernel, part):
     launches = [op[2] for op in dev.log() if op[0] == "launch"]
     assert part in launches[-1] and dev.lib.fake_live() == live
     assert dev.lib.jarq_selftest_stalled_kernel(b"no such kernel", ctypes.c_void_p(STREAM)) == 1
+
+
+@pytest.mark.parametrize("g", [64, 128])
+def test_band_holds_what_the_sweep_reads(dev, g):
+    """The blocks of Ht beside the diagonal that a group's changes act on: the
+    other groups of a block of 256 columns, no more."""
+    rc, _ = dev.prepare(512, g)
+    assert rc == 0
+    grid = [op[2].split("grid=")[1] for op in dev.log() if op[0] == "launch" and "band_kernel" in op[2]]
+    assert grid == [f"{(g // 32) ** 2},{512 // g},{256 // g - 1}"]
