@@ -47,9 +47,7 @@ DTYPE = "f32 (integer-digit fp16/bf16 tensor-core products with exact partial su
 # valid while the kernel's source file is unchanged (first 12 hex digits of
 # its SHA-1); otherwise the bench reports null.
 TRAFFIC = {
-    "target": ("k_tc_target.cu", "0e24dd5faf51", 42.625e6 + 0.140e6),
     "sweep_product": ("k_tc_target.cu", "0e24dd5faf51", 42.625e6 + 0.140e6),
-    "babai": ("k_babai.cu", "672bc1eb4b99", 19.160e6 + 0.0),
     "sweep_babai": ("k_babai.cu", "672bc1eb4b99", 19.160e6 + 0.0),
     "gram": ("k_tc_gram.cu", "caa812655db4", 141.735e6 + 22.765e6),
     "proj": ("k_tc_proj.cu", "18c811b3e91e", 1350.252e6 + 139.033e6),
@@ -256,8 +254,6 @@ def kernel_model(kernel, lay, nsplit_bytes=0):
     Memory-bound kernels count the bytes they must move once.
     """
     p, d, g, G = lay.dout, lay.din, lay.g, lay.din // lay.g
-    if kernel == "target":
-        return dict(bound="tensor", work=2.0 * p * g * d, issued=4 * 2.0 * p * g * d)
     # the sweep's blocks of 256 columns: the average launch of a sweep
     launches = -(-d // 256)
     if kernel == "sweep_product":
@@ -270,8 +266,6 @@ def kernel_model(kernel, lay, nsplit_bytes=0):
     if kernel == "gram":
         blocks = G * (G + 1) / 2
         return dict(bound="tensor", work=2.0 * p * g * g * blocks, issued=4 * 2.0 * p * g * g * blocks)
-    if kernel == "babai":
-        return dict(bound="alu", work=1.0 * g * g * p)
     if kernel == "ptilde":
         return dict(bound="tensor", work=2.0 * p * d * g, issued=21 * 2.0 * p * d * g)
     if kernel == "scale_solve":

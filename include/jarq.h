@@ -328,10 +328,12 @@ const char *jarq_status_string(jarq_status s);
  * on.  When enabled, the library records a CUDA event pair around every
  * kernel launch it makes; durations are accumulated per kernel name when the
  * enclosing call synchronises.  Names: "validate", "residual", "init_rows",
- * "hr_full", "grad", "gram", "scale_solve", "phase_hr", "babai",
- * "symmetrize", "group_factor", "slices", "slice_rows", "proj", "whw", "rhs",
- * "htilde", "ptilde", "target", "syrk", "mu_combine", "own_rhs", "scale_fit",
- * "probe", "sweep_product", "sweep_babai".  Not thread-safe. */
+ * "hr_full", "grad", "gram", "scale_solve", "symmetrize", "group_factor",
+ * "slices", "slice_rows", "proj", "whw", "rhs", "htilde", "ptilde", "syrk",
+ * "mu_combine", "own_rhs", "scale_fit", "probe", "sweep_product",
+ * "sweep_babai"; also read: "target" and "babai" (the last two, whose launches
+ * once covered a group instead of a block of 256 columns) and "phase_hr" (no
+ * launches).  Not thread-safe. */
 void jarq_profile_enable(int on);
 void jarq_profile_reset(void);
 /* Accumulated launches and total device milliseconds of one kernel name since

@@ -658,7 +658,7 @@ jarq_status jarq_multicode_probe(jarq_hessian *h, const float *W, const float *S
     RUN("proj", 1, launch_tc_proj(w.mapWd, h->mapD8, w.Phi, w.Plo, w.wexp, h->expo, p, w.p_pad, d,
                                   h->d_pad, g, h->dstatus, st));
     // T = sum_h s_h H_ih c_h: the phase product with H's own digits
-    RUN("target", 1, launch_tc_target(w.mapC, h->mapD10, w.t_hi, w.t_lo, la.S, h->expo, nullptr, p,
+    RUN("sweep_product", 1, launch_tc_target(w.mapC, h->mapD10, w.t_hi, w.t_lo, la.S, h->expo, nullptr, p,
                                       w.p_pad, h->d_pad, g, G, group, 1, 0, nsplit, (1 << bits) - 1, h->dstatus, st,
                                       false));
     uint8_t *qo = reinterpret_cast<uint8_t *>(w.Hr);

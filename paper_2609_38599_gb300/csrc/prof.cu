@@ -9,11 +9,16 @@ namespace jarq {
 namespace {
 
 const char *const kNames[] = {"validate", "residual", "init_rows", "hr_full", "grad", "gram",
-                              "scale_solve", "phase_hr", "babai", "symmetrize", "group_factor",
-                              "slices", "slice_rows", "proj", "whw", "rhs", "htilde", "ptilde",
-                              "target", "syrk", "mu_combine", "own_rhs",
+                              "scale_solve", "symmetrize", "group_factor", "slices", "slice_rows",
+                              "proj", "whw", "rhs", "htilde", "ptilde", "syrk", "mu_combine", "own_rhs",
                               "scale_fit", "probe", "sweep_product", "sweep_babai"};
 constexpr int kNumNames = sizeof(kNames) / sizeof(kNames[0]);
+
+// Earlier names, still read: what is recorded under them now (null: nothing).
+struct Alias {
+    const char *name, *now;
+};
+constexpr Alias kAliases[] = {{"target", "sweep_product"}, {"babai", "sweep_babai"}, {"phase_hr", nullptr}};
 
 struct Pending {
     int id;
@@ -99,7 +104,18 @@ void jarq_profile_reset(void) {
 
 int jarq_profile_read(const char *kernel, long long *launches, double *total_ms) {
     jarq::prof_collect();
-    int id = kernel ? jarq::name_id(kernel) : -1;
+    if (!kernel) return -1;
+    for (const auto &a : jarq::kAliases)
+        if (!strcmp(a.name, kernel)) {
+            kernel = a.now;
+            break;
+        }
+    if (!kernel) {
+        if (launches) *launches = 0;
+        if (total_ms) *total_ms = 0.0;
+        return 0;
+    }
+    const int id = jarq::name_id(kernel);
     if (id < 0) return -1;
     if (launches) *launches = jarq::g_count[id];
     if (total_ms) *total_ms = jarq::g_ms[id];

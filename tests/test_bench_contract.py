@@ -23,9 +23,9 @@ Q_PROJ = _Shape(bench.WORKLOAD, 4096, 4096, 128, 3, 10)
 def test_kernel_work_closed_forms():
     p, d, g = 4096, 4096, 128
     G = d // g
-    # phase product: one (p x d) x (d x g) product of useful work, four digit planes issued
-    m = bench.kernel_model("target", Q_PROJ)
-    assert m["bound"] == "tensor" and m["work"] == 2.0 * p * g * d == 4294967296.0
+    # sweep product: one (p x d) x (d x 256) product of useful work, four digit planes issued
+    m = bench.kernel_model("sweep_product", Q_PROJ)
+    assert m["bound"] == "tensor" and m["work"] == 2.0 * p * 256 * d == 8589934592.0
     assert m["issued"] == 4 * m["work"]
     # Gram: the G (G + 1) / 2 blocks h <= i of c_h^T H_hi c_i, 2 p g^2 each
     m = bench.kernel_model("gram", Q_PROJ)
@@ -33,8 +33,8 @@ def test_kernel_work_closed_forms():
     # target projection P = W H and its 18 digit pairs
     m = bench.kernel_model("proj", Q_PROJ)
     assert m["work"] == 2.0 * p * d * d and m["issued"] == 18 * m["work"]
-    # Babai: the dense triangular back substitution, g^2 flops per (row, group)
-    assert bench.kernel_model("babai", Q_PROJ) == {"bound": "alu", "work": 1.0 * g * g * p}
+    # Babai: the dense triangular back substitution, g^2 flops per (row, group), two groups a launch
+    assert bench.kernel_model("sweep_babai", Q_PROJ) == {"bound": "alu", "work": 2.0 * g * g * p}
     # the scale solve moves each row's float64 Gram matrix once
     m = bench.kernel_model("scale_solve", Q_PROJ)
     assert m["bound"] == "hbm" and m["work"] >= 8.0 * p * G * G
@@ -44,8 +44,8 @@ def test_kernel_work_closed_forms():
 def test_roofline_arithmetic():
     pk = {"hbm_gbs": 6789.0, "bf16_tflops": 1942.2, "bf16_tflops_sustained": 1736.3}
     # 10 launches of 35 us each
-    e = bench.roofline_entry("target", {"launches": 10, "total_ms": 0.35}, Q_PROJ, pk, "measured")
-    achieved = 2.0 * 4096 * 128 * 4096 / 35e-6 / 1e12
+    e = bench.roofline_entry("sweep_product", {"launches": 10, "total_ms": 0.35}, Q_PROJ, pk, "measured")
+    achieved = 2.0 * 4096 * 256 * 4096 / 35e-6 / 1e12
     assert e["bound"] == "tensor" and e["unit"] == "TFLOP/s"
     assert e["achieved"] == pytest.approx(achieved) and e["peak"] == 1736.3
     assert e["frac"] == pytest.approx(achieved / 1736.3)
@@ -56,11 +56,11 @@ def test_roofline_arithmetic():
     assert e["unit"] == "GB/s" and e["peak"] == 6789.0
     assert e["frac"] == pytest.approx(e["achieved"] / 6789.0)
     # Babai against the float32 FMA rate of 152 SMs at 2070 MHz
-    e = bench.roofline_entry("babai", {"launches": 1, "total_ms": 0.0186}, Q_PROJ, pk, "measured")
+    e = bench.roofline_entry("sweep_babai", {"launches": 1, "total_ms": 0.0186}, Q_PROJ, pk, "measured")
     assert e["bound"] == "alu"
     assert e["peak"] == pytest.approx(152 * 128 * 2 * 2070e6 / 1e12)
     # no launches, no entry
-    assert bench.roofline_entry("target", {"launches": 0, "total_ms": 0.0}, Q_PROJ, pk, "x") is None
+    assert bench.roofline_entry("sweep_product", {"launches": 0, "total_ms": 0.0}, Q_PROJ, pk, "x") is None
 
 
 def test_traffic_is_reported_only_for_an_unchanged_source(tmp_path, monkeypatch):
@@ -73,21 +73,21 @@ def test_traffic_is_reported_only_for_an_unchanged_source(tmp_path, monkeypatch)
     # a changed source file withdraws its figure
     csrc = tmp_path / "paper_2609_38599_gb300" / "csrc"
     csrc.mkdir(parents=True)
-    fname = bench.TRAFFIC["target"][0]
+    fname = bench.TRAFFIC["sweep_product"][0]
     shutil.copy(os.path.join(bench.ROOT, "paper_2609_38599_gb300", "csrc", fname), csrc / fname)
     monkeypatch.setattr(bench, "ROOT", str(tmp_path))
-    unchanged = bench.traffic_for("target")
+    unchanged = bench.traffic_for("sweep_product")
     with open(csrc / fname, "a") as fh:
         fh.write("\n// changed\n")
-    assert bench.traffic_for("target") is None
-    assert unchanged in (None, bench.TRAFFIC["target"][2])
+    assert bench.traffic_for("sweep_product") is None
+    assert unchanged in (None, bench.TRAFFIC["sweep_product"][2])
     assert bench.traffic_for("not_in_table") is None
 
 
 def test_roofline_traffic_only_for_the_main_workload():
     pk = {"hbm_gbs": 6789.0, "bf16_tflops": 1942.2, "bf16_tflops_sustained": 1736.3}
     other = _Shape("llama2_7b_down_proj_4096x11008_g128_w4", 11008, 4096, 128, 4, 10)
-    e = bench.roofline_entry("target", {"launches": 1, "total_ms": 0.07}, other, pk, "measured")
+    e = bench.roofline_entry("sweep_product", {"launches": 1, "total_ms": 0.07}, other, pk, "measured")
     assert e["traffic"] is None
 
 

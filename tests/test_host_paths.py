@@ -227,3 +227,25 @@ def test_band_holds_what_the_sweep_reads(dev, g):
     assert rc == 0
     grid = [op[2].split("grid=")[1] for op in dev.log() if op[0] == "launch" and "band_kernel" in op[2]]
     assert grid == [f"{(g // 32) ** 2},{512 // g},{256 // g - 1}"]
+
+
+def test_profile_names_of_a_refinement(dev):
+    """The sweep's kernels are recorded once per block of 256 columns, and read
+    under the names that they had when a launch covered one group as well."""
+    lib, n, ms = dev.lib, ctypes.c_longlong(), ctypes.c_double()
+    _, h = dev.prepare(640, 128)
+    lay = dev.layer(640, 40, 128)
+
+    def read(name):
+        assert lib.jarq_profile_read(name, ctypes.byref(n), ctypes.byref(ms)) == 0, name
+        return n.value
+
+    lib.jarq_profile_reset()
+    lib.jarq_profile_enable(1)
+    assert dev.refine(h, lay, 40) == 0                  # three iterations
+    assert lib.jarq_multicode_probe(h, *lay, 40, 3, 1, None, None, None, None, None, ctypes.c_void_p(STREAM)) == 0
+    lib.jarq_profile_enable(0)
+    assert [read(k) for k in (b"sweep_product", b"target")] == [3 * 3 + 1] * 2      # and the probe's
+    assert [read(k) for k in (b"sweep_babai", b"babai")] == [3 * 3] * 2
+    assert read(b"gram") == 3 and read(b"phase_hr") == 0
+    assert lib.jarq_profile_read(b"no such kernel", ctypes.byref(n), ctypes.byref(ms)) == -1
