@@ -6,13 +6,18 @@ off) from its host state: the whole hot path (once the target projection
 P = W H and its folded form; per iteration the Gram matrices, right-hand
 sides and joint scale solve, then the sweep, a product and a Babai step per
 block of two groups).  Inputs are seeded synthetic tensors resident in HBM; the
-working set per step (W, P and the folded P 64 MB each, the digit planes of
-H 336 MB) exceeds the 129 MB L2.
+working set per step (W 64 MB, P and the folded P 128 MB each, digit planes
+448 MB) exceeds the 129 MB L2.
 
 ``value`` is weights refined per second over all ranks; ``e2e`` is the same
 metric through the C ABI with host buffers (host-to-device and back inside
 the timed region).  ``--impl reference`` times the float64 oracle (the
 reference arm of this build) on the host cores.
+
+The line printed is short (below 2600 characters, so that it survives a log
+that keeps the end of a program's output): the main workload in full, of the
+other workloads and legs the figures.  ``--details FILE`` writes the whole
+record, with every kernel's roofline.
 """
 from __future__ import annotations
 
@@ -88,6 +93,8 @@ def parse_args():
                          "extra legs, end-to-end pass or CPU baseline (profiling runs)")
     ap.add_argument("--tokens", type=int, default=None,
                     help="calibration tokens of the Hessian workload (default: 128 x 2048)")
+    ap.add_argument("--details", default=None, metavar="FILE",
+                    help="write the whole record (rooflines and kernel times of every workload) here")
     ap.add_argument("--cpu-seconds", type=float, default=12.0,
                     help="target CPU time of the oracle baseline sample")
     return ap.parse_args()
@@ -470,10 +477,51 @@ def run_ours(args, rank, world):
                                           f"{t:.1f} s"}
     hess.close()
     if rank == 0:
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as fh:
+                json.dump(line, fh)
+        print(json.dumps(short_line(line)))
     if dist:
         dist.destroy_process_group()
     return 0
+
+
+def _digits(x):
+    """Floats of a nested record to five significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.5g}")
+    if isinstance(x, dict):
+        return {k: _digits(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_digits(v) for v in x]
+    return x
+
+
+def short_line(full):
+    """The printed line: the whole record without the parts that only explain
+    it, kernels as [launches, us a launch] and the other legs reduced to their
+    figures."""
+    drop = ("roofline_all", "kernel_timing", "kernels", "postpass", "configs", "hessian", "early_stop",
+            "mu_target", "ablations")
+    out = {k: v for k, v in full.items() if k not in drop}
+    extra = {}
+    if "kernels" in full:
+        extra["kernels"] = {k: [v["launches"], v["avg_us"]] for k, v in full["kernels"].items()}
+    if "postpass" in full:
+        extra["postpass_ms"] = {k: v["ms"] for k, v in full["postpass"].items()}
+    if "configs" in full:
+        extra["configs_s"] = {k: v.get("s_per_layer", v.get("s_per_block")) for k, v in full["configs"].items()}
+    if "hessian" in full:
+        h = full["hessian"]
+        extra["hessian"] = {"kernel_ms": h["kernel_ms"], "tokens_per_s": h["tokens_per_s"],
+                            "frac": h["roofline"]["frac"]}
+    pick = {"early_stop": ("s_per_layer", "iters_mean"), "mu_target": ("ms_per_layer_mu_0.5", "ms_per_layer_mu_1.0"),
+            "ablations": ("gap_independent_pct_median", "gap_coordinate_pct_median", "probe_ms_per_group",
+                          "joint_over_fixed_heldout_pct_median")}
+    for leg, keys in pick.items():
+        if leg in full:
+            extra[leg] = {k: full[leg][k] for k in keys}
+    return {**out, **_digits(extra)}
 
 
 def flush_l2(buf):
@@ -643,8 +691,8 @@ def hessian_leg(args, jarq, dev, standalone=False):
     ``jarq_accumulate_hessian`` call: the step before refinement.  Timed by
     the library's CUDA event pair on its stream (kernel) and around the call
     (which synchronises).  Algorithmic work counts each unordered feature
-    pair once: n d (d + 1) flops; the kernel issues whole 128 x 256 tiles
-    meeting the upper triangle."""
+    pair once: n d (d + 1) flops; the kernel issues whole 256 x 256 tiles
+    on and above the diagonal."""
     import torch
     from synth import ACT_CONFIGS, config_activations
     X = config_activations(HESSIAN_WORKLOAD, device=dev, tokens=args.tokens)
@@ -665,9 +713,8 @@ def hessian_leg(args, jarq, dev, standalone=False):
     k_ms = tot / max(1, nl)
     pk, peak_kind = peaks()
     work = float(n) * d * (d + 1)
-    rt, ct = (d + 127) // 128, (d + 255) // 256
-    tiles = sum(min(rt, 2 * cj + 2) for cj in range(ct))
-    issued = tiles * 2.0 * 128 * 256 * (-(-n // 64) * 64)
+    ct = (d + 255) // 256
+    issued = ct * (ct + 1) // 2 * 2.0 * 256 * 256 * (-(-n // 64) * 64)
     achieved = work / (k_ms / 1e3) / 1e12
     peak = pk["bf16_tflops"]
     out = {"workload": HESSIAN_WORKLOAD, "tokens": n, "din": d, "call_ms": call_ms,
@@ -790,9 +837,9 @@ def early_stop_leg(args, jarq, dev, lay, hess, fixed_ms):
     """The main layer with the early stop of App. E (Eq. strict_stopping,
     default thresholds) against the fixed K-iteration run of the main line:
     seconds per layer, the rows' last solved iteration and, per iteration k,
-    the share of rows and of 128-row tiles still solved at k (a tile whose
-    rows have all stopped skips its phase products; stopped rows skip the
-    Babai step and the Gram)."""
+    the share of rows and of the pairs of row tiles (256 rows) still solved at
+    k (a pair whose rows have all stopped skips its products and Gram blocks;
+    stopped rows skip the scale solve and the Babai step)."""
     import torch
     opts = jarq.default_options(max_iters=lay.K, early_stop=1)
     S = lay.S0.clone()
@@ -820,10 +867,10 @@ def early_stop_leg(args, jarq, dev, lay, hess, fixed_ms):
     Q.copy_(lay.Q0)
     st = jarq.refine(hess, lay.W, S, Q, lay.Z, lay.bits, options=opts, collect_stats=True)
     it = st.iters.cpu().numpy().astype(np.int64)
-    ntile = (len(it) + 127) // 128
-    tile_max = np.zeros(ntile * 128, np.int64)
+    ntile = (len(it) + 255) // 256
+    tile_max = np.zeros(ntile * 256, np.int64)
     tile_max[:len(it)] = it
-    tile_max = tile_max.reshape(ntile, 128).max(axis=1)
+    tile_max = tile_max.reshape(ntile, 256).max(axis=1)
     K = lay.K
     return {"K": K, "tau_rel": opts.tau_rel, "tau_abs": opts.tau_abs, "steps": steps,
             "s_per_layer": ms / 1e3, "weights_per_s": lay.din * lay.dout / (ms / 1e3),

@@ -99,3 +99,46 @@ def test_config_names_the_workload_and_its_l2_note():
     # W 64 MB, P and the folded P 128 MB each, digit planes 448 MB: all larger than L2
     assert "W 64 MB" in c["l2"] and "128 MB" in c["l2"] and "448 MB" in c["l2"]
     assert bench.config_dict(Q_PROJ, note="x")["note"] == "x"
+
+
+def test_printed_line_is_short_and_keeps_the_contract():
+    """A record as long as a full run's, printed in fewer than 2600 characters
+    with every key of the contract unrounded."""
+    import json
+    x = 1.0 / 3
+    kernels = {k: {"launches": 7160, "total_ms": 1e3 * x, "avg_us": 1e4 * x, "share": x}
+               for k in ("validate", "residual", "init_rows", "gram", "scale_solve", "slice_rows", "proj", "whw",
+                         "rhs", "ptilde", "sweep_product", "sweep_babai")}
+    roof = bench.roofline_entry("sweep_product", {"launches": 10, "total_ms": x}, Q_PROJ,
+                                {"bf16_tflops_sustained": 1736.3}, "measured")
+    cfg = {"din": 4096, "dout": 14336, "s_per_layer": x, "weights_per_s": 1e9 * x, "launches_per_step": 358.0,
+           "roofline": roof, "roofline_all": {k: roof for k in kernels}, "kernels": kernels}
+    full = {"metric": bench.METRIC, "value": 1e9 * x, "unit": bench.UNIT, "n_gpus": 1, "steps": 20, "warmup": 5,
+            "ms_per_step": 40 * x, "s_per_layer": x, "higher_is_better": True, "scaling": "weak",
+            "vs_baseline": None, "dtype": bench.DTYPE, "data": "synthetic (seeded Llama-2-7B-shaped layer, RTN host)",
+            "config": bench.config_dict(Q_PROJ), "roofline": roof, "roofline_all": {k: roof for k in kernels},
+            "gpu_launches": 7160, "kernel_timing": "x" * 130, "launches_per_step": 358.0,
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "samples": 12, "reasons": ["sw_power_cap"]},
+            "kernels": kernels,
+            "postpass": {k: {"ms": x, "bytes": 51380224, "GB_s": 1e3 * x, "hbm_frac": x, "note": "y" * 50}
+                         for k in ("dequantize_f16", "pack_codes", "canonicalize")},
+            "configs": {k: cfg for k in ("tiny_256x256_g64_w3", "llama2_7b_down_proj_4096x11008_g128_w4",
+                                         "llama3_8b_gate_proj_14336x4096_g128_w3", "llama2_7b_block")},
+            "hessian": {"kernel_ms": 10 * x, "tokens_per_s": 1e8 * x, "roofline": roof, "cpu_baseline": {}},
+            "early_stop": {"s_per_layer": x, "iters_mean": 28 * x, "rows_solved_at_k": [x] * 10},
+            "mu_target": {"ms_per_layer_mu_0.5": 50 * x, "ms_per_layer_mu_1.0": 40 * x, "workload": "z"},
+            "ablations": {k: 100 * x for k in ("gap_independent_pct_median", "gap_coordinate_pct_median",
+                                               "probe_ms_per_group", "babai_after_single_code_pct",
+                                               "joint_over_fixed_heldout_pct_median", "rows_improved_by_joint")},
+            "e2e": {"value": 1e9 * x, "unit": bench.UNIT, "h2d_bytes_per_step": 84934656,
+                    "d2h_bytes_per_step": 17301504, "ms_per_step": 40 * x},
+            "cpu_baseline": {"value": 1e5 * x, "unit": bench.UNIT, "cores": 16, "kind": "oracle",
+                             "sample": "94 of 4096 rows, K=10, full din, 15.5 s"}}
+    short = bench.short_line(full)
+    text = json.dumps(short)
+    assert len(text) < 2600 and "\n" not in text, len(text)
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "roofline", "gpu_launches", "clocks", "e2e",
+                "cpu_baseline"):
+        assert short[key] == full[key], key
+    assert short["configs_s"]["llama2_7b_block"] == 0.33333 and short["kernels"]["gram"] == [7160, 3333.3]
