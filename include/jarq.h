@@ -188,7 +188,7 @@ jarq_status jarq_objective(jarq_hessian *h, const float *W, const float *S, cons
  * (H r_j)_i of Sec. 3.3.2, Eq. conditional_residual, for every group at
  * once.  It is computed by the split-precision tensor-core kernel behind
  * jarq_objective (the refinement's sweep forms its Babai targets with the
- * exact folded phase product instead), and it exists so that tests can
+ * exact product of the folded rows instead), and it exists so that tests can
  * compare that contraction element by element with a reference.  Same
  * layouts and checks as jarq_refine_layer. */
 jarq_status jarq_residual_product(jarq_hessian *h, const float *W, const float *S,

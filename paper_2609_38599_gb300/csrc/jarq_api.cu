@@ -490,8 +490,8 @@ jarq_status jarq_prepare_hessian(const float *H, int din, int group_size, float 
         layout_hessian(m, h);
         // the folded rows R_i^{-T} H[grp i, :] as float pairs, only needed to
         // form their digits, and the inverse factors as float pairs, only
-        // needed to form those: in the memory of H's own digits, which are
-        // formed last
+        // needed to form those: 8 d^2 + 8 d g bytes in the 20 d_pad^2 of H's own
+        // digits (Hdig8 and behind it Hdig10), which are formed last
         float *const Ht_hi = reinterpret_cast<float *>(h->Hdig8), *const Ht_lo = Ht_hi + dd;
         float2 *const RinvF = reinterpret_cast<float2 *>(Ht_lo + dd);
         // columns beyond din are read as zeros by the products
@@ -657,7 +657,7 @@ jarq_status jarq_multicode_probe(jarq_hessian *h, const float *W, const float *S
     RUN("slice_rows", 1, launch_slice_rows(la.W, w.wdig, w.wexp, p, d, h->d_pad, w.p_pad, g, st));
     RUN("proj", 1, launch_tc_proj(w.mapWd, h->mapD8, w.Phi, w.Plo, w.wexp, h->expo, p, w.p_pad, d,
                                   h->d_pad, g, h->dstatus, st));
-    // T = sum_h s_h H_ih c_h: the phase product with H's own digits
+    // T = sum_h s_h H_ih c_h: the sweep's product with H's own digits
     RUN("sweep_product", 1, launch_tc_target(w.mapC, h->mapD10, w.t_hi, w.t_lo, la.S, h->expo, nullptr, p,
                                       w.p_pad, h->d_pad, g, G, group, 1, 0, nsplit, (1 << bits) - 1, h->dstatus, st,
                                       false));
@@ -808,8 +808,8 @@ jarq_status refine_impl(jarq_hessian *h, const float *W, float *S, uint8_t *Q, c
         RUN("scale_solve", 1, launch_scale_solve(w.gram, w.rhs, w.wHw, la.S, w.L_prev, L_out,
                                                  w.active, w.iters, w.ridge, w.rstat, h->dstatus,
                                                  p, d, g, k, false, o, st, chained));
-        // The phase product reads the active flags only with the early stop
-        // on (to skip tiles whose rows all stopped); a row marked numerical
+        // The product reads the active flags only with the early stop on (to
+        // skip pairs of tiles whose rows all stopped); a row marked numerical
         // by the scale solve is skipped by Babai, and its partials go unread.
         for (int i0 = 0; i0 < G; i0 += nblk) {
             const int nb = G - i0 < nblk ? G - i0 : nblk;

@@ -24,12 +24,12 @@ enum : int {
 
 constexpr int kMaxGroups = 128;    // largest supported G for the scale solve
 constexpr int kMaxGroupSize = 128; // the larger of the two group sizes
-constexpr int kMaxSplit = 16;      // largest split-K factor of the phase product
+constexpr int kMaxSplit = 16;      // largest split-K factor of the sweep's product
 
 // Groups of one block of the sweep for group size g: 256 columns.  The Babai
 // kernel holds the factors of two groups and the blocks Ht_i'i of one group i
 // in shared memory, which for g = 128 leaves room for one such block.  Two
-// groups of 128 in one launch take 36.7 us of product and 27.6 us of Babai
+// groups of 128 in one launch take 32.8 us of product and 27.6 us of Babai
 // steps on 4096 x 4096; with a launch per group the start of each launch
 // (about 8 us of a product, 4 us of a Babai step) is paid twice.
 __host__ __device__ constexpr int sweep_block(int g) { return 256 / g; }
@@ -95,8 +95,8 @@ struct Workspace {
     float *r = nullptr;          // [p][d]  residual r = w - D_s (q - z)
     float2 *gram = nullptr;      // [p][G][G]  Gram matrices of the current codes (float pairs)
     double *rhs = nullptr;       // [p][G]  rhs_i = c_i^T P_i (also the scratch of grad)
-    float *t_hi = nullptr;       // [nsplit][p_pad][nb g]  split-K partials of the phase
-    float *t_lo = nullptr;       //   product of nb groups (double-float)
+    float *t_hi = nullptr;       // [nsplit][p_pad][nb g]  split-K partials of the
+    float *t_lo = nullptr;       //   product of a block's nb groups (double-float)
     __nv_bfloat16 *rplanes = nullptr;  // [3][p_pad][d_pad] bf16 split of r
     __half *cplane = nullptr;          // [p_pad][d_pad] codes c = q - z
     CUtensorMap mapR;            // tensor map of rplanes, 128 x 64 boxes

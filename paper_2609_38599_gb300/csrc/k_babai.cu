@@ -2,7 +2,7 @@
 // sweep, every active row (Sec. 3.3.2, Eqs. conditional_residual, group_bils,
 // group_qr, babai_update; App. E "Small scales").
 //
-// The sweep runs in blocks of a few groups (sweep_block).  The phase product
+// The sweep runs in blocks of a few groups (sweep_block).  The product
 // (k_tc_target.cu) has formed T_i = sum_h s_h R_i^{-T} H_ih c_h for every
 // group i of the block from the codes before the block; this kernel takes
 // each row through the block's groups in order.  A proposal that is accepted
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(32 * (kMaxWarps + 1), 1) babai_kernel(BabaiArg
             if (*abort_f) atomicOr(a.status, ST_TIMEOUT);
         }
     } else {
-        // The phase product (previous kernel) must be complete before its
+        // The block's product (previous kernel) must be complete before its
         // partials are read and before the codes it reads are rewritten.  The
         // next grid is released only after this wait: by then every grid before
         // this one has completed, so the next product may read the codes of the

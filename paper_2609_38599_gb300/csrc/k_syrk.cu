@@ -30,9 +30,9 @@
 // Each unordered pair {i, j} belongs to exactly one tile element with
 // col >= row, so every element of H is written exactly once.
 //
-// What bounds it: for many tokens the MMAs (d = 11008, 32768 tokens: 2.56 ms; 2.43
+// What bounds it: for many tokens the MMAs (d = 11008, 32768 tokens: 2.54 ms; 2.43
 // ms without the additions to H; the same flops at the 1.75 PFLOP/s that a long
-// run sustains take 2.3 ms), for few the additions to H (d = 4096, 2048 tokens: 61
+// run sustains take 2.3 ms), for few the additions to H (d = 4096, 2048 tokens: 58
 // us; 30 us without them).  One CTA per 128 x 256 tile, its ring reused to stage
 // the whole tile, took 2.87 ms and 72 us: 192 bytes of shared memory were written
 // and read per cycle of the MMAs, now 128.  Measured and not kept: tiles in

@@ -35,7 +35,7 @@
 // and operand reads 128 KB of shared-memory traffic.  Two accumulators keep MMA
 // and drain of consecutive groups overlapped, but a group's MMAs start only when
 // all 32 drain warps have read the accumulator two groups back.  Per launch of
-// two groups (256 columns, CUDA events): 33.1 us at K = 4096, 73 us at K = 11008;
+// two groups (256 columns, CUDA events): 32.8 us at K = 4096, 72 us at K = 11008;
 // with 17 operations in the drain (the integer part of D_1 split off by adding a
 // constant, the product's error formed apart) 36.7 and 82 us.  One CTA per tile
 // took 58.9 us at K = 4096 (192 KB of shared-memory traffic per group, and an
@@ -155,7 +155,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // own wait it reads nothing that this grid or the previous one writes.
     tc::pdl_launch_dependents();
     // a pair of tiles none of whose rows is still active (early stop, App. E)
-    // does no work: the Babai step reads the partials of active rows only
+    // does no work: the Babai step reads the partials of active rows only.
+    // Flags are optional in the later branch too: without the early stop the
+    // first block has none, nor has the multi-code probe's group 0, and reading
+    // them without the null check is a memory fault.
     const bool live = early ? jp < a.p
                             : __syncthreads_or(threadIdx.x < 256 && jp + (int)threadIdx.x < a.p &&
                                                (!a.active || a.active[jp + threadIdx.x] != 0));

@@ -157,11 +157,12 @@ def test_block_solve_group_edges(jarq, G):
 
 
 @pytest.mark.parametrize("early_stop", [False, True])
-def test_two_chain_sweep_parity(jarq, early_stop):
-    """10200 rows, din 256, g = 128: one phase product needs 80 x 2 = 160 CTAs,
-    more than one wave, so the sweep runs as two chains over the row halves
-    (5120 and 5080 rows, the second ending in a ragged tile).  Every row is
-    compared; with the early stop on, also the stopping iterations."""
+def test_many_row_tiles_parity(jarq, early_stop):
+    """10200 rows, din 256, g = 128: 40 pairs of row tiles (the last ends in a
+    ragged tile of 88 rows) by four column tiles, 160 pairs of CTAs where the
+    chip holds 76, so a product takes three waves; a Babai step's warps take
+    several rows each.  Every row is compared; with the early stop on, also the
+    stopping iterations."""
     K = 4 if early_stop else 2
     lay = small_layer(256, 10200, 128, 3, K=K, seed=77)
     prep, res = oracle_run(lay, K, early_stop)
