@@ -52,15 +52,15 @@ DTYPE = "f32 (integer-digit fp16/bf16 tensor-core products with exact partial su
 # valid while the kernel's source file is unchanged (first 12 hex digits of
 # its SHA-1); otherwise the bench reports null.
 TRAFFIC = {
-    "sweep_product": ("k_tc_target.cu", "0e24dd5faf51", 42.625e6 + 0.140e6),
-    "sweep_babai": ("k_babai.cu", "672bc1eb4b99", 19.160e6 + 0.0),
-    "gram": ("k_tc_gram.cu", "caa812655db4", 141.735e6 + 22.765e6),
-    "proj": ("k_tc_proj.cu", "18c811b3e91e", 1350.252e6 + 139.033e6),
-    "ptilde": ("k_tc_proj.cu", "18c811b3e91e", 134.258e6 + 143.617e6 + 288.578e6 + 97.168e6),
-    "rhs": ("k_tc_proj.cu", "18c811b3e91e", 151.551e6 + 0.272e6),
-    "whw": ("k_tc_proj.cu", "18c811b3e91e", 201.350e6 + 0.297e6),
-    "slice_rows": ("k_tc_proj.cu", "18c811b3e91e", 67.122e6 + 73.267e6),
-    "scale_solve": ("k_solve.cu", "c4ababeb8bae", 35.289e6 + 0.0),
+    "sweep_product": ("k_tc_target.cu", "7ff0bf5bd113", 42.495e6 + 0.005e6),
+    "sweep_babai": ("k_babai.cu", "1f2c6eaf91b0", 19.161e6 + 0.002e6),
+    "gram": ("k_tc_gram.cu", "040880dfa541", 140.947e6 + 22.452e6),
+    "proj": ("k_tc_proj.cu", "7359153c6634", 1336.274e6 + 137.113e6),
+    "ptilde": ("k_tc_proj.cu", "7359153c6634", 134.262e6 + 143.167e6 + 293.427e6 + 97.857e6),
+    "rhs": ("k_tc_proj.cu", "7359153c6634", 151.546e6 + 0.272e6),
+    "whw": ("k_tc_proj.cu", "7359153c6634", 201.340e6 + 0.220e6),
+    "slice_rows": ("k_tc_proj.cu", "7359153c6634", 67.128e6 + 72.345e6),
+    "scale_solve": ("k_solve.cu", "c4ababeb8bae", 35.323e6 + 0.0),
 }
 HESSIAN_WORKLOAD = "llama2_7b_attn_in_4096_n262144"
 

@@ -645,7 +645,7 @@ __device__ __forceinline__ void df_warp_sum(float &sh, float &sl) {
 // NT = g/32 consecutive entries of every group; NB groups are loaded and reduced
 // together.  What bounds it: memory (9 bytes an entry), at the loads that a row's
 // warp keeps in flight.  4096 x 4096: 37 us for g = 128 (NB = 8; 39 with 4), 47 us
-// for g = 64 (NB = 2; 52 and 57 with 4 and 8); 14336 x 4096 83 us, 4096 x 11008 96
+// for g = 64 (NB = 2; 52 and 57 with 4 and 8); 14336 x 4096 97 us, 4096 x 11008 86
 // us.  One group at a time: 42, 68, 102 and 98 us.
 constexpr int kRhsThreads = 64;
 
