@@ -26,7 +26,7 @@ struct Pending {
 };
 
 bool g_enabled = false;
-long long g_launches = 0;
+std::atomic<long long> g_launches{0};     // calls may overlap on several threads
 long long g_count[kNumNames] = {};
 double g_ms[kNumNames] = {};
 std::vector<Pending> g_pending;
@@ -54,7 +54,7 @@ int name_id(const char *name) {
 
 }  // namespace
 
-void count_launches(int n) { g_launches += n; }
+void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 ProfScope::ProfScope(const char *name, cudaStream_t s) : id_(-1), s_(s), a_(nullptr) {
     if (!g_enabled) return;
@@ -122,6 +122,6 @@ int jarq_profile_read(const char *kernel, long long *launches, double *total_ms)
     return 0;
 }
 
-long long jarq_launch_count(void) { return jarq::g_launches; }
+long long jarq_launch_count(void) { return jarq::g_launches.load(std::memory_order_relaxed); }
 
 }  // extern "C"

@@ -249,3 +249,24 @@ def test_profile_names_of_a_refinement(dev):
     assert [read(k) for k in (b"sweep_babai", b"babai")] == [3 * 3] * 2
     assert read(b"gram") == 3 and read(b"phase_hr") == 0
     assert lib.jarq_profile_read(b"no such kernel", ctypes.byref(n), ctypes.byref(ms)) == -1
+
+
+def test_launch_count_of_overlapping_calls(dev):
+    """Calls that may overlap on several host threads all count."""
+    import threading
+    lib = dev.lib
+    lib.jarq_launch_count.restype = ctypes.c_longlong
+    bufs = [(dev.buf(128), dev.buf(128)) for _ in range(8)]
+    n0, calls = lib.jarq_launch_count(), 6000
+    call = ctypes.CDLL(lib._name).jarq_pack_codes
+
+    def run(q, out):
+        for _ in range(calls):
+            call(q, 1, 128, 3, out, None)
+
+    threads = [threading.Thread(target=run, args=b) for b in bufs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert lib.jarq_launch_count() - n0 == 2 * calls * len(bufs)
